@@ -227,18 +227,28 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   const size_t J = (size_t)cfg->num_jobs, P = (size_t)cfg->population;
   int rc;
   if ((rc = dev_alloc(ctx, &ctx->d_cap, ((size_t)cfg->num_nodes + 7) & ~(size_t)7)) != SCHED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_kfit, (size_t)ctx->ND)) != SCHED_OK) return fail(rc);
+  if ((rc = dev_alloc(ctx, &ctx->d_kfit, (size_t)ctx->ND + ctx->KD)) != SCHED_OK) return fail(rc);
+  ctx->d_nmin = ctx->d_kfit + ctx->ND;
+  // fewest nodes (at least two) that K replicas fit on; n_max + 1: none
+  for (int K = 0, n = 2; K < ctx->KD; ++K) {
+    while (n < ctx->ND && kfit[n] < K) ++n;
+    kfit.push_back(n < ctx->ND ? n : ctx->ND);
+  }
   // (K, class) pairs that exist: class 0 (one node) needs K <= largest node; class 1 (several
-  // nodes) needs K >= 2 and K <= the min(K, n_max) largest nodes together
-  std::vector<int32_t> pairs;
+  // nodes) needs K >= 2 and K <= the min(K, n_max) largest nodes together; class 2 (several racks)
+  // is tabulated where class 1 is
+  std::vector<int32_t> pairs, rack_pairs;
   for (int K = 1; K <= cfg->k_max; ++K) {
-    if (K <= kfit[1]) pairs.push_back(K * 2);
-    if (cfg->n_max >= 2 && K >= 2 && K <= kfit[std::min(K, cfg->n_max)]) pairs.push_back(K * 2 + 1);
+    if (K <= kfit[1]) pairs.push_back(K * 4);
+    if (cfg->n_max >= 2 && K >= 2 && K <= kfit[std::min(K, cfg->n_max)]) {
+      pairs.push_back(K * 4 + 1);
+      rack_pairs.push_back(K * 4 + 2);
+    }
   }
   ctx->num_pairs = (int)pairs.size();
+  ctx->num_rack_pairs = (int)rack_pairs.size();
+  pairs.insert(pairs.end(), rack_pairs.begin(), rack_pairs.end());
   if ((rc = dev_alloc(ctx, &ctx->d_pairs, pairs.size())) != SCHED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_gmax, J * ctx->KD * 2)) != SCHED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_amax, J * ctx->KD * 2)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_rank, P)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_order, P)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_pen, J)) != SCHED_OK) return fail(rc);
@@ -251,12 +261,10 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   e = cudaMemcpyAsync(ctx->d_cap, h_node_capacity, sizeof(int16_t) * cfg->num_nodes,
                       cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(ctx->d_kfit, kfit.data(), sizeof(int32_t) * ctx->ND, cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync(ctx->d_kfit, kfit.data(), sizeof(int32_t) * kfit.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess && !pairs.empty())
     e = cudaMemcpyAsync(ctx->d_pairs, pairs.data(), sizeof(int32_t) * pairs.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_gmax, 0, sizeof(float) * std::max<size_t>(J * ctx->KD * 2, 1), ctx->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_amax, 0xFF, sizeof(uint16_t) * std::max<size_t>(J * ctx->KD * 2, 1), ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);   // host vectors go out of scope
   if (e != cudaSuccess) {
     set_error(ctx, "sched_init: upload failed: %s", cudaGetErrorString(e));
@@ -289,12 +297,11 @@ int sched_fair_share(const int16_t *h_node_capacity, int32_t num_nodes, int32_t 
 int sched_destroy(sched_ctx *ctx) {
   if (!ctx) return SCHED_OK;
   cudaStreamSynchronize(ctx->stream);
-  void *ptrs[] = {ctx->d_cap, ctx->d_kfit, ctx->d_pairs, ctx->d_gmax, ctx->d_amax, ctx->d_rank, ctx->d_order,
+  void *ptrs[] = {ctx->d_cap, ctx->d_kfit, ctx->d_pairs, ctx->d_rank, ctx->d_order,
                   ctx->d_dflag, ctx->d_pen, ctx->d_partial, ctx->d_ticket, ctx->d_status,
                   ctx->d_popA, ctx->d_popB, ctx->d_fit_buf, ctx->d_tab_goodput, ctx->d_tab_speedup,
                   ctx->d_rf, ctx->d_best_idx, ctx->d_stage, ctx->d_stage_fit, ctx->d_colsum, ctx->d_summ, ctx->d_collist, ctx->d_colcount, ctx->d_rowticket, ctx->d_round, ctx->d_occcount, ctx->d_occlist,
-                  ctx->d_colelig, ctx->rs_pool, ctx->rs_rec, ctx->rs_ptr, ctx->rs_state, ctx->d_gmax_rack,
-                  ctx->d_amax_rack, ctx->d_rack, ctx->d_tab_speedup_rack};
+                  ctx->d_colelig, ctx->rs_pool, ctx->rs_rec, ctx->rs_ptr, ctx->rs_state, ctx->d_rack, ctx->d_tab_speedup_rack};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
@@ -386,7 +393,7 @@ int build_speedup_table_rack(sched_ctx *ctx, const sched_jobs *d_jobs, const flo
   if (rc != SCHED_OK) return rc;
   REQUIRE(ctx, d_alpha_rack && d_beta_rack && d_speedup, SCHED_ERR_INVALID_ARG,
           "build_speedup_table_rack: d_alpha_rack, d_beta_rack and d_speedup must be non-NULL");
-  return launch_speedup_table_rack(ctx, d_jobs, d_alpha_rack, d_beta_rack, d_goodput, d_speedup, d_argmax);
+  return launch_speedup_table(ctx, d_jobs, nullptr, nullptr, nullptr, d_alpha_rack, d_beta_rack, d_goodput, d_speedup, d_argmax);
 }
 
 int eval_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
@@ -576,16 +583,14 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
                       int16_t *d_best, float *d_best_fitness) {
   int rc;
   const bool penalise = d_cur && d_jobs->age_sec && d_jobs->num_restarts;
-  if ((rc = launch_speedup_table(ctx, d_jobs, ctx->d_tab_goodput, ctx->d_tab_speedup, nullptr)) != SCHED_OK) return rc;
   // Rack-level locality: a second table for allocations that span racks; the round then runs on
   // dense matrices with the fitness read from them (the row summaries carry no rack count).
   const bool racks = ctx->d_rack != nullptr;
-  if (racks) {
-    const float *ar = ctx->d_alpha_rack ? ctx->d_alpha_rack : d_jobs->alpha_node;
-    const float *br = ctx->d_beta_rack ? ctx->d_beta_rack : d_jobs->beta_node;
-    if ((rc = launch_speedup_table_rack(ctx, d_jobs, ar, br, nullptr, ctx->d_tab_speedup_rack, nullptr)) != SCHED_OK)
-      return rc;
-  }
+  const float *ar = ctx->d_alpha_rack ? ctx->d_alpha_rack : d_jobs->alpha_node;
+  const float *br = ctx->d_beta_rack ? ctx->d_beta_rack : d_jobs->beta_node;
+  if ((rc = launch_speedup_table(ctx, d_jobs, ctx->d_tab_goodput, ctx->d_tab_speedup, nullptr, ar, br, nullptr,
+                                 racks ? ctx->d_tab_speedup_rack : nullptr, nullptr)) != SCHED_OK)
+    return rc;
   if (penalise && (rc = launch_realloc_factor(ctx, d_jobs, ctx->d_rf)) != SCHED_OK) return rc;
   const float *rf = penalise ? ctx->d_rf : nullptr;
   int16_t *pa = ctx->d_popA, *pb = ctx->d_popB;

@@ -50,12 +50,10 @@ struct sched_ctx {
   // device scratch owned by the context
   int16_t *d_cap;        // [num_nodes]
   int32_t *d_kfit;       // [ND] replicas that fit on the N largest nodes
-  int32_t *d_pairs;      // [num_pairs] K * 2 + class of every (K, class) that exists on this cluster
-  int num_pairs;
-  float *d_gmax;         // [J][KD][2] compact goodput maxima (class local / node)
-  uint16_t *d_amax;      // [J][KD][2]
-  float *d_gmax_rack;    // [J][KD][2] the same with the rack pair in the node pair's place (allocated on first use)
-  uint16_t *d_amax_rack;
+  int32_t *d_nmin;       // [KD] fewest nodes, two or more, that K replicas fit on (behind d_kfit)
+  int32_t *d_pairs;      // K * 4 + class of every (K, class) that exists on this cluster: the local and node
+                         // pairs, then the rack pairs
+  int num_pairs, num_rack_pairs;
   // rack-level locality (sched_set_racks): rack of every node, the third synchronisation pair
   int16_t *d_rack;       // [num_nodes] or NULL when the cluster is not split into racks
   const float *d_alpha_rack, *d_beta_rack;   // caller-owned device arrays [J]
@@ -278,10 +276,10 @@ __device__ __forceinline__ int nth_occupied(const int16_t *row, int num_nodes, u
 }
 
 // kernels' launchers (defined in table.cu / fitness.cu / ga.cu / rowstore.cu)
-int launch_speedup_table(sched_ctx *ctx, const sched_jobs *jobs, float *d_goodput, float *d_speedup,
-                         uint16_t *d_argmax);
-int launch_speedup_table_rack(sched_ctx *ctx, const sched_jobs *jobs, const float *d_alpha_rack,
-                              const float *d_beta_rack, float *d_goodput, float *d_speedup, uint16_t *d_argmax);
+int launch_speedup_table(sched_ctx *ctx, const sched_jobs *jobs, float *d_goodput, float *d_speedup, uint16_t *d_argmax,
+                         const float *d_alpha_rack = nullptr, const float *d_beta_rack = nullptr,
+                         float *d_goodput_rack = nullptr, float *d_speedup_rack = nullptr,
+                         uint16_t *d_argmax_rack = nullptr);
 int launch_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
                          const float *d_speedup_rack, const int16_t *d_cur, const float *d_rf,
                          const uint8_t *d_active, float p, float *d_fitness);

@@ -114,3 +114,27 @@ def test_single_job_and_custom_dims(gpu, oracle):
     gp_r, sp_r, am_r = oracle.build_speedup_table(jobs, cl.node_capacity, 20, 2, 8)
     assert gp.shape == (1, 21, 3)
     check_table(oracle, jobs, 8, gp, sp, am, gp_r, sp_r, am_r)
+
+
+@pytest.mark.parametrize("grid_m,grid_s,case", [(1, 8, ""), (3, 32, ""), (128, 9, "flat"), (129, 4, "flat"), (300, 3, ""),
+                                                (1030, 2, ""), (64, 8, "big"), (16, 200, "steps")])
+def test_screened_sweep_edges(gpu, oracle, grid_m, grid_s, case):
+    """Lengths of the grid around what a thread and a block can screen, jobs whose goodput hardly
+    depends on m (dozens of points within the screening margin), batch sizes beyond the screening's
+    exact quotients, many accumulation steps; slabs of a width that is no multiple of four."""
+    cl = synth.Cluster(np.array([8, 8, 4, 4, 2], np.int16))
+    jobs = synth.draw_jobs(5, 33, grid_m, max(grid_s, 8), cl.k_max)
+    if case == "flat":
+        jobs.alpha_grad[:] = 1e-6
+        jobs.alpha_local[:] = jobs.alpha_node[:] = 1e-7
+        jobs.beta_local[:] = jobs.beta_node[:] = 0.0
+        jobs.phi[:] = 1e6
+    if case == "big":
+        jobs.m0[:] = 1 << 20
+        jobs.m_max_total[:] = 12 << 20
+        jobs.m_max_gpu[:] = 1 << 18
+        jobs.m_grid = synth.make_m_grid(jobs.m_max_gpu, grid_m)
+    jobs = with_fair_share(jobs, cl)
+    gp, sp, am = _gpu_table(gpu, cl, jobs, grid_s, k_max=14, n_max=4)
+    gp_r, sp_r, am_r = oracle.build_speedup_table(jobs, cl.node_capacity, 14, 4, grid_s)
+    check_table(oracle, jobs, grid_s, gp, sp, am, gp_r, sp_r, am_r)
