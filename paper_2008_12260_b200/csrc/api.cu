@@ -77,9 +77,9 @@ int ensure_round_scratch(sched_ctx *ctx) {
   const size_t pop = (size_t)c.population * c.num_jobs * c.num_nodes;
   const size_t tab = (size_t)c.num_jobs * ctx->KD * ctx->ND;
   int rc;
-  // Large problems keep the round's population in the row store, whose pool starts with the
-  // dense initial population; if it cannot be allocated the round runs on dense matrices.
-  if (rowstore_eligible(ctx, nullptr) && !ctx->rs_off && !ctx->d_rack) {
+  // Most problems keep the round's population in the row store; if it cannot be allocated the round
+  // runs on dense matrices.
+  if (rowstore_eligible(ctx) && !ctx->rs_off) {
     if (rowstore_ensure(ctx) != SCHED_OK) ctx->rs_off = true;
   }
   if (!ctx->rs_ready) {
@@ -258,8 +258,10 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   if ((rc = dev_alloc(ctx, &ctx->d_round, 1)) != SCHED_OK) return fail(rc);
   ctx->graphs_enabled = true;
   ctx->rs_budget = 12ull << 30;
-  e = cudaMemcpyAsync(ctx->d_cap, h_node_capacity, sizeof(int16_t) * cfg->num_nodes,
-                      cudaMemcpyHostToDevice, ctx->stream);
+  e = cudaMemsetAsync(ctx->d_cap, 0, sizeof(int16_t) * (((size_t)cfg->num_nodes + 7) & ~(size_t)7), ctx->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ctx->d_cap, h_node_capacity, sizeof(int16_t) * cfg->num_nodes,
+                        cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ctx->d_kfit, kfit.data(), sizeof(int32_t) * kfit.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess && !pairs.empty())
@@ -583,8 +585,7 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
                       int16_t *d_best, float *d_best_fitness) {
   int rc;
   const bool penalise = d_cur && d_jobs->age_sec && d_jobs->num_restarts;
-  // Rack-level locality: a second table for allocations that span racks; the round then runs on
-  // dense matrices with the fitness read from them (the row summaries carry no rack count).
+  // Rack-level locality: a second table for allocations that span racks.
   const bool racks = ctx->d_rack != nullptr;
   const float *ar = ctx->d_alpha_rack ? ctx->d_alpha_rack : d_jobs->alpha_node;
   const float *br = ctx->d_beta_rack ? ctx->d_beta_rack : d_jobs->beta_node;
@@ -598,6 +599,7 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
   // from the current allocation); the in-round fitness reads those instead of the matrices
   // whenever the batched kernels were used, with bit-identical results.
   ctx->round_cur = rf ? d_cur : nullptr;
+  // (the row summaries carry no rack count: with racks, dense matrices are evaluated as a whole)
   ctx->round_summ = racks ? nullptr : ctx->d_summ;
   ctx->round_summ_in = nullptr;
   uint32_t *summ_other = ctx->d_summ + (size_t)ctx->cfg.population * ctx->cfg.num_jobs;

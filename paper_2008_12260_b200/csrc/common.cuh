@@ -311,7 +311,8 @@ int launch_penalty_prep(sched_ctx *ctx, const int16_t *d_cur, const float *d_rf)
 int ensure_colscratch(sched_ctx *ctx, size_t ints);
 void fitness_chunking(const sched_ctx *ctx, int32_t count, int &rows_per_block, int &chunks);
 // row store (rowstore.cu)
-bool rowstore_eligible(const sched_ctx *ctx, const int16_t *d_cur);
+bool rowstore_eligible(const sched_ctx *ctx);
+bool round_is_small(const sched_ctx *ctx);
 int rowstore_ensure(sched_ctx *ctx);
 int rowstore_build_current(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, const int16_t *d_seed,
                            const int16_t *d_cur, const float *d_pen);

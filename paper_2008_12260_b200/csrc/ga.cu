@@ -1779,6 +1779,12 @@ RowsArgs base_rows_args(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
 
 }  // namespace
 
+// Rounds whose generations generation_small_kernel runs: rows short enough for a thread each.
+bool round_is_small(const sched_ctx *ctx) {
+  const sched_config &c = ctx->cfg;
+  return c.num_jobs <= 256 && c.num_nodes <= SMALL_MAX_NODES && c.num_nodes % 8 == 0 && ctx->cap_max <= 2047 && !ctx->d_rack;
+}
+
 int launch_repair(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
                   int32_t count, uint32_t first_candidate, uint32_t generation) {
   int rc = ensure_dflag(ctx, count);

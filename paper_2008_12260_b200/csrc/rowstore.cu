@@ -33,8 +33,11 @@ constexpr int GEN_GROUPS = GEN_THREADS / 16;  // rows worked on at a time by a b
 constexpr int STORE_MAX_JOBS = 8192;          // job index must fit 13 bits of an occupant entry
 constexpr int COW_RESERVE = 16;               // slots a block takes up front for rows the column pass changes
 
+// rows of the pool are whole 16-byte pieces: entries beyond the cluster's last node are zero
+__host__ __device__ inline int row_stride(int NN) { return (NN + 7) & ~7; }
+
 struct StoreView {
-  int16_t *pool;
+  int16_t *pool;            // [slots][row_stride(nodes)]
   uint32_t *rec;
   unsigned long long half_cap;
   uint32_t zero_slot;       // also the largest valid slot
@@ -82,7 +85,7 @@ __device__ __forceinline__ Grp make_group(int lane, int NN) {
   Grp g;
   g.sub = lane & (GROUP - 1);
   g.mask = 0xFFFFu << (lane & GROUP);
-  g.row_vecs = NN >> 3;
+  g.row_vecs = (NN + 7) >> 3;
   return g;
 }
 
@@ -99,6 +102,19 @@ __device__ __forceinline__ uint4 load_piece(const int16_t *src, int v) {
     const uint32_t lo = (uint16_t)(CG ? __ldcg(src + 8 * v + 2 * k) : src[8 * v + 2 * k]);
     const uint32_t hi = (uint16_t)(CG ? __ldcg(src + 8 * v + 2 * k + 1) : src[8 * v + 2 * k + 1]);
     w[k] = lo | (hi << 16);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// the same of a row of NN entries in an array of the caller's (rows back to back: the last piece
+// of a row may be cut short, and reads as zeros from there on)
+__device__ __forceinline__ uint4 load_user_piece(const int16_t *src, int v, int NN) {
+  if (8 * v + 8 <= NN) return load_piece<false>(src, v);
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int n = 8 * v + 2 * k;
+    w[k] = (n < NN ? (uint32_t)(uint16_t)src[n] : 0u) | ((n + 1 < NN ? (uint32_t)(uint16_t)src[n + 1] : 0u) << 16);
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -154,14 +170,14 @@ struct CurPieces {
 
 // this lane's pieces of the current allocation's row (NULL: none), fetched ahead of their use
 template <int PPL>
-__device__ __forceinline__ CurPieces<PPL> cur_pieces(const Grp &g, const int16_t *cur_row) {
+__device__ __forceinline__ CurPieces<PPL> cur_pieces(const Grp &g, const int16_t *cur_row, int NN) {
   CurPieces<PPL> c;
   c.have = cur_row != nullptr;
 #pragma unroll
   for (int q = 0; q < PPL; ++q) {
     const int v = g.sub * PPL + q;
     c.x[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (c.have && v < g.row_vecs) c.x[q] = load_piece<false>(cur_row, v);
+    if (c.have && v < g.row_vecs) c.x[q] = load_user_piece(cur_row, v, NN);
   }
   return c;
 }
@@ -229,6 +245,43 @@ __device__ __forceinline__ uint32_t pack_summary(int K, int N, int ndiff) {
   return (uint32_t)K | ((uint32_t)N << 11) | ((uint32_t)ndiff << 22);
 }
 
+// Rack-level locality: a row whose occupied nodes lie in two racks or more takes its speedup from the
+// third table (rack NULL: the cluster is one rack).
+struct RackView {
+  const int16_t *rack;      // [NN]
+  const float *table;
+};
+
+// lowest and highest rack of the nodes seen so far
+struct RackSpan {
+  int lo, hi;
+  __device__ __forceinline__ void add(const RackView &v, int node) {
+    const int r = v.rack ? (int)__ldg(v.rack + node) : 0;
+    lo = min(lo, r);
+    hi = max(hi, r);
+  }
+  __device__ __forceinline__ const float *table(const RackView &v, const float *one_rack) const {
+    return lo < hi ? v.table : one_rack;
+  }
+};
+__device__ __forceinline__ RackSpan no_racks() { return {0x7fffffff, -1}; }
+
+// the span of a row held in shared memory, for its group
+template <int PPL>
+__device__ __forceinline__ RackSpan row_racks(const Grp &g, const RackView &v, const RowPieces<PPL> &p) {
+  RackSpan s = no_racks();
+  if (!v.rack) return s;
+#pragma unroll
+  for (int q = 0; q < PPL; ++q)
+    for (uint32_t m = p.mask[q]; m; m &= m - 1) s.add(v, 8 * (g.sub * PPL + q) + __ffs(m) - 1);
+#pragma unroll
+  for (int off = GROUP / 2; off >= 1; off >>= 1) {
+    s.lo = min(s.lo, __shfl_xor_sync(g.mask, s.lo, off, GROUP));
+    s.hi = max(s.hi, __shfl_xor_sync(g.mask, s.hi, off, GROUP));
+  }
+  return s;
+}
+
 // ---------------------------------------------------------------------------------------
 // Start of a round on the store: the current allocation's rows become slots 0 .. 2J - 1.
 // Slot j holds job j's row as an unperturbed child of the initial population has it (entries
@@ -246,6 +299,7 @@ struct BuildCurArgs {
   const int16_t *cap;
   const int32_t *k_cap;
   TermParams tp;
+  RackView racks;
   int J, NN, k_max, n_max;
 };
 
@@ -255,12 +309,13 @@ __global__ void __launch_bounds__(256) rowstore_build_cur_kernel(BuildCurArgs a)
   __shared__ uint32_t s_rec[16][REC_WORDS];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 4;
   const Grp g = make_group(lane, a.NN);
+  const int NS = row_stride(a.NN);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.state[0] = 2u * (unsigned int)a.J;
     a.state[1] = 0u;
   }
   if (blockIdx.x == 0) {    // the empty row: contents and record all zero
-    for (int n = threadIdx.x; n < a.NN; n += blockDim.x) a.st.pool[(size_t)a.st.zero_slot * a.NN + n] = 0;
+    for (int n = threadIdx.x; n < NS; n += blockDim.x) a.st.pool[(size_t)a.st.zero_slot * NS + n] = 0;
     if (threadIdx.x < REC_WORDS) a.st.rec[(size_t)a.st.zero_slot * REC_WORDS + threadIdx.x] = 0u;
   }
   for (int j = blockIdx.x * 16 + grp; j < a.J; j += gridDim.x * 16) {
@@ -270,7 +325,7 @@ __global__ void __launch_bounds__(256) rowstore_build_cur_kernel(BuildCurArgs a)
     for (int v = g.sub; v < g.row_vecs; v += GROUP) {
       uint4 x = make_uint4(0u, 0u, 0u, 0u);
       if (a.seed) {
-        x = load_piece<false>(a.seed + (size_t)j * a.NN, v);
+        x = load_user_piece(a.seed + (size_t)j * a.NN, v, a.NN);
         const uint4 cp = *((const uint4 *)a.cap + v);
         x.x = __vimin_s16x2_relu(x.x, __vimax_s16x2_relu(cp.x, 0u));
         x.y = __vimin_s16x2_relu(x.y, __vimax_s16x2_relu(cp.y, 0u));
@@ -279,20 +334,22 @@ __global__ void __launch_bounds__(256) rowstore_build_cur_kernel(BuildCurArgs a)
       }
       ((uint4 *)s_row[grp])[v] = x;
     }
-    const CurPieces<PPL> cur = cur_pieces<PPL>(g, a.cur ? a.cur + (size_t)j * a.NN : nullptr);
+    const CurPieces<PPL> cur = cur_pieces<PPL>(g, a.cur ? a.cur + (size_t)j * a.NN : nullptr, a.NN);
     __syncwarp(g.mask);
     const int kc = max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max));
     for (int pass = 0; pass < 2; ++pass) {              // before the row caps (slot J + j), after them (slot j)
       int K, N, nd;
-      summarise_row<PPL>(g, s_row[grp], cur, K, N, nd, s_rec[grp]);
+      const RowPieces<PPL> p = summarise_row<PPL>(g, s_row[grp], cur, K, N, nd, s_rec[grp]);
+      TermParams tp = a.tp;
+      tp.table = row_racks<PPL>(g, a.racks, p).table(a.racks, a.tp.table);
       const size_t slot = pass == 0 ? (size_t)a.J + j : (size_t)j;
       if (g.sub == 0) {
         // (before the row caps K may exceed its field: the row is only a perturbation's source then,
         // and that path adds the entries up itself)
         s_rec[grp][REC_SUMM] = pack_summary(min(K, 2047), N, nd);
-        s_rec[grp][REC_TERM] = __float_as_uint(fitness_term(a.tp, j, K, N, nd != 0));
+        s_rec[grp][REC_TERM] = __float_as_uint(fitness_term(tp, j, K, N, nd != 0));
       }
-      if (N > REC_ENTRIES) store_row(g, a.st.pool + slot * a.NN, s_row[grp]);
+      if (N > REC_ENTRIES) store_row(g, a.st.pool + slot * NS, s_row[grp]);
       __syncwarp(g.mask);
       if (g.sub < REC_WORDS) a.st.rec[slot * REC_WORDS + g.sub] = s_rec[grp][g.sub];
       __syncwarp(g.mask);
@@ -359,7 +416,7 @@ __global__ void __launch_bounds__(256) rowstore_compact_kernel(CompactArgs a) {
     atomicAdd(a.moves, 1u);
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int row_vecs = a.NN >> 3;
+  const int NS = row_stride(a.NN), row_vecs = NS >> 3;
   for (unsigned long long r = (unsigned long long)blockIdx.x * 8 + warp; r < rows; r += (unsigned long long)gridDim.x * 8) {
     const uint32_t slot = a.ptr[r];
     if (slot == a.st.zero_slot) continue;
@@ -367,8 +424,8 @@ __global__ void __launch_bounds__(256) rowstore_compact_kernel(CompactArgs a) {
     if (!sched_index_ok(a.st.status, slot < a.st.zero_slot && dst < a.st.zero_slot, SCHED_CHK_SLOT)) continue;
     const uint32_t w = (lane < REC_WORDS) ? a.st.rec[(size_t)slot * REC_WORDS + lane] : 0u;
     if (__shfl_sync(0xffffffffu, w, 0) == REC_OVERFLOW) {   // the record does not hold the row: its contents move too
-      const uint4 *s4 = (const uint4 *)(a.st.pool + (size_t)slot * a.NN);
-      uint4 *d4 = (uint4 *)(a.st.pool + dst * a.NN);
+      const uint4 *s4 = (const uint4 *)(a.st.pool + (size_t)slot * NS);
+      uint4 *d4 = (uint4 *)(a.st.pool + dst * NS);
       for (int v = lane; v < row_vecs; v += 32) d4[v] = s4[v];
     }
     if (lane < REC_WORDS) a.st.rec[dst * REC_WORDS + lane] = w;
@@ -385,8 +442,8 @@ rowstore_gather_kernel(StoreView st, const uint32_t *__restrict__ ptr, int first
                        const int32_t *__restrict__ index, int J, int NN, int16_t *__restrict__ out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long first = (long long)(index ? *index : first_candidate) * J;
-  const int row_vecs = NN >> 3;
-  const bool aligned = ((uintptr_t)out & 15) == 0;
+  const int NS = row_stride(NN), row_vecs = NS >> 3;
+  const bool aligned = ((uintptr_t)out & 15) == 0 && NS == NN;
   for (long long r = (long long)blockIdx.x * 8 + warp; r < rows; r += (long long)gridDim.x * 8) {
     uint32_t slot = ptr[first + r];
     if (!sched_index_ok(st.status, slot <= st.zero_slot, SCHED_CHK_SLOT)) slot = st.zero_slot;
@@ -395,11 +452,11 @@ rowstore_gather_kernel(StoreView st, const uint32_t *__restrict__ ptr, int first
     const uint4 hi = *((const uint4 *)(st.rec + (size_t)slot * REC_WORDS) + 1);
     if (lo.x == REC_OVERFLOW) {          // more occupied nodes than a record holds: the contents are in the pool
       if (aligned) {
-        const uint4 *s4 = (const uint4 *)(st.pool + (size_t)slot * NN);
+        const uint4 *s4 = (const uint4 *)(st.pool + (size_t)slot * NS);
         uint4 *d4 = (uint4 *)(out + (size_t)r * NN);
         for (int v = lane; v < row_vecs; v += 32) d4[v] = s4[v];
       } else {
-        for (int n = lane; n < NN; n += 32) out[(size_t)r * NN + n] = st.pool[(size_t)slot * NN + n];
+        for (int n = lane; n < NN; n += 32) out[(size_t)r * NN + n] = st.pool[(size_t)slot * NS + n];
       }
       continue;
     }
@@ -420,8 +477,9 @@ rowstore_gather_kernel(StoreView st, const uint32_t *__restrict__ ptr, int first
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          out[(size_t)r * NN + 8 * v + 2 * q] = (int16_t)(w[q] & 0xFFFFu);
-          out[(size_t)r * NN + 8 * v + 2 * q + 1] = (int16_t)(w[q] >> 16);
+          const int n = 8 * v + 2 * q;
+          if (n < NN) out[(size_t)r * NN + n] = (int16_t)(w[q] & 0xFFFFu);
+          if (n + 1 < NN) out[(size_t)r * NN + n + 1] = (int16_t)(w[q] >> 16);
         }
       }
     }
@@ -446,6 +504,7 @@ struct GenArgs {
   uint32_t init_src;        // initial population: slot of job 0's row before the row caps (perturbation source)
   RngKey key;
   TermParams tp;
+  RackView racks;
   int rows_per_chunk, chunks;   // the dense fitness kernel's chunking, reproduced for identical sums
   float *fitness_out;       // [P]
   int *status;
@@ -667,6 +726,15 @@ __device__ __forceinline__ void list_from_record(RowList &r, uint32_t *words, ui
   r.pn = 0;
 }
 
+__device__ __forceinline__ RackSpan list_racks(const RowList &r, const RackView &v) {
+  RackSpan s = no_racks();
+  if (v.rack) {
+#pragma unroll 1
+    for (int k = 0; k < r.n; ++k) s.add(v, ent_node(r.e[k]));
+  }
+  return s;
+}
+
 // a record written by one thread: two 16-byte stores
 __device__ __forceinline__ void store_record(uint32_t *rec, const RowList &r, float term, uint32_t word) {
   ((uint4 *)rec)[0] = make_uint4(r.e[0], r.e[1], r.e[2], r.e[3]);
@@ -686,7 +754,7 @@ __device__ __forceinline__ uint4 piece_with(uint4 x, int h, int val) {   // entr
 // the record does not hold the row (read from L2: the row may be new in this kernel)
 __device__ __noinline__ int row_value_at(const uint32_t *rec, const int16_t *pool, int NN, uint32_t slot, int nn) {
   const uint4 lo = __ldcg((const uint4 *)(rec + (size_t)slot * REC_WORDS));
-  if (lo.x == REC_OVERFLOW) return (int)__ldcg(pool + (size_t)slot * NN + nn);
+  if (lo.x == REC_OVERFLOW) return (int)__ldcg(pool + (size_t)slot * row_stride(NN) + nn);
   const uint4 hi = __ldcg((const uint4 *)(rec + (size_t)slot * REC_WORDS) + 1);
   const uint32_t e[REC_ENTRIES] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y};
   int v = 0;
@@ -756,8 +824,8 @@ __host__ __device__ inline GenSmem gen_smem_layout(int J, int NN) {
   TAKE(viol, (size_t)NN);
   TAKE(occ, (size_t)NN * OCC * 4);
   // a row per group of 16 lanes; at other times eight words per thread for the list form of a row
-  TAKE(rowbuf, (size_t)GEN_GROUPS * NN * 2 > (size_t)GEN_THREADS * LIST_WORDS * 4 ? (size_t)GEN_GROUPS * NN * 2
-                                                                                     : (size_t)GEN_THREADS * LIST_WORDS * 4);
+  const size_t group_rows = (size_t)GEN_GROUPS * row_stride(NN) * 2, thread_lists = (size_t)GEN_THREADS * LIST_WORDS * 4;
+  TAKE(rowbuf, group_rows > thread_lists ? group_rows : thread_lists);
   TAKE(mut, (size_t)J * 2);
   TAKE(ovf, (size_t)J * 2);
   TAKE(slow, (size_t)J * 2);
@@ -812,10 +880,11 @@ __device__ __forceinline__ int block_exscan(int v, int *s_red, int &total) {
   return before + incl - v;
 }
 
-template <int PPL, bool INIT>
+template <int PPL, bool INIT, bool RACKS>
 __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int J = a.J, NN = a.NN, P = a.P;
+  const RackView racks = RACKS ? a.racks : RackView{nullptr, nullptr};
+  const int J = a.J, NN = a.NN, NS = row_stride(NN), P = a.P;
   const GenSmem L = gen_smem_layout(J, NN);
   uint32_t *s_slot = (uint32_t *)(smem + L.slot);
   int *s_mark = (int *)(smem + L.mark);
@@ -1125,7 +1194,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
       if (!slow) {
         // K and N are final: the speedup, the penalty factor and the current allocation's values on
         // the nodes the perturbation touched are fetched together
-        const float x_sp = __ldg(a.tp.table + fitness_table_index(a.tp, j, rl.K, rl.n));
+        const float x_sp = __ldg(list_racks(rl, racks).table(racks, a.tp.table) + fitness_table_index(a.tp, j, rl.K, rl.n));
         const float x_pen = a.tp.pen ? __ldg(a.tp.pen + j) : 1.f;
         int cv0 = 0, cv1 = 0;
         if (a.cur && rl.pn > 0) cv0 = (int)__ldg(a.cur + (size_t)j * NN + rl.pnode0);
@@ -1154,7 +1223,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
   // ---- the few rows that need their contents: a group of 16 lanes each --------------------------
   const Grp g = make_group(lane, NN);
   const int grp = tid >> 4;
-  int16_t *row = s_rowbuf + (size_t)grp * NN;   // this group's row
+  int16_t *row = s_rowbuf + (size_t)grp * NS;   // this group's row
   uint32_t *recw = s_rec + grp * REC_WORDS;
   if (s_nslow | s_novf) {
     // perturbed rows whose record does not hold them (before or after): contents from the pool, or
@@ -1165,12 +1234,12 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
       const int j = (int)s_slow[i];
       const uint32_t old = s_slot[j];
       if (g.sub < REC_WORDS) recw[g.sub] = __ldcg(a.st.rec + (size_t)old * REC_WORDS + g.sub);
-      const CurPieces<PPL> cur = cur_pieces<PPL>(g, a.cur ? a.cur + (size_t)j * NN : nullptr);
+      const CurPieces<PPL> cur = cur_pieces<PPL>(g, a.cur ? a.cur + (size_t)j * NN : nullptr, NN);
       const int kc_in = a.k_cap ? a.k_cap[j] : a.k_max;
       __syncwarp(g.mask);
       const int rN = (int)((recw[REC_SUMM] >> 11) & 0x7FFu);
       if (recw[0] == REC_OVERFLOW) {
-        load_row<true>(g, row, a.st.pool + (size_t)old * NN);
+        load_row<true>(g, row, a.st.pool + (size_t)old * NS);
       } else {
         for (int v = g.sub; v < g.row_vecs; v += GROUP) ((uint4 *)row)[v] = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp(g.mask);
@@ -1219,9 +1288,10 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
       }
       const uint32_t slot = s_base_mut + (uint32_t)(s_mark[j] >> 4);
       float term = 0.f;
+      const float *table = row_racks<PPL>(g, racks, p).table(racks, a.tp.table);
       if (g.sub == 0)
-        term = row_term_of(a.tp.table, a.tp.pen, a.tp.k_max, a.tp.n_max, a.tp.mode, a.tp.p, a.tp.floor_, j, K, N, nd);
-      if (N > REC_ENTRIES) store_row(g, a.st.pool + (size_t)slot * NN, row);
+        term = row_term_of(table, a.tp.pen, a.tp.k_max, a.tp.n_max, a.tp.mode, a.tp.p, a.tp.floor_, j, K, N, nd);
+      if (N > REC_ENTRIES) store_row(g, a.st.pool + (size_t)slot * NS, row);
       const uint32_t word = pack_summary(K, N, nd);
       __syncwarp(g.mask);
       if (g.sub == 0) {
@@ -1240,7 +1310,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
 #pragma unroll 1
     for (int i = grp; i < s_novf; i += GEN_GROUPS) {
       const int j = (int)s_ovf[i];
-      load_row<true>(g, row, a.st.pool + (size_t)s_slot[j] * NN);
+      load_row<true>(g, row, a.st.pool + (size_t)s_slot[j] * NS);
       __syncwarp(g.mask);
       const RowPieces<PPL> p = row_pieces<PPL>(g, row);
       add_row_occupants(g, j, p, (s_mark[j] & MARK_DIST) != 0);
@@ -1390,7 +1460,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
         }
         rl.n = m;
         // K and N are final: speedup, penalty factor and the current allocation's values travel together
-        const float x_sp = __ldg(a.tp.table + fitness_table_index(a.tp, j, rl.K, rl.n));
+        const float x_sp = __ldg(list_racks(rl, racks).table(racks, a.tp.table) + fitness_table_index(a.tp, j, rl.K, rl.n));
         const float x_pen = a.tp.pen ? __ldg(a.tp.pen + j) : 1.f;
         int cv0 = 0, cv1 = 0;
         if (a.cur && rl.pn > 0) cv0 = (int)__ldg(a.cur + (size_t)j * NN + rl.pnode0);
@@ -1401,13 +1471,14 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
       } else {
         // contents only: pieces pass through this thread, patched on the way; the occupied nodes
         // that remain are listed, so that a row that now fits a record becomes one again
-        const int16_t *from = a.st.pool + (size_t)src * NN;
-        int16_t *to = a.st.pool + (size_t)dst * NN;
+        const int16_t *from = a.st.pool + (size_t)src * NS;
+        int16_t *to = a.st.pool + (size_t)dst * NS;
         int kept = 0;                   // occupied nodes that remain
+        RackSpan span = no_racks();
 #pragma unroll
         for (int k = 0; k <= LIST_MAX; ++k) rl.e[k] = 0u;
 #pragma unroll 1
-        for (int v = 0; v < (NN >> 3); ++v) {
+        for (int v = 0; v < (NS >> 3); ++v) {
           uint4 x = load_piece<true>(from, v);
           const uint4 x0 = x;
           uint32_t m = piece_mask(x);
@@ -1423,6 +1494,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
               x = piece_with(x, h, v_new);
             }
             if (v_new > 0) {
+              span.add(racks, node);
               if (kept < REC_ENTRIES) rl.e[kept] = (uint32_t)node | ((uint32_t)v_new << 12);
               ++kept;
             }
@@ -1434,7 +1506,8 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
 #pragma unroll
           for (int k = 1; k < LIST_MAX; ++k) rl.e[k] = 0u;
         }
-        term = row_term_of(a.tp.table, a.tp.pen, a.tp.k_max, a.tp.n_max, a.tp.mode, a.tp.p, a.tp.floor_, j, rl.K, rl.n, rl.nd);
+        term = row_term_of(span.table(racks, a.tp.table), a.tp.pen, a.tp.k_max, a.tp.n_max, a.tp.mode, a.tp.p, a.tp.floor_, j, rl.K,
+                           rl.n, rl.nd);
       }
       const uint32_t word = pack_summary(rl.K, rl.n, rl.nd);
       store_record(a.st.rec + (size_t)dst * REC_WORDS, rl, term, word);
@@ -1565,8 +1638,22 @@ __global__ void __launch_bounds__(GEN_THREADS, 4) generation_store_kernel(GenArg
 
 // pieces per lane of a row's group: 1, 2 or 4 (a lane's pieces beyond the row's end are empty)
 int store_pieces_per_lane(int num_nodes) {
-  const int need = ((num_nodes >> 3) + GROUP - 1) / GROUP;
+  const int need = ((row_stride(num_nodes) >> 3) + GROUP - 1) / GROUP;
   return need <= 1 ? 1 : need == 2 ? 2 : 4;
+}
+
+template <bool RACKS>
+void (*generation_kernel_of(int ppl, bool init))(GenArgs) {
+  if (init)
+    return ppl == 1 ? generation_store_kernel<1, true, RACKS> : ppl == 2 ? generation_store_kernel<2, true, RACKS>
+                                                                         : generation_store_kernel<4, true, RACKS>;
+  return ppl == 1 ? generation_store_kernel<1, false, RACKS> : ppl == 2 ? generation_store_kernel<2, false, RACKS>
+                                                                        : generation_store_kernel<4, false, RACKS>;
+}
+
+void (*generation_kernel(const sched_ctx *ctx, bool init))(GenArgs) {
+  const int ppl = store_pieces_per_lane(ctx->cfg.num_nodes);
+  return ctx->d_rack ? generation_kernel_of<true>(ppl, init) : generation_kernel_of<false>(ppl, init);
 }
 
 StoreView store_view(const sched_ctx *ctx) {
@@ -1594,7 +1681,7 @@ static unsigned long long store_base_rows(const sched_config &c) {
 static int store_units(const sched_config &c, unsigned long long budget) {
   const unsigned long long rows = store_base_rows(c);
   const unsigned long long worst = store_worst_case(c.population, c.num_jobs);
-  const unsigned long long row_bytes = (unsigned long long)c.num_nodes * 2 + REC_WORDS * 4;
+  const unsigned long long row_bytes = (unsigned long long)row_stride(c.num_nodes) * 2 + REC_WORDS * 4;
   const unsigned long long half_rows = budget / 2 / row_bytes;
   const unsigned long long index_rows = ((1ull << 32) - 2) / 2;      // slot indices are 32-bit
   const unsigned long long room = half_rows < index_rows ? half_rows : index_rows;
@@ -1603,13 +1690,12 @@ static int store_units(const sched_config &c, unsigned long long budget) {
   return (int)(units < 24 ? units : 24);
 }
 
-// The row store serves rounds whose candidates span several row batches of the dense
-// kernels (J > 256; smaller problems run a generation as one dense kernel already), with
-// rows of whole 16-byte vectors and sizes that fit the packed fields.
-bool rowstore_eligible(const sched_ctx *ctx, const int16_t *) {
+// The row store serves rounds of at most 512 nodes and sizes that fit the packed fields - except those
+// that one block per candidate runs faster on dense rows (round_is_small).
+bool rowstore_eligible(const sched_ctx *ctx) {
   const sched_config &c = ctx->cfg;
-  if (c.num_jobs <= 256 || c.num_jobs > STORE_MAX_JOBS) return false;
-  if (c.num_nodes % 8 != 0 || c.num_nodes > 512 || ctx->cap_max > 2047) return false;
+  if (round_is_small(ctx) || c.num_jobs > STORE_MAX_JOBS) return false;
+  if (c.num_nodes > 512 || ctx->cap_max > 2047) return false;
   if (c.k_max > 2047 || c.n_max > 2047) return false;
   if (gen_smem_layout(c.num_jobs, c.num_nodes).total > 200 * 1024) return false;
   // a half holds the population plus at least two generations' worst case; if that does not fit
@@ -1631,7 +1717,7 @@ int rowstore_ensure(sched_ctx *ctx) {
   ctx->rs_check_every = check;
   ctx->rs_half_cap = (size_t)(store_base_rows(c) + (unsigned long long)units * worst);
   const size_t slots = 2 * ctx->rs_half_cap + 1;
-  cudaError_t e = cudaMalloc((void **)&ctx->rs_pool, slots * c.num_nodes * sizeof(int16_t));
+  cudaError_t e = cudaMalloc((void **)&ctx->rs_pool, slots * row_stride(c.num_nodes) * sizeof(int16_t));
   if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->rs_rec, slots * REC_WORDS * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->rs_ptr, 2 * (size_t)rows * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->rs_state, 5 * sizeof(unsigned int));
@@ -1639,10 +1725,8 @@ int rowstore_ensure(sched_ctx *ctx) {
   if (e == cudaSuccess) {
     const size_t smem = gen_smem_layout(c.num_jobs, c.num_nodes).total;
     if (smem > 48 * 1024)
-    for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
-      void (*kernel)(GenArgs) = k == 0 ? generation_store_kernel<1, false> : k == 1 ? generation_store_kernel<2, false>
-                                : k == 2 ? generation_store_kernel<4, false> : k == 3 ? generation_store_kernel<1, true>
-                                : k == 4 ? generation_store_kernel<2, true> : generation_store_kernel<4, true>;
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      void (*kernel)(GenArgs) = generation_kernel(ctx, k != 0);
       e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
   }
@@ -1670,6 +1754,7 @@ int rowstore_build_current(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t
   a.tp.table = ctx->d_tab_speedup; a.tp.pen = d_pen; a.tp.active = d_active;
   a.tp.k_max = c.k_max; a.tp.n_max = c.n_max; a.tp.mode = fitness_mode(c.p); a.tp.p = c.p;
   a.tp.floor_ = c.speedup_floor;
+  a.racks = {ctx->d_rack, ctx->d_tab_speedup_rack};
   a.J = c.num_jobs; a.NN = c.num_nodes; a.k_max = c.k_max; a.n_max = c.n_max;
   {
     TimedLaunch tl_(ctx, KK_STORE_BUILD);
@@ -1740,6 +1825,7 @@ int rowstore_generation(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
   a.tp.table = ctx->d_tab_speedup; a.tp.pen = d_pen; a.tp.active = d_active;
   a.tp.k_max = c.k_max; a.tp.n_max = c.n_max; a.tp.mode = fitness_mode(c.p); a.tp.p = c.p;
   a.tp.floor_ = c.speedup_floor;
+  a.racks = {ctx->d_rack, ctx->d_tab_speedup_rack};
   fitness_chunking(ctx, c.population, a.rows_per_chunk, a.chunks);
   a.fitness_out = d_fitness_out;
   a.status = ctx->d_status;
@@ -1748,11 +1834,7 @@ int rowstore_generation(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
     TimedLaunch tl_(ctx, KK_GENSTORE);
     // launched so that it may start while the previous kernel of the stream still runs: the kernel
     // does its draws first and waits for that kernel before it reads anything it wrote
-    const int ppl = store_pieces_per_lane(c.num_nodes);
-    void (*kernel)(GenArgs) = init ? (ppl == 1 ? generation_store_kernel<1, true>
-                                      : ppl == 2 ? generation_store_kernel<2, true> : generation_store_kernel<4, true>)
-                                   : (ppl == 1 ? generation_store_kernel<1, false>
-                                      : ppl == 2 ? generation_store_kernel<2, false> : generation_store_kernel<4, false>);
+    void (*kernel)(GenArgs) = generation_kernel(ctx, init);
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)c.population);
     lc.blockDim = dim3(GEN_THREADS);
