@@ -40,8 +40,8 @@ extern "C" {
 #define SCHED_ERR_INVALID_ARG (-1) /* null pointer, negative size, misaligned buffer   */
 #define SCHED_ERR_BAD_CONFIG (-2)  /* a sched_config field outside its documented range */
 #define SCHED_ERR_CUDA (-3)        /* a CUDA runtime call failed                        */
-#define SCHED_ERR_TIMEOUT (-4)     /* a bounded device-side wait ran out (reserved: no
-                                      kernel of this version waits on another)          */
+#define SCHED_ERR_TIMEOUT (-4)     /* a bounded device-side wait ran out (a round's blocks wait
+                                      for one another's candidates)                     */
 #define SCHED_ERR_NOT_FINITE (-5)  /* a host input array holds a NaN or an infinity     */
 #define SCHED_ERR_TOO_LARGE (-6)   /* a size exceeds a documented fixed maximum         */
 
@@ -287,25 +287,25 @@ int ga_generation_shard(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t 
  * fitness, `generations` x (ga_generation, eval_fitness), then the best candidate of the
  * last population.  d_cur: int16 [J][num_nodes] or NULL.  d_best: int16 [J][num_nodes],
  * d_best_fitness: fp32 [1].  Population and table buffers are context scratch allocated
- * on the first call.  Problems with more than 256 jobs (rows of whole 16-byte pieces, at
- * most 512 nodes and 8192 jobs) keep the population of the round as shared rows - row
- * indices per candidate into a pool of rows, copy on write - instead of dense matrices;
- * the results are the same bit for bit, the scratch is larger (see sched_set_store_budget),
- * and a pool overflow
- * (not expected: the pool is compacted before it can run out) would be reported as device
- * status SCHED_ERR_TOO_LARGE by sched_sync_status.  If the pool cannot be allocated the
- * round runs on dense matrices. */
+ * on the first call.  The search runs as one launch whose blocks stay on the GPU and pass the
+ * population on among themselves (at most 512 nodes and 8192 jobs; a cooperative launch); every
+ * wait in it is bounded, and one that runs out is reported as device status SCHED_ERR_TIMEOUT by
+ * sched_sync_status.  With a budget too small for it (see sched_set_store_budget) the population is
+ * kept as shared rows - row indices per candidate into a pool of rows, copy on write; a pool overflow
+ * (not expected: the pool is compacted before it can run out) would be reported as device status
+ * SCHED_ERR_TOO_LARGE.  Where neither fits, the round runs on dense matrices.  The results are the
+ * same bit for bit. */
 int schedule_round(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_cur, uint32_t round,
                    int32_t generations, int16_t *d_best, float *d_best_fitness);
 
-/* Memory the shared-row pool of schedule_round may take (rows + records; default 12 GiB), to be
- * set before the first schedule_round of the context.  The pool is sized at twice (the
- * population + as many worst-case generations as the budget allows, at most 24); with less
- * room the live rows move between the halves more often (same results, more time), and when
- * not even two worst-case generations fit, rounds run on dense matrices.  The paper has no
- * counterpart: a deployment knob.  sched_store_moves: how often the rows have moved since the
- * context was made (waits for the stream; 0 when rounds run on dense matrices, -1 on a CUDA
- * error). */
+/* Memory the rows of schedule_round may take (default 12 GiB), to be set before the first
+ * schedule_round of the context.  The rows of four generations, with room for every row's contents,
+ * are kept where they fit half of it.  With less, the shared-row pool is sized at twice (the population +
+ * as many worst-case generations as the budget allows, at most 24); the less room, the more often the
+ * live rows move between the halves (same results, more time), and when not even two worst-case
+ * generations fit, rounds run on dense matrices.  The paper has no counterpart: a deployment knob.
+ * sched_store_moves: how often the pool's rows have moved since the context was made (waits for the
+ * stream; 0 when rounds do not use the pool, -1 on a CUDA error). */
 int sched_set_store_budget(sched_ctx *ctx, uint64_t bytes);
 int64_t sched_store_moves(sched_ctx *ctx);
 

@@ -77,6 +77,11 @@ int ensure_round_scratch(sched_ctx *ctx) {
   const size_t pop = (size_t)c.population * c.num_jobs * c.num_nodes;
   const size_t tab = (size_t)c.num_jobs * ctx->KD * ctx->ND;
   int rc;
+  if ((rc = round_flow_ensure(ctx)) != SCHED_OK) return rc;
+  if (ctx->fl_blocks) {
+    ctx->round_ready = true;
+    return SCHED_OK;
+  }
   // Most problems keep the round's population in the row store; if it cannot be allocated the round
   // runs on dense matrices.
   if (rowstore_eligible(ctx) && !ctx->rs_off) {
@@ -299,6 +304,10 @@ int sched_fair_share(const int16_t *h_node_capacity, int32_t num_nodes, int32_t 
 int sched_destroy(sched_ctx *ctx) {
   if (!ctx) return SCHED_OK;
   cudaStreamSynchronize(ctx->stream);
+  if (ctx->fl_arena) {      // these lie in the one allocation
+    ctx->d_tab_goodput = ctx->d_tab_speedup = ctx->d_tab_speedup_rack = ctx->d_fit_buf = nullptr;
+    cudaFree(ctx->fl_arena);
+  }
   void *ptrs[] = {ctx->d_cap, ctx->d_kfit, ctx->d_pairs, ctx->d_rank, ctx->d_order,
                   ctx->d_dflag, ctx->d_pen, ctx->d_partial, ctx->d_ticket, ctx->d_status,
                   ctx->d_popA, ctx->d_popB, ctx->d_fit_buf, ctx->d_tab_goodput, ctx->d_tab_speedup,
@@ -580,18 +589,22 @@ int ga_generation_shard(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t 
                            d_fitness_in, d_children, generation, first_child, num_children);
 }
 
+// The tables of a round; rack-level locality: a second one for allocations that span racks.
+static int launch_round_tables(sched_ctx *ctx, const sched_jobs *d_jobs) {
+  const float *ar = ctx->d_alpha_rack ? ctx->d_alpha_rack : d_jobs->alpha_node;
+  const float *br = ctx->d_beta_rack ? ctx->d_beta_rack : d_jobs->beta_node;
+  return launch_speedup_table(ctx, d_jobs, ctx->d_tab_goodput, ctx->d_tab_speedup, nullptr, ar, br, nullptr,
+                              ctx->d_rack ? ctx->d_tab_speedup_rack : nullptr, nullptr);
+}
+
 // Everything a round enqueues on the stream (the round number is already in d_round).
 static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_cur, int32_t generations,
                       int16_t *d_best, float *d_best_fitness) {
   int rc;
   const bool penalise = d_cur && d_jobs->age_sec && d_jobs->num_restarts;
-  // Rack-level locality: a second table for allocations that span racks.
   const bool racks = ctx->d_rack != nullptr;
-  const float *ar = ctx->d_alpha_rack ? ctx->d_alpha_rack : d_jobs->alpha_node;
-  const float *br = ctx->d_beta_rack ? ctx->d_beta_rack : d_jobs->beta_node;
-  if ((rc = launch_speedup_table(ctx, d_jobs, ctx->d_tab_goodput, ctx->d_tab_speedup, nullptr, ar, br, nullptr,
-                                 racks ? ctx->d_tab_speedup_rack : nullptr, nullptr)) != SCHED_OK)
-    return rc;
+  if ((rc = launch_round_tables(ctx, d_jobs)) != SCHED_OK) return rc;
+  if (ctx->fl_blocks) return launch_round_flow(ctx, d_jobs, d_cur, generations, d_best, d_best_fitness);
   if (penalise && (rc = launch_realloc_factor(ctx, d_jobs, ctx->d_rf)) != SCHED_OK) return rc;
   const float *rf = penalise ? ctx->d_rf : nullptr;
   int16_t *pa = ctx->d_popA, *pb = ctx->d_popB;
@@ -608,17 +621,9 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
   rc = SCHED_OK;
   if (rf) rc = launch_penalty_prep(ctx, d_cur, rf);
   ctx->pen_ready = (rc == SCHED_OK) && rf;
-  // problems whose candidates fit one block get row pass, column pass and fitness in one kernel
-  ctx->ff_on = !racks;
-  ctx->ff_table = ctx->d_tab_speedup;
-  ctx->ff_pen = rf ? ctx->d_pen : nullptr;
-  ctx->ff_active = d_jobs->active;
-  ctx->ff_p = ctx->cfg.p;
   // parents' fitness is read while children's is written: the two alternate between buffers
   float *fit_cur = ctx->d_fit_buf, *fit_next = ctx->d_fit_buf + ctx->cfg.population;
-  ctx->ff_out = fit_cur;
   auto fitness_of = [&](const int16_t *pop, float *out) {
-    if (ctx->fit_done) return (int)SCHED_OK;
     if (racks)
       return launch_fitness_racks(ctx, pop, ctx->cfg.population, ctx->d_tab_speedup, ctx->d_tab_speedup_rack, d_cur, rf,
                                   d_jobs->active, ctx->cfg.p, out);
@@ -658,7 +663,6 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
     if (rc == SCHED_OK) rc = fitness_of(pa, fit_cur);
   }
   for (int g = 0; g < generations && rc == SCHED_OK && !store; ++g) {
-    ctx->ff_out = fit_next;
     // children's summaries go to the other half; the parents' feed the unperturbed rows
     ctx->round_summ_in = ctx->summ_valid ? ctx->round_summ : nullptr;
     if (!racks) std::swap(ctx->round_summ, summ_other);
@@ -670,8 +674,6 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
   }
   ctx->d_fit = fit_cur;
   ctx->pen_ready = false;
-  ctx->ff_on = false;
-  ctx->fit_done = false;
   ctx->round_cur = nullptr;
   ctx->round_summ = nullptr;
   ctx->round_summ_in = nullptr;
@@ -769,7 +771,10 @@ int sched_get_population(sched_ctx *ctx, int16_t *d_pop_out, float *d_fitness_ou
   REQUIRE(nullptr, ctx, SCHED_ERR_INVALID_ARG, "sched_get_population: ctx is NULL");
   REQUIRE(ctx, ctx->d_pop_last, SCHED_ERR_INVALID_ARG, "sched_get_population: no round has run yet");
   const sched_config &c = ctx->cfg;
-  if (d_pop_out && ctx->rs_ptr_last) {
+  if (d_pop_out && ctx->fl_blocks) {
+    int rc = flow_gather(ctx, d_pop_out);
+    if (rc != SCHED_OK) return rc;
+  } else if (d_pop_out && ctx->rs_ptr_last) {
     int rc = rowstore_gather(ctx, ctx->rs_ptr_last, 0, c.population, nullptr, d_pop_out);
     if (rc != SCHED_OK) return rc;
   } else if (d_pop_out)

@@ -80,13 +80,6 @@ struct sched_ctx {
   const uint32_t *round_summ_in;  // summaries of the parent population (the other half), or NULL
   uint32_t *d_summ;          // [2][P][J]: parents' and children's summaries alternate
   bool summ_valid;           // the last row/column pass filled d_summ
-  // fitness fused into the generation kernel (single-batch problems): inputs set by
-  // schedule_round, fit_done reports that the last row/column pass also wrote the fitness
-  const float *ff_table, *ff_pen;
-  const uint8_t *ff_active;
-  float ff_p;
-  float *ff_out;
-  bool ff_on, fit_done;
   bool pen_ready;        // d_pen already holds this round's factors (set by schedule_round)
   int *d_status;         // device status word
   uint32_t *d_round;     // round number read by the operator kernels
@@ -115,6 +108,12 @@ struct sched_ctx {
   bool rs_ready;           // the buffers above exist
   bool rs_off;             // the store could not be allocated: rounds run on dense matrices
   const uint32_t *rs_ptr_last;  // indices of the last round's final population, or NULL when it is dense
+
+  // Rounds whose blocks stay on the GPU (round_flow.cu): one allocation, with the tables in it
+  void *fl_arena;
+  int fl_blocks;           // blocks of the launch, 0: rounds run on the other kernels
+  int fl_generations;      // generations of the last round
+  bool fl_ahead;           // blocks have threads that draw a step ahead
 
   // staging for the *_host entry points (allocated on first use)
   void *d_stage;         // job arrays + cur + best
@@ -310,9 +309,13 @@ int ensure_dflag(sched_ctx *ctx, int32_t count);
 int launch_penalty_prep(sched_ctx *ctx, const int16_t *d_cur, const float *d_rf);
 int ensure_colscratch(sched_ctx *ctx, size_t ints);
 void fitness_chunking(const sched_ctx *ctx, int32_t count, int &rows_per_block, int &chunks);
+// rounds whose blocks stay on the GPU (round_flow.cu)
+int round_flow_ensure(sched_ctx *ctx);
+int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_cur, int32_t generations, int16_t *d_best,
+                      float *d_best_fitness);
+int flow_gather(sched_ctx *ctx, int16_t *d_out);
 // row store (rowstore.cu)
 bool rowstore_eligible(const sched_ctx *ctx);
-bool round_is_small(const sched_ctx *ctx);
 int rowstore_ensure(sched_ctx *ctx);
 int rowstore_build_current(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, const int16_t *d_seed,
                            const int16_t *d_cur, const float *d_pen);

@@ -27,18 +27,21 @@ __device__ __forceinline__ size_t fitness_table_index(const TermParams &tp, int 
   return ((size_t)j * (tp.k_max + 1) + K) * (tp.n_max + 1) + N;
 }
 
+// The forms that the common exponents do not use, as calls: inlined at every use they would multiply the
+// kernels' code, and the small kernels' time is instruction fetch as much as anything.
+static __device__ __noinline__ float fitness_term_rare(int mode, float p, float x) {
+  return mode == MODE_GEO ? logf(x) : powf(x, p);
+}
+
 // x_j^p from the looked-up speedup x and the job's penalty factor (used when the row changed):
 // re-allocation penalty, floor, and the form that the mode sums (x, 1/x, ln x, sqrt x or x^p).
 __device__ __forceinline__ float fitness_term_with(const TermParams &tp, float x, float pen, bool changed) {
   if (tp.pen && changed) x *= pen;
   x = fmaxf(x, tp.floor_);
-  switch (tp.mode) {
-    case MODE_ARITH: return x;
-    case MODE_HARM: return 1.f / x;
-    case MODE_GEO: return logf(x);
-    case MODE_SQRT: return sqrtf(x);
-    default: return powf(x, tp.p);
-  }
+  if (tp.mode == MODE_HARM) return 1.f / x;
+  if (tp.mode == MODE_ARITH) return x;
+  if (tp.mode == MODE_SQRT) return sqrtf(x);
+  return fitness_term_rare(tp.mode, tp.p, x);
 }
 
 __device__ __forceinline__ float fitness_term_of(const TermParams &tp, int j, float x, bool changed) {
@@ -85,18 +88,25 @@ __device__ __forceinline__ void block_term_sum(const float *s_term, int nrows, i
 }
 
 // ((1/J) sum x^p)^(1/p) from the summed terms; 0 when no job is active.
+static __device__ __noinline__ double fitness_finalise_rare(int mode, float p, double mean) {
+  return mode == MODE_GEO ? exp(mean) : pow(mean, 1.0 / (double)p);
+}
+
 __device__ __forceinline__ float fitness_finalise(int mode, float p, double sum, double count) {
   if (count == 0.0) return 0.f;
   const double mean = sum / count;
-  double f;
-  switch (mode) {
-    case MODE_ARITH: f = mean; break;
-    case MODE_HARM: f = 1.0 / mean; break;
-    case MODE_GEO: f = exp(mean); break;
-    case MODE_SQRT: f = mean * mean; break;
-    default: f = pow(mean, 1.0 / (double)p); break;
-  }
-  return (float)f;
+  if (mode == MODE_HARM) return (float)(1.0 / mean);
+  if (mode == MODE_ARITH) return (float)mean;
+  if (mode == MODE_SQRT) return (float)(mean * mean);
+  return (float)fitness_finalise_rare(mode, p, mean);
+}
+
+// REALLOC_FACTOR(delta) = (T - R delta) / (T + delta), clamped to [0, 1] (Sec. 4.2)
+__device__ __forceinline__ float realloc_factor(float T, int restarts, float delta) {
+  const float R = (float)restarts;
+  float f = (T - R * delta) / (T + delta);
+  if (!(f >= 0.f)) f = 0.f;
+  return fminf(f, 1.f);
 }
 
 constexpr int FITNESS_MAX_ROWS_PER_BLOCK = 2048;

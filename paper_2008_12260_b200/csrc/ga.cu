@@ -3,14 +3,14 @@
 // avoidance (Sec. 4.2).  Integer work only; all randomness comes from the counter-based
 // stream, so every output is a pure function of the inputs.
 //
-// Three implementations of the same operators on dense matrices, chosen by shape:
+// Implementations of the same operators on dense matrices, chosen by shape:
 //  * rows_kernel + cols_kernel (+ rank_kernel): the general pair - a warp per (candidate, job)
 //    row through shared memory, then a thread per (candidate, node) column;
 //  * rows2_kernel + colrepair_kernel: rows of whole 16-byte vectors and at most 512 nodes -
 //    batched rows with fused column sums and occupant lists, a work list of violating nodes;
-//    for at most 256 jobs the row kernel also does the column pass and the fitness (FUSE);
-//  * generation_small_kernel: at most 256 jobs and 32 nodes inside a round - a thread per row.
-// Rounds of more than 256 jobs do not use dense matrices for their generations at all (rowstore.cu).
+//  * rows_stream_kernel + colrepair_kernel: the same without per-row summaries (entry points).
+// Rounds do not use dense matrices for their generations (round_flow.cu, rowstore.cu) unless neither the
+// blocks nor the memory of those fit.
 #include "common.cuh"
 #include "fitness_common.cuh"
 
@@ -319,11 +319,6 @@ struct Rows2Args {
   int32_t *occ_count;        // [count][nbatch][num_nodes] rows of the batch that occupy the node
   uint32_t *occ_list;        // [count][nbatch][num_nodes][OCC_SLOTS] job | GPUs << 20 | distributed << 31
   int nbatch, lpr_log2;
-  // Single-batch candidates (J <= 256): the block also does the column pass and the fitness of
-  // its candidate, so a whole generation is one kernel.
-  int fuse;
-  TermParams tp;
-  float *fitness_out;        // [count]
 };
 
 __device__ __forceinline__ uint4 clamp_vec(uint4 x, uint4 cp) {
@@ -538,7 +533,7 @@ __device__ void repair_column_list(const ColfixArgs &a, int cl, int nn, int tot,
 
 // VPL = 16-byte vectors per lane; a row is split over LPR = 1 << LPR_LOG2 lanes
 // (LPR * VPL >= row_vecs, FULL when equal), so a warp works on 32 / LPR rows at a time.
-template <int LPR_LOG2, int VPL, bool FULL, bool FUSE>
+template <int LPR_LOG2, int VPL, bool FULL>
 __global__ void __launch_bounds__(256, 4) rows2_kernel(Rows2Args aa) {
   const RowsArgs &a = aa.r;
   constexpr int MAXN = 8 * (1 << LPR_LOG2) * VPL;   // nodes this instantiation can hold
@@ -548,8 +543,6 @@ __global__ void __launch_bounds__(256, 4) rows2_kernel(Rows2Args aa) {
   __shared__ int32_t s_tot[MAXN], s_el[MAXN], s_cnt[MAXN];
   __shared__ uint32_t s_occ[MAXN * OCC_SLOTS];
   __shared__ int s_parent[2];
-  __shared__ uint32_t s_summ[256];   // row summaries of the block's rows
-  __shared__ float s_term[256];
   // per-warp queue of non-empty vectors waiting to be expanded into occupants
   __shared__ __align__(16) uint4 s_qvec[8][QCAP];
   __shared__ uint32_t s_qmeta[8][QCAP];
@@ -642,7 +635,7 @@ __global__ void __launch_bounds__(256, 4) rows2_kernel(Rows2Args aa) {
   // An unperturbed child row is a verbatim copy of a parent's row, whose summary (K, N, entries
   // differing from the current allocation; kept exact by the column pass) is already known:
   // such rows skip the row totals and the comparison with the current allocation.
-  const bool inherit = !FUSE && a.mode == ROWS_GENERATION && a.summ_in != nullptr;
+  const bool inherit = a.mode == ROWS_GENERATION && a.summ_in != nullptr;
   const uint32_t *sin_a = inherit ? a.summ_in + (size_t)s_parent[0] * J + j0 : nullptr;
   const uint32_t *sin_b = inherit ? a.summ_in + (size_t)s_parent[1] * J + j0 : nullptr;
   uint4 raw[VPL];
@@ -829,53 +822,11 @@ __global__ void __launch_bounds__(256, 4) rows2_kernel(Rows2Args aa) {
       a.dflag[(size_t)cl * J + j] = (on && dist) ? 1 : 0;
       // row summary for the fitness: K | N << 11 | (entries that differ from current) << 22
       const uint32_t word = on ? ((uint32_t)K | ((uint32_t)N << 11) | ((uint32_t)ndiff << 22)) : 0u;
-      if (FUSE) s_summ[warp * 32 + r] = word;
-      if (!FUSE && a.summ) a.summ[(size_t)cl * J + j] = word;
+      if (a.summ) a.summ[(size_t)cl * J + j] = word;
     }
   }
 
   __syncthreads();
-  if (FUSE) {
-    // ---- the whole candidate lives in this block: column pass and fitness right here ---------
-    ColfixArgs f;
-    f.pop = a.dst; f.dflag = a.dflag; f.cap = a.cap; f.cur = a.cur;
-    f.colsum = nullptr; f.colelig = nullptr; f.summ = nullptr; f.occ_count = nullptr; f.occ_list = nullptr;
-    f.list = nullptr; f.list_count = nullptr;
-    f.J = J; f.num_nodes = NN; f.nbatch = 1; f.gen = a.gen; f.first_cand = a.first_cand; f.key = a.key;
-    for (int nb = warp * 32; nb < NN; nb += 256) {
-      const int n = nb + lane;
-      const int total = (n < NN) ? s_tot[n] : 0, nelig = (n < NN) ? s_el[n] : 0;
-      const int cp = (n < NN) ? (int)s_cap[n] : 0;
-      unsigned todo = __ballot_sync(0xffffffffu, n < NN && (nelig >= 2 || total > cp));
-      while (todo) {
-        const int srcl = __ffs(todo) - 1;
-        todo &= todo - 1;
-        const int nn = nb + srcl;
-        const int tot_n = __shfl_sync(0xffffffffu, total, srcl), ne_n = __shfl_sync(0xffffffffu, nelig, srcl);
-        const int cap_n = __shfl_sync(0xffffffffu, cp, srcl);
-        const int have_n = s_cnt[nn];
-        if (have_n > OCC_SLOTS) {
-          repair_column_any(f, s_summ, cl, nn, tot_n, ne_n, cap_n, lane);
-        } else {
-          const uint32_t entry = (lane < have_n) ? s_occ[nn * OCC_SLOTS + lane] : 0u;
-          repair_column_entries(f, s_summ, cl, nn, tot_n, ne_n, cap_n, lane, entry, have_n);
-        }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < J; j += blockDim.x) {
-      if (!aa.tp.active || aa.tp.active[j]) {
-        const uint32_t w = s_summ[j];
-        s_term[j] = fitness_term(aa.tp, j, (int)(w & 0x7FFu), (int)((w >> 11) & 0x7FFu), (w >> 22) != 0u);
-      }
-    }
-    __syncthreads();
-    double tsum, tcount;
-    block_term_sum(s_term, J, 0, aa.tp.active, tsum, tcount);
-    if (threadIdx.x == 0) aa.fitness_out[cl] = fitness_finalise(aa.tp.mode, aa.tp.p, tsum, tcount);
-    return;
-  }
   // ---- column partials and occupant lists of the block -------------------------------------
   const size_t base = ((size_t)cl * aa.nbatch + batch) * NN;
   for (int i = threadIdx.x; i < NN; i += blockDim.x) {
@@ -1232,343 +1183,6 @@ __global__ void __launch_bounds__(256, 4) rows_stream_kernel(Rows2Args aa) {
   }
 }
 
-// ---------------------------------------------------------------------------------------
-// Small problems (at most 256 jobs, at most 32 nodes): one block per candidate, one THREAD
-// per row.  A row is 16 to 64 bytes, so a thread reads its parent's row with one to four
-// vector loads, keeps it in its own line of shared memory, perturbs and caps it there, and
-// adds its occupants to per-node lists; warps then repair the violating nodes from the
-// lists (or from the rows in shared memory when a list overflows), the threads write their
-// rows out and the block sums the fitness.  Same operators, draws and sums as the kernels
-// above: identical populations and fitness bits, with far fewer dependent steps.
-// ---------------------------------------------------------------------------------------
-constexpr int SMALL_MAX_NODES = 32;
-constexpr int SMALL_OCC = 32;   // occupants listed per node: one lane each in the repair
-
-__global__ void __launch_bounds__(256) generation_small_kernel(Rows2Args aa) {
-  const RowsArgs &a = aa.r;
-  __shared__ __align__(16) int16_t s_rows[256][SMALL_MAX_NODES];   // child rows, a line per job
-  __shared__ __align__(16) int16_t s_cap[SMALL_MAX_NODES];
-  __shared__ uint32_t s_tot[SMALL_MAX_NODES], s_cnt[SMALL_MAX_NODES];  // GPUs placed; distributed jobs | occupants << 16
-  __shared__ uint32_t s_occ[SMALL_MAX_NODES][SMALL_OCC];               // job | GPUs << 13 | distributed << 31
-  __shared__ uint32_t s_summ[256];
-  __shared__ uint8_t s_dirty[256];
-  __shared__ float s_term[256];
-  __shared__ int s_parent[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cl = blockIdx.x;
-  const uint32_t c = a.first_cand + (uint32_t)cl;
-  const int NN = a.num_nodes, J = a.J, P = a.P;
-  const int row_vecs = NN >> 3;
-  const bool elite = (int)c < a.num_elite;
-
-  // The next generation's grid may be set up while this one runs (programmatic dependent launch):
-  // its blocks do their own parent-independent prologue and then wait, below, for this grid to
-  // finish.  Nothing this kernel writes to global memory is written before its own wait.
-  asm volatile("griddepcontrol.launch_dependents;");
-  // Everything that does not depend on the parents is asked for first, so that the waits overlap:
-  // the job's flags and caps, the fitness keys (staged in shared memory), and the row's draws.
-  const int j = tid;
-  bool on = false;
-  int kc = a.k_max;
-  if (j < J) {
-    on = !a.active || a.active[j];
-    if (a.k_cap) kc = a.k_cap[j];
-  }
-  __shared__ __align__(16) uint32_t s_keys[256];
-  const bool staged = P <= 256;
-  if (tid < NN) {
-    s_cap[tid] = (int16_t)max((int)a.cap[tid], 0);
-    s_tot[tid] = 0u;
-    s_cnt[tid] = 0u;
-  }
-  bool second = false, mut = false;
-  u32x4 mw = {0, 0, 0, 0};
-  if (on && !elite) {
-    second = (draw(a.key, (uint32_t)j, c, a.gen, SLOT_XOVER).x >> 31) != 0u;
-    mw = draw(a.key, (uint32_t)j, c, a.gen, SLOT_MUTATE);
-    mut = mw.x < a.thr;
-  }
-  uint4 cur4[SMALL_MAX_NODES / 8];
-#pragma unroll
-  for (int v = 0; v < SMALL_MAX_NODES / 8; ++v) {
-    cur4[v] = make_uint4(0u, 0u, 0u, 0u);
-    if (a.cur && j < J && v < row_vecs) cur4[v] = __ldg((const uint4 *)(a.cur + (size_t)j * NN) + v);
-  }
-  // from here on the parents' population and fitness are read: the grid that wrote them must be done
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (elite) {
-    if (staged && tid < P) s_keys[tid] = order_key(__ldcg(a.fitness_bits + tid));
-    __syncthreads();
-  }
-  const bool early = !elite && row_vecs <= 2;
-  uint4 cand[2][2] = {{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)},
-                      {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)}};
-  int pair0 = -1;
-  // ---- parents (rank = candidates ordered before, fitness descending, index ascending) --------
-  if (elite) {
-    for (int i = tid; i < P; i += blockDim.x) {
-      const uint32_t ki = staged ? s_keys[i] : order_key(__ldcg(a.fitness_bits + i));
-      int rk = 0, o = 0;
-      if (staged) {
-        for (; o + 4 <= P; o += 4) {   // four staged keys per step
-          const uint4 k4 = *(const uint4 *)(s_keys + o);
-          rk += (k4.x > ki || (k4.x == ki && o < i)) ? 1 : 0;
-          rk += (k4.y > ki || (k4.y == ki && o + 1 < i)) ? 1 : 0;
-          rk += (k4.z > ki || (k4.z == ki && o + 2 < i)) ? 1 : 0;
-          rk += (k4.w > ki || (k4.w == ki && o + 3 < i)) ? 1 : 0;
-        }
-      }
-      for (; o < P; ++o) {
-        const uint32_t ko = staged ? s_keys[o] : order_key(__ldcg(a.fitness_bits + o));
-        rk += (ko > ki || (ko == ki && o < i)) ? 1 : 0;
-      }
-      if (rk == (int)c) s_parent[0] = s_parent[1] = i;
-    }
-  } else {
-    const u32x4 sel = draw(a.key, 0u, c, a.gen, SLOT_SELECT);
-    const int idx[4] = {(int)bounded(sel.x, P), (int)bounded(sel.y, P), (int)bounded(sel.z, P), (int)bounded(sel.w, P)};
-    // short rows: this thread's row of both candidates of its pair is fetched together with the
-    // candidates' keys
-    if (early && j < J && on) {
-      pair0 = idx[second ? 2 : 0];
-      const uint4 *r0 = (const uint4 *)(a.src + ((size_t)pair0 * J + j) * NN);
-      const uint4 *r1 = (const uint4 *)(a.src + ((size_t)idx[second ? 3 : 1] * J + j) * NN);
-      cand[0][0] = __ldcg(r0);
-      cand[1][0] = __ldcg(r1);
-      if (row_vecs > 1) { cand[0][1] = __ldcg(r0 + 1); cand[1][1] = __ldcg(r1 + 1); }
-    }
-    if (tid == 0) {
-      uint32_t k4[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) k4[q] = order_key(__ldcg(a.fitness_bits + idx[q]));
-      s_parent[0] = tournament_winner(k4[0], idx[0], k4[1], idx[1]);
-      s_parent[1] = tournament_winner(k4[2], idx[2], k4[3], idx[3]);
-    }
-  }
-  __syncthreads();
-
-  // ---- rows: thread j builds row j of the child ----------------------------------------------
-  // K and N of the row in this thread's line of shared memory, from its 16-byte pieces
-  auto row_totals = [&](const int16_t *r, int &k_out, int &n_out) {
-    uint32_t part = 0;
-    for (int v = 0; v < row_vecs; ++v) part += row_partial(((const uint4 *)r)[v]);
-    k_out = (int)(part & 0x3FFFFFu);
-    n_out = (int)(part >> 22);
-  };
-  int16_t *row = s_rows[tid];
-  int K = 0, N = 0, ndiff = 0;
-  if (j < J) {
-    const int parent = s_parent[second ? 1 : 0];
-    const uint4 *src = (const uint4 *)(a.src + ((size_t)parent * J + j) * NN);
-    const int which = (parent == pair0) ? 0 : 1;   // when the row was fetched early
-#pragma unroll
-    for (int v = 0; v < SMALL_MAX_NODES / 8; ++v) {
-      uint4 x = make_uint4(0u, 0u, 0u, 0u);
-      if (v < row_vecs) {
-        if (on) {
-          const uint4 raw = (early && v < 2) ? (which == 0 ? cand[0][v] : cand[1][v]) : __ldcg(src + v);
-          x = clamp_vec(raw, ((const uint4 *)s_cap)[v]);   // entries into [0, node size]
-        }
-        ((uint4 *)row)[v] = x;
-      }
-    }
-    if (on) {
-      row_totals(row, K, N);
-      if (mut) {
-        const uint32_t op = bounded(mw.y, 3u);
-        if (op == 0u) {
-          const int n = (int)bounded(mw.w, (uint32_t)NN);
-          row[n] = (int16_t)min((int)row[n] + 1, (int)s_cap[n]);
-        } else if (N > 0) {
-          int t = (int)bounded(mw.z, (uint32_t)N), ns = 0;
-          for (int n = 0; n < NN; ++n) {
-            if (row[n] > 0 && t-- == 0) { ns = n; break; }
-          }
-          if (op == 1u) {
-            row[ns] = (int16_t)(row[ns] - 1);
-          } else {
-            const int nd = (int)bounded(mw.w, (uint32_t)NN);
-            if (nd != ns) {
-              row[nd] = (int16_t)min((int)row[nd] + (int)row[ns], (int)s_cap[nd]);
-              row[ns] = 0;
-            }
-          }
-        }
-        row_totals(row, K, N);
-      }
-      // per-row caps: replicas above the job's cap leave from the highest node index down, then
-      // occupied nodes beyond n_max are cleared from the highest index down
-      kc = max(0, min(kc, a.k_max));
-      if (K > kc || N > a.n_max) {
-        int excess = K - kc;
-        for (int n = NN - 1; n >= 0 && excess > 0; --n) {
-          const int take = min((int)row[n], excess);
-          row[n] = (int16_t)(row[n] - take);
-          excess -= take;
-        }
-        int occ = 0;
-        K = 0;
-        for (int n = 0; n < NN; ++n) {
-          if (row[n] > 0) {
-            ++occ;
-            if (occ > a.n_max) row[n] = 0;
-          }
-          K += row[n];
-        }
-        N = min(occ, a.n_max);
-      }
-      // occupants into the nodes' totals and lists; entries differing from the current allocation
-      const bool dist = N >= 2;
-#pragma unroll
-      for (int v = 0; v < SMALL_MAX_NODES / 8; ++v) {
-        if (v >= row_vecs) break;
-        const uint4 x = ((const uint4 *)row)[v];
-        if (a.cur) {
-          // each half of the xor is a non-negative int16, so min(half, 1) counts the halves that differ
-          const uint32_t d = __vimin_s16x2_relu(x.x ^ cur4[v].x, 0x00010001u) + __vimin_s16x2_relu(x.y ^ cur4[v].y, 0x00010001u) +
-                             __vimin_s16x2_relu(x.z ^ cur4[v].z, 0x00010001u) + __vimin_s16x2_relu(x.w ^ cur4[v].w, 0x00010001u);
-          ndiff += (int)((d & 0xFFFFu) + (d >> 16));
-        }
-        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int h = 0; h < 8; ++h) {
-          const int g = (int)((w[h >> 1] >> ((h & 1) * 16)) & 0xFFFFu);
-          if (g > 0) {
-            const int n = 8 * v + h;
-            atomicAdd(&s_tot[n], (uint32_t)g);
-            const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
-            if (k < SMALL_OCC) s_occ[n][k] = (uint32_t)j | ((uint32_t)g << 13) | (dist ? 0x80000000u : 0u);
-          }
-        }
-      }
-    }
-    s_summ[j] = on ? ((uint32_t)K | ((uint32_t)N << 11) | ((uint32_t)ndiff << 22)) : 0u;
-    s_dirty[j] = 0;
-  }
-  __syncthreads();
-
-  // ---- repair, a warp per violating node -------------------------------------------------------
-  for (int nn = warp; nn < NN; nn += 8) {
-    int tot = (int)s_tot[nn];
-    const int ne = (int)(s_cnt[nn] & 0xFFFFu), have_n = (int)(s_cnt[nn] >> 16), cap_n = (int)s_cap[nn];
-    if (ne < 2 && tot <= cap_n) continue;
-    if (have_n <= SMALL_OCC) {
-      // one occupant per lane
-      const bool have = lane < have_n;
-      const uint32_t entry = have ? s_occ[nn][lane] : 0u;
-      const int jj = (int)(entry & 0x1FFFu);
-      const int v_old = have ? (int)((entry >> 13) & 0x7FFu) : 0;
-      int v = v_old;
-      const bool dist = have && (entry >> 31);
-      if (ne >= 2) {
-        const int o = (int)bounded(draw(a.key, (uint32_t)nn, c, a.gen, SLOT_REPAIR_INTF).x, (uint32_t)J);
-        int t = J;
-        if (dist && v > 0) { t = jj - o; if (t < 0) t += J; }
-        int best = t;
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
-        int removed = 0;
-        if (dist && v > 0 && t != best) { removed = v; v = 0; }
-        tot -= warp_sum(removed);
-      }
-      const int excess = tot - cap_n;
-      if (excess > 0) {
-        const int o = (int)bounded(draw(a.key, (uint32_t)nn, c, a.gen, SLOT_REPAIR_CAP).x, (uint32_t)J);
-        int rot = 0x7fffffff;
-        if (have) { rot = jj - o; if (rot < 0) rot += J; }
-        int ahead = 0;                       // GPUs of the occupants that come first in rotated order
-        for (int k = 0; k < have_n; ++k) {
-          const int rk = __shfl_sync(0xffffffffu, rot, k);
-          const int vk = __shfl_sync(0xffffffffu, v, k);
-          if (rk < rot) ahead += vk;
-        }
-        if (have) v -= min(v, max(excess - ahead, 0));
-      }
-      if (have && v != v_old) {
-        s_rows[jj][nn] = (int16_t)v;
-        s_dirty[jj] = 1;
-      }
-    } else {
-      // more occupants than the list holds: the column of the rows in shared memory
-      int keep = -1;
-      const bool intf = ne >= 2;
-      if (intf) {
-        const int o = (int)bounded(draw(a.key, (uint32_t)nn, c, a.gen, SLOT_REPAIR_INTF).x, (uint32_t)J);
-        int best = J;
-        for (int jj = lane; jj < J; jj += 32) {
-          if (s_rows[jj][nn] > 0 && ((s_summ[jj] >> 11) & 0x7FFu) >= 2u) {
-            int t = jj - o;
-            if (t < 0) t += J;
-            best = min(best, t);
-          }
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
-        keep = o + best;
-        if (keep >= J) keep -= J;
-        int removed = 0;
-        for (int jj = lane; jj < J; jj += 32) {
-          const int v = s_rows[jj][nn];
-          if (v > 0 && ((s_summ[jj] >> 11) & 0x7FFu) >= 2u && jj != keep) removed += v;
-        }
-        tot -= warp_sum(removed);
-      }
-      int excess = tot - cap_n;
-      const int o = (excess > 0) ? (int)bounded(draw(a.key, (uint32_t)nn, c, a.gen, SLOT_REPAIR_CAP).x, (uint32_t)J) : 0;
-      for (int t0 = 0; t0 < J; t0 += 32) {
-        const int t = t0 + lane;
-        int jj = o + t;
-        if (jj >= J) jj -= J;
-        int v_old = 0, v_eff = 0;
-        if (t < J) {
-          v_old = s_rows[jj][nn];
-          const bool dist = ((s_summ[jj] >> 11) & 0x7FFu) >= 2u;
-          v_eff = (intf && dist && v_old > 0 && jj != keep) ? 0 : v_old;
-        }
-        int sfx = v_eff;                              // inclusive prefix over the 32 jobs
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, sfx, off);
-          if (lane >= off) sfx += u;
-        }
-        const int take = (excess > 0) ? min(v_eff, max(excess - (sfx - v_eff), 0)) : 0;
-        const int v_new = v_eff - take;
-        if (t < J && v_new != v_old) {
-          s_rows[jj][nn] = (int16_t)v_new;
-          s_dirty[jj] = 1;
-        }
-        excess -= __shfl_sync(0xffffffffu, sfx, 31);
-      }
-    }
-  }
-  __syncthreads();
-
-  // ---- rows out, fitness -----------------------------------------------------------------------
-  if (j < J) {
-    if (s_dirty[j]) {
-      row_totals(row, K, N);
-      ndiff = 0;
-      if (a.cur) {
-#pragma unroll
-        for (int v = 0; v < SMALL_MAX_NODES / 8; ++v) {
-          if (v >= row_vecs) break;
-          const uint4 x = ((const uint4 *)row)[v];
-          const uint32_t d = __vimin_s16x2_relu(x.x ^ cur4[v].x, 0x00010001u) + __vimin_s16x2_relu(x.y ^ cur4[v].y, 0x00010001u) +
-                             __vimin_s16x2_relu(x.z ^ cur4[v].z, 0x00010001u) + __vimin_s16x2_relu(x.w ^ cur4[v].w, 0x00010001u);
-          ndiff += (int)((d & 0xFFFFu) + (d >> 16));
-        }
-      }
-    }
-    uint4 *dst = (uint4 *)(a.dst + ((size_t)cl * J + j) * NN);
-    for (int v = 0; v < row_vecs; ++v) dst[v] = ((const uint4 *)row)[v];
-    if (on && (!aa.tp.active || aa.tp.active[j])) s_term[j] = fitness_term(aa.tp, j, K, N, ndiff != 0);
-  }
-  __syncthreads();
-  double tsum, tcount;
-  block_term_sum(s_term, J, 0, aa.tp.active, tsum, tcount);
-  if (tid == 0) aa.fitness_out[cl] = fitness_finalise(aa.tp.mode, aa.tp.p, tsum, tcount);
-}
-
 // Column pass: warps take nodes from the work list the row kernel built (any order: columns are
 // independent) and repair them.
 __global__ void __launch_bounds__(128, 4) colrepair_kernel(ColfixArgs a) {
@@ -1640,7 +1254,6 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   const bool fused = (NN % 8 == 0) && NN <= 512 && aligned && ctx->cap_max <= 2047 && count <= 65535 &&
                      a.J <= (1 << 20);
   ctx->summ_valid = fused && a.summ != nullptr;
-  ctx->fit_done = false;
   if (!fused) {
     if (a.mode == ROWS_GENERATION) {
       {
@@ -1661,15 +1274,9 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   aa.colsum = ctx->d_colsum; aa.colelig = ctx->d_colelig; aa.nbatch = nbatch;
   aa.list_count = ctx->d_colcount; aa.list = ctx->d_collist; aa.cand_ticket = ctx->d_rowticket;
   aa.occ_count = ctx->d_occcount; aa.occ_list = ctx->d_occlist;
-  aa.fuse = (nbatch == 1 && ctx->ff_on) ? 1 : 0;
-  aa.tp.table = ctx->ff_table; aa.tp.pen = ctx->ff_pen; aa.tp.active = ctx->ff_active;
-  aa.tp.k_max = ctx->cfg.k_max; aa.tp.n_max = ctx->cfg.n_max; aa.tp.mode = fitness_mode(ctx->ff_p);
-  aa.tp.p = ctx->ff_p; aa.tp.floor_ = ctx->cfg.speedup_floor;
-  aa.fitness_out = ctx->ff_out;
-  ctx->fit_done = aa.fuse != 0;
   dim3 grid((unsigned)nbatch, (unsigned)count);
   const int row_vecs_all = NN / 8;
-  if (!aa.fuse && a.summ == nullptr && (row_vecs_all & (row_vecs_all - 1)) == 0) {
+  if (a.summ == nullptr && (row_vecs_all & (row_vecs_all - 1)) == 0) {
     // no per-row summaries wanted (the entry points called on their own): the streaming kernel
     const size_t smem = stream_smem_bytes(NN);
     if (smem > 24 * 1024) {
@@ -1696,30 +1303,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
     SCHED_LAUNCH_CHECK(ctx);
     return SCHED_OK;
   }
-  if (aa.fuse && a.mode == ROWS_GENERATION && NN <= SMALL_MAX_NODES && a.J <= 8192) {
-    // small problem inside a round: thread-per-row kernel, fitness included
-    {
-      TimedLaunch tl_(ctx, KK_ROWS);
-      // launched so that it may overlap the tail of the kernel before it (see the kernel's top)
-      cudaLaunchConfig_t lc = {};
-      lc.gridDim = dim3((unsigned)count);
-      lc.blockDim = dim3(256);
-      lc.dynamicSmemBytes = 0;
-      lc.stream = ctx->stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      lc.attrs = attr;
-      lc.numAttrs = 1;
-      if (cudaLaunchKernelEx(&lc, generation_small_kernel, aa) != cudaSuccess) {
-        cudaGetLastError();
-        generation_small_kernel<<<(unsigned)count, 256, 0, ctx->stream>>>(aa);
-      }
-    }
-    SCHED_LAUNCH_CHECK(ctx);
-    return SCHED_OK;
-  }
-  if (!aa.fuse) SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(ctx->d_colcount, 0, sizeof(unsigned int), ctx->stream));
+  SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(ctx->d_colcount, 0, sizeof(unsigned int), ctx->stream));
   {
     TimedLaunch tl_(ctx, KK_ROWS);
     // about four vectors per lane: several loads in flight and the per-row overhead shared
@@ -1729,15 +1313,10 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
     aa.lpr_log2 = lpr_log2;
     const int vpl = (row_vecs + (1 << lpr_log2) - 1) >> lpr_log2;
     const bool full = (vpl << lpr_log2) == row_vecs && (vpl == 1 || vpl == 2 || vpl == 4);
-#define ROWS2(L, V)                                                            \
-  do {                                                                         \
-    if (aa.fuse) {                                                             \
-      if (full) rows2_kernel<L, V, true, true><<<grid, 256, 0, ctx->stream>>>(aa);    \
-      else rows2_kernel<L, V, false, true><<<grid, 256, 0, ctx->stream>>>(aa);        \
-    } else {                                                                   \
-      if (full) rows2_kernel<L, V, true, false><<<grid, 256, 0, ctx->stream>>>(aa);   \
-      else rows2_kernel<L, V, false, false><<<grid, 256, 0, ctx->stream>>>(aa);       \
-    }                                                                          \
+#define ROWS2(L, V)                                                      \
+  do {                                                                   \
+    if (full) rows2_kernel<L, V, true><<<grid, 256, 0, ctx->stream>>>(aa); \
+    else rows2_kernel<L, V, false><<<grid, 256, 0, ctx->stream>>>(aa);     \
   } while (0)
     if (lpr_log2 == 0) {
       if (vpl <= 1) ROWS2(0, 1);
@@ -1750,7 +1329,6 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
 #undef ROWS2
   }
   SCHED_LAUNCH_CHECK(ctx);
-  if (aa.fuse) return SCHED_OK;   // the block did the column pass and the fitness itself
   ColfixArgs f;
   f.pop = pop; f.dflag = ctx->d_dflag; f.cap = ctx->d_cap;
   f.colsum = ctx->d_colsum; f.colelig = ctx->d_colelig; f.summ = a.summ;
@@ -1778,12 +1356,6 @@ RowsArgs base_rows_args(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
 }
 
 }  // namespace
-
-// Rounds whose generations generation_small_kernel runs: rows short enough for a thread each.
-bool round_is_small(const sched_ctx *ctx) {
-  const sched_config &c = ctx->cfg;
-  return c.num_jobs <= 256 && c.num_nodes <= SMALL_MAX_NODES && c.num_nodes % 8 == 0 && ctx->cap_max <= 2047 && !ctx->d_rack;
-}
 
 int launch_repair(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
                   int32_t count, uint32_t first_candidate, uint32_t generation) {

@@ -1690,11 +1690,11 @@ static int store_units(const sched_config &c, unsigned long long budget) {
   return (int)(units < 24 ? units : 24);
 }
 
-// The row store serves rounds of at most 512 nodes and sizes that fit the packed fields - except those
-// that one block per candidate runs faster on dense rows (round_is_small).
+// The row store serves rounds of at most 512 nodes and sizes that fit the packed fields, where the four
+// generations that round_flow.cu keeps do not fit the budget, or its blocks the GPU.
 bool rowstore_eligible(const sched_ctx *ctx) {
   const sched_config &c = ctx->cfg;
-  if (round_is_small(ctx) || c.num_jobs > STORE_MAX_JOBS) return false;
+  if (c.num_jobs < 1 || c.num_jobs > STORE_MAX_JOBS) return false;
   if (c.num_nodes > 512 || ctx->cap_max > 2047) return false;
   if (c.k_max > 2047 || c.n_max > 2047) return false;
   if (gen_smem_layout(c.num_jobs, c.num_nodes).total > 200 * 1024) return false;

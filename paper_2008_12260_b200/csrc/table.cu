@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fitness_common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -669,10 +670,7 @@ __global__ void realloc_factor_kernel(const float *__restrict__ age, const int32
                                       float delta, int J, float *__restrict__ out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= J) return;
-  const float T = age[j], R = (float)restarts[j];
-  float f = (T - R * delta) / (T + delta);
-  if (!(f >= 0.f)) f = 0.f;
-  out[j] = fminf(f, 1.f);
+  out[j] = realloc_factor(age[j], restarts[j], delta);
 }
 
 // Goodput-driven auto-scaling rule (Sec. 5.3): one thread per job.  All products are

@@ -1,5 +1,5 @@
 """Rounds at the shapes where their kernels change: node counts that are no multiple of a row's
-pieces, racks, few and many jobs, inactive jobs.  A round must equal, bit for bit, the same round made of the
+pieces, racks, few and many jobs, inactive jobs, populations larger than the GPU holds blocks, elites.  A round must equal, bit for bit, the same round made of the
 dense entry points called one by one (which other tests pin to the oracle)."""
 import numpy as np
 import pytest
@@ -16,6 +16,9 @@ SHAPES = [
     (129, 4, 257, 16, 5, 0, 1.0, 0.3), (505, 2, 270, 9, 4, 100, 1.0, 0.4), (512, 4, 33, 12, 5, 64, 1.0, 1.0),
     (40, 2, 6, 24, 40, 10, 1.0, 0.9), (16, 4, 256, 64, 6, 0, 0.3, 0.2), (32, 4, 96, 100, 12, 8, 1.0, 0.08),
     (13, 96, 300, 24, 6, 0, 1.0, 0.3), (9, 200, 50, 24, 6, 4, 1.0, 0.5),
+    # more candidates than blocks fit the GPU at once; one candidate; more elites than a warp has lanes
+    (16, 4, 270, 700, 3, 0, 1.0, 0.05), (8, 4, 40, 2500, 3, 0, 1.0, 0.1), (8, 4, 20, 1, 5, 0, 1.0, 0.5),
+    (24, 4, 70, 90, 6, 6, 0.6, 0.2),
 ]
 
 
@@ -26,7 +29,7 @@ def test_round_equals_stepwise(shape, start):
     from paper_2008_12260_b200 import api
 
     NN, gpn, J, P, gens, per_rack, active, mutate = shape
-    cfg = synth.Config("shape", NN, gpn, J, NN + J, 16, 8, P, gens, num_elite=min(2, P), mutate_prob=mutate, init_prob=0.3,
+    cfg = synth.Config("shape", NN, gpn, J, NN + J, 16, 8, P, gens, num_elite=min(P, 40 if P == 90 else J % 3), mutate_prob=mutate, init_prob=0.3,
                        with_history=True, p=-1.0 if J % 2 else 0.5)
     cl = cfg.cluster()
     jobs = cfg.jobs()
