@@ -256,7 +256,8 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   if ((rc = dev_alloc(ctx, &ctx->d_pairs, pairs.size())) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_rank, P)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_order, P)) != SCHED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_pen, J)) != SCHED_OK) return fail(rc);
+  if ((rc = dev_alloc(ctx, &ctx->d_pen, 2 * J)) != SCHED_OK) return fail(rc);
+  ctx->d_cur_nz = (int32_t *)(ctx->d_pen + J);
   if ((rc = dev_alloc(ctx, &ctx->d_status, 1)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_best_idx, 1)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_colcount, 1)) != SCHED_OK) return fail(rc);
@@ -421,8 +422,8 @@ int eval_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, cons
           SCHED_ERR_INVALID_ARG, "eval_fitness_racks: a buffer is not aligned to its element size");
   REQUIRE(ctx, (long long)count * ctx->cfg.num_jobs < (1LL << 31), SCHED_ERR_TOO_LARGE,
           "eval_fitness_racks: count * num_jobs must be below 2^31");
-  return launch_fitness_racks(ctx, d_pop, count, d_speedup, d_speedup_rack, d_cur, d_realloc_factor, d_active, p,
-                              d_fitness);
+  return launch_fitness(ctx, d_pop, count, d_speedup, d_cur, d_realloc_factor, d_active, p, d_fitness, nullptr,
+                        d_speedup_rack);
 }
 
 int sched_num_kernel_kinds(void) { return KK_COUNT; }
@@ -624,11 +625,9 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
   // parents' fitness is read while children's is written: the two alternate between buffers
   float *fit_cur = ctx->d_fit_buf, *fit_next = ctx->d_fit_buf + ctx->cfg.population;
   auto fitness_of = [&](const int16_t *pop, float *out) {
-    if (racks)
-      return launch_fitness_racks(ctx, pop, ctx->cfg.population, ctx->d_tab_speedup, ctx->d_tab_speedup_rack, d_cur, rf,
-                                  d_jobs->active, ctx->cfg.p, out);
     return launch_fitness(ctx, pop, ctx->cfg.population, ctx->d_tab_speedup, d_cur, rf, d_jobs->active,
-                          ctx->cfg.p, out, ctx->summ_valid ? ctx->round_summ : nullptr);
+                          ctx->cfg.p, out, ctx->summ_valid ? ctx->round_summ : nullptr,
+                          racks ? ctx->d_tab_speedup_rack : nullptr);
   };
   const bool store = ctx->rs_ready && generations > 0;
   int parity = 0;

@@ -62,6 +62,7 @@ struct sched_ctx {
   int32_t *d_order;      // [P] inverse of rank
   uint8_t *d_dflag;      // [P][J] "row spans >= 2 nodes" after the row pass
   float *d_pen;          // [J] effective penalty factor (1 when none applies)
+  int32_t *d_cur_nz;     // [J] entries of the current allocation's rows that are not 0 (behind d_pen)
   double *d_partial;     // [count][chunks] partial sums of the fitness reduction
   unsigned int *d_ticket;  // [count] arrival counters of the fitness reduction
   uint32_t *d_collist;   // [count * num_nodes] columns that need repair
@@ -279,9 +280,6 @@ int launch_speedup_table(sched_ctx *ctx, const sched_jobs *jobs, float *d_goodpu
                          const float *d_alpha_rack = nullptr, const float *d_beta_rack = nullptr,
                          float *d_goodput_rack = nullptr, float *d_speedup_rack = nullptr,
                          uint16_t *d_argmax_rack = nullptr);
-int launch_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
-                         const float *d_speedup_rack, const int16_t *d_cur, const float *d_rf,
-                         const uint8_t *d_active, float p, float *d_fitness);
 int launch_speedup_table_msample(sched_ctx *ctx, const sched_jobs *jobs, const int32_t *d_m_samples, int G,
                                  const int32_t *d_m_max_gpu, const uint8_t *d_adaptive, float *d_goodput,
                                  float *d_speedup, uint16_t *d_argmax);
@@ -290,7 +288,7 @@ int launch_autoscale(sched_ctx *ctx, const float *d_goodput, const int32_t *d_cu
                      int32_t *d_target_nodes);
 int launch_fitness(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
                    const int16_t *d_cur, const float *d_rf, const uint8_t *d_active, float p,
-                   float *d_fitness, const uint32_t *d_summ = nullptr);
+                   float *d_fitness, const uint32_t *d_summ = nullptr, const float *d_speedup_rack = nullptr);
 int launch_repair(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
                   int32_t count, uint32_t first_candidate, uint32_t generation);
 int launch_init_population(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active,

@@ -2,51 +2,24 @@
 // nodes, "row differs from the current allocation"), speedup gather, re-allocation
 // penalty, floor, and the power-mean reduction over the active jobs.
 //
-// The kernel streams the dense int16 population once with wide loads.  Rows are split
-// over LPR lanes (a power of two <= 32); a warp summarises 32 rows, parks each row's
-// packed (K, N, changed) in one lane, and then all 32 lanes do the gather / penalty /
-// power term for their row at once.  A block covers a contiguous chunk of one
-// candidate's rows; chunk sums go to a scratch array and the last block to arrive adds
-// them in index order, so results are bitwise reproducible.
+// Two kernels stream the dense int16 population once with wide loads.
+//  * fitness_kernel: rows of whole 16-byte vectors, no penalty.  Rows are split over LPR lanes (a power of
+//    two <= 32); a warp summarises 32 rows, parks each row's packed (K, N) in one lane, and then
+//    all 32 lanes do the gather / power term for their row at once.
+//  * fitness_flat_kernel: everything else - rows of any width and alignment, the penalty, racks.  A block's
+//    rows are one flat run of aligned vectors, and only those that hold something are looked at.
+// A block covers a contiguous chunk of one candidate's rows; chunk sums go to a scratch array and the last
+// block to arrive adds them in index order, so results are bitwise reproducible.
 #include "common.cuh"
 #include "fitness_common.cuh"
 
 namespace {
 
-template <int W>
-struct VecLoad;
-template <>
-struct VecLoad<16> {
-  static __device__ __forceinline__ uint4 ld(const void *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-  }
-  static __device__ __forceinline__ uint4 ld_cached(const void *p) { return __ldg((const uint4 *)p); }
-};
-template <>
-struct VecLoad<8> {
-  static __device__ __forceinline__ uint4 ld(const void *p) {
-    const uint2 t = __ldg((const uint2 *)p);
-    return make_uint4(t.x, t.y, 0u, 0u);
-  }
-  static __device__ __forceinline__ uint4 ld_cached(const void *p) { return ld(p); }
-};
-template <>
-struct VecLoad<4> {
-  static __device__ __forceinline__ uint4 ld(const void *p) {
-    return make_uint4(__ldg((const uint32_t *)p), 0u, 0u, 0u);
-  }
-  static __device__ __forceinline__ uint4 ld_cached(const void *p) { return ld(p); }
-};
-template <>
-struct VecLoad<2> {
-  static __device__ __forceinline__ uint4 ld(const void *p) {
-    return make_uint4((uint32_t)__ldg((const uint16_t *)p), 0u, 0u, 0u);
-  }
-  static __device__ __forceinline__ uint4 ld_cached(const void *p) { return ld(p); }
-};
+__device__ __forceinline__ uint4 stream_load(const void *p) {
+  uint4 v;
+  asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
 
 // per 32-bit word (two int16 entries): signed sum, and count of entries > 0
 __device__ __forceinline__ void summarise_word(uint32_t w, int &ksum, uint32_t &npos) {
@@ -59,8 +32,11 @@ struct FitnessArgs {
   const int16_t *cur;
   const float *table;
   const float *pen;       // [J] factor applied to changed rows, or NULL
+  const int32_t *cur_nz;  // [J] entries of the current allocation's row that are not 0 (with pen)
   const uint8_t *active;  // or NULL
   const uint32_t *summ;   // [count][J] row summaries from the row/column kernels (SUMMARY mode)
+  const float *table_rack;   // with rack: table of rows whose nodes lie in two racks or more
+  const int16_t *rack;    // [num_nodes] or NULL
   int J, num_nodes, k_max, n_max;
   int lpr_log2;           // lanes per row = 1 << lpr_log2
   int rows_per_block, chunks;
@@ -99,24 +75,20 @@ __device__ __forceinline__ void block_finish(const FitnessArgs &a, int cand, int
   }
 }
 
-template <int W>
 __global__ void __launch_bounds__(256) fitness_kernel(FitnessArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int cand = blockIdx.y, chunk = blockIdx.x;
   const int LPR = 1 << a.lpr_log2, RPW = 32 >> a.lpr_log2;
   const int group = lane >> a.lpr_log2, sub = lane & (LPR - 1);
-  const unsigned gmask = (LPR == 32) ? 0xffffffffu : (((1u << LPR) - 1u) << (group * LPR));
-  const int row_vecs = (a.num_nodes * 2) / W;
+  const int row_vecs = a.num_nodes / 8;
   const int j0 = chunk * a.rows_per_block;
   const int j1 = min(a.J, j0 + a.rows_per_block);
-  const int KD = a.k_max + 1, ND = a.n_max + 1;
   const char *cand_base = (const char *)(a.pop + (size_t)cand * a.J * a.num_nodes);
-  const char *cur_base = (const char *)a.cur;
   const size_t row_bytes = (size_t)a.num_nodes * 2;
 
   __shared__ float s_term[FITNESS_MAX_ROWS_PER_BLOCK];
   TermParams tp;
-  tp.table = a.table; tp.pen = a.pen; tp.active = a.active;
+  tp.table = a.table; tp.pen = nullptr; tp.active = a.active;
   tp.k_max = a.k_max; tp.n_max = a.n_max; tp.mode = a.mode; tp.p = a.p; tp.floor_ = a.floor_;
   uint32_t mine = 0;
   int myrow = -1;
@@ -128,52 +100,26 @@ __global__ void __launch_bounds__(256) fitness_kernel(FitnessArgs a) {
     const int j = jb + group;
     const bool live = j < j1;
     int ksum = 0;
-    uint32_t npos = 0, diff = 0;
+    uint32_t npos = 0;
     if (live) {
       const char *row = cand_base + (size_t)j * row_bytes;
-      const char *crow = cur_base ? cur_base + (size_t)j * row_bytes : nullptr;
       // batches of vectors per lane: all loads of a batch are issued before any is used
-      if (!crow) {
-        constexpr int B = 8;
-        for (int v0 = sub; v0 < row_vecs; v0 += LPR * B) {
-          uint4 x[B];
+      constexpr int B = 8;
+      for (int v0 = sub; v0 < row_vecs; v0 += LPR * B) {
+        uint4 x[B];
 #pragma unroll
-          for (int k = 0; k < B; ++k) {
-            const int v = v0 + k * LPR;
-            x[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (v < row_vecs) x[k] = VecLoad<W>::ld(row + (size_t)v * W);
-          }
-#pragma unroll
-          for (int k = 0; k < B; ++k) {
-            if ((x[k].x | x[k].y | x[k].z | x[k].w) != 0u) {
-              summarise_word(x[k].x, ksum, npos);
-              if (W >= 8) summarise_word(x[k].y, ksum, npos);
-              if (W >= 16) { summarise_word(x[k].z, ksum, npos); summarise_word(x[k].w, ksum, npos); }
-            }
-          }
+        for (int k = 0; k < B; ++k) {
+          const int v = v0 + k * LPR;
+          x[k] = make_uint4(0u, 0u, 0u, 0u);
+          if (v < row_vecs) x[k] = stream_load(row + (size_t)v * 16);
         }
-      } else {
-        constexpr int B = 4;   // the current allocation's vectors travel with the candidate's
-        for (int v0 = sub; v0 < row_vecs; v0 += LPR * B) {
-          uint4 x[B], c[B];
 #pragma unroll
-          for (int k = 0; k < B; ++k) {
-            const int v = v0 + k * LPR;
-            x[k] = make_uint4(0u, 0u, 0u, 0u);
-            c[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (v < row_vecs) {
-              x[k] = VecLoad<W>::ld(row + (size_t)v * W);
-              c[k] = VecLoad<W>::ld_cached(crow + (size_t)v * W);
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < B; ++k) {
-            if ((x[k].x | x[k].y | x[k].z | x[k].w) != 0u) {
-              summarise_word(x[k].x, ksum, npos);
-              if (W >= 8) summarise_word(x[k].y, ksum, npos);
-              if (W >= 16) { summarise_word(x[k].z, ksum, npos); summarise_word(x[k].w, ksum, npos); }
-            }
-            diff |= (x[k].x ^ c[k].x) | (x[k].y ^ c[k].y) | (x[k].z ^ c[k].z) | (x[k].w ^ c[k].w);
+        for (int k = 0; k < B; ++k) {
+          if ((x[k].x | x[k].y | x[k].z | x[k].w) != 0u) {
+            summarise_word(x[k].x, ksum, npos);
+            summarise_word(x[k].y, ksum, npos);
+            summarise_word(x[k].z, ksum, npos);
+            summarise_word(x[k].w, ksum, npos);
           }
         }
       }
@@ -185,22 +131,177 @@ __global__ void __launch_bounds__(256) fitness_kernel(FitnessArgs a) {
     nl = min(nl, 2047);
     uint32_t packed = (uint32_t)ksum | ((uint32_t)nl << 16);
     for (int off = LPR >> 1; off >= 1; off >>= 1) packed += __shfl_xor_sync(0xffffffffu, packed, off);
-    const unsigned changed = __ballot_sync(0xffffffffu, diff != 0u) & gmask;
     // lane `sub` of each group parks the row its group summarised in iteration `sub`
     if (live && sub == (it & (LPR - 1))) {
-      // K <= 32*2047 < 2^16, N likewise; keep "changed" in the top bit of the N field
-      mine = (packed & 0x7FFFFFFFu) | (changed ? 0x80000000u : 0u);
+      mine = packed;
       myrow = j;
     }
     const bool flush = ((it + 1) % slots_per_fill == 0) || (jb + nwarps * RPW >= j1);
     if (flush) {
       if (myrow >= 0 && (!a.active || a.active[myrow]))
-        s_term[myrow - j0] = fitness_term(tp, myrow, (int)(mine & 0xFFFFu), (int)((mine >> 16) & 0x7FFFu),
-                                          (mine >> 31) != 0u);
+        s_term[myrow - j0] = fitness_term(tp, myrow, (int)(mine & 0xFFFFu), (int)(mine >> 16), false);
       myrow = -1;
     }
   }
 
+  block_finish(a, cand, chunk, j0, j1, s_term);
+}
+
+// Rows of any width and alignment, with the re-allocation penalty and racks.
+//
+// Almost every entry of a population is zero, so a block's rows are read as one flat run of aligned
+// 16-byte vectors, whatever the rows' width, and only vectors that hold something are looked at: they are
+// compacted into a per-warp queue (ballot + popc) and their entries added to their rows' sums in shared
+// memory.  The current allocation is read at the candidate's own entries only: a row equals it when those
+// agree and it has no more entries than they (cur_nz).  Same chunks and fixed-order sums as above.
+// Candidates are taken last to first: what a column repair has just written last is still in L2.
+// Bound: a block's loads wait for its looking, so how many blocks an SM holds and how full the last wave is;
+// 3.9 TB/s.  Measured for 300 candidates of 777 x 251 with the penalty: 31 us (98 us with loads of one
+// entry); for 512 of 1024 x 256: 58 us (60 us).
+constexpr int FLAT_QUEUE = 64;
+__host__ __device__ constexpr int flat_blocks_per_sm(int batch) { return batch == 8 ? 4 : 5; }
+
+__host__ __device__ inline size_t flat_smem_bytes(int rows, bool racks) { return (size_t)rows * (racks ? 16 : 8); }
+
+template <bool RACKS, int B>
+__global__ void __launch_bounds__(256, flat_blocks_per_sm(B)) fitness_flat_kernel(FitnessArgs a) {
+  extern __shared__ float flat_smem[];
+  __shared__ __align__(16) uint4 s_qvec[8][FLAT_QUEUE];
+  __shared__ int s_qat[8][FLAT_QUEUE];
+  const int rows_max = a.rows_per_block;
+  float *s_term = flat_smem;                             // at the end, over the row's GPUs
+  int *s_k = (int *)flat_smem;
+  uint32_t *s_n = (uint32_t *)(s_k + rows_max);          // entries above 0 | entries not 0 << 14 | one differs << 31
+  int *s_lo = (int *)(s_n + rows_max), *s_hi = s_lo + rows_max;   // (RACKS) lowest and highest rack
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cand = gridDim.y - 1 - blockIdx.y, chunk = blockIdx.x, NN = a.num_nodes;
+  const int j0 = chunk * a.rows_per_block;
+  const int j1 = min(a.J, j0 + a.rows_per_block), rows = j1 - j0;
+  for (int r = tid; r < rows; r += 256) {
+    s_k[r] = 0;
+    s_n[r] = 0u;
+    if (RACKS) { s_lo[r] = 0x7fffffff; s_hi[r] = -1; }
+  }
+  __syncthreads();
+  const int16_t *first = a.pop + ((size_t)cand * a.J + j0) * NN;
+  const int16_t *cur = a.cur ? a.cur + (size_t)j0 * NN : nullptr;
+  const int entries = rows * NN;                         // at most 2048 x 8192
+  const int skew = (int)(((uintptr_t)first & 15) >> 1);  // vector i holds entries 8 i - skew ..
+  const int vecs = (entries + skew + 7) / 8;
+  const uint4 *base = (const uint4 *)(first - skew);
+
+  uint4 *qvec = s_qvec[warp];
+  int *qat = s_qat[warp];
+  int queued = 0;
+  auto look = [&](int count) {       // the first `count` queued vectors, one per lane
+    __syncwarp();
+    if (lane < count) {
+      const uint4 x = qvec[lane];
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+      const int e = 8 * qat[lane] - skew;
+      int row = e < 0 ? 0 : e / NN, n = e - row * NN;
+      unsigned set = 0u, other = 0u;   // bit h: entry h is not 0; it is not the current allocation's
+      int c[8];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const int v = (int)(int16_t)(w[h >> 1] >> (16 * (h & 1)));
+        set |= (v != 0 ? 1u : 0u) << h;
+        c[h] = v;
+        if (v != 0 && cur) c[h] = (int)__ldg(cur + e + h);
+      }
+#pragma unroll
+      for (int h = 0; h < 8; ++h) other |= (c[h] != (int)(int16_t)(w[h >> 1] >> (16 * (h & 1))) ? 1u : 0u) << h;
+      // the vector's part in each of its rows
+      for (int h0 = 0; h0 < 8 && (set >> h0);) {
+        const int h1 = min(8, NN - n);
+        const unsigned part = ((1u << h1) - 1u) & ~((1u << h0) - 1u);
+        if (set & part) {
+          int k = 0;
+          uint32_t npos = 0u;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const unsigned m = part >> (2 * q);
+            summarise_word(w[q] & ((m & 1u ? 0xFFFFu : 0u) | (m & 2u ? 0xFFFF0000u : 0u)), k, npos);
+          }
+          atomicAdd(&s_k[row], k);
+          atomicAdd(&s_n[row], (npos & 0xFFFFu) + (npos >> 16) + ((uint32_t)__popc(set & part) << 14));
+          if (other & part) atomicOr(&s_n[row], 1u << 31);
+          if (RACKS) {
+            int lo = 0x7fffffff, hi = -1;
+#pragma unroll
+            for (int h = 0; h < 8; ++h)
+              if (((set & part) >> h & 1u) && (int)(int16_t)(w[h >> 1] >> (16 * (h & 1))) > 0) {
+                const int r = (int)__ldg(a.rack + n + h);
+                lo = min(lo, r);
+                hi = max(hi, r);
+              }
+            atomicMin(&s_lo[row], lo);
+            atomicMax(&s_hi[row], hi);
+          }
+        }
+        ++row;
+        n -= NN;                     // of entry 0, by the next row
+        h0 = h1;
+      }
+    }
+    __syncwarp();
+  };
+  for (int v0 = 0; v0 < vecs; v0 += 256 * B) {
+    uint4 x[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const int i = v0 + q * 256 + tid, e = 8 * i - skew;
+      x[q] = make_uint4(0u, 0u, 0u, 0u);
+      if (e >= 0 && e + 8 <= entries) {
+        x[q] = stream_load(base + i);
+      } else if (i < vecs) {          // the run's ragged ends
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int h = 0; h < 8; ++h)
+          if (e + h >= 0 && e + h < entries) w[h >> 1] |= (uint32_t)(uint16_t)first[e + h] << (16 * (h & 1));
+        x[q] = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const bool nz = (x[q].x | x[q].y | x[q].z | x[q].w) != 0u;
+      const unsigned bal = __ballot_sync(0xffffffffu, nz);
+      if (nz) {
+        const int pos = queued + __popc(bal & ((1u << lane) - 1u));
+        qvec[pos] = x[q];
+        qat[pos] = v0 + q * 256 + tid;
+      }
+      queued += __popc(bal);
+      if (queued >= 32) {
+        look(32);
+        queued -= 32;
+        if (lane < queued) {          // what is left moves to the front
+          const uint4 y = qvec[32 + lane];
+          const int at = qat[32 + lane];
+          qvec[lane] = y;
+          qat[lane] = at;
+        }
+        __syncwarp();
+      }
+    }
+  }
+  look(queued);
+  // penalty factors and counts of the current allocation come from the kernel before this one
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncthreads();
+  TermParams tp;
+  tp.table = a.table; tp.pen = a.pen; tp.active = a.active;
+  tp.k_max = a.k_max; tp.n_max = a.n_max; tp.mode = a.mode; tp.p = a.p; tp.floor_ = a.floor_;
+  for (int r = tid; r < rows; r += 256) {
+    const int j = j0 + r;
+    if (a.active && !a.active[j]) continue;
+    const uint32_t c = s_n[r];
+    const int K = max(0, s_k[r]), N = (int)(c & 0x3FFFu);
+    const bool changed = a.cur && ((c >> 31) || (int)((c >> 14) & 0x3FFFu) != __ldcg(a.cur_nz + j));
+    const float *table = RACKS && N >= 1 && s_lo[r] != s_hi[r] ? a.table_rack : a.table;
+    const float x = __ldg(table + fitness_table_index(tp, j, K, N));
+    s_term[r] = fitness_term_with(tp, x, tp.pen && changed ? __ldcg(tp.pen + j) : 1.f, changed);
+  }
   block_finish(a, cand, chunk, j0, j1, s_term);
 }
 
@@ -224,78 +325,36 @@ __global__ void __launch_bounds__(256) fitness_summary_kernel(FitnessArgs a) {
   block_finish(a, cand, chunk, j0, j1, s_term);
 }
 
-// Eq. 14 with rack-level locality: a row whose occupied nodes lie in two or more racks takes its
-// speedup from the rack-class table.  A plain warp-per-row pass (this variant is not the
-// streaming kernel above); same chunks and the same fixed-order sums.
-__global__ void __launch_bounds__(256)
-fitness_racks_kernel(FitnessArgs a, const float *__restrict__ table_rack, const int16_t *__restrict__ rack) {
-  __shared__ float s_term[FITNESS_MAX_ROWS_PER_BLOCK];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int cand = blockIdx.y, chunk = blockIdx.x;
-  const int j0 = chunk * a.rows_per_block;
-  const int j1 = min(a.J, j0 + a.rows_per_block);
-  TermParams tp;
-  tp.table = a.table; tp.pen = a.pen; tp.active = a.active;
-  tp.k_max = a.k_max; tp.n_max = a.n_max; tp.mode = a.mode; tp.p = a.p; tp.floor_ = a.floor_;
-  for (int j = j0 + warp; j < j1; j += nwarps) {
-    if (a.active && !a.active[j]) continue;
-    const int16_t *row = a.pop + ((size_t)cand * a.J + j) * a.num_nodes;
-    const int16_t *crow = a.cur ? a.cur + (size_t)j * a.num_nodes : nullptr;
-    long long K = 0;
-    int N = 0, rmin = 0x7fffffff, rmax = -1, diff = 0;
-    for (int n = lane; n < a.num_nodes; n += 32) {
-      const int v = row[n];
-      K += v;
-      if (v > 0) {
-        ++N;
-        const int r = rack[n];
-        rmin = min(rmin, r);
-        rmax = max(rmax, r);
-      }
-      if (crow) diff |= (v != (int)crow[n]) ? 1 : 0;
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      K += __shfl_xor_sync(0xffffffffu, K, off);
-      N += __shfl_xor_sync(0xffffffffu, N, off);
-      rmin = min(rmin, __shfl_xor_sync(0xffffffffu, rmin, off));
-      rmax = max(rmax, __shfl_xor_sync(0xffffffffu, rmax, off));
-      diff |= __shfl_xor_sync(0xffffffffu, diff, off);
-    }
-    if (lane == 0) {
-      const int Kc = (int)max(0ll, min(K, (long long)a.k_max));
-      const bool several = N >= 1 && rmin != rmax;
-      const float x = __ldg((several ? table_rack : a.table) + fitness_table_index(tp, j, Kc, N));
-      s_term[j - j0] = fitness_term_of(tp, j, x, diff != 0);
-    }
-  }
-  block_finish(a, cand, chunk, j0, j1, s_term);
-}
-
 // Effective penalty per job: the re-allocation factor when the job currently holds GPUs,
-// else 1 (pending jobs are never penalised).  One warp per job.
-__global__ void penalty_prep_kernel(const int16_t *__restrict__ cur, const float *__restrict__ rf,
-                                    int J, int num_nodes, float *__restrict__ pen) {
+// else 1 (pending jobs are never penalised); and how many entries of its current row are not 0.
+// One warp per job.  The fitness kernel behind it streams the population meanwhile.
+__global__ void __launch_bounds__(256) penalty_prep_kernel(const int16_t *__restrict__ cur, const float *__restrict__ rf,
+                                                           int J, int num_nodes, float *__restrict__ pen,
+                                                           int32_t *__restrict__ cur_nz) {
+  asm volatile("griddepcontrol.launch_dependents;");
   const int lane = threadIdx.x & 31;
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (j >= J) return;
   long long k = 0;
-  for (int n = lane; n < num_nodes; n += 32) k += cur[(size_t)j * num_nodes + n];
+  int nz = 0;
+  for (int n = lane; n < num_nodes; n += 32) {
+    const int v = cur[(size_t)j * num_nodes + n];
+    k += v;
+    nz += v != 0;
+  }
   for (int off = 16; off >= 1; off >>= 1) k += __shfl_xor_sync(0xffffffffu, k, off);
-  if (lane == 0) pen[j] = (k > 0) ? rf[j] : 1.f;
+  nz = __reduce_add_sync(0xffffffffu, nz);
+  if (lane == 0) {
+    pen[j] = (k > 0) ? rf[j] : 1.f;
+    cur_nz[j] = nz;
+  }
 }
 
-// Launch geometry shared by the entry points: the widest vector that divides a row and
-// keeps every row aligned; lanes per row so that a lane owns about four vectors (several
-// loads in flight, few shuffle steps); rows per block of about 1 MB of population, shrunk
+// Launch geometry shared by the entry points: lanes per row so that a lane owns about four vectors
+// (several loads in flight, few shuffle steps; fitness_kernel only); rows per block of about 1 MB of population, shrunk
 // while the grid would leave SMs idle.
-void fitness_geometry(size_t row_bytes, uintptr_t align_bits, int J, int count, int num_sms, int &W,
-                      int &lpr_log2, int &rows_per_block, int &chunks) {
-  W = 2;
-  if (row_bytes % 16 == 0 && align_bits % 16 == 0) W = 16;
-  else if (row_bytes % 8 == 0 && align_bits % 8 == 0) W = 8;
-  else if (row_bytes % 4 == 0 && align_bits % 4 == 0) W = 4;
-  const int row_vecs = (int)(row_bytes / W);
+void fitness_geometry(size_t row_bytes, int J, int count, int num_sms, int &lpr_log2, int &rows_per_block, int &chunks) {
+  const int row_vecs = (int)(row_bytes / 16);
   lpr_log2 = 0;
   while ((4 << lpr_log2) < row_vecs && lpr_log2 < 5) ++lpr_log2;
   rows_per_block = (int)((1u << 20) / row_bytes);
@@ -308,13 +367,49 @@ void fitness_geometry(size_t row_bytes, uintptr_t align_bits, int J, int count, 
   chunks = J > 0 ? (J + rows_per_block - 1) / rows_per_block : 1;
 }
 
+// The kernel for the arguments: whole aligned vectors and nothing to compare with go to fitness_kernel
+// (which sums a row's vectors where they are), everything else to the flat one (which first finds the
+// vectors that hold something).  after_prep: launched behind penalty_prep_kernel, so that it may start
+// while that still runs.
+cudaError_t launch_fitness_kernel(const FitnessArgs &a, int count, int num_sms, bool after_prep, cudaStream_t stream) {
+  const dim3 grid((unsigned)a.chunks, (unsigned)count);
+  const size_t row_bytes = (size_t)a.num_nodes * 2;
+  if (a.summ) {
+    fitness_summary_kernel<<<grid, 256, 0, stream>>>(a);
+    return cudaGetLastError();
+  }
+  if (!a.cur && !a.rack && row_bytes % 16 == 0 && (uintptr_t)a.pop % 16 == 0) {
+    fitness_kernel<<<grid, 256, 0, stream>>>(a);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(256);
+  lc.dynamicSmemBytes = flat_smem_bytes(a.rows_per_block, a.rack != nullptr);
+  lc.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = after_prep ? 1 : 0;
+  // Eight vectors per thread at once, or four and a fifth block per SM where that makes the grid a wave shorter
+  const long long blocks = (long long)a.chunks * count;
+  auto waves = [&](int batch) {
+    const long long resident = (long long)flat_blocks_per_sm(batch) * num_sms;
+    return (blocks + resident - 1) / resident;
+  };
+  const bool wide = waves(8) <= waves(4);
+  void (*const kernel)(FitnessArgs) = a.rack ? (wide ? fitness_flat_kernel<true, 8> : fitness_flat_kernel<true, 4>)
+                                             : (wide ? fitness_flat_kernel<false, 8> : fitness_flat_kernel<false, 4>);
+  return cudaLaunchKernelEx(&lc, kernel, a);
+}
+
 }  // namespace
 
 // Rows per block and blocks per candidate that launch_fitness uses for `count` candidates.
 void fitness_chunking(const sched_ctx *ctx, int32_t count, int &rows_per_block, int &chunks) {
-  int W, lpr_log2;
-  fitness_geometry((size_t)ctx->cfg.num_nodes * 2, 0, ctx->cfg.num_jobs, count, ctx->num_sms, W, lpr_log2,
-                   rows_per_block, chunks);
+  int lpr_log2;
+  fitness_geometry((size_t)ctx->cfg.num_nodes * 2, ctx->cfg.num_jobs, count, ctx->num_sms, lpr_log2, rows_per_block, chunks);
 }
 
 int launch_penalty_prep(sched_ctx *ctx, const int16_t *d_cur, const float *d_rf) {
@@ -322,15 +417,17 @@ int launch_penalty_prep(sched_ctx *ctx, const int16_t *d_cur, const float *d_rf)
   if (J == 0) return SCHED_OK;
   {
     TimedLaunch tl_(ctx, KK_PENPREP);
-    penalty_prep_kernel<<<(J * 32 + 255) / 256, 256, 0, ctx->stream>>>(d_cur, d_rf, J, ctx->cfg.num_nodes, ctx->d_pen);
+    penalty_prep_kernel<<<(J * 32 + 255) / 256, 256, 0, ctx->stream>>>(d_cur, d_rf, J, ctx->cfg.num_nodes, ctx->d_pen,
+                                                                       ctx->d_cur_nz);
   }
   SCHED_LAUNCH_CHECK(ctx);
   return SCHED_OK;
 }
 
+// d_speedup_rack: table of rows whose occupied nodes lie in two or more racks, or NULL (one rack)
 int launch_fitness(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
                    const int16_t *d_cur, const float *d_rf, const uint8_t *d_active, float p,
-                   float *d_fitness, const uint32_t *d_summ) {
+                   float *d_fitness, const uint32_t *d_summ, const float *d_speedup_rack) {
   const sched_config &c = ctx->cfg;
   const int J = c.num_jobs;
   if (count == 0) return SCHED_OK;
@@ -338,110 +435,36 @@ int launch_fitness(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const fl
     SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(d_fitness, 0, (size_t)count * sizeof(float), ctx->stream));
     return SCHED_OK;
   }
-
-  const bool penalise = d_cur && d_rf;
-  if (penalise && J > 0 && !ctx->pen_ready) {
-    {
-    TimedLaunch tl_(ctx, KK_PENPREP);
-    penalty_prep_kernel<<<(J * 32 + 255) / 256, 256, 0, ctx->stream>>>(d_cur, d_rf, J, c.num_nodes,
-                                                                       ctx->d_pen);
-    }
-    SCHED_LAUNCH_CHECK(ctx);
-  }
-
-  int W, lpr_log2, rows_per_block, chunks;
-  fitness_geometry((size_t)c.num_nodes * 2, (uintptr_t)d_pop | (penalise ? (uintptr_t)d_cur : 0), J, count,
-                   ctx->num_sms, W, lpr_log2, rows_per_block, chunks);
+  int lpr_log2, rows_per_block, chunks;
+  fitness_geometry((size_t)c.num_nodes * 2, J, count, ctx->num_sms, lpr_log2, rows_per_block, chunks);
   int rc = ensure_fitness_scratch(ctx, count, chunks);
   if (rc != SCHED_OK) return rc;
+  const bool penalise = d_cur && d_rf, prep = penalise && !ctx->pen_ready;
+  if (prep && (rc = launch_penalty_prep(ctx, d_cur, d_rf)) != SCHED_OK) return rc;
 
-  FitnessArgs a;
-  a.pop = d_pop;
+  FitnessArgs a = {};
   a.cur = penalise ? d_cur : nullptr;
   a.table = d_speedup;
+  a.table_rack = d_speedup_rack; a.rack = d_speedup_rack ? ctx->d_rack : nullptr;
   a.pen = penalise ? ctx->d_pen : nullptr;
+  a.cur_nz = ctx->d_cur_nz;
   a.active = d_active;
-  a.summ = d_summ;
   a.J = J; a.num_nodes = c.num_nodes; a.k_max = c.k_max; a.n_max = c.n_max;
   a.lpr_log2 = lpr_log2;
   a.rows_per_block = rows_per_block; a.chunks = chunks;
   a.p = p; a.floor_ = c.speedup_floor;
   a.mode = fitness_mode(p);
-  a.partial = ctx->d_partial;
-  a.ticket = ctx->d_ticket;
-  a.fitness = d_fitness;
-
   // grid.y is limited to 65535 candidates per launch
   for (int32_t first = 0; first < count; first += 65535) {
     const int32_t n = (count - first < 65535) ? (count - first) : 65535;
-    FitnessArgs b = a;
-    b.pop = d_pop + (size_t)first * J * c.num_nodes;
-    b.partial = ctx->d_partial + (size_t)first * chunks * 2;
-    b.ticket = ctx->d_ticket + first;
-    b.fitness = d_fitness + first;
-    if (d_summ) b.summ = d_summ + (size_t)first * J;
-    dim3 grid((unsigned)chunks, (unsigned)n);
-    {
-    TimedLaunch tl_(ctx, KK_FITNESS);
-    if (d_summ) fitness_summary_kernel<<<grid, 256, 0, ctx->stream>>>(b);
-    else
-    switch (W) {
-      case 16: fitness_kernel<16><<<grid, 256, 0, ctx->stream>>>(b); break;
-      case 8: fitness_kernel<8><<<grid, 256, 0, ctx->stream>>>(b); break;
-      case 4: fitness_kernel<4><<<grid, 256, 0, ctx->stream>>>(b); break;
-      default: fitness_kernel<2><<<grid, 256, 0, ctx->stream>>>(b); break;
-    }
-    }
-    SCHED_LAUNCH_CHECK(ctx);
-  }
-  return SCHED_OK;
-}
-
-int launch_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
-                         const float *d_speedup_rack, const int16_t *d_cur, const float *d_rf,
-                         const uint8_t *d_active, float p, float *d_fitness) {
-  const sched_config &c = ctx->cfg;
-  const int J = c.num_jobs;
-  if (count == 0) return SCHED_OK;
-  if (J == 0) {     // the mean over no jobs: 0 by definition
-    SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(d_fitness, 0, (size_t)count * sizeof(float), ctx->stream));
-    return SCHED_OK;
-  }
-  const bool penalise = d_cur && d_rf;
-  if (penalise && J > 0 && !ctx->pen_ready) {
-    int rc = launch_penalty_prep(ctx, d_cur, d_rf);
-    if (rc != SCHED_OK) return rc;
-  }
-  int W, lpr_log2, rows_per_block, chunks;
-  fitness_geometry((size_t)c.num_nodes * 2, 0, J, count, ctx->num_sms, W, lpr_log2, rows_per_block, chunks);
-  int rc = ensure_fitness_scratch(ctx, count, chunks);
-  if (rc != SCHED_OK) return rc;
-  FitnessArgs a;
-  a.pop = d_pop;
-  a.cur = penalise ? d_cur : nullptr;
-  a.table = d_speedup;
-  a.pen = penalise ? ctx->d_pen : nullptr;
-  a.active = d_active;
-  a.summ = nullptr;
-  a.J = J; a.num_nodes = c.num_nodes; a.k_max = c.k_max; a.n_max = c.n_max;
-  a.lpr_log2 = 0;
-  a.rows_per_block = rows_per_block; a.chunks = chunks;
-  a.p = p; a.floor_ = c.speedup_floor;
-  a.mode = fitness_mode(p);
-  a.partial = ctx->d_partial;
-  a.ticket = ctx->d_ticket;
-  a.fitness = d_fitness;
-  for (int32_t first = 0; first < count; first += 65535) {
-    const int32_t n = (count - first < 65535) ? (count - first) : 65535;
-    FitnessArgs b = a;
-    b.pop = d_pop + (size_t)first * J * c.num_nodes;
-    b.partial = ctx->d_partial + (size_t)first * chunks * 2;
-    b.ticket = ctx->d_ticket + first;
-    b.fitness = d_fitness + first;
-    dim3 grid((unsigned)chunks, (unsigned)n);
+    a.pop = d_pop + (size_t)first * J * c.num_nodes;
+    a.summ = d_summ ? d_summ + (size_t)first * J : nullptr;
+    a.partial = ctx->d_partial + (size_t)first * chunks * 2;
+    a.ticket = ctx->d_ticket + first;
+    a.fitness = d_fitness + first;
     {
       TimedLaunch tl_(ctx, KK_FITNESS);
-      fitness_racks_kernel<<<grid, 256, 0, ctx->stream>>>(b, d_speedup_rack, ctx->d_rack);
+      SCHED_CUDA_CHECK(ctx, launch_fitness_kernel(a, n, ctx->num_sms, prep && first == 0, ctx->stream));
     }
     SCHED_LAUNCH_CHECK(ctx);
   }
@@ -468,6 +491,7 @@ struct NoAllocScratch {
   double partial[NOALLOC_MAX_PARTIALS * 2];
   unsigned int ticket[NOALLOC_MAX_COUNT];
   float pen[NOALLOC_MAX_JOBS];
+  int32_t cur_nz[NOALLOC_MAX_JOBS];
 };
 
 // Lives in every GPU that loads the library, from load to exit (about 2.2 MB).  In host code
@@ -540,24 +564,23 @@ int eval_fitness_noalloc(const int16_t *d_pop, int32_t count, int32_t num_jobs, 
   const bool penalise = d_cur && d_realloc_factor;
   if (penalise) {
     penalty_prep_kernel<<<(J * 32 + 255) / 256, 256, 0, stream>>>(d_cur, d_realloc_factor, J, num_nodes,
-                                                                 scratch->pen);
+                                                                 scratch->pen, scratch->cur_nz);
     e = cudaGetLastError();
     if (e != cudaSuccess) return noalloc_fail(SCHED_ERR_CUDA, "penalty_prep_kernel launch", e);
   }
 
-  int W, lpr_log2, rows_per_block, chunks;
-  fitness_geometry((size_t)num_nodes * 2, (uintptr_t)d_pop | (penalise ? (uintptr_t)d_cur : 0), J, count,
-                   g_noalloc_sms[device], W, lpr_log2, rows_per_block, chunks);
+  int lpr_log2, rows_per_block, chunks;
+  fitness_geometry((size_t)num_nodes * 2, J, count, g_noalloc_sms[device], lpr_log2, rows_per_block, chunks);
   if ((size_t)count * (size_t)chunks > NOALLOC_MAX_PARTIALS)   // cannot happen within the limits above
     return noalloc_fail(SCHED_ERR_TOO_LARGE, "eval_fitness_noalloc: chunk sums exceed the scratch array");
 
-  FitnessArgs a;
+  FitnessArgs a = {};
   a.pop = d_pop;
   a.cur = penalise ? d_cur : nullptr;
   a.table = d_speedup;
   a.pen = penalise ? scratch->pen : nullptr;
   a.active = d_active;
-  a.summ = nullptr;
+  a.cur_nz = scratch->cur_nz;
   a.J = J; a.num_nodes = num_nodes; a.k_max = k_max; a.n_max = n_max;
   a.lpr_log2 = lpr_log2;
   a.rows_per_block = rows_per_block; a.chunks = chunks;
@@ -566,14 +589,7 @@ int eval_fitness_noalloc(const int16_t *d_pop, int32_t count, int32_t num_jobs, 
   a.partial = scratch->partial;
   a.ticket = scratch->ticket;
   a.fitness = d_fitness;
-  dim3 grid((unsigned)chunks, (unsigned)count);
-  switch (W) {
-    case 16: fitness_kernel<16><<<grid, 256, 0, stream>>>(a); break;
-    case 8: fitness_kernel<8><<<grid, 256, 0, stream>>>(a); break;
-    case 4: fitness_kernel<4><<<grid, 256, 0, stream>>>(a); break;
-    default: fitness_kernel<2><<<grid, 256, 0, stream>>>(a); break;
-  }
-  e = cudaGetLastError();
+  e = launch_fitness_kernel(a, count, g_noalloc_sms[device], penalise, stream);
   if (e != cudaSuccess) return noalloc_fail(SCHED_ERR_CUDA, "fitness_kernel launch", e);
   return SCHED_OK;
 }

@@ -147,3 +147,23 @@ def test_stress_workload_full_row_size(gpu, oracle, p):
     assert np.all(got > 0) and np.all(np.isfinite(got))
     rows = pop[0].to(torch.int64)
     assert int((rows > 0).sum(-1).max()) <= 64 and float((rows.sum(-1) == 0).float().mean()) > 0.4
+
+
+@pytest.mark.parametrize("nodes,P,J,skew", [
+    (1, 3, 1, 1),         # less than a vector
+    (5, 4, 517, 3),       # vectors of up to three rows; rows in three blocks
+    (8, 2, 256, 7),       # whole vectors, the run off by one entry
+    (33, 3, 513, 0),      # a last block of one row
+    (9, 660, 70, 5),      # more blocks than four to an SM
+])
+def test_flat_rows(gpu, oracle, nodes, P, J, skew):
+    torch, _ = gpu
+    cl, table, pop, cur, rf, active = _case(nodes + P, P=P, J=J, nodes=nodes, density=0.4)
+    flat = torch.full((pop.size + 16,), 9, dtype=torch.int16, device="cuda:0")   # neighbours that must not be read as entries
+    flat[skew:skew + pop.size] = torch.from_numpy(pop.reshape(-1)).to("cuda:0")
+    moved = flat[skew:skew + pop.size].view(P, J, nodes)
+    for c, r in ((cur, rf), (None, None)):
+        got = _run(gpu, moved, table, cl.node_capacity, -1.0, cur=c, rf=r, active=active)
+        ref = oracle.eval_fitness(pop, table.astype(np.float64), cl.k_max, cl.n_max, -1.0, 1e-3, cur=c,
+                                  realloc=None if r is None else r.astype(np.float64), active=active)
+        assert_close(got, ref, what="fitness of %d x %d x %d at %d" % (P, J, nodes, skew))
