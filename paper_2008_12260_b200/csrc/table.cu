@@ -710,26 +710,30 @@ int launch_autoscale(sched_ctx *ctx, const float *d_goodput, const int32_t *d_cu
   return SCHED_OK;
 }
 
-// A cluster of blocks per job: one block where the jobs alone give every SM two, more where they do
-// not, up to eight (large tables of few jobs gain as much as their sweep: each block writes its share of
-// the slab).  A (K, class) is shared by two threads where jobs are many - a block's pairs then fill
-// its warps better - and by up to eight where they are few.
+// A cluster of blocks per job: one block where the jobs alone give every SM two or where a job's (K, class)
+// pairs fill no more than one, more otherwise, up to eight (large tables of few jobs gain as much as their
+// sweep: each block writes its share of the slab).  A pair is shared by up to eight threads while all of
+// them fit the GPU at once (registers: some 1170 threads per SM).  At least four warps, whatever the pairs
+// are: pairs with several close points are spread over them (700 jobs x 11 pairs x 87 samples: 28.7 us
+// with one warp and two threads per pair, 16.5 us).
 static int launch_table(sched_ctx *ctx, void (*kernel)(TableArgs), TableArgs &a) {
   const int J = ctx->cfg.num_jobs;
   for (int j0 = 0; j0 < J; j0 += 65536) {
     const int jobs = std::min(65536, J - j0);
     int nb = 1;
-    while (nb < 8 && jobs * nb < 2 * ctx->num_sms) nb *= 2;
+    while (nb < 8 && jobs * nb < 2 * ctx->num_sms && a.pair_count * MAX_PARTS > 128 * nb) nb *= 2;
     const int pairs = std::max(1, (a.pair_count + nb - 1) / nb);
     // (at least two: the second evaluates a second point)
-    int parts = jobs * nb >= 4 * ctx->num_sms ? 2 : MAX_PARTS;
-    while (parts > 2 && (a.G < 4 * parts || pairs * parts > 512)) parts /= 2;
+    int parts = MAX_PARTS;
+    while (parts > 2 && (a.G < 4 * parts || pairs * parts > 512 ||
+                         (long long)jobs * nb * pairs * parts > 1024LL * ctx->num_sms))
+      parts /= 2;
     while (parts < MAX_PARTS && (a.G + parts - 1) / parts > (1 << IDX_BITS)) parts *= 2;
     const int ppp = (((a.G + parts - 1) / parts) + 3) & ~3;
     a.parts = parts;
     a.points = a.G <= MAX_POINTS ? ppp * parts : 0;
     a.j_first = j0;
-    const int threads = std::min(512, (pairs * parts + 31) & ~31);
+    const int threads = std::max(128, std::min(512, (pairs * parts + 31) & ~31));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(jobs * nb));
     lc.blockDim = dim3((unsigned)threads);
