@@ -724,6 +724,7 @@ int schedule_round(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_cu
     ctx->d_fit = ctx->graph_fit;
     ctx->d_pop_last = ctx->graph_pop_last;
     ctx->rs_ptr_last = ctx->graph_ptr_last;
+    ctx->fl_generations = generations;      // (the key's: which of the kept generations is the last one)
     return SCHED_OK;
   }
   const bool capture = graphs_ok && ctx->seen_valid && same_round_key(key, ctx->seen_key);

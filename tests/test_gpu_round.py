@@ -200,6 +200,43 @@ def test_graph_replay_gives_the_same_rounds(gpu):
     assert len({r[1] for r in outs[True][0]}) > 1    # the round number reaches the kernels
 
 
+@pytest.mark.parametrize("counts", [(100, 50), (7, 6), (4, 8), (3, 0)], ids=str)
+def test_population_after_replayed_rounds_of_two_lengths(gpu, counts):
+    """A graph holds one generation count; a round of another count runs plainly and leaves the graph
+    standing.  The population handed out after the next replay must be the replayed round's, with its
+    fitness, whatever ran in between."""
+    torch, api = gpu
+    cfg = synth.TINY
+    cl, jobs = setup(cfg)
+    cur = cfg.cur()
+    a, b = counts
+    outs = {}
+    for graphs in (False, True):
+        st = torch.cuda.Stream()
+        s = api.scheduler_for(cfg, stream=st.cuda_stream)
+        s.set_graphs(graphs)
+        dj = api.DeviceJobs(jobs, "cuda:0", torch)
+        d_cur = torch.from_numpy(cur).cuda()
+        best = torch.empty((cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
+        bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
+        pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
+        fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")
+        torch.cuda.synchronize()
+        res = []
+        for rnd, gens in enumerate((a, a, a, b, a, b, b, b, a, b)):
+            s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=gens)
+            s.get_population(pop, fit)
+            s.sync_status()
+            res.append([x.cpu().numpy().copy() for x in (pop, fit, best, bf)])
+        outs[graphs] = res
+        s.close()
+    for k, (plain, replayed) in enumerate(zip(outs[False], outs[True])):
+        for x, y in zip(plain, replayed):
+            assert np.array_equal(x, y), "round %d" % k
+        pop, fit, best, bf = replayed
+        assert np.array_equal(pop[int(np.argmax(fit))], best) and fit.max() == bf[0]
+
+
 def test_graph_survives_scratch_reallocation(gpu):
     """A captured round holds raw scratch pointers; a later call that makes the context grow
     its scratch must not leave a stale graph behind."""
