@@ -46,7 +46,7 @@ CONFIG = {
     "per_rank": "one independent cluster per rank",
     "arithmetic": "int16 matrices, fp32 tables and fitness on the GPU (the oracle computes in fp64)",
     "l2": "every round rebuilds its 17 MB tables and a fresh population; inside a round the generations work on "
-          "the row store (records + indices, about 40 MB), L2-resident by design; the single-kernel sections flush "
+          "32-byte row records (17 MB each, four kept in turn), L2-resident by design; the single-kernel sections flush "
           "L2 or stream more than L2 per pass",
 }
 
@@ -57,8 +57,8 @@ CONFIG = {
 # written: some parent rows are shared by several children and come from L2).
 # "fitness_stress": 16 dense stress candidates moved 544.8 + 3.5 MB; every candidate is streamed
 # once, so the figure is scaled by candidates / 16 to the chunk that is timed.
-# "generation_store": no counters of the one-launch search yet.
-NCU_TRAFFIC_BYTES = {"rows": 461.4e6, "fitness_stress_per_candidate": 548.3e6 / 16, "generation_store": None}
+# "round_search": its records stay in L2; what it moves to and from DRAM has not been counted.
+NCU_TRAFFIC_BYTES = {"rows": 461.4e6, "fitness_stress_per_candidate": 548.3e6 / 16, "round_search": None}
 
 
 def measured_peaks():
@@ -286,8 +286,7 @@ def run_ours(args):
     units = float(P) * (G + 1) * args.steps
     value, t_max, u_sum = pdist.throughput(elapsed_ms, units, device=dev)
     # The generation kernel inside the clean region: rounds of G and of G / 2 generations, both
-    # replayed as graphs, differ by G / 2 generations (kernel, launch gap and the compaction
-    # checks that fall among them) and by nothing else.
+    # replayed as graphs, differ by G / 2 generations of the one launch and by nothing else.
     def clean_round_ms(gens):
         for k in range(3):                                  # plain, capture, first replay
             sched.schedule_round(dj, d_cur, d_best, d_bf, round=200 + k, generations=gens)
@@ -301,7 +300,6 @@ def run_ours(args):
     half_ms = clean_round_ms(G // 2)
     full_ms = clean_round_ms(G)
     gen_us_clean = 1e3 * (full_ms - half_ms) / (G - G // 2)
-    moves = sched.store_moves()
 
     # ---- end to end through the host-buffer entry point (pinned host memory) -------------
     hj = api.HostJobs(jobs, torch)
@@ -330,7 +328,7 @@ def run_ours(args):
         "rows": 2 * pop_bytes + P * J * 5 + J * NN * 2,
         # the round's search is one launch of G + 1 generations: per generation and (candidate, job) a
         # 32-byte record in and one out, and the candidate's fitness
-        "generation_store": (G + 1) * (float(P) * J * (32 + 32) + 4 * P),
+        "round_search": (G + 1) * (float(P) * J * (32 + 32) + 4 * P),
     }
     kernels = []
     for name, (ms, n) in sorted(kernel_ms.items(), key=lambda kv: -kv[1][0]):
@@ -345,15 +343,15 @@ def run_ours(args):
         kernels.append(k)
     dom = next((k for k in kernels if "achieved_gbs" in k), None)
     roofline = None
-    if dom and dom["kernel"] == "generation_store":
+    if dom and dom["kernel"] == "round_search":
         # the dominant kernel, timed inside the clean region (see clean_round_ms above); the
         # per-kernel pass only gives the shares
         gen_bytes = dom["algorithmic_bytes"] / (G + 1)
         gbs = gen_bytes / (gen_us_clean * 1e-6) / 1e9
-        roofline = {"kernel": "generation_store", "bound": "hbm", "achieved": round(gbs, 1), "peak": hbm_peak,
+        roofline = {"kernel": "round_search", "bound": "hbm", "achieved": round(gbs, 1), "peak": hbm_peak,
                     "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peak_src == "measured" else "recipe fallback",
                     "unit": "GB/s", "frac": round(gbs / hbm_peak, 4),
-                    "traffic": NCU_TRAFFIC_BYTES.get("generation_store"),
+                    "traffic": NCU_TRAFFIC_BYTES.get("round_search"),
                     "algorithmic_bytes_per_generation": gen_bytes,
                     "generation_us": round(gen_us_clean, 2),
                     "generation_us_how": "(round of %d generations - round of %d) / %d, both replayed as graphs in a "
@@ -390,7 +388,7 @@ def run_ours(args):
         "kernel_timing": {"how": "second pass over the same steps with a CUDA-event pair around every kernel (no "
                                  "graph replay, no overlap between consecutive kernels): shares only",
                           "ms_per_step": profiled_ms / args.steps},
-        "row_store": {"pool_moves_so_far": moves, "clean_round_ms": full_ms, "clean_half_round_ms": half_ms},
+        "clean_rounds": {"ms": full_ms, "half_the_generations_ms": half_ms},
         "best_fitness": float(h_bf.item()),
         "best_allocation": allocation_summary(h_best.numpy(), jobs, cl),
     }
@@ -414,7 +412,7 @@ def run_ours(args):
 
 
 def bench_dense_generation(api, torch, dev, stream, cfg, cl, jobs, cur, hbm_peak, peak_src):
-    """ga_generation on dense matrices (the entry point; a round of this size uses the row store
+    """ga_generation on dense matrices (the entry point; a round of this size works on row records
     instead): the row pass streams 268 MB of parents in and 268 MB of children out."""
     P, J, NN = cfg.population, cfg.num_jobs, cfg.num_nodes
     sched = api.scheduler_for(cfg, stream=stream.cuda_stream)
@@ -492,12 +490,11 @@ def bench_table(api, torch, dev, stream, cfg, cl, jobs, sm_max_mhz, clocks):
         flush.fill_(1)
         sched.build_speedup_table_msample(dj, ms, mm, gp, sp, am)
     t2 = sched.read_kernel_timing()
-    msample_ms = t2["goodput_sweep"][0] / reps
+    msample_ms = t2["speedup_table"][0] / reps
     sched.set_kernel_timing(False)
     fma_peak, mufu_peak, _ = sched.measure_peaks(None, reps=5)
     sched.close()
-    sweep_ms = t["goodput_sweep"][0] / reps
-    expand_ms = t["speedup_expand"][0] / reps
+    sweep_ms = t["speedup_table"][0] / reps
     classes = distinct_classes(cl)
     points = float(cfg.num_jobs) * classes * cfg.grid_m * cfg.grid_s
     num_sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -520,13 +517,11 @@ def bench_table(api, torch, dev, stream, cfg, cl, jobs, sm_max_mhz, clocks):
         oracle.set_threads(0)
     return {
         "workload": "large", "distinct_points": points, "sweep_us": round(sweep_ms * 1e3, 2),
-        "expand_us": round(expand_ms * 1e3, 2),
-        "evals_per_sec": points / ((sweep_ms + expand_ms) * 1e-3),
-        "evals_per_sec_sweep_only": points / (sweep_ms * 1e-3),
+        "evals_per_sec": points / (sweep_ms * 1e-3),
         "msample_search": {"candidates_per_job": 128, "sweep_us": round(msample_ms * 1e3, 2),
                            "evals_per_sec": float(cfg.num_jobs) * classes * 128 / (msample_ms * 1e-3),
                            "note": "integer (m, s) derivation + 3 MUFU per candidate; latency-sized at this size"},
-        "roofline": {"kernel": "goodput_sweep", "bound": "special-function unit", "achieved": mufu_ops / (sweep_ms * 1e-3) / 1e12,
+        "roofline": {"kernel": "speedup_table", "bound": "special-function unit", "achieved": mufu_ops / (sweep_ms * 1e-3) / 1e12,
                      "peak": mufu_peak / 1e12, "unit": "T op/s", "frac": mufu_ops / mufu_peak / (sweep_ms * 1e-3),
                      "peak_source": "lg2 / ex2 chains, same process (nominal %.2f)" % (num_sms * 16 * sm_max_mhz * 1e6 / 1e12),
                      "output_bytes": out_bytes, "output_floor_us": out_bytes / (hbm_peak * 1e9) * 1e6,

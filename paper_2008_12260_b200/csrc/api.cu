@@ -429,10 +429,10 @@ int eval_fitness_racks(sched_ctx *ctx, const int16_t *d_pop, int32_t count, cons
 int sched_num_kernel_kinds(void) { return KK_COUNT; }
 
 const char *sched_kernel_kind_name(int kind) {
-  static const char *names[KK_COUNT] = {"goodput_sweep", "speedup_expand", "realloc_factor",
-                                        "penalty_prep", "fitness", "rank", "rows", "cols",
-                                        "best_index", "copy_best", "colscan", "fit_theta",
-                                        "generation_store", "store_build", "store_compact", "store_gather"};
+  static const char *names[KK_COUNT] = {"speedup_table", "realloc_factor", "penalty_prep", "fitness", "rank", "rows", "cols",
+                                        "best_index", "copy_best", "fit_theta", "round_build", "round_search",
+                                        "round_finish", "round_gather", "generation_store", "store_build",
+                                        "store_compact", "store_gather"};
   return (kind >= 0 && kind < KK_COUNT) ? names[kind] : "";
 }
 

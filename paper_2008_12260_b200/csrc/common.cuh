@@ -20,8 +20,9 @@
 
 // kernel classes, for launch accounting and optional per-kernel timing
 enum KernelKind {
-  KK_SWEEP = 0, KK_EXPAND, KK_REALLOC, KK_PENPREP, KK_FITNESS, KK_RANK, KK_ROWS, KK_COLS, KK_BEST,
-  KK_COPY, KK_COLSCAN, KK_FIT, KK_GENSTORE, KK_STORE_BUILD, KK_STORE_COMPACT, KK_STORE_GATHER, KK_COUNT
+  KK_TABLE = 0, KK_REALLOC, KK_PENPREP, KK_FITNESS, KK_RANK, KK_ROWS, KK_COLS, KK_BEST, KK_COPY, KK_FIT,
+  KK_FLOW_BUILD, KK_FLOW, KK_FLOW_FINISH, KK_FLOW_GATHER, KK_GENSTORE, KK_STORE_BUILD, KK_STORE_COMPACT,
+  KK_STORE_GATHER, KK_COUNT
 };
 
 struct TimedSpan {

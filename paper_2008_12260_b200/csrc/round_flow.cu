@@ -1406,7 +1406,7 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   a.generations = generations;
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
-    TimedLaunch tl_(ctx, KK_STORE_BUILD);
+    TimedLaunch tl_(ctx, KK_FLOW_BUILD);
     flow_build_kernel<<<(c.num_jobs + 3) / 4, 128, 0, ctx->stream>>>(a);
   }
   SCHED_LAUNCH_CHECK(ctx);
@@ -1421,12 +1421,12 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   lc.attrs = attr;
   lc.numAttrs = 1;
   {
-    TimedLaunch tl_(ctx, KK_GENSTORE);
+    TimedLaunch tl_(ctx, KK_FLOW);
     SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, flow_kernel, a));
   }
   SCHED_LAUNCH_CHECK(ctx);
   {
-    TimedLaunch tl_(ctx, KK_BEST);
+    TimedLaunch tl_(ctx, KK_FLOW_FINISH);
     flow_finish_kernel<<<std::min((c.num_jobs + 7) / 8, ctx->num_sms), 256, 0, ctx->stream>>>(a);
   }
   SCHED_LAUNCH_CHECK(ctx);
@@ -1439,7 +1439,7 @@ int flow_gather(sched_ctx *ctx, int16_t *d_out) {
   const sched_config &c = ctx->cfg;
   const long long want = ((long long)c.population * c.num_jobs + 7) / 8;
   {
-    TimedLaunch tl_(ctx, KK_STORE_GATHER);
+    TimedLaunch tl_(ctx, KK_FLOW_GATHER);
     flow_gather_kernel<<<(unsigned)std::min<long long>(want, (long long)ctx->num_sms * 8), 256, 0, ctx->stream>>>(
         flow_arena(ctx, (char *)ctx->fl_arena).r, c.population, c.num_jobs, c.num_nodes, ctx->fl_generations, d_out);
   }

@@ -748,7 +748,7 @@ static int launch_table(sched_ctx *ctx, void (*kernel)(TableArgs), TableArgs &a)
     if (lc.dynamicSmemBytes > 48 * 1024)
       SCHED_CUDA_CHECK(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes));
     {
-      TimedLaunch tl_(ctx, KK_SWEEP);
+      TimedLaunch tl_(ctx, KK_TABLE);
       SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, kernel, a));
     }
     SCHED_LAUNCH_CHECK(ctx);

@@ -53,6 +53,18 @@ def check_table(oracle, jobs, grid_s, gp_gpu, sp_gpu, am_gpu, gp_ref, sp_ref, am
     return len(diff)
 
 
+def store_budget(cfg):
+    """A budget (set_store_budget) under which a round of this size keeps its rows in the row pool: room for
+    two worst-case generations in each half.  The four generations that the one-launch search keeps do not
+    fit it once there are more than about 40 jobs."""
+    stride = (cfg.num_nodes + 7) // 8 * 8
+    rows = max(cfg.population, 2) * cfg.num_jobs
+    worst = cfg.population * (cfg.num_jobs + 16)
+    budget = 2 * (stride * 2 + 32) * (rows + 2 * worst + 64)
+    assert 8 * cfg.population * cfg.num_jobs * (stride * 2 + 32) > budget, "the one-launch search fits this budget"
+    return budget
+
+
 def feasible(A, cap, k_cap, n_max):
     A = A.astype(np.int64)
     occ = A > 0

@@ -3,7 +3,7 @@ feasible, consistent with the oracle's fitness, and the host-buffer variant."""
 import numpy as np
 import pytest
 
-from helpers import REL_TOL, assert_close, feasible, setup
+from helpers import REL_TOL, assert_close, feasible, setup, store_budget
 from paper_2008_12260_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -265,6 +265,29 @@ def test_graph_survives_scratch_reallocation(gpu):
         s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=6)
         s.sync_status()
         assert np.array_equal(best.cpu().numpy(), ref[rnd][0]) and float(bf.item()) == ref[rnd][1]
+    s.close()
+
+
+@pytest.mark.parametrize("route,search", [("default", "round_search"), ("store", "generation_store"), ("dense", "rows")])
+def test_kernel_timing_names_the_kernels_that_ran(gpu, route, search):
+    torch, api = gpu
+    cfg = synth.TESTBED
+    cl, jobs = setup(cfg)
+    s = api.scheduler_for(cfg, stream=torch.cuda.Stream().cuda_stream)
+    if route != "default":
+        s.set_store_budget(store_budget(cfg) if route == "store" else 0)
+    dj = api.DeviceJobs(jobs, "cuda:0", torch)
+    d_cur = torch.from_numpy(cfg.cur()).cuda()
+    best = torch.empty((cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
+    bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
+    torch.cuda.synchronize()
+    s.set_kernel_timing(True)
+    s.schedule_round(dj, d_cur, best, bf, round=0, generations=6)
+    s.sync_status()
+    ran = {name: n for name, (ms, n) in s.read_kernel_timing().items() if n}
+    assert ran["speedup_table"] == 1
+    assert [k for k in ("round_search", "generation_store", "rows") if k in ran] == [search]
+    assert ran[search] == (1 if route == "default" else 7)         # the search, or a launch per population
     s.close()
 
 
