@@ -65,6 +65,13 @@ def store_budget(cfg):
     return budget
 
 
+def check_route(s, route):
+    """What a round ran on, from the kernel timing that was on meanwhile ("flow": the one-launch search,
+    "store": the row pool)."""
+    ran = {name for name, (ms, n) in s.read_kernel_timing().items() if n}
+    assert ("round_search" in ran, "generation_store" in ran, "rows" in ran) == (route == "flow", route == "store", False)
+
+
 def feasible(A, cap, k_cap, n_max):
     A = A.astype(np.int64)
     occ = A > 0

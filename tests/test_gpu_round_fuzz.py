@@ -1,5 +1,5 @@
-"""Randomly drawn problem shapes through a whole round: the round's specialised kernels (row store,
-thread-per-row kernel, fused batched kernel) against the same round made of the dense entry points
+"""Randomly drawn problem shapes through a whole round: the round's specialised kernels (the one-launch
+search, the row store) against the same round made of the dense entry points
 called one by one - populations and fitness bit for bit - and the last generation against the
 oracle.  Shapes, probabilities, the current allocation (none / feasible / breaking every rule),
 inactive jobs and small replica caps all vary with the seed.  POLLUX_FUZZ_CASES raises the number
@@ -9,7 +9,7 @@ import os
 import numpy as np
 import pytest
 
-from helpers import assert_close, feasible, with_fair_share
+from helpers import assert_close, check_route, feasible, store_budget, with_fair_share
 from paper_2008_12260_b200 import synth
 from test_gpu_round_kernels import _stepwise
 
@@ -23,9 +23,9 @@ def draw_case(seed):
     nodes = int(g.choice([8, 16, 24, 32, 40, 64, 128, 256]))
     gpn = int(g.choice([1, 2, 4, 8, 16, 96]))
     if g.uniform() < 0.35 and nodes <= 32:
-        jobs = int(g.integers(3, 257))            # thread-per-row kernel
+        jobs = int(g.integers(3, 257))            # the child's records in shared memory, too
     else:
-        jobs = int(g.integers(257, 900))          # row store
+        jobs = int(g.integers(257, 900))
     cfg = synth.Config("fuzz-%d" % seed, nodes, gpn, jobs, 5000 + seed, 16, 8, int(g.integers(6, 40)),
                        int(g.integers(2, 12)), p=float(g.choice([-1.0, -1.0, 0.5, 1.0, 0.0])),
                        num_elite=int(g.integers(0, 4)), mutate_prob=float(g.choice([0.02, 0.1, 0.3, 0.7, 1.0])),
@@ -43,10 +43,13 @@ def gpu():
     return torch, api
 
 
+@pytest.mark.parametrize("route", ["flow", "store"])
 @pytest.mark.parametrize("seed", range(N_CASES))
-def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed):
+def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed, route):
     torch, api = gpu
     cfg, kind, g = draw_case(seed)
+    if route == "store" and cfg.num_jobs <= 48:
+        pytest.skip("four generations of so few rows fit any budget the row pool fits")
     cl = cfg.cluster()
     jobs = cfg.jobs()
     if g.uniform() < 0.5:
@@ -66,12 +69,17 @@ def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed):
     penalise = cur is not None
     rnd = int(g.integers(0, 5))
     s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
+    if route == "store":
+        s.set_store_budget(store_budget(cfg))
+    s.set_kernel_timing(True)
     dj = api.DeviceJobs(jobs, "cuda:0", torch)
     d_cur = None if cur is None else torch.from_numpy(cur).cuda()
     best = torch.full((cfg.num_jobs, cfg.num_nodes), -1, dtype=torch.int16, device="cuda:0")
     bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
     s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=cfg.generations)
     s.sync_status()
+    check_route(s, route)
+    s.set_kernel_timing(False)
     pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
     fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")
     s.get_population(pop, fit)

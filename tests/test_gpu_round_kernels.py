@@ -1,6 +1,6 @@
-"""Inside a round the generations run on specialised kernels: problems with more than 256 jobs
-keep their population as shared rows (indices into a row pool, copy on write), problems with
-at most 256 jobs and 32 nodes use a thread-per-row kernel.  Either way the round must equal,
+"""Inside a round the generations run on specialised kernels: one launch that keeps four generations of
+row records, or, where a budget leaves no room for those, shared rows (indices into a row pool, copy
+on write; a launch per generation).  Every case runs on both.  Either way the round must equal,
 bit for bit, the same round made of the dense entry points called one by one, which the other
 tests pin to the oracle; the last generation is also checked against the oracle directly
 (teacher-forced)."""
@@ -9,7 +9,7 @@ import dataclasses
 import numpy as np
 import pytest
 
-from helpers import REL_TOL, assert_close, feasible, setup
+from helpers import REL_TOL, assert_close, check_route, feasible, setup, store_budget
 from paper_2008_12260_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -17,19 +17,20 @@ pytestmark = pytest.mark.gpu
 # name, nodes, GPUs per node, jobs, seed, grid, population, generations, mutation, what it exercises
 CASES = [
     # half of the rows perturbed per generation: the pool's half in use fills up and the live
-    # rows move to the other half several times
+    # rows move to the other half several times (the budget of all cases leaves room for two worst-case
+    # generations per half)
     synth.Config("store-compaction", 32, 8, 300, 11, 16, 8, 48, 24, num_elite=3, mutate_prob=0.5,
                  init_prob=0.3, with_history=True, random_cur=True),
-    # every row perturbed in every generation and a pool with room for two worst-case generations only:
-    # a candidate may take its full J + 16 slots per generation without the pool running out
+    # every row perturbed in every generation: a candidate may take its full J + 16 slots per generation
+    # without the pool running out
     synth.Config("store-all-perturbed", 16, 4, 280, 21, 16, 8, 20, 10, num_elite=1, mutate_prob=1.0,
                  init_prob=1.0, with_history=True, random_cur=True),
     # a current allocation that breaks every rule (node sizes, replica caps, interference) on large
     # nodes: rows hold more GPUs before the row caps than a summary can say
     synth.Config("store-infeasible-current", 8, 1500, 300, 22, 16, 8, 24, 6, num_elite=2, mutate_prob=0.3,
                  init_prob=0.6, with_history=True, random_cur=False),
-    # few large nodes: more jobs on a node than a block lists per node (column scan through the
-    # indices), and many GPUs per job
+    # few large nodes: more jobs on a node than a block lists per node (the block walks the
+    # column), and many GPUs per job
     synth.Config("store-crowded-nodes", 8, 64, 400, 12, 16, 8, 32, 12, num_elite=2, mutate_prob=0.3,
                  init_prob=0.5, with_history=True, random_cur=True),
     # many small nodes and frequent growth: rows that occupy more nodes than a record holds
@@ -37,7 +38,7 @@ CASES = [
                  init_prob=0.9, with_history=True, random_cur=False),
     # no current allocation, inactive jobs, ragged job count
     synth.Config("store-plain", 16, 8, 257, 14, 16, 8, 20, 6, num_elite=1, mutate_prob=0.1),
-    # the widest rows the store takes (512 nodes: four 16-byte pieces per lane of a row's group)
+    # the widest rows these kernels take (512 nodes: four 16-byte pieces per lane of a row's group in the store)
     synth.Config("store-512-nodes", 512, 2, 600, 15, 16, 8, 12, 10, num_elite=2, mutate_prob=0.2,
                  init_prob=0.3, with_history=True, random_cur=True),
     # rows whose pieces do not fill the lanes evenly (17 pieces), many jobs per candidate
@@ -45,13 +46,13 @@ CASES = [
                  init_prob=0.3, with_history=True, random_cur=True),
     # the large workload itself (the configuration the benchmark times), ten generations
     dataclasses.replace(synth.LARGE, name="store-large", generations=10),
-    # thread-per-row kernel: more jobs on a node than its list holds (column scan in shared memory)
+    # as many jobs as keep their child's records in shared memory, too; crowded nodes
     synth.Config("small-crowded-nodes", 8, 128, 256, 17, 16, 8, 24, 30, num_elite=2, mutate_prob=0.3,
                  init_prob=0.9, with_history=True, random_cur=True),
-    # thread-per-row kernel: the widest rows it takes (32 nodes), row caps at work, inactive jobs
+    # fewer jobs, row caps at work, inactive jobs
     synth.Config("small-32-nodes", 32, 4, 120, 18, 16, 8, 20, 15, num_elite=3, mutate_prob=0.6,
                  init_prob=0.6, with_history=True, random_cur=True),
-    # thread-per-row kernel: three 16-byte pieces per row, no current allocation
+    # three 16-byte pieces per row, no current allocation
     synth.Config("small-24-nodes", 24, 2, 90, 19, 16, 8, 16, 10, num_elite=1, mutate_prob=0.4, init_prob=0.4),
 ]
 
@@ -89,8 +90,9 @@ def _stepwise(torch, s, dj, cfg, d_cur, rnd, gens, penalise):
     return a.cpu().numpy(), f.cpu().numpy(), sp.cpu().numpy(), prev
 
 
+@pytest.mark.parametrize("route", ["flow", "store"])
 @pytest.mark.parametrize("cfg", CASES, ids=lambda c: c.name)
-def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg):
+def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg, route):
     torch, api = gpu
     cl, jobs = setup(cfg)
     if cfg.name in ("store-plain", "small-32-nodes"):
@@ -107,17 +109,17 @@ def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg):
     penalise = cur is not None
     rnd = 3
     s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
-    if cfg.name in ("store-compaction", "store-all-perturbed"):
-        # a pool with room for two worst-case generations per half: the rows have to move every
-        # other generation or so
-        rows, worst = cfg.population * cfg.num_jobs, cfg.population * (cfg.num_jobs + 16)
-        s.set_store_budget(2 * (cfg.num_nodes * 2 + 32) * (rows + 2 * worst + 64))
+    if route == "store":
+        s.set_store_budget(store_budget(cfg))
+    s.set_kernel_timing(True)
     dj = api.DeviceJobs(jobs, "cuda:0", torch)
     d_cur = None if cur is None else torch.from_numpy(cur).cuda()
     best = torch.full((cfg.num_jobs, cfg.num_nodes), -1, dtype=torch.int16, device="cuda:0")
     bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
     s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=cfg.generations)
     s.sync_status()
+    check_route(s, route)
+    s.set_kernel_timing(False)
     pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
     fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")
     s.get_population(pop, fit)
@@ -130,9 +132,9 @@ def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg):
     assert np.array_equal(best.cpu().numpy(), pop[i]) and float(bf.item()) == fit[i]
     for c in range(cfg.population):
         assert feasible(pop[c], cl.node_capacity, jobs.k_cap, cl.n_max)
-    if cfg.name in ("store-compaction", "store-all-perturbed"):
+    if route == "store" and cfg.name in ("store-compaction", "store-all-perturbed"):
         assert s.store_moves() >= 3
-    elif cfg.name.startswith("store-"):
+    elif route == "flow":
         assert s.store_moves() == 0
     if cfg.name == "store-crowded-nodes":
         assert (pop > 0).sum(axis=1).max() > 16      # more jobs on a node than a block lists
@@ -158,7 +160,8 @@ def setup_fair(jobs, cl):
     return with_fair_share(jobs, cl)
 
 
-def test_store_round_replays_as_graph_and_is_reproducible(gpu):
+@pytest.mark.parametrize("route", ["flow", "store"])
+def test_store_round_replays_as_graph_and_is_reproducible(gpu, route):
     torch, api = gpu
     cfg = CASES[0]
     cl, jobs = setup(cfg)
@@ -167,6 +170,8 @@ def test_store_round_replays_as_graph_and_is_reproducible(gpu):
     for graphs in (False, True):
         s = api.scheduler_for(cfg, stream=torch.cuda.Stream().cuda_stream)
         s.set_graphs(graphs)
+        if route == "store":
+            s.set_store_budget(store_budget(cfg))
         dj = api.DeviceJobs(jobs, "cuda:0", torch)
         d_cur = torch.from_numpy(cur).cuda()
         best = torch.empty((cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
