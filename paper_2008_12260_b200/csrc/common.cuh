@@ -184,7 +184,7 @@ extern char g_init_error[256];
 // (first one wins, read by sched_sync_status) and the access is skipped.  Nothing traps.  In the
 // normal build the test compiles away.
 // ---------------------------------------------------------------------------------------
-#define SCHED_CHK_SLOT (-101)     /* a row slot beyond the pool                           */
+#define SCHED_CHK_SLOT (-101)     /* a row slot beyond the pool, a candidate beyond the population */
 #define SCHED_CHK_NODE (-102)     /* a node (or job) number beyond the cluster (the jobs)  */
 #define SCHED_CHK_LIST (-103)     /* a position beyond a block's work list                 */
 #define SCHED_CHK_ENTRY (-104)    /* a position beyond a row's list of occupied nodes      */

@@ -269,7 +269,7 @@ __device__ __forceinline__ const float *list_table(const FlowArgs &a, const uint
   int lo = 0x7fffffff, hi = -1;
 #pragma unroll
   for (int k = 0; k < ENTRIES; ++k)
-    if (e[k] != NO_NODE) {
+    if (e[k] != NO_NODE && sched_index_ok(a.status, entry_node(e[k]) < a.NN, SCHED_CHK_NODE)) {
       const int r = (int)__ldg(a.rack + entry_node(e[k]));
       lo = min(lo, r);
       hi = max(hi, r);
@@ -294,6 +294,7 @@ __device__ __forceinline__ TermLoads list_loads(const FlowArgs &a, const uint32_
     t.hi = __ldg((const uint2 *)(a.r.same + (size_t)j * REC_WORDS + 4));
     t.pen = __ldg(a.r.pen + j);
   }
+  if (!sched_index_ok(a.status, j < a.J && K >= 0 && N >= 0 && N <= ENTRIES, SCHED_CHK_ENTRY)) K = N = 0;
   t.speedup = __ldg(list_table(a, e) + fitness_table_index(a.tp, j, K, N));
   return t;
 }
@@ -308,12 +309,13 @@ __device__ __forceinline__ Record list_record(const FlowArgs &a, const uint32_t 
 }
 
 // ---- rows laid out in shared memory, a warp each (wide rows, and lists that overflow) --------------
-__device__ __forceinline__ void dense_from_list(int16_t *row, int NS, const Record &r, int lane) {
+__device__ __forceinline__ void dense_from_list(int16_t *row, int NS, const Record &r, int lane, int *status) {
   for (int n = lane; n < NS; n += 32) row[n] = 0;
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < ENTRIES; ++k)
-    if (lane == k && r.w[k] != NO_NODE) row[entry_node(r.w[k])] = (int16_t)entry_gpus(r.w[k]);
+    if (lane == k && r.w[k] != NO_NODE && sched_index_ok(status, entry_node(r.w[k]) < NS, SCHED_CHK_NODE))
+      row[entry_node(r.w[k])] = (int16_t)entry_gpus(r.w[k]);
   __syncwarp();
 }
 
@@ -679,6 +681,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
       s_flag[jc] = (sec ? 1 : 0) | (mut ? 2 : 0);
       if (mut) {
         const int i = atomicAdd(&s_nmut2[set], 1);
+        if (!sched_index_ok(a.status, i < J, SCHED_CHK_LIST)) continue;
         s_mut[i] = (uint16_t)(jc | (sec ? 0x8000 : 0));
         if (i < STASH) s_stash2[set * STASH + i] = make_uint4(m.y, m.z, m.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)));
       }
@@ -753,6 +756,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
       }
       __syncthreads();
       if (!s_ok) return;                        // (a wait ran out: the status says so)
+      if (!sched_index_ok(a.status, w.init || (s_par[0] < (uint32_t)P && s_par[1] < (uint32_t)P), SCHED_CHK_SLOT)) return;
       const uint32_t elite_key = elite ? s_keys[s_par[0]] : 0u;
       // (initial population: an unperturbed row is the current allocation's after the row caps, a perturbed one
       // starts from it before them; rows of the current allocation lie by job)
@@ -764,6 +768,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
       // a row's occupants into the nodes' totals and lists
       auto add_occupant = [&](int jc, int k_rec, uint32_t e, uint32_t dist) {
         const int n = entry_node(e);
+        if (!sched_index_ok(a.status, n < NN && jc < JA && entry_gpus(e) <= 2047, SCHED_CHK_NODE)) return;
         atomicAdd(&s_tot[n], entry_gpus(e));
         const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
         if (k < (uint32_t)a.occ) s_occ[n * a.occ + k] = (uint32_t)jc | ((uint32_t)entry_gpus(e) << 13) | ((uint32_t)k_rec << 25) | dist;
@@ -805,7 +810,8 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
             s_term[s_act[jc]] = __uint_as_float(rec[q].w[REC_TERM]);
             if (rec[q].w[0] == WIDE) {
               s_info[jc] = INFO_DIST | INFO_WIDE;
-              s_wide[atomicAdd(&s_nwide, 1)] = (uint16_t)(jc | ((flag[q] & 1u) ? 0x8000 : 0));
+              const int at = atomicAdd(&s_nwide, 1);
+              if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_wide[at] = (uint16_t)(jc | ((flag[q] & 1u) ? 0x8000 : 0));
               continue;
             }
             const uint32_t dist = rec[q].w[1] != NO_NODE ? 0x80000000u : 0u;
@@ -828,7 +834,9 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
         // ---- perturbed rows: the last warp, a lane each --------------------------------------------------
 #pragma unroll 1
         for (int i = lane; i < nmut; i += 32) {
-          const int jc = s_mut[i] & 0x7FFF, j = s_act[jc];
+          const int jc = s_mut[i] & 0x7FFF;
+          if (!sched_index_ok(a.status, i < J && jc < JA, SCHED_CHK_LIST)) continue;
+          const int j = s_act[jc];
           const uint32_t *src = (w.init || (s_mut[i] >> 15)) ? w.src_b : w.src_a;
           const Record rec = load_record(src + (size_t)(w.init ? j : jc) * REC_WORDS);
           uint4 st;
@@ -870,7 +878,10 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
               s_term[j] = __uint_as_float(out.w[REC_TERM]);
             }
           }
-          if (slow) s_slow[atomicAdd(&s_nslow, 1)] = s_mut[i];
+          if (slow) {
+            const int at = atomicAdd(&s_nslow, 1);
+            if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_slow[at] = s_mut[i];
+          }
         }
       }
       __syncthreads();
@@ -888,7 +899,9 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
 #pragma unroll 1
         for (int i = warp; i < s_nwide + s_nslow; i += nwarps) {
           const bool slow = i >= s_nwide;
-          const int x = slow ? s_slow[i - s_nwide] : s_wide[i], jc = x & 0x7FFF, j = s_act[jc];
+          const int x = slow ? s_slow[i - s_nwide] : s_wide[i], jc = x & 0x7FFF;
+          if (!sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST)) continue;
+          const int j = s_act[jc];
           const bool sec = (x >> 15) || (w.init && slow);
           const int at = w.init ? j : jc;
           const Record rec = load_record((sec ? w.src_b : w.src_a) + (size_t)at * REC_WORDS);
@@ -902,7 +915,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
             }
             __syncwarp();
           } else {
-            dense_from_list(s_dense, NS, rec, lane);
+            dense_from_list(s_dense, NS, rec, lane, a.status);
           }
           if (slow) {
             int K, N;
@@ -913,7 +926,8 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
             if (op == 0u) {
               if (lane == 0) s_dense[nd] = (int16_t)min((int)s_dense[nd] + 1, (int)s_cap[nd]);
             } else if (N > 0) {
-              const int ns = nth_occupied(s_dense, NN, bounded(m.z, (uint32_t)N), lane);
+              int ns = nth_occupied(s_dense, NN, bounded(m.z, (uint32_t)N), lane);
+              if (!sched_index_ok(a.status, ns >= 0 && ns < NN && nd < NN, SCHED_CHK_NODE)) ns = nd;
               if (lane == 0 && op == 1u) s_dense[ns] = (int16_t)(s_dense[ns] - 1);
               if (lane == 0 && op == 2u && nd != ns) {
                 s_dense[nd] = (int16_t)min((int)s_dense[nd] + (int)s_dense[ns], (int)s_cap[nd]);
@@ -951,6 +965,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
       // A decision goes straight into the row: entry k of its record (0 GPUs: taken out when the row is
       // finished), or its contents.  Decisions of different nodes touch different words.
       auto set_entry = [&](int jc, int k, int n, int v) {
+        if (!sched_index_ok(a.status, jc < JA && n < NN && (k == 7 || k < ENTRIES), SCHED_CHK_ENTRY)) return;
         if (k == 7) w.wide[(size_t)jc * NS + n] = (int16_t)v;
         else if (s_rec) s_rec[jc * REC_WORDS + k] = ((uint32_t)n << 16) | (uint32_t)v;
         else w.rec[(size_t)jc * REC_WORDS + k] = ((uint32_t)n << 16) | (uint32_t)v;
@@ -990,7 +1005,8 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
           const int n = n0 + max(b, 0) * nwarps, count = b >= 0 ? (int)(s_cnt[n] >> 16) : 0;
           const bool listed = count <= a.occ, have = listed && sub < count;   // else: walked below
           const uint32_t e = have ? s_occ[n * a.occ + sub] : 0u;
-          const int jc = (int)(e & 0x1FFFu), j = have ? (int)s_act[jc] : 0;
+          const int jc = (int)(e & 0x1FFFu);
+          const int j = have && sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) ? (int)s_act[jc] : 0;
           int ri = j - (int)(rep & 0xFFFFu), rc = have ? j - (int)(rep >> 16) : 0x3fffffff;
           if (ri < 0) ri += J;
           if (rc < 0) rc += J;
@@ -1001,7 +1017,10 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
             set_entry(jc, (int)((e >> 25) & 7u), n, v);
             // (bytes, so the word around it is updated as a whole)
             const uint32_t bit = (uint32_t)INFO_CHANGED << (8 * (jc & 3));
-            if ((atomicOr((uint32_t *)s_info + (jc >> 2), bit) & bit) == 0u) s_mod[atomicAdd(&s_nmod, 1)] = (uint16_t)jc;
+            if (sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) && (atomicOr((uint32_t *)s_info + (jc >> 2), bit) & bit) == 0u) {
+              const int at = atomicAdd(&s_nmod, 1);
+              if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_mod[at] = (uint16_t)jc;
+            }
           }
           if (b >= 0 && sub == 0 && !listed) { s_viol[n] = 1; s_walk = 1; }
           __syncwarp();
@@ -1217,7 +1236,8 @@ __global__ void __launch_bounds__(256) flow_finish_kernel(FlowArgs a) {
   __syncthreads();
 #pragma unroll 1
   for (int w = 0; w < 8; ++w) best = s_best[w] > best ? s_best[w] : best;
-  const int c = (int)(0xFFFFFFFFu - (uint32_t)best), JA = *a.r.num_act;
+  const int found = (int)(0xFFFFFFFFu - (uint32_t)best), JA = *a.r.num_act;
+  const int c = sched_index_ok(a.status, found >= 0 && found < P, SCHED_CHK_SLOT) ? found : 0;
 #pragma unroll 1
   for (int i = tid; i < JA; i += 256) s_place[a.r.act[i]] = (uint16_t)i;
   __syncthreads();
