@@ -144,9 +144,8 @@ __device__ __noinline__ void draw_two(uint32_t k0, uint32_t k1, uint32_t idx, ui
 
 // ---- waiting and publishing --------------------------------------------------------------------
 // The key published under `tag`; false when it has not come within the limit (the caller returns: the
-// other blocks' waits run out the same way).  The rows behind it are read through L2 (ld.cg, issued after
-// this load has answered), which the publisher's fence has them in; an acquire here would throw away the
-// tables' lines in this SM's L1 once more in every step.
+// other blocks' waits run out the same way).  A thread that has waited calls waited() before the barrier
+// behind which the block reads the rows, or before it publishes in its turn.
 __device__ __noinline__ bool wait_tag(const unsigned long long *p, uint32_t tag, uint32_t &key, int *status) {
 #pragma unroll 1
   for (unsigned int n = 0; n < WAIT_LIMIT; ++n) {
@@ -161,6 +160,12 @@ __device__ __noinline__ bool wait_tag(const unsigned long long *p, uint32_t tag,
   key = 0u;
   return false;
 }
+// Acquire: with the publisher's fence (release) and the block's barrier, what was written before the tag
+// was published is seen by every thread of this block, and what was read before it lies behind it.  One
+// fence after the polls that succeeded, not an acquire in each poll.  The one-way fence costs nothing that
+// can be measured (testbed round 663 us with it and without, large 3.87 ms), fence.acq_rel, which also waits
+// for this thread's own writes, 4 to 10 % (732 us, 4.03 ms).
+__device__ __forceinline__ void waited() { asm volatile("fence.acquire.gpu;" ::: "memory"); }
 __device__ __forceinline__ void publish(unsigned long long *p, uint32_t tag, uint32_t key) {
   const unsigned long long v = ((unsigned long long)tag << 32) | key;
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
@@ -736,6 +741,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
             ok = wait_tag(pub_of(s - 1, i), base + (uint32_t)(s - 1), k, a.status);
             s_keys[i] = k;
           }
+          waited();
           if (!ok) s_ok = 0;
           __syncthreads();
           if (elite && warp == 0 && s_ok) {
@@ -749,6 +755,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
           const uint32_t mine = s_sel[set][lane & 3];
           if (lane < 4 && !elite) ok = wait_tag(pub_of(s - 1, mine), base + (uint32_t)(s - 1), k, a.status);
           if (lane == 4 && s >= DEPTH) ok = wait_tag(pub_of(s - 2, 0u), base + (uint32_t)(s - 2), k, a.status);
+          waited();
           if (!__all_sync(0xffffffffu, ok) && lane == 0) s_ok = 0;
           const uint32_t other = __shfl_down_sync(0xffffffffu, mine, 1), ko = __shfl_down_sync(0xffffffffu, k, 1);
           if (!elite && (lane == 0 || lane == 2)) s_par[lane >> 1] = (uint32_t)tournament_winner(k, (int)mine, ko, (int)other);

@@ -99,3 +99,45 @@ def test_round_equals_stepwise(route, shape, start):
     for c in range(0, P, 3):
         assert feasible(pop[c].cpu().numpy(), cl.node_capacity, k_cap, cl.n_max)
     s.close()
+
+
+@pytest.mark.parametrize("shape", [(16, 4, 48, 148, 60), (75, 8, 300, 700, 12), (8, 4, 20, 2500, 20)],
+                         ids=lambda s: "-".join(str(x) for x in s))
+def test_rows_handed_from_block_to_block_arrive(shape):
+    """Blocks read rows that other blocks have just published, for many generations and many times over:
+    every repetition must be the same round, bit for bit, and the first the dense entry points'."""
+    import torch
+    from paper_2008_12260_b200 import api
+
+    NN, gpn, J, P, gens = shape
+    cfg = synth.Config("hand-over", NN, gpn, J, 3, 16, 8, P, gens, num_elite=4, mutate_prob=0.3, init_prob=0.5,
+                       with_history=True)
+    cl = cfg.cluster()
+    jobs = with_fair_share(cfg.jobs(), cl)
+    cur = synth.random_feasible_allocation(cl, J, 5, active=jobs.active)
+    st = torch.cuda.Stream()
+    s = api.scheduler_for(cfg, stream=st.cuda_stream)
+    with torch.cuda.stream(st):
+        dj = api.DeviceJobs(jobs, "cuda", torch)
+        d_cur = torch.from_numpy(cur).cuda()
+        best, bf = torch.empty((J, NN), dtype=torch.int16, device="cuda"), torch.zeros(1, device="cuda")
+        pop, fit = torch.empty((P, J, NN), dtype=torch.int16, device="cuda"), torch.empty(P, device="cuda")
+        sp, rf = torch.empty(s.table_shape, device="cuda"), torch.empty(J, device="cuda")
+        s.build_speedup_table(dj, None, sp, None)
+        s.compute_realloc_factor(dj, rf)
+        a, b, f = torch.empty_like(pop), torch.empty_like(pop), torch.empty_like(fit)
+        kw = dict(p=cfg.p, cur=d_cur, realloc_factor=rf, active=dj.tensors["active"])
+        s.init_population(dj, d_cur, a, round=1)
+        s.eval_fitness(a, sp, f, **kw)
+        for g in range(gens):
+            s.ga_generation(dj, a, f, b, round=1, generation=g)
+            a, b = b, a
+            s.eval_fitness(a, sp, f, **kw)
+        for k in range(20):
+            s.schedule_round(dj, d_cur, best, bf, round=1 + k % 2, generations=gens)
+            if k % 2:
+                continue
+            s.get_population(pop, fit)
+            s.sync_status()
+            assert torch.equal(pop, a) and torch.equal(fit.view(torch.int32), f.view(torch.int32)), k
+    s.close()
