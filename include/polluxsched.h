@@ -309,6 +309,13 @@ int schedule_round(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_cu
 int sched_set_store_budget(sched_ctx *ctx, uint64_t bytes);
 int64_t sched_store_moves(sched_ctx *ctx);
 
+/* How often a block of a round's one-launch search looks for another's candidate before it gives up
+ * (some 0.15 us each; default SCHED_WAIT_LIMIT, about a third of a second, where a candidate takes a few
+ * microseconds).  A wait that runs out ends the launch: d_best and d_best_fitness are then undefined, the
+ * status is SCHED_ERR_TIMEOUT, and the next round starts afresh.  0: every wait gives up at once. */
+#define SCHED_WAIT_LIMIT (1u << 21)
+int sched_set_wait_limit(sched_ctx *ctx, uint32_t polls);
+
 /* schedule_round replays a CUDA graph of the whole round from the third call on that passes
  * the same pointers and generation count (the second such call captures it); this removes
  * the per-kernel launch cost that dominates small problems.  Results are identical with

@@ -23,7 +23,7 @@ EXPORTS = (
     "init_population", "ga_generation", "ga_generation_shard", "schedule_round", "schedule_round_host",
     "sched_get_population", "sched_get_round_tables", "sched_round_speedup_table", "eval_fitness_host",
     "sched_set_kernel_timing", "sched_num_kernel_kinds", "sched_kernel_kind_name",
-    "sched_read_kernel_timing", "sched_measure_peaks", "sched_set_graphs", "sched_set_store_budget", "sched_store_moves", "eval_fitness_noalloc", "eval_fitness_noalloc_last_error",
+    "sched_read_kernel_timing", "sched_measure_peaks", "sched_set_graphs", "sched_set_store_budget", "sched_store_moves", "sched_set_wait_limit", "eval_fitness_noalloc", "eval_fitness_noalloc_last_error",
 )
 
 
@@ -93,6 +93,7 @@ def load_library(path: str = LIB_PATH):
                                         C.POINTER(C.c_double)]
     lib.sched_set_store_budget.argtypes = [vp, C.c_uint64]
     lib.sched_store_moves.argtypes = [vp]
+    lib.sched_set_wait_limit.argtypes = [vp, u32]
     lib.sched_store_moves.restype = C.c_int64
     lib.sched_num_kernel_kinds.argtypes = []
     lib.sched_kernel_kind_name.argtypes = [i32]
@@ -232,6 +233,9 @@ class Scheduler:
 
     def store_moves(self) -> int:
         return int(_lib.sched_store_moves(self._ctx))
+
+    def set_wait_limit(self, polls: int):
+        self._check(_lib.sched_set_wait_limit(self._ctx, int(polls)))
 
     def read_kernel_timing(self):
         """{kernel class: (total ms, timed launches)} since the previous read-out"""

@@ -264,6 +264,7 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   if ((rc = dev_alloc(ctx, &ctx->d_round, 1)) != SCHED_OK) return fail(rc);
   ctx->graphs_enabled = true;
   ctx->rs_budget = 12ull << 30;
+  ctx->fl_wait_limit = SCHED_WAIT_LIMIT;
   e = cudaMemsetAsync(ctx->d_cap, 0, sizeof(int16_t) * (((size_t)cfg->num_nodes + 7) & ~(size_t)7), ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ctx->d_cap, h_node_capacity, sizeof(int16_t) * cfg->num_nodes,
@@ -357,6 +358,13 @@ int sched_set_store_budget(sched_ctx *ctx, uint64_t bytes) {
   REQUIRE(ctx, !ctx->round_ready, SCHED_ERR_INVALID_ARG,
           "sched_set_store_budget: the round scratch exists already (call before the first schedule_round)");
   ctx->rs_budget = bytes;
+  return SCHED_OK;
+}
+
+int sched_set_wait_limit(sched_ctx *ctx, uint32_t polls) {
+  REQUIRE(nullptr, ctx, SCHED_ERR_INVALID_ARG, "sched_set_wait_limit: ctx is NULL");
+  ctx->fl_wait_limit = polls;
+  ctx->scratch_epoch++;      // (a captured round holds the limit)
   return SCHED_OK;
 }
 

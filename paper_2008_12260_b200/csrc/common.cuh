@@ -116,6 +116,7 @@ struct sched_ctx {
   int fl_blocks;           // blocks of the launch, 0: rounds run on the other kernels
   int fl_generations;      // generations of the last round
   bool fl_ahead;           // blocks have threads that draw a step ahead
+  unsigned int fl_wait_limit;   // sched_set_wait_limit
 
   // staging for the *_host entry points (allocated on first use)
   void *d_stage;         // job arrays + cur + best

@@ -34,7 +34,6 @@ constexpr int MAX_ROW_THREADS = 256;            // as the dense fitness kernel: 
 constexpr int STASH = 128;                      // perturbed rows whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
 constexpr int FLOW_MAX_JOBS = 8192, FLOW_MAX_NODES = 512;
-constexpr unsigned int WAIT_LIMIT = 1u << 21;   // polls (a few hundred cycles each) before a wait gives up
 
 __host__ __device__ inline int wide_stride(int NN) { return (NN + 7) & ~7; }
 
@@ -73,6 +72,7 @@ struct FlowArgs {
   float *fitness;            // [P]
   int16_t *best;             // [J][NN]
   float *best_fitness;
+  unsigned int wait_limit;   // polls (a few hundred cycles each) before a wait gives up
   int *status;
 };
 
@@ -146,9 +146,9 @@ __device__ __noinline__ void draw_two(uint32_t k0, uint32_t k1, uint32_t idx, ui
 // The key published under `tag`; false when it has not come within the limit (the caller returns: the
 // other blocks' waits run out the same way).  A thread that has waited calls waited() before the barrier
 // behind which the block reads the rows, or before it publishes in its turn.
-__device__ __noinline__ bool wait_tag(const unsigned long long *p, uint32_t tag, uint32_t &key, int *status) {
+__device__ __noinline__ bool wait_tag(const unsigned long long *p, uint32_t tag, uint32_t &key, unsigned int limit, int *status) {
 #pragma unroll 1
-  for (unsigned int n = 0; n < WAIT_LIMIT; ++n) {
+  for (unsigned int n = 0; n < limit; ++n) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     if ((uint32_t)(v >> 32) == tag) {
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
 #pragma unroll 1
           for (int i = tid; i < P && ok; i += blockDim.x) {
             uint32_t k;
-            ok = wait_tag(pub_of(s - 1, i), base + (uint32_t)(s - 1), k, a.status);
+            ok = wait_tag(pub_of(s - 1, i), base + (uint32_t)(s - 1), k, a.wait_limit, a.status);
             s_keys[i] = k;
           }
           waited();
@@ -753,8 +753,8 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
           uint32_t k = 0u;
           bool ok = true;
           const uint32_t mine = s_sel[set][lane & 3];
-          if (lane < 4 && !elite) ok = wait_tag(pub_of(s - 1, mine), base + (uint32_t)(s - 1), k, a.status);
-          if (lane == 4 && s >= DEPTH) ok = wait_tag(pub_of(s - 2, 0u), base + (uint32_t)(s - 2), k, a.status);
+          if (lane < 4 && !elite) ok = wait_tag(pub_of(s - 1, mine), base + (uint32_t)(s - 1), k, a.wait_limit, a.status);
+          if (lane == 4 && s >= DEPTH) ok = wait_tag(pub_of(s - 2, 0u), base + (uint32_t)(s - 2), k, a.wait_limit, a.status);
           waited();
           if (!__all_sync(0xffffffffu, ok) && lane == 0) s_ok = 0;
           const uint32_t other = __shfl_down_sync(0xffffffffu, mine, 1), ko = __shfl_down_sync(0xffffffffu, k, 1);
@@ -1421,6 +1421,7 @@ static FlowArgs flow_args(const sched_ctx *ctx, const sched_jobs *jobs, const in
   a.key = make_key(c.seed, ctx->d_round);
   fitness_chunking(ctx, c.population, a.rows_per_chunk, a.chunks);
   a.fitness = ctx->d_fit;
+  a.wait_limit = ctx->fl_wait_limit;
   a.status = ctx->d_status;
   return a;
 }

@@ -291,6 +291,54 @@ def test_kernel_timing_names_the_kernels_that_ran(gpu, route, search):
     s.close()
 
 
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("limit", [0, 1])
+def test_a_wait_that_runs_out_ends_the_round_with_a_status(gpu, limit, graphs):
+    """No polls at all, or one (some blocks get on, some do not): every block leaves, the status says so, and
+    the next round on the same context is right again."""
+    torch, api = gpu
+    cfg = synth.TESTBED
+    cl, jobs = setup(cfg)
+    s = api.scheduler_for(cfg, stream=torch.cuda.Stream().cuda_stream)
+    s.set_graphs(graphs)
+    dj = api.DeviceJobs(jobs, "cuda:0", torch)
+    d_cur = torch.from_numpy(cfg.cur()).cuda()
+    best = torch.empty((cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
+    bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
+    pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
+    fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")
+    torch.cuda.synchronize()
+    res = []
+    for k in range(4):
+        if k == 2:
+            s.set_wait_limit(limit)
+            for rnd in range(3):
+                s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=30)
+                with pytest.raises(api.SchedError) as e:
+                    s.sync_status()
+                assert e.value.code == -4
+            s.sync_status()                                # reported once
+            s.set_wait_limit(1 << 21)
+        s.schedule_round(dj, d_cur, best, bf, round=7, generations=30)
+        s.get_population(pop, fit)
+        s.sync_status()
+        res.append([x.cpu().numpy().copy() for x in (pop, fit, best, bf)])
+    for r in res[1:]:
+        for x, y in zip(res[0], r):
+            assert np.array_equal(x, y)
+    hj = api.HostJobs(jobs, torch)
+    h_cur, h_best = torch.from_numpy(cfg.cur()).pin_memory(), torch.empty(best.shape, dtype=torch.int16).pin_memory()
+    h_bf = torch.zeros(1, dtype=torch.float32).pin_memory()
+    s.set_wait_limit(limit)
+    with pytest.raises(api.SchedError) as e:               # the host-buffer call waits, so the status is its result
+        s.schedule_round_host(hj, h_cur, h_best, h_bf, round=7, generations=30)
+    assert e.value.code == -4
+    s.set_wait_limit(1 << 21)
+    s.schedule_round_host(hj, h_cur, h_best, h_bf, round=7, generations=30)
+    assert np.array_equal(h_best.numpy(), res[0][2]) and h_bf.item() == res[0][3][0]
+    s.close()
+
+
 def test_argument_errors(gpu):
     torch, api = gpu
     cfg = synth.TINY
