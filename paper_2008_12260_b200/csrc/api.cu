@@ -886,8 +886,8 @@ int schedule_round_host(sched_ctx *ctx, const sched_jobs *h_jobs, const int16_t 
   if ((rc = validate_host_jobs(ctx, h_jobs, h_cur)) != SCHED_OK) return rc;
   const sched_config &c = ctx->cfg;
   const size_t J = (size_t)c.num_jobs, mat = J * c.num_nodes * sizeof(int16_t);
-  // layout of the staging buffer: 10 fp32 arrays, m_grid, k_cap, fair_k, fair_n, age,
-  // restarts, active, cur, best, best_fitness - each 256-byte aligned
+  // layout of the staging buffer: 10 fp32 arrays, k_cap, fair_k, fair_n, age, restarts, active, m_grid,
+  // cur, best, best_fitness - each 256-byte aligned
   const size_t f32 = align256(J * 4), grid = align256(J * c.grid_m * 4), u8 = align256(J);
   const size_t need = 10 * f32 + grid + 5 * f32 + u8 + 2 * align256(mat) + 256;
   if (need > ctx->stage_bytes) {
@@ -902,27 +902,30 @@ int schedule_round_host(sched_ctx *ctx, const sched_jobs *h_jobs, const int16_t 
   }
   char *base = (char *)ctx->d_stage;
   size_t off = 0;
-  // The inputs are first gathered in a pinned buffer laid out like the device one and go up in a
+  // The arrays that end within the layout's first 256 KB are gathered in a pinned buffer and go up in a
   // single copy: 18 copies from pageable memory, each of which waits, cost 0.2 ms of the largest
-  // configuration's round.  Beyond 4 MB the bytes are what takes the time, and the buffer would only be
-  // held.  The fitness and the status come back through its first words.
-  const size_t input_bytes = need - 2 * align256(mat) - 256 + align256(mat);   // everything up to and including cur
-  const bool gather = input_bytes <= (4u << 20);
-  const size_t h_need = 256 + (gather ? input_bytes : 0);
+  // configuration's round.  Longer ones (there its grid and its matrix, 0.5 MB each) are copied from where
+  // they are: gathering them saves nothing (3.83 ms a round from pinned and 3.87 from pageable arrays with
+  // it, 3.85 and 3.83 so), and a pinned buffer of a megabyte is dear to make, where one of this size comes
+  // out of a pool of the runtime's (a context's first large round 6.2 to 9.5 ms with everything gathered,
+  // 4.4 to 5.0 so).  The fitness and the status come back through its first words.
+  const size_t staged = std::min<size_t>(256u << 10, need);
+  const size_t h_need = 256 + staged;
   if (h_need > ctx->h_stage_bytes) {
     if (ctx->h_stage) { cudaFreeHost(ctx->h_stage); ctx->h_stage = nullptr; ctx->h_stage_bytes = 0; }
     if (cudaMallocHost(&ctx->h_stage, h_need) == cudaSuccess) ctx->h_stage_bytes = h_need;
     else { cudaGetLastError(); ctx->h_stage = nullptr; }
   }
-  char *hbase = (gather && ctx->h_stage) ? (char *)ctx->h_stage + 256 : nullptr;
+  char *hbase = ctx->h_stage ? (char *)ctx->h_stage + 256 : nullptr;
+  size_t gathered = 0;
   struct Back { float fitness; int status; } pageable;
   Back *const back = ctx->h_stage ? (Back *)ctx->h_stage : &pageable;
   auto up = [&](const void *h, size_t bytes, size_t slot) -> const void * {
     void *d = base + off;
-    char *hs = hbase ? hbase + off : nullptr;
+    char *hs = hbase && off + bytes <= staged ? hbase + off : nullptr;
     off += slot;
     if (!h) return nullptr;
-    if (hs) { memcpy(hs, h, bytes); return d; }
+    if (hs) { memcpy(hs, h, bytes); gathered = (size_t)(hs - hbase) + bytes; return d; }
     if (cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) return (const void *)-1;
     return d;
   };
@@ -937,18 +940,19 @@ int schedule_round_host(sched_ctx *ctx, const sched_jobs *h_jobs, const int16_t 
     *df[i] = (const float *)up(hf[i], J * 4, f32);
     bad |= (*df[i] == (const float *)-1);
   }
-  dj.m_grid = (const int32_t *)up(h_jobs->m_grid, J * c.grid_m * 4, grid);
   dj.k_cap = (const int32_t *)up(h_jobs->k_cap, J * 4, f32);
   dj.fair_k = (const int32_t *)up(h_jobs->fair_k, J * 4, f32);
   dj.fair_n = (const int32_t *)up(h_jobs->fair_n, J * 4, f32);
   dj.age_sec = (const float *)up(h_jobs->age_sec, J * 4, f32);
   dj.num_restarts = (const int32_t *)up(h_jobs->num_restarts, J * 4, f32);
   dj.active = (const uint8_t *)up(h_jobs->active, J, u8);
+  dj.m_grid = (const int32_t *)up(h_jobs->m_grid, J * c.grid_m * 4, grid);
   const int16_t *d_cur = (const int16_t *)up(h_cur, mat, align256(mat));
   bad |= dj.m_grid == (const void *)-1 || dj.k_cap == (const void *)-1 || dj.fair_k == (const void *)-1 ||
          dj.fair_n == (const void *)-1 || dj.age_sec == (const void *)-1 ||
          dj.num_restarts == (const void *)-1 || dj.active == (const void *)-1 || d_cur == (const void *)-1;
-  if (hbase && cudaMemcpyAsync(base, hbase, off, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) bad = true;
+  // (the gathered arrays are the first ones of the layout: one that ends beyond `staged` has none behind it that does not)
+  if (gathered && cudaMemcpyAsync(base, hbase, gathered, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) bad = true;
   REQUIRE(ctx, !bad, SCHED_ERR_CUDA, "schedule_round_host: a host-to-device copy failed: %s",
           cudaGetErrorString(cudaGetLastError()));
   int16_t *d_best = (int16_t *)(base + off);

@@ -121,7 +121,7 @@ struct sched_ctx {
   // staging for the *_host entry points (allocated on first use)
   void *d_stage;         // job arrays + cur + best
   size_t stage_bytes;
-  void *h_stage;         // pinned: results (256 bytes), then a mirror of the inputs' part of d_stage (one copy instead of 18)
+  void *h_stage;         // pinned: results (256 bytes), then a mirror of d_stage's first 256 KB (one copy instead of one per array)
   size_t h_stage_bytes;
   void *d_stage_fit;     // eval_fitness_host staging
   size_t stage_fit_bytes;

@@ -171,6 +171,30 @@ def test_host_buffer_round(gpu):
     s.close()
 
 
+@pytest.mark.parametrize("pin", [True, False])
+@pytest.mark.parametrize("jobs,nodes,grid", [(48, 16, 64), (64, 8, 900), (64, 8, 1100), (1500, 40, 16), (5000, 8, 16)])
+def test_host_buffer_round_of_any_size(gpu, jobs, nodes, grid, pin):
+    """Arrays up to 256 KB in all go up together, longer ones by themselves: everything gathered; the grid just
+    below and just above the line, the matrix beyond it; grid and matrix beyond; job arrays beyond (some optional
+    arrays left out)."""
+    torch, api = gpu
+    cfg = synth.Config("host", nodes, 4, jobs, 5, grid, 16, 12, 4, num_elite=1, mutate_prob=0.2,
+                       with_history=jobs != 64)
+    cl, host_jobs = setup(cfg)
+    cur = synth.random_feasible_allocation(cl, jobs, 3)
+    s, dj, best, bf, pop, fit = _round(gpu, cfg, host_jobs, cur, 4, rnd=1)
+    hj = api.HostJobs(host_jobs, torch, pin=pin)
+    h_cur, h_best = torch.from_numpy(cur), torch.empty((jobs, nodes), dtype=torch.int16)
+    h_bf = torch.zeros(1, dtype=torch.float32)
+    if pin:
+        h_cur, h_best, h_bf = h_cur.pin_memory(), h_best.pin_memory(), h_bf.pin_memory()
+    for _ in range(3):
+        h_best.fill_(-1)
+        s.schedule_round_host(hj, h_cur, h_best, h_bf, round=1, generations=4)
+        assert np.array_equal(h_best.numpy(), best) and float(h_bf.item()) == bf
+    s.close()
+
+
 def test_graph_replay_gives_the_same_rounds(gpu):
     """Rounds 3+ with unchanged buffers replay a captured CUDA graph; they must equal the same
     rounds run kernel by kernel, for every round number."""
