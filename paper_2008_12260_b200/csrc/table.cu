@@ -280,6 +280,7 @@ __device__ __forceinline__ void write_slab(const TableRow *rows, int e0, int e1,
     K += step_k;
     N += step_n;
     if (N >= ND) { N -= ND; ++K; }
+    else if (N < 0) { N += ND; --K; }       // (the thread's first four began before the slab)
   }
 }
 

@@ -138,3 +138,15 @@ def test_screened_sweep_edges(gpu, oracle, grid_m, grid_s, case):
     gp, sp, am = _gpu_table(gpu, cl, jobs, grid_s, k_max=14, n_max=4)
     gp_r, sp_r, am_r = oracle.build_speedup_table(jobs, cl.node_capacity, 14, 4, grid_s)
     check_table(oracle, jobs, grid_s, gp, sp, am, gp_r, sp_r, am_r)
+
+
+@pytest.mark.parametrize("nodes,gpus,jobs", [(32, 1, 300), (17, 4, 300), (28, 8, 60), (9, 8, 150), (50, 1, 300), (22, 4, 1000),
+                                             (6, 2, 37), (16, 4, 48)])
+def test_slabs_of_any_width_and_place(gpu, oracle, nodes, gpus, jobs):
+    """A slab's fours of entries are aligned in the whole table, so a thread's first one may begin before the
+    slab; widths at which its next ones would still be counted from there, and others."""
+    cl = synth.uniform_cluster(nodes, gpus)
+    j = with_fair_share(synth.draw_jobs(jobs, 5, 32, 8, cl.k_max), cl)
+    gp, sp, am = _gpu_table(gpu, cl, j, 8)
+    gp_r, sp_r, am_r = oracle.build_speedup_table(j, cl.node_capacity, cl.k_max, cl.n_max, 8)
+    check_table(oracle, j, 8, gp, sp, am, gp_r, sp_r, am_r)
