@@ -254,6 +254,12 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
   ctx->num_rack_pairs = (int)rack_pairs.size();
   pairs.insert(pairs.end(), rack_pairs.begin(), rack_pairs.end());
   if ((rc = dev_alloc(ctx, &ctx->d_pairs, pairs.size())) != SCHED_OK) return fail(rc);
+  // results of a table in two launches (table.cu: beyond 50 thousand pairs no list of points takes those)
+  const size_t results = J * ctx->num_pairs <= 50000 ? J * ctx->KD * 3 : 0;
+  if (results) {
+    if ((rc = dev_alloc(ctx, &ctx->d_gmax, results + (results + 1) / 2)) != SCHED_OK) return fail(rc);
+    ctx->d_amax = (uint16_t *)(ctx->d_gmax + results);
+  }
   if ((rc = dev_alloc(ctx, &ctx->d_rank, P)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_order, P)) != SCHED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_pen, 2 * J)) != SCHED_OK) return fail(rc);
@@ -273,6 +279,8 @@ int sched_init(const sched_config *cfg, const int16_t *h_node_capacity, void *cu
     e = cudaMemcpyAsync(ctx->d_kfit, kfit.data(), sizeof(int32_t) * kfit.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess && !pairs.empty())
     e = cudaMemcpyAsync(ctx->d_pairs, pairs.data(), sizeof(int32_t) * pairs.size(), cudaMemcpyHostToDevice, ctx->stream);
+  if (e == cudaSuccess && results) e = cudaMemsetAsync(ctx->d_gmax, 0, sizeof(float) * results, ctx->stream);
+  if (e == cudaSuccess && results) e = cudaMemsetAsync(ctx->d_amax, 0xFF, sizeof(uint16_t) * results, ctx->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);   // host vectors go out of scope
   if (e != cudaSuccess) {
@@ -310,7 +318,7 @@ int sched_destroy(sched_ctx *ctx) {
     ctx->d_tab_goodput = ctx->d_tab_speedup = ctx->d_tab_speedup_rack = ctx->d_fit_buf = nullptr;
     cudaFree(ctx->fl_arena);
   }
-  void *ptrs[] = {ctx->d_cap, ctx->d_kfit, ctx->d_pairs, ctx->d_rank, ctx->d_order,
+  void *ptrs[] = {ctx->d_cap, ctx->d_kfit, ctx->d_pairs, ctx->d_gmax, ctx->d_rank, ctx->d_order,
                   ctx->d_dflag, ctx->d_pen, ctx->d_partial, ctx->d_ticket, ctx->d_status,
                   ctx->d_popA, ctx->d_popB, ctx->d_fit_buf, ctx->d_tab_goodput, ctx->d_tab_speedup,
                   ctx->d_rf, ctx->d_best_idx, ctx->d_stage, ctx->d_stage_fit, ctx->d_colsum, ctx->d_summ, ctx->d_collist, ctx->d_colcount, ctx->d_rowticket, ctx->d_round, ctx->d_occcount, ctx->d_occlist,

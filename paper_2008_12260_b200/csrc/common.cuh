@@ -55,6 +55,8 @@ struct sched_ctx {
   int32_t *d_pairs;      // K * 4 + class of every (K, class) that exists on this cluster: the local and node
                          // pairs, then the rack pairs
   int num_pairs, num_rack_pairs;
+  float *d_gmax;         // [J][KD][3] goodput per (K, class) and (behind it) the index of its maximiser, of a
+  uint16_t *d_amax;      // table that is being built in two launches; NULL where there are too many pairs for that
   // rack-level locality (sched_set_racks): rack of every node, the third synchronisation pair
   int16_t *d_rack;       // [num_nodes] or NULL when the cluster is not split into racks
   const float *d_alpha_rack, *d_beta_rack;   // caller-owned device arrays [J]

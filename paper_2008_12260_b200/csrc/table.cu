@@ -54,6 +54,8 @@ __device__ __forceinline__ float overlap_time(float tg, float ts, float gamma, f
   return __fmul_rn(hi, ex2_approx(lg2_approx(1.f + x) * inv_gamma));
 }
 
+__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+
 // A candidate optimum: goodput = num / den; tie = (s << 16) | grid index (smaller wins).
 struct Best {
   float num, den;
@@ -93,6 +95,9 @@ struct TableArgs {
   float *goodput, *speedup;     // [J][KD][ND] of the local and node classes (speedup NULL: not wanted)
   uint16_t *argmax;
   float *goodput_rack, *speedup_rack;   // the same of the rack class
+  float one, zero;              // 1 and 0 (see grid_points)
+  float *g;                     // [J][KD][3] results per (K, class) between the launches of a small table:
+  uint16_t *a;                  // 0 and 0xFFFF where there is no such pair (nothing ever writes those)
   uint16_t *argmax_rack;
 };
 
@@ -168,11 +173,69 @@ __device__ __forceinline__ void batch_window(float km, float M0, float Mmax, flo
   uhi = fminf(uhi, gs);
 }
 
-// The best s of one grid point m, exactly as tabulated: with u = s + 1
+// The best s of each of MQ grid points (m[q], index i + 32 q; only the first `count` of them exist), exactly
+// as tabulated: with u = s + 1
 //   T_iter = ta + u tg,  1/EFFICIENCY = c0 + u kr  (kr = K m / (phi + M0)),
 //   goodput = K m * u / den(u),  den(u) = (ta + u tg)(c0 + u kr),
 // the maximiser over ALL s by cross-multiplied compares (den(u)/u is convex in u, so goodput is
-// unimodal in s), clamped into the window M0 <= K m u <= Mmax.
+// unimodal in s), clamped into the window M0 <= K m u <= Mmax.  Several points go two by two through packed
+// arithmetic, and what a compare chooses is moved by predicated multiply-adds with a one and a zero that the
+// compiler does not know: compares and selects share the half-rate integer pipe (1024 jobs x 19 pairs x 300
+// points: 67 us with plain selects, 63 us so).
+template <int MQ>
+__device__ __forceinline__ void grid_points(const JobModel &jm, float ts, float Kf, float rinv, float c0, const int (&m)[MQ],
+                                            int i, int count, int Gs, float one, float zero, Best &best) {
+  float tg[MQ], ta[MQ], kr[MQ], bu[MQ], bd[MQ];
+#pragma unroll
+  for (int q = 0; q < MQ; ++q) {
+    tg[q] = fmaf(jm.b_g, (float)m[q], jm.a_g);
+    ta[q] = __fsub_rn(overlap_time(tg[q], ts, jm.gamma, jm.inv_gamma), tg[q]);
+    kr[q] = __fmul_rn(Kf * (float)m[q], rinv);
+    bu[q] = 0.f;
+    bd[q] = 1.f;
+  }
+  float u = 1.f;
+#pragma unroll 4
+  for (int s = 0; s < Gs; ++s, u += 1.f) {
+    if (MQ == 1) {
+      const float den = __fmul_rn(fmaf(u, tg[0], ta[0]), fmaf(u, kr[0], c0));
+      if (__fmul_rn(u, bd[0]) > __fmul_rn(bu[0], den)) { bu[0] = u; bd[0] = den; }
+    }
+#pragma unroll
+    for (int q = 0; q + 1 < MQ; q += 2) {
+      const float2 u2 = f2(u);
+      const float2 den = __fmul2_rn(__ffma2_rn(u2, make_float2(tg[q], tg[q + 1]), make_float2(ta[q], ta[q + 1])),
+                                    __ffma2_rn(u2, make_float2(kr[q], kr[q + 1]), f2(c0)));
+      const float2 l = __fmul2_rn(u2, make_float2(bd[q], bd[q + 1])), r = __fmul2_rn(make_float2(bu[q], bu[q + 1]), den);
+      asm("{\n"
+          " .reg .pred pa, pb;\n"
+          " setp.gt.f32 pa, %4, %6;\n"
+          " setp.gt.f32 pb, %5, %7;\n"
+          " @pa fma.rn.f32 %0, %8, %11, %12;\n"
+          " @pa fma.rn.f32 %2, %9, %11, %12;\n"
+          " @pb fma.rn.f32 %1, %8, %11, %12;\n"
+          " @pb fma.rn.f32 %3, %10, %11, %12;\n"
+          "}"
+          : "+f"(bu[q]), "+f"(bu[q + 1]), "+f"(bd[q]), "+f"(bd[q + 1])
+          : "f"(l.x), "f"(l.y), "f"(r.x), "f"(r.y), "f"(u), "f"(den.x), "f"(den.y), "f"(one), "f"(zero));
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < MQ; ++q) {
+    const float km = Kf * (float)m[q], rkm = __frcp_rn(km);
+    float ulo, uhi;
+    batch_window(km, jm.M0, jm.Mmax, jm.M0 * rkm, jm.Mmax * rkm, (float)Gs, ulo, uhi);
+    if (q >= count || !(ulo <= uhi)) continue;
+    const float us = fminf(fmaxf(bu[q], ulo), uhi);
+    Best b;
+    b.num = km * us;
+    b.den = (us == bu[q]) ? bd[q] : __fmul_rn(fmaf(us, tg[q], ta[q]), fmaf(us, kr[q], c0));
+    b.tie = ((uint32_t)(us - 1.f) << 16) | (uint32_t)(i + 32 * q);
+    if (beats(b, best)) best = b;
+  }
+}
+
+// One grid point (a point of which no s is feasible is not scanned).
 __device__ __noinline__ Best grid_point(const JobModel &jm, float ts, float Kf, float rinv, float c0, int m, int i,
                                         int Gs) {
   Best b = {0.f, 1.f, 0xFFFFFFFFu};
@@ -201,8 +264,8 @@ __device__ __noinline__ Best grid_point(const JobModel &jm, float ts, float Kf, 
 // ceil(per_gpu / m_max) - 1 (the fewest accumulation steps that fit the per-GPU limit), m =
 // ceil(per_gpu / (s + 1)); the batch actually run is M' = K m (s + 1), feasible when M0 <= M' <=
 // M_max.  A non-adaptive job has the single candidate M0 and EFFICIENCY fixed to 1 (Sec. 4.2).
-__device__ __noinline__ Best sample_point(const JobModel &jm, float ts, int K, float rinv, float c0, int mmax, long long M,
-                                             int i) {
+__device__ __forceinline__ Best sample_point_inline(const JobModel &jm, float ts, int K, float rinv, float c0, int mmax,
+                                                    long long M, int i) {
   Best b = {0.f, 1.f, 0xFFFFFFFFu};
   if (M < 1) return b;
   long long s, m;
@@ -225,6 +288,11 @@ __device__ __noinline__ Best sample_point(const JobModel &jm, float ts, int K, f
   b.den = __fmul_rn(tit, fmaf(Mrun, rinv, c0));
   b.tie = (uint32_t)i;
   return b;
+}
+
+__device__ __noinline__ Best sample_point(const JobModel &jm, float ts, int K, float rinv, float c0, int mmax, long long M,
+                                          int i) {
+  return sample_point_inline(jm, ts, K, rinv, c0, mmax, M, i);
 }
 
 __device__ __forceinline__ bool kn_valid(int K, int N, int k_max, int n_max, const int32_t *__restrict__ kfit) {
@@ -284,11 +352,16 @@ __device__ __forceinline__ void write_slab(const TableRow *rows, int e0, int e1,
   }
 }
 
-__device__ __forceinline__ void write_tables(const TableArgs &a, const TableSmem &t, TableRow *rows, int j, int rank, int nb) {
-  const int KD = a.k_max + 1, ND = a.n_max + 1;
+// where the job's fair-share goodput is (K * 3 + class), -1: there is none
+__device__ __forceinline__ int fair_place(const TableArgs &a, int j) {
   const int kf = a.fair_k[j], nf = a.fair_n[j];
-  float denom = 0.f;
-  if (kn_valid(kf, nf, a.k_max, a.n_max, a.kfit)) denom = t.g[kf * 3 + (nf >= 2 ? CLS_NODE : CLS_LOCAL)];
+  return kn_valid(kf, nf, a.k_max, a.n_max, a.kfit) ? kf * 3 + (nf >= 2 ? CLS_NODE : CLS_LOCAL) : -1;
+}
+
+__device__ __forceinline__ void write_tables(const TableArgs &a, const TableSmem &t, TableRow *rows, int j, int rank, int nb,
+                                             int fair) {
+  const int KD = a.k_max + 1, ND = a.n_max + 1;
+  const float denom = fair >= 0 ? t.g[fair] : 0.f;
   const int entries = KD * ND;
   const int e0 = (int)((long long)entries * rank / nb), e1 = (int)((long long)entries * (rank + 1) / nb);
 #pragma unroll 1
@@ -344,7 +417,6 @@ constexpr float EXACT_QUOTIENT = 1048576.f;
 constexpr float LOW = 1.f - 4e-7f, HIGH = 1.f + 4e-7f;
 constexpr float MAGIC = 12582912.f;
 
-__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
 
@@ -663,7 +735,65 @@ __global__ void __maxnreg__(56) table_kernel(TableArgs a) {
     }
   }
   cl.sync();          // all results are in every block's shared memory
-  write_tables(a, t, (TableRow *)(smem + L.rows), j, rank, nb);
+  write_tables(a, t, (TableRow *)(smem + L.rows), j, rank, nb, fair_place(a, j));
+}
+
+// ---- small tables, long lists of points ------------------------------------------------------------
+// Where there are few (job, K, class), evaluating every point by a warp each is a shorter chain than
+// screening them: no table of points, no hand-over of the near ones, no blocks that wait for one another.
+// Two launches then, the results per (K, class) in between in global memory; the second is launched beside the
+// first (programmatic) and has its job's fair share ready when the results are there (0.6 us less than two launches
+// one behind the other).  A warp's lanes evaluate the points lane, lane + 32, ..., MQ of them side by side.
+template <bool SAMPLES, int MQ>
+__global__ void __launch_bounds__(256, 4) sweep_kernel(TableArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int j = a.j_first + (int)blockIdx.x, lane = threadIdx.x & 31;
+  const int x = (int)(blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5));
+  int pr;
+  if (x < a.pair_count) {
+    pr = __ldg(a.pairs + a.pair_first + x);
+  } else {            // (rack table alone: the pair that holds the fair share is wanted too)
+    const int fair = x == a.pair_count && !a.speedup ? fair_place(a, j) : -1;
+    if (fair < 0) return;
+    pr = fair / 3 * 4 + fair % 3;
+  }
+  const JobModel jm = job_model(a.jp, j);
+  const int32_t *grid = a.m_grid + (size_t)j * a.G;
+  const bool adapt = !SAMPLES || !a.adaptive || a.adaptive[j];
+  const int mmax = SAMPLES ? a.m_max_gpu[j] : 1;
+  const int G = !SAMPLES ? a.G : mmax < 1 ? 0 : adapt ? a.G : 1;
+  const float rinv = adapt ? 1.f / (jm.phi + jm.M0) : 0.f;   // (phi + M) rinv = 1 / EFFICIENCY; 1 when fixed
+  const float c0 = adapt ? jm.phi * rinv : 1.f;
+  const int K = pr >> 2;
+  const float ts = sync_time(jm, K, pr & 3);
+  Best best = {0.f, 1.f, 0xFFFFFFFFu};
+  for (int i = lane; i < G; i += 32 * MQ) {
+    if (SAMPLES) {
+      const Best p = sample_point_inline(jm, ts, K, rinv, c0, mmax, adapt ? (long long)__ldg(grid + i) : (long long)jm.M0, i);
+      if (beats(p, best)) best = p;
+    } else {
+      int m[MQ];
+#pragma unroll
+      for (int q = 0; q < MQ; ++q) m[q] = __ldg(grid + min(i + 32 * q, G - 1));
+      grid_points<MQ>(jm, ts, (float)K, rinv, c0, m, i, (G - i + 31) / 32, a.Gs, a.one, a.zero, best);
+    }
+  }
+  best = warp_best(best);
+  if (lane == 0) {
+    const size_t at = (size_t)j * (a.k_max + 1) * 3 + K * 3 + (pr & 3);
+    const bool found = best.num > 0.f;
+    a.g[at] = found ? best.num / best.den : 0.f;
+    a.a[at] = !found ? (uint16_t)0xFFFFu : (uint16_t)(SAMPLES ? best.tie : (best.tie & 0xFFFFu) * a.Gs + (best.tie >> 16));
+  }
+}
+
+__global__ void __launch_bounds__(256) slab_kernel(TableArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int KD = a.k_max + 1, j = a.j_first + (int)blockIdx.x;
+  const int fair = fair_place(a, j);
+  const TableSmem t = {a.g + (size_t)j * KD * 3, a.a + (size_t)j * KD * 3};
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  write_tables(a, t, (TableRow *)smem, j, 0, 1, fair);
 }
 
 // REALLOC_FACTOR_j(delta) = (T_j - R_j delta) / (T_j + delta), clamped to [0, 1].
@@ -711,16 +841,69 @@ int launch_autoscale(sched_ctx *ctx, const float *d_goodput, const int32_t *d_cu
   return SCHED_OK;
 }
 
+// A block of at most eight warps per job and eight pairs; then one per job, an aligned four of the slab per
+// thread (fewer than four warps make its first phase longer: 8 x 4, 64 jobs: 7.9 us with three, 6.6 so).
+template <bool SAMPLES>
+static int launch_small_table(sched_ctx *ctx, const TableArgs &a, int jobs) {
+  const int warps = a.pair_count + (a.speedup ? 0 : 1);      // (the fair share's pair)
+  if (warps > 0) {
+    const int threads = 32 * std::min(8, warps);
+    const dim3 grid((unsigned)jobs, (unsigned)((warps + 7) / 8));
+    TimedLaunch tl_(ctx, KK_TABLE);
+    if (SAMPLES || a.G <= 32) sweep_kernel<SAMPLES, 1><<<grid, threads, 0, ctx->stream>>>(a);
+    else if (a.G <= 64) sweep_kernel<false, 2><<<grid, threads, 0, ctx->stream>>>(a);
+    else sweep_kernel<false, 4><<<grid, threads, 0, ctx->stream>>>(a);
+    SCHED_LAUNCH_CHECK(ctx);
+  }
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)jobs);
+  lc.blockDim = dim3((unsigned)std::max(128, std::min(256, (ctx->KD * ctx->ND / 4 + 32) & ~31)));
+  lc.dynamicSmemBytes = (size_t)(ctx->KD + 1) * sizeof(TableRow);
+  lc.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = warps > 0 ? 1 : 0;
+  {
+    TimedLaunch tl_(ctx, KK_TABLE);
+    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, slab_kernel, a));
+  }
+  SCHED_LAUNCH_CHECK(ctx);
+  return SCHED_OK;
+}
+
+// Whether the two launches above are the shorter way: the sweep's work (groups of 32 points, each with its
+// steps) against the time of the one launch, which hardly depends on it up to 64 points, is a jump longer up to 128
+// (several points come near one another) and far longer beyond (no room to note those: all points again).
+// The lines lie where the two take the same time, measured for 2 x 2 to 128 x 8 GPUs and 8 to 1024 jobs (two
+// launches / one, us): 4 x 4 GPUs with 32 points and 16 steps: 8 jobs 4.8 / 7.9, 384 jobs 8.5 / 8.9, 512 jobs 9.7 / 9.0;
+// 16 x 4 with 64 points: 48 jobs 7.1 / 9.2, 96 jobs 10.5 / 9.5; 4 x 4 with 128 points: 256 jobs 12 / 14.5, 384
+// jobs 14.1 / 16.0; 300 points, 4 x 4, 384 jobs: 29 / 46, 32 x 8, 256 jobs: 60 / 54; 300 samples, 16 x 4, 512 jobs: 82 / 106.
+// (Contexts too large for any of this have no room for the results in between; a list too long for the screening
+// takes this way wherever there is.)
+static bool small_table(const sched_ctx *ctx, long long job_pairs, int G, int Gs, bool samples) {
+  const long long work = job_pairs * ((G + 31) / 32) * (samples ? 32 : 32 + Gs);
+  return ctx->d_gmax && (G > MAX_POINTS || work <= (G <= 64 ? 400000 : G <= 128 ? 1000000 : samples ? 20000000 : 8000000));
+}
+
 // A cluster of blocks per job: one block where the jobs alone give every SM two or where a job's (K, class)
 // pairs fill no more than one, more otherwise, up to eight (large tables of few jobs gain as much as their
 // sweep: each block writes its share of the slab).  A pair is shared by up to eight threads while all of
 // them fit the GPU at once (registers: some 1170 threads per SM).  At least four warps, whatever the pairs
 // are: pairs with several close points are spread over them (700 jobs x 11 pairs x 87 samples: 28.7 us
 // with one warp and two threads per pair, 16.5 us).
-static int launch_table(sched_ctx *ctx, void (*kernel)(TableArgs), TableArgs &a) {
+template <bool SAMPLES>
+static int launch_table(sched_ctx *ctx, TableArgs &a) {
   const int J = ctx->cfg.num_jobs;
   for (int j0 = 0; j0 < J; j0 += 65536) {
     const int jobs = std::min(65536, J - j0);
+    a.j_first = j0;
+    if (small_table(ctx, (long long)jobs * a.pair_count, a.G, a.Gs, SAMPLES)) {
+      const int rc = launch_small_table<SAMPLES>(ctx, a, jobs);
+      if (rc != SCHED_OK) return rc;
+      continue;
+    }
     int nb = 1;
     while (nb < 8 && jobs * nb < 2 * ctx->num_sms && a.pair_count * MAX_PARTS > 128 * nb) nb *= 2;
     const int pairs = std::max(1, (a.pair_count + nb - 1) / nb);
@@ -733,7 +916,6 @@ static int launch_table(sched_ctx *ctx, void (*kernel)(TableArgs), TableArgs &a)
     const int ppp = (((a.G + parts - 1) / parts) + 3) & ~3;
     a.parts = parts;
     a.points = a.G <= MAX_POINTS ? ppp * parts : 0;
-    a.j_first = j0;
     const int threads = std::max(128, std::min(512, (pairs * parts + 31) & ~31));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(jobs * nb));
@@ -747,10 +929,10 @@ static int launch_table(sched_ctx *ctx, void (*kernel)(TableArgs), TableArgs &a)
     lc.attrs = attr;
     lc.numAttrs = 1;
     if (lc.dynamicSmemBytes > 48 * 1024)
-      SCHED_CUDA_CHECK(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes));
+      SCHED_CUDA_CHECK(ctx, cudaFuncSetAttribute(table_kernel<SAMPLES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes));
     {
       TimedLaunch tl_(ctx, KK_TABLE);
-      SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, kernel, a));
+      SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, table_kernel<SAMPLES>, a));
     }
     SCHED_LAUNCH_CHECK(ctx);
   }
@@ -765,6 +947,8 @@ static TableArgs table_args(const sched_ctx *ctx, const sched_jobs *jobs) {
   a.m_grid = jobs->m_grid;
   a.pairs = ctx->d_pairs;
   a.pair_count = ctx->num_pairs;
+  a.g = ctx->d_gmax; a.a = ctx->d_amax;
+  a.one = 1.f; a.zero = 0.f;
   a.kfit = ctx->d_kfit; a.nmin = ctx->d_nmin; a.fair_k = jobs->fair_k; a.fair_n = jobs->fair_n;
   a.k_max = c.k_max; a.n_max = c.n_max; a.G = c.grid_m; a.Gs = c.grid_s;
   return a;
@@ -784,7 +968,7 @@ int launch_speedup_table(sched_ctx *ctx, const sched_jobs *jobs, float *d_goodpu
     if (d_speedup) a.pair_count += ctx->num_rack_pairs;
     else { a.pair_first = ctx->num_pairs; a.pair_count = ctx->num_rack_pairs; }
   }
-  return launch_table(ctx, table_kernel<false>, a);
+  return launch_table<false>(ctx, a);
 }
 
 int launch_speedup_table_msample(sched_ctx *ctx, const sched_jobs *jobs, const int32_t *d_m_samples, int G,
@@ -794,7 +978,7 @@ int launch_speedup_table_msample(sched_ctx *ctx, const sched_jobs *jobs, const i
   TableArgs a = table_args(ctx, jobs);
   a.m_grid = d_m_samples; a.m_max_gpu = d_m_max_gpu; a.adaptive = d_adaptive; a.G = G;
   a.goodput = d_goodput; a.speedup = d_speedup; a.argmax = d_argmax;
-  return launch_table(ctx, table_kernel<true>, a);
+  return launch_table<true>(ctx, a);
 }
 
 int launch_realloc_factor(sched_ctx *ctx, const sched_jobs *jobs, float *d_out) {

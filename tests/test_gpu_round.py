@@ -309,7 +309,7 @@ def test_kernel_timing_names_the_kernels_that_ran(gpu, route, search):
     s.schedule_round(dj, d_cur, best, bf, round=0, generations=6)
     s.sync_status()
     ran = {name: n for name, (ms, n) in s.read_kernel_timing().items() if n}
-    assert ran["speedup_table"] == 1
+    assert ran["speedup_table"] in (1, 2)
     assert [k for k in ("round_search", "generation_store", "rows") if k in ran] == [search]
     assert ran[search] == (1 if route == "default" else 7)         # the search, or a launch per population
     s.close()

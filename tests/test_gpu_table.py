@@ -150,3 +150,58 @@ def test_slabs_of_any_width_and_place(gpu, oracle, nodes, gpus, jobs):
     gp, sp, am = _gpu_table(gpu, cl, j, 8)
     gp_r, sp_r, am_r = oracle.build_speedup_table(j, cl.node_capacity, cl.k_max, cl.n_max, 8)
     check_table(oracle, j, 8, gp, sp, am, gp_r, sp_r, am_r)
+
+
+@pytest.mark.parametrize("kind,nodes,gpus,points,steps,many,few", [
+    ("grid", 4, 4, 32, 16, 900, 7), ("grid", 6, 2, 100, 8, 2500, 30), ("grid", 17, 4, 64, 16, 400, 21), ("grid", 32, 8, 128, 32, 100, 24),
+    ("grid", 4, 4, 300, 8, 3000, 40), ("grid", 1, 1, 33, 8, 9000, 3), ("flat", 6, 4, 128, 9, 900, 20), ("flat", 6, 4, 129, 4, 5000, 20),
+    ("big", 5, 8, 64, 8, 500, 11), ("samples", 8, 4, 48, 1, 400, 20), ("samples", 5, 8, 128, 1, 700, 50),
+    ("samples", 3, 2, 300, 1, 9000, 9), ("fixed", 8, 4, 90, 1, 600, 20), ("rack", 9, 8, 64, 16, 200, 12), ("rack", 4, 4, 31, 8, 2000, 5)])
+def test_tables_in_two_launches_equal_those_in_one(gpu, oracle, kind, nodes, gpus, points, steps, many, few):
+    """Few (job, K, class): a sweep of all points and the slabs, two launches; many: one launch that screens.  The
+    same job's table is the same bit for bit, and a sample agrees with the oracle."""
+    torch, api = gpu
+    cl = synth.uniform_cluster(nodes, gpus)
+    samples = kind in ("samples", "fixed")
+    jobs = synth.draw_jobs(many, 5, 32 if samples else points, max(steps, 8), cl.k_max)
+    if kind == "flat":
+        jobs.alpha_grad[:] = 1e-6
+        jobs.alpha_local[:] = jobs.alpha_node[:] = 1e-7
+        jobs.beta_local[:] = jobs.beta_node[:] = 0.0
+        jobs.phi[:] = 1e6
+    if kind == "big":
+        jobs.m0[:] = 1 << 20
+        jobs.m_max_total[:] = 12 << 20
+        jobs.m_max_gpu[:] = 1 << 18
+        jobs.m_grid = synth.make_m_grid(jobs.m_max_gpu, points)
+    jobs = with_fair_share(jobs, cl)
+    adaptive = (np.arange(many) % 3 != 0).astype(np.uint8) if kind == "fixed" else None
+    ar, br = synth.draw_rack_pair(jobs, 8)
+    idx = np.unique(np.linspace(0, many - 1, few).astype(int))
+    out = []
+    for take, launches in ((np.arange(many), 1), (idx, 2)):
+        j = jobs.take(take)
+        dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+        s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=j.num_jobs, grid_m=j.m_grid.shape[1], grid_s=max(steps, 1),
+                          population=1, stream=torch.cuda.current_stream().cuda_stream)
+        dj = api.DeviceJobs(j, "cuda", torch)
+        gp = torch.full(s.table_shape, -1.0, device="cuda")
+        sp, am = torch.full_like(gp, -1.0), torch.full(s.table_shape, 7, dtype=torch.uint16, device="cuda")
+        s.set_kernel_timing(True)
+        if samples:
+            s.build_speedup_table_msample(dj, dev(synth.make_m_samples(j.m0, j.m_max_total, points)), dev(j.m_max_gpu), gp, sp, am,
+                                          adaptive=None if adaptive is None else dev(adaptive[take]))
+        elif kind == "rack":
+            s.build_speedup_table_rack(dj, dev(ar[take]), dev(br[take]), gp, sp, am)
+        else:
+            s.build_speedup_table(dj, gp, sp, am)
+        s.sync_status()
+        assert s.read_kernel_timing()["speedup_table"][1] == launches
+        out.append([x.cpu().numpy() for x in (gp, sp, am)])
+        s.close()
+    for one, two in zip(*out):
+        assert np.array_equal(one[idx], two)
+    if kind in ("grid", "flat", "big"):
+        ref = oracle.build_speedup_table(jobs.take(idx), cl.node_capacity, cl.k_max, cl.n_max, steps)
+        check_table(oracle, jobs.take(idx), steps, *out[1], *ref)
+    assert (out[0][0] > 0).any()
