@@ -1,9 +1,9 @@
 // Speedup-table builder: goodput sweep over the (m, s) grid (Eq. 4-11, 13) and
-// normalisation by the fair-share goodput (Eq. 15), one launch per table.
+// normalisation by the fair-share goodput (Eq. 15): one launch per table, two for small ones.
 //
 // The goodput of an allocation depends on the allocation only through K = SUM(a) and its
 // placement class (one node, several nodes, several racks; Eq. 9), so a job's sweep runs once
-// per (K, class).  One cluster of thread blocks serves one job: its blocks share the job's
+// per (K, class).  In one launch, a cluster of thread blocks serves one job: its blocks share the job's
 // (K, class) pairs, every result goes to all of them (distributed shared memory), and each
 // then writes its part of the job's [K][N] slabs from shared memory.
 #include <cooperative_groups.h>
@@ -402,8 +402,7 @@ __device__ __forceinline__ void write_tables(const TableArgs &a, const TableSmem
 // compares them in the order of its lanes.
 // Bound: special-function unit (five operations a point, an eighth of the issue rate) beside the
 // table's own bytes.  Measured for 1024 jobs x 71 pairs x 128 points (x 32 steps), all three outputs (43 MB):
-// 134 us with a scan over s at every point and a launch of its own for the slabs, 42 us now; 48 jobs x 67
-// pairs x 64 points: 12.3 us and 10.2 us, latency.
+// 134 us with a scan over s at every point and a launch of its own for the slabs, 44 us so.
 constexpr int IDX_BITS = 7;               // points a thread can tell apart
 constexpr int MAX_PARTS = 8;
 constexpr int MAX_POINTS = MAX_PARTS << IDX_BITS;   // longer lists are evaluated exactly, all points
@@ -879,7 +878,7 @@ static int launch_small_table(sched_ctx *ctx, const TableArgs &a, int jobs) {
 // The lines lie where the two take the same time, measured for 2 x 2 to 128 x 8 GPUs and 8 to 1024 jobs (two
 // launches / one, us): 4 x 4 GPUs with 32 points and 16 steps: 8 jobs 4.8 / 7.9, 384 jobs 8.5 / 8.9, 512 jobs 9.7 / 9.0;
 // 16 x 4 with 64 points: 48 jobs 7.1 / 9.2, 96 jobs 10.5 / 9.5; 4 x 4 with 128 points: 256 jobs 12 / 14.5, 384
-// jobs 14.1 / 16.0; 300 points, 4 x 4, 384 jobs: 29 / 46, 32 x 8, 256 jobs: 60 / 54; 300 samples, 16 x 4, 512 jobs: 82 / 106.
+// jobs 14.1 / 16.0; 300 points, 4 x 4, 384 jobs: 29 / 46, 32 x 8, 256 jobs: 60 / 54; 300 samples, 16 x 4, 512 jobs: 77 / 106.
 // (Contexts too large for any of this have no room for the results in between; a list too long for the screening
 // takes this way wherever there is.)
 static bool small_table(const sched_ctx *ctx, long long job_pairs, int G, int Gs, bool samples) {

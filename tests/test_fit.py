@@ -48,6 +48,59 @@ def test_oracle_fit_recovers_the_noise_floor():
     assert np.all(xz[2:6] == 0.0) and fz >= f * 0.999
 
 
+DIVIDE = r"""
+#include <stdio.h>
+#include <stdint.h>
+#include <string.h>
+#include "divide.cuh"
+
+static uint64_t state = 12345;
+static uint64_t next64() {                       // splitmix64
+  uint64_t z = (state += 0x9E3779B97F4A7C15ull);
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return z ^ (z >> 31);
+}
+static double number(uint64_t bits, int exponent) {    // significand: random, or one where rounding is close
+  uint64_t f = next64() & 0xFFFFFFFFFFFFFull;
+  if (bits % 4 == 1) f = 0xFFFFFFFFFFFFFull - (next64() & 7);
+  if (bits % 4 == 2) f = next64() & 7;
+  if (bits % 4 == 3) f = (next64() & 7) << 49 | (next64() & 3);
+  const double v = ldexp(1.0 + ldexp((double)f, -52), exponent);
+  return bits & 64 ? -v : v;
+}
+int main() {
+  long long n = 0, bad = 0;
+  for (int k = 0; k < 20000000; ++k) {
+    const uint64_t r = next64();
+    int ea, eb;
+    do {
+      ea = -968 + (int)(next64() % 1988);
+      eb = -1021 + (int)(next64() % 2041);
+      if (r & 128) { ea = -40 + ea % 40; eb = -40 + eb % 40; }      // the usual exponents
+    } while (ea - eb < -1019 || ea - eb > 1019);
+    const double b = number(r >> 10, eb), a = k % 1000 ? number(r >> 20, ea) : 0.0, q = a / b, got = divide_by(a, b, 1.0 / b);
+    ++n;
+    bad += q != got;
+  }
+  printf("%lld %lld\n", n, bad);
+  return 0;
+}
+"""
+
+
+def test_division_by_a_reciprocal_is_the_division(tmp_path):
+    """The quotient of two corrected multiplications equals the division's, bit for bit, over the exponents
+    the method is stated for (fma and reciprocal are correctly rounded here as on the GPU)."""
+    import subprocess
+    from paper_2008_12260_b200 import build
+    src, exe = tmp_path / "divide.cpp", tmp_path / "divide"
+    src.write_text(DIVIDE)
+    subprocess.check_call(["g++", "-O2", "-ffp-contract=off", "-I", build.CSRC, "-o", str(exe), str(src)])
+    n, bad = subprocess.check_output([str(exe)]).split()
+    assert int(n) == 20000000 and int(bad) == 0
+
+
 def _problem(J, per_job, seed):
     fit = _fit()
     jobs = synth.draw_jobs(J, seed, 8, 4, 16)
