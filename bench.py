@@ -57,8 +57,9 @@ CONFIG = {
 # written: some parent rows are shared by several children and come from L2).
 # "fitness_stress": 16 dense stress candidates moved 544.8 + 3.5 MB; every candidate is streamed
 # once, so the figure is scaled by candidates / 16 to the chunk that is timed.
-# "round_search": its records stay in L2; what it moves to and from DRAM has not been counted.
-NCU_TRAFFIC_BYTES = {"rows": 461.4e6, "fitness_stress_per_candidate": 548.3e6 / 16, "round_search": None}
+# "round_search": per generation, a 201st of one large round's 12.0 MB read and 2328 MB written (records stay in
+# L2 or are written back from it).
+NCU_TRAFFIC_BYTES = {"rows": 461.4e6, "fitness_stress_per_candidate": 548.3e6 / 16, "round_search": 2340.3e6 / 201}
 
 
 def measured_peaks():
@@ -359,8 +360,8 @@ def run_ours(args):
                     "avg_launch_us_with_event_pairs": dom["avg_us"],
                     "launches_per_step": 1, "share_of_step": round(gen_us_clean * (G + 1) / (1e3 * t_max / args.steps), 3),
                     "note": "one launch runs the round's search, one block at a time to a candidate, on L2-resident "
-                            "32-byte records: bound by the length of a block's chain of dependent steps and by "
-                            "instruction issue, not by DRAM (the dense operator "
+                            "32-byte records: bound by the length of a block's chain of dependent steps beside "
+                            "instruction issue (45 % of the slots), not by DRAM (the dense operator "
                             "kernel, which is, is reported under dense_generation)",
                     # what the same generation costs on dense matrices (parents read, children written, the
                     # repair's row and column passes: about four population sweeps): the bytes this kernel

@@ -82,8 +82,8 @@ int ensure_round_scratch(sched_ctx *ctx) {
     ctx->round_ready = true;
     return SCHED_OK;
   }
-  // Most problems keep the round's population in the row store; if it cannot be allocated the round
-  // runs on dense matrices.
+  // Where the one-launch search does not fit, the row store; if that does not fit or cannot be allocated,
+  // dense matrices.
   if (rowstore_eligible(ctx) && !ctx->rs_off) {
     if (rowstore_ensure(ctx) != SCHED_OK) ctx->rs_off = true;
   }

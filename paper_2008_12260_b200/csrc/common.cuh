@@ -98,7 +98,7 @@ struct sched_ctx {
   int16_t *d_pop_last;   // points at d_popA or d_popB after a round
   bool round_ready;
 
-  // Row store of a running round (large problems): rows live once in a pool and candidates
+  // Row store of a running round (budgets that the one-launch search does not fit): rows live once in a pool and candidates
   // hold row indices, so a child row that equals its parent's costs one index.
   int16_t *rs_pool;        // [2 * rs_half_cap + 1][num_nodes] row contents (last slot: the empty row)
   uint32_t *rs_rec;        // [slots][8] up to 7 occupied nodes of the row (node | GPUs << 12, or an overflow
@@ -279,7 +279,7 @@ __device__ __forceinline__ int nth_occupied(const int16_t *row, int num_nodes, u
   return -1;
 }
 
-// kernels' launchers (defined in table.cu / fitness.cu / ga.cu / rowstore.cu)
+// kernels' launchers (defined in table.cu / fitness.cu / ga.cu / fit.cu)
 int launch_speedup_table(sched_ctx *ctx, const sched_jobs *jobs, float *d_goodput, float *d_speedup, uint16_t *d_argmax,
                          const float *d_alpha_rack = nullptr, const float *d_beta_rack = nullptr,
                          float *d_goodput_rack = nullptr, float *d_speedup_rack = nullptr,

@@ -1,6 +1,6 @@
-// Pieces of the fitness evaluation (Eq. 14) shared by the dense fitness kernel and the
-// fused small-problem generation kernel, so that both produce identical bits: the term of
-// one row, the reduction of a block's terms in a fixed order, and the final power mean.
+// Pieces of the fitness evaluation (Eq. 14) shared by the dense fitness kernels, the one-launch search and
+// the row store, so that all produce identical bits: the term of one row, the reduction of a block's terms in
+// a fixed order, and the final power mean.
 #pragma once
 
 #include "common.cuh"
