@@ -550,9 +550,7 @@ int repair_population(sched_ctx *ctx, const sched_jobs *d_jobs, int16_t *d_pop, 
   REQUIRE(ctx, (long long)count * ctx->cfg.num_jobs < (1LL << 31), SCHED_ERR_TOO_LARGE,
           "repair_population: count * num_jobs must be below 2^31");
   if (ctx->cfg.num_jobs == 0) return SCHED_OK;
-  int rc = launch_set_round(ctx, round);
-  if (rc != SCHED_OK) return rc;
-  return launch_repair(ctx, d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr, d_pop,
+  return launch_repair(ctx, make_key_of_round(ctx->cfg.seed, round), d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr, d_pop,
                        count, first_candidate, generation);
 }
 
@@ -563,9 +561,7 @@ int init_population(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_c
   REQUIRE(ctx, ((uintptr_t)d_pop_out & 1) == 0 && ((uintptr_t)d_cur & 1) == 0, SCHED_ERR_INVALID_ARG,
           "init_population: a buffer is misaligned");
   if (ctx->cfg.num_jobs == 0) return SCHED_OK;
-  int rc = launch_set_round(ctx, round);
-  if (rc != SCHED_OK) return rc;
-  return launch_init_population(ctx, d_jobs ? d_jobs->k_cap : nullptr,
+  return launch_init_population(ctx, make_key_of_round(ctx->cfg.seed, round), d_jobs ? d_jobs->k_cap : nullptr,
                                 d_jobs ? d_jobs->active : nullptr, d_cur, d_pop_out);
 }
 
@@ -578,9 +574,7 @@ int ga_generation(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d_pop
   REQUIRE(ctx, (((uintptr_t)d_pop_in | (uintptr_t)d_pop_out) & 1) == 0 && ((uintptr_t)d_fitness_in & 3) == 0,
           SCHED_ERR_INVALID_ARG, "ga_generation: a buffer is misaligned");
   if (ctx->cfg.num_jobs == 0) return SCHED_OK;
-  int rc = launch_set_round(ctx, round);
-  if (rc != SCHED_OK) return rc;
-  return launch_generation(ctx, d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr,
+  return launch_generation(ctx, make_key_of_round(ctx->cfg.seed, round), d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr,
                            d_pop_in, d_fitness_in, d_pop_out, generation);
 }
 
@@ -600,9 +594,7 @@ int ga_generation_shard(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t 
           SCHED_ERR_INVALID_ARG, "ga_generation_shard: parents and children must not overlap");
   REQUIRE(ctx, (((uintptr_t)d_pop_in | (uintptr_t)d_children) & 1) == 0 && ((uintptr_t)d_fitness_in & 3) == 0,
           SCHED_ERR_INVALID_ARG, "ga_generation_shard: a buffer is misaligned");
-  int rc = launch_set_round(ctx, round);
-  if (rc != SCHED_OK) return rc;
-  return launch_generation(ctx, d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr, d_pop_in,
+  return launch_generation(ctx, make_key_of_round(ctx->cfg.seed, round), d_jobs ? d_jobs->k_cap : nullptr, d_jobs ? d_jobs->active : nullptr, d_pop_in,
                            d_fitness_in, d_children, generation, first_child, num_children);
 }
 
@@ -674,14 +666,14 @@ static int round_body(sched_ctx *ctx, const sched_jobs *d_jobs, const int16_t *d
     }
   } else {
     if (ctx->rs_ready) pa = ctx->rs_pool;   // no generations: the dense initial population sits at the start of the pool
-    if (rc == SCHED_OK) rc = launch_init_population(ctx, d_jobs->k_cap, d_jobs->active, d_cur, pa);
+    if (rc == SCHED_OK) rc = launch_init_population(ctx, make_key(ctx->cfg.seed, ctx->d_round), d_jobs->k_cap, d_jobs->active, d_cur, pa);
     if (rc == SCHED_OK) rc = fitness_of(pa, fit_cur);
   }
   for (int g = 0; g < generations && rc == SCHED_OK && !store; ++g) {
     // children's summaries go to the other half; the parents' feed the unperturbed rows
     ctx->round_summ_in = ctx->summ_valid ? ctx->round_summ : nullptr;
     if (!racks) std::swap(ctx->round_summ, summ_other);
-    rc = launch_generation(ctx, d_jobs->k_cap, d_jobs->active, pa, fit_cur, pb, (uint32_t)g);
+    rc = launch_generation(ctx, make_key(ctx->cfg.seed, ctx->d_round), d_jobs->k_cap, d_jobs->active, pa, fit_cur, pb, (uint32_t)g);
     if (rc != SCHED_OK) break;
     std::swap(pa, pb);
     rc = fitness_of(pa, fit_next);

@@ -230,24 +230,35 @@ __host__ __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, uint32_t k0, ui
 }
 
 // Random stream of the operators: key = (seed_lo ^ seed_hi, round),
-// counter = (idx, candidate, generation, slot).  The round number is read from device
-// memory so that a captured CUDA graph of a round can be replayed for any round.
+// counter = (idx, candidate, generation, slot).  Inside a round the round number is read from device
+// memory so that a captured CUDA graph of a round can be replayed for any round; an entry point
+// called on its own hands it over by value (round_ptr NULL).
 struct RngKey {
   uint32_t k0;
   const uint32_t *round_ptr;
+  uint32_t round;
 };
 
 inline RngKey make_key(uint64_t seed, const uint32_t *d_round) {
   RngKey k;
   k.k0 = (uint32_t)seed ^ (uint32_t)(seed >> 32);
   k.round_ptr = d_round;
+  k.round = 0u;
   return k;
 }
+
+inline RngKey make_key_of_round(uint64_t seed, uint32_t round) {
+  RngKey k = make_key(seed, nullptr);
+  k.round = round;
+  return k;
+}
+
+__device__ __forceinline__ uint32_t round_of(const RngKey &k) { return k.round_ptr ? __ldg(k.round_ptr) : k.round; }
 
 __device__ __forceinline__ u32x4 draw(RngKey k, uint32_t idx, uint32_t cand, uint32_t gen,
                                       uint32_t slot) {
   u32x4 c = {idx, cand, gen, slot};
-  return philox4x32_10(c, k.k0, __ldg(k.round_ptr));
+  return philox4x32_10(c, k.k0, round_of(k));
 }
 
 // floor(w * n / 2^32): an integer in [0, n)
@@ -271,9 +282,10 @@ __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xffff
 __device__ __forceinline__ int nth_occupied(const int16_t *row, int num_nodes, uint32_t t, int lane) {
   for (int base = 0; base < num_nodes; base += 32) {
     const int n = base + lane;
-    const unsigned m = __ballot_sync(0xffffffffu, n < num_nodes && row[n] > 0);
+    const bool on = n < num_nodes && row[n] > 0;
+    const unsigned m = __ballot_sync(0xffffffffu, on);
     const uint32_t c = __popc(m);
-    if (t < c) return base + (int)__fns(m, 0, (int)t + 1);
+    if (t < c) return base + __ffs(__ballot_sync(0xffffffffu, on && __popc(m & ((1u << lane) - 1u)) == (int)t)) - 1;
     t -= c;
   }
   return -1;
@@ -293,11 +305,11 @@ int launch_autoscale(sched_ctx *ctx, const float *d_goodput, const int32_t *d_cu
 int launch_fitness(sched_ctx *ctx, const int16_t *d_pop, int32_t count, const float *d_speedup,
                    const int16_t *d_cur, const float *d_rf, const uint8_t *d_active, float p,
                    float *d_fitness, const uint32_t *d_summ = nullptr, const float *d_speedup_rack = nullptr);
-int launch_repair(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
+int launch_repair(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
                   int32_t count, uint32_t first_candidate, uint32_t generation);
-int launch_init_population(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active,
+int launch_init_population(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active,
                            const int16_t *d_cur, int16_t *d_pop_out);
-int launch_generation(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active,
+int launch_generation(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active,
                       const int16_t *d_pop_in, const float *d_fitness_in, int16_t *d_pop_out,
                       uint32_t generation, int first_child = 0, int num_children = -1);
 int launch_set_round(sched_ctx *ctx, uint32_t round);

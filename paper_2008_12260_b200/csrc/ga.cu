@@ -4,15 +4,21 @@
 // stream, so every output is a pure function of the inputs.
 //
 // Implementations of the same operators on dense matrices, chosen by shape:
-//  * rows_kernel + cols_kernel (+ rank_kernel): the general pair - a warp per (candidate, job)
-//    row through shared memory, then a thread per (candidate, node) column;
-//  * rows2_kernel + colrepair_kernel: rows of whole 16-byte vectors and at most 512 nodes -
+//  * child_kernel: one launch, a block or a cluster of blocks per child, rows of any width up to 512 nodes (the
+//    entry points called on their own);
+//  * rows2_kernel + colrepair_kernel: rows of whole 16-byte vectors and at most 512 nodes, with per-row summaries -
 //    batched rows with fused column sums and occupant lists, a work list of violating nodes;
-//  * rows_stream_kernel + colrepair_kernel: the same without per-row summaries (entry points).
+//  * rows_kernel + cols_kernel (+ rank_kernel): the general pair - a warp per (candidate, job)
+//    row through shared memory, then a thread per (candidate, node) column.
 // Rounds do not use dense matrices for their generations (round_flow.cu, rowstore.cu) unless neither the
 // blocks nor the memory of those fit.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "common.cuh"
 #include "fitness_common.cuh"
+#include "search_common.cuh"
 
 namespace {
 
@@ -863,326 +869,6 @@ __global__ void __launch_bounds__(256, 4) rows2_kernel(Rows2Args aa) {
   }
 }
 
-// ---------------------------------------------------------------------------------------
-// Streaming row kernel: the row pass when no per-row summaries are wanted (the dense entry
-// points called on their own) and a row is a power-of-two number of 16-byte vectors.
-//
-// Almost every entry of a population is zero and almost every row is copied unchanged, so the
-// rows are moved as a stream - a warp reads its 32 rows as one flat run of vectors, four loads
-// per lane in flight, and stores them straight back out - and only the vectors that hold
-// something are looked at: they are compacted into a per-warp queue (ballot + popc) and
-// expanded one lane per entry, once to get each row's K, N and whether any entry leaves
-// [0, node size], and once more for the column totals and occupant lists.  A row that is
-// perturbed, has an entry out of range or breaks a row cap is rebuilt in shared memory by the
-// whole warp, written again, and its queue entries are replaced.  Same operators, draws and
-// results as rows2_kernel; block and grid shapes, column partials and the work list are shared
-// with it.
-// ---------------------------------------------------------------------------------------
-constexpr int STREAM_QCAP = 128;        // vectors a warp queues per tile
-
-// dynamic shared memory of the streaming kernel: per-node arrays sized by the cluster
-__host__ __device__ inline size_t stream_smem_bytes(int NN) {
-  return (size_t)8 * NN * 2          // a row per warp (rebuilt rows)
-         + (size_t)NN * 2            // node sizes
-         + (size_t)NN * 4 * 3        // GPUs placed, distributed jobs, occupants per node
-         + (size_t)NN * OCC_SLOTS * 4;
-}
-
-__global__ void __launch_bounds__(256, 4) rows_stream_kernel(Rows2Args aa) {
-  const RowsArgs &a = aa.r;
-  extern __shared__ __align__(16) unsigned char stream_smem[];
-  const int NN = a.num_nodes, J = a.J;
-  int16_t *s_rows = (int16_t *)stream_smem;                       // [8][NN] per-warp buffer for a row that is rebuilt
-  int16_t *s_cap = s_rows + (size_t)8 * NN;                       // node sizes floored at 0
-  int32_t *s_tot = (int32_t *)(s_cap + NN), *s_el = s_tot + NN, *s_cnt = s_el + NN;
-  uint32_t *s_occ = (uint32_t *)(s_cnt + NN);
-  __shared__ int s_parent[2];
-  __shared__ __align__(16) uint4 s_qvec[8][STREAM_QCAP];
-  __shared__ uint32_t s_qmeta[8][STREAM_QCAP];       // row (bits 0..4) | vector of the row (8..13) | alive (31)
-  __shared__ int s_rowK[8][32], s_rowN[8][32], s_rowbad[8][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cl = blockIdx.y, batch = blockIdx.x;
-  const uint32_t c = a.first_cand + (uint32_t)cl;
-  const int row_vecs = NN >> 3;                      // a power of two, 1 .. 64
-  const int rv_log2 = 31 - __clz(row_vecs);
-  for (int i = threadIdx.x; i < NN; i += blockDim.x) {
-    s_tot[i] = 0; s_el[i] = 0; s_cnt[i] = 0;
-    s_cap[i] = (int16_t)max((int)a.cap[i], 0);
-  }
-  // ---- parents of this candidate (generation mode), found by the block itself (as rows2_kernel) ----
-  if (a.mode == ROWS_GENERATION) {
-    const int P = a.P;
-    if ((int)c < a.num_elite) {
-      for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const uint32_t ki = order_key(a.fitness_bits[i]);
-        int rk = 0;
-        for (int o = 0; o < P; ++o) {
-          const uint32_t ko = order_key(__ldg(a.fitness_bits + o));
-          rk += (ko > ki || (ko == ki && o < i)) ? 1 : 0;
-        }
-        if (rk == (int)c) s_parent[0] = s_parent[1] = i;
-      }
-    } else {
-      const u32x4 sel = draw(a.key, 0u, c, a.gen, SLOT_SELECT);
-      const int idx[4] = {(int)bounded(sel.x, P), (int)bounded(sel.y, P), (int)bounded(sel.z, P),
-                          (int)bounded(sel.w, P)};
-      if (threadIdx.x == 0) {
-        uint32_t k4[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) k4[q] = order_key(__ldg(a.fitness_bits + idx[q]));
-        s_parent[0] = tournament_winner(k4[0], idx[0], k4[1], idx[1]);
-        s_parent[1] = tournament_winner(k4[2], idx[2], k4[3], idx[3]);
-      }
-    }
-  }
-  __syncthreads();
-
-  const int j0 = batch * 256 + warp * 32;
-  const int nrows = min(32, J - j0);          // may be <= 0 for trailing warps
-  // ---- per-lane set-up for row j0 + lane: the row's draws, 32 side by side ---------------------
-  bool act_l = false, mut_l = false, sec_l = false;
-  int kc_l = 0;
-  u32x4 mw = {0, 0, 0, 0};
-  if (lane < nrows) {
-    const int j = j0 + lane;
-    act_l = !a.active || a.active[j];
-    kc_l = max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max));
-    if (a.mode == ROWS_GENERATION) {
-      if ((int)c >= a.num_elite) {
-        sec_l = (draw(a.key, (uint32_t)j, c, a.gen, SLOT_XOVER).x >> 31) != 0u;
-        mw = draw(a.key, (uint32_t)j, c, a.gen, SLOT_MUTATE);
-        mut_l = mw.x < a.thr;
-      }
-    } else if (a.mode == ROWS_INIT && c > 0) {
-      mw = draw(a.key, (uint32_t)j, c, GEN_INIT, SLOT_INIT);
-      mut_l = mw.x < a.thr;
-    }
-  }
-  const unsigned act_mask = __ballot_sync(0xffffffffu, act_l);
-  const unsigned sec_mask = __ballot_sync(0xffffffffu, sec_l);
-  const unsigned mut_mask = __ballot_sync(0xffffffffu, mut_l && act_l);
-
-  // row j0 of the possible sources; per row only the offset r * NN is added
-  const size_t roff0 = (size_t)j0 * NN;
-  const int16_t *src_a = nullptr, *src_b = nullptr;
-  if (a.mode == ROWS_GENERATION) {
-    src_a = a.src + (size_t)s_parent[0] * J * NN + roff0;
-    src_b = a.src + (size_t)s_parent[1] * J * NN + roff0;
-  } else if (a.mode == ROWS_INIT) {
-    src_a = src_b = a.src ? a.src + roff0 : nullptr;
-  } else {
-    src_a = src_b = a.dst + (size_t)cl * J * NN + roff0;
-  }
-  int16_t *dst0 = a.dst + (size_t)cl * J * NN + roff0;
-  int16_t *row = s_rows + (size_t)warp * NN;
-  uint4 *qvec = s_qvec[warp];
-  uint32_t *qmeta = s_qmeta[warp];
-
-  const int total_vecs = max(nrows, 0) << rv_log2;      // the warp's rows as one run of vectors
-  // Rows are contiguous, so the warp's rows are one flat array of vectors in each source and in the
-  // destination: vector t of the run is element t of all three.  What depends on the lane and the
-  // slot q only (a tile never splits a row) is worked out once: the vector's row within the tile and
-  // its place in that row.
-  const uint4 *flat_a = (const uint4 *)src_a, *flat_b = (const uint4 *)src_b;
-  uint4 *flat_d = (uint4 *)dst0;
-  uint32_t meta_q[4];
-  int rel_row[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int u = q * 32 + lane;
-    rel_row[q] = u >> rv_log2;
-    meta_q[q] = (uint32_t)rel_row[q] | ((uint32_t)(u & (row_vecs - 1)) << 8) | 0x80000000u;
-  }
-  for (int t0 = 0; t0 < total_vecs; t0 += 128) {
-    // rows of this tile: [r_first, r_first + rows_here)
-    const int r_first = t0 >> rv_log2;
-    const int rows_here = min(nrows - r_first, max(128 >> rv_log2, 1));
-    s_rowK[warp][lane] = 0; s_rowN[warp][lane] = 0; s_rowbad[warp][lane] = 0;
-    // ---- the stream: four vectors per lane in, queued if they hold anything, out ---------------
-    // (rows that are inactive or have no source read as empty)
-    uint4 x[4];
-    bool in[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = t0 + q * 32 + lane;
-      const int r = r_first + rel_row[q];
-      in[q] = t < total_vecs;
-      x[q] = make_uint4(0u, 0u, 0u, 0u);
-      if (in[q] && ((act_mask >> (r & 31)) & 1u) && flat_a) x[q] = __ldg((((sec_mask >> (r & 31)) & 1u) ? flat_b : flat_a) + t);
-    }
-    int qn = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const bool nz = (x[q].x | x[q].y | x[q].z | x[q].w) != 0u;      // vectors outside the run are empty
-      const unsigned bal = __ballot_sync(0xffffffffu, nz);
-      if (nz) {
-        const int pos = qn + __popc(bal & ((1u << lane) - 1u));
-        qvec[pos] = x[q];
-        qmeta[pos] = meta_q[q];
-      }
-      qn += __popc(bal);
-      if (in[q]) flat_d[t0 + q * 32 + lane] = x[q];       // final for every row that is not rebuilt below
-    }
-    __syncwarp();
-    // ---- first look at the queued entries: each row's K and N, entries outside [0, node size] ----
-    for (int e = lane; e < qn * 8; e += 32) {
-      const int val = (int)((const int16_t *)qvec)[e];
-      if (val != 0) {
-        const uint32_t meta = qmeta[e >> 3];
-        const int rr = (int)(meta & 31u), n = (int)((meta >> 8) & 63u) * 8 + (e & 7);
-        const int cv = min(max(val, 0), (int)s_cap[n]);
-        if (cv != val) s_rowbad[warp][rr] = 1;
-        if (cv > 0) { atomicAdd(&s_rowK[warp][rr], cv); atomicAdd(&s_rowN[warp][rr], 1); }
-      }
-    }
-    __syncwarp();
-    // ---- rows that have to be rebuilt: perturbed, an entry out of range, or a row cap broken ----
-    bool need_l = false;
-    const int kc_r = __shfl_sync(0xffffffffu, kc_l, (r_first + lane) & 31);   // the cap of the tile's lane-th row
-    if (lane < rows_here) {
-      const int r = r_first + lane;
-      need_l = ((act_mask >> r) & 1u) &&
-               (((mut_mask >> r) & 1u) || s_rowbad[warp][lane] || s_rowK[warp][lane] > kc_r || s_rowN[warp][lane] > a.n_max);
-    }
-    unsigned need = __ballot_sync(0xffffffffu, need_l);
-    while (need) {
-      const int rl = __ffs(need) - 1;           // row within the tile
-      need &= need - 1;
-      const int rr = r_first + rl;
-      const int16_t *src = ((sec_mask >> rr) & 1u) ? src_b : src_a;
-      // the row, every entry forced into [0, node size]
-      for (int v = lane; v < row_vecs; v += 32) {
-        uint4 y = make_uint4(0u, 0u, 0u, 0u);
-        if (src) y = clamp_vec(__ldg((const uint4 *)(src + (size_t)rr * NN) + v), ((const uint4 *)s_cap)[v]);
-        ((uint4 *)row)[v] = y;
-      }
-      __syncwarp();
-      int rK = 0, rN = 0;
-      for (int n = lane; n < NN; n += 32) { rK += row[n]; rN += row[n] > 0; }
-      rK = __reduce_add_sync(0xffffffffu, rK);
-      rN = __reduce_add_sync(0xffffffffu, rN);
-      if ((mut_mask >> rr) & 1u) {
-        const uint32_t m1 = __shfl_sync(0xffffffffu, mw.y, rr), m2 = __shfl_sync(0xffffffffu, mw.z, rr),
-                       m3 = __shfl_sync(0xffffffffu, mw.w, rr);
-        const uint32_t op = bounded(m1, 3u);
-        if (op == 0u) {
-          const int n = (int)bounded(m3, (uint32_t)NN);
-          if (lane == 0) row[n] = (int16_t)min((int)row[n] + 1, (int)s_cap[n]);
-        } else if (rN > 0) {
-          const int ns = nth_occupied(row, NN, bounded(m2, (uint32_t)rN), lane);
-          if (op == 1u) {
-            if (lane == 0) row[ns] = (int16_t)(row[ns] - 1);
-          } else {
-            const int nd = (int)bounded(m3, (uint32_t)NN);
-            if (nd != ns && lane == 0) {
-              row[nd] = (int16_t)min((int)row[nd] + (int)row[ns], (int)s_cap[nd]);
-              row[ns] = 0;
-            }
-          }
-        }
-        __syncwarp();
-        rK = 0; rN = 0;
-        for (int n = lane; n < NN; n += 32) { rK += row[n]; rN += row[n] > 0; }
-        rK = __reduce_add_sync(0xffffffffu, rK);
-        rN = __reduce_add_sync(0xffffffffu, rN);
-      }
-      const int rkc = __shfl_sync(0xffffffffu, kc_l, rr);
-      if (rK > rkc || rN > a.n_max) {
-        if (lane == 0) {
-          int excess = rK - rkc;
-          rK = min(rK, rkc);
-          for (int n = NN - 1; n >= 0 && excess > 0; --n) {
-            const int take = min((int)row[n], excess);
-            row[n] = (int16_t)(row[n] - take);
-            excess -= take;
-          }
-          int occ = 0;
-          for (int n = 0; n < NN; ++n) {
-            if (row[n] > 0) {
-              ++occ;
-              if (occ > a.n_max) { rK -= row[n]; row[n] = 0; }
-            }
-          }
-          rN = min(occ, a.n_max);
-        }
-        rN = __shfl_sync(0xffffffffu, rN, 0);
-        rK = __shfl_sync(0xffffffffu, rK, 0);
-        __syncwarp();
-      }
-      if (lane == 0) { s_rowK[warp][rl] = rK; s_rowN[warp][rl] = rN; }
-      // the row's queued vectors are dropped; the row is written again and its occupants go
-      // straight into the column totals and lists
-      for (int e = lane; e < qn; e += 32)
-        if ((qmeta[e] & 31u) == (uint32_t)rl) qmeta[e] &= 0x7FFFFFFFu;
-      for (int v = lane; v < row_vecs; v += 32) ((uint4 *)(dst0 + (size_t)rr * NN))[v] = ((const uint4 *)row)[v];
-      for (int n = lane; n < NN; n += 32) {
-        const int val = row[n];
-        if (val > 0) {
-          atomicAdd(&s_tot[n], val);
-          if (rN >= 2) atomicAdd(&s_el[n], 1);
-          const int slot = atomicAdd(&s_cnt[n], 1);
-          if (slot < OCC_SLOTS)
-            s_occ[n * OCC_SLOTS + slot] = (uint32_t)(j0 + rr) | ((uint32_t)val << 20) | (rN >= 2 ? 0x80000000u : 0u);
-        }
-      }
-      __syncwarp();
-    }
-    // ---- second look: column totals, distributed-job counts and occupant lists --------------------
-    for (int e = lane; e < qn * 8; e += 32) {
-      const uint32_t meta = qmeta[e >> 3];
-      const int val = (int)((const int16_t *)qvec)[e];
-      if ((meta >> 31) && val > 0) {
-        const int rl = (int)(meta & 31u), n = (int)((meta >> 8) & 63u) * 8 + (e & 7);
-        const bool dist = s_rowN[warp][rl] >= 2;
-        atomicAdd(&s_tot[n], val);
-        if (dist) atomicAdd(&s_el[n], 1);
-        const int slot = atomicAdd(&s_cnt[n], 1);
-        if (slot < OCC_SLOTS)
-          s_occ[n * OCC_SLOTS + slot] = (uint32_t)(j0 + r_first + rl) | ((uint32_t)val << 20) | (dist ? 0x80000000u : 0u);
-      }
-    }
-    if (lane < rows_here) {
-      const int r = r_first + lane;
-      a.dflag[(size_t)cl * J + j0 + r] = (((act_mask >> r) & 1u) && s_rowN[warp][lane] >= 2) ? 1 : 0;
-    }
-    __syncwarp();
-  }
-
-  __syncthreads();
-  // ---- column partials and occupant lists of the block (as rows2_kernel) ----------------------
-  const size_t base = ((size_t)cl * aa.nbatch + batch) * NN;
-  for (int i = threadIdx.x; i < NN; i += blockDim.x) {
-    aa.colsum[base + i] = s_tot[i];
-    aa.colelig[base + i] = s_el[i];
-    aa.occ_count[base + i] = s_cnt[i];
-    const int cnt = min(s_cnt[i], OCC_SLOTS);
-    for (int k = 0; k < cnt; ++k) aa.occ_list[(base + i) * OCC_SLOTS + k] = s_occ[i * OCC_SLOTS + k];
-  }
-  __shared__ bool s_last_block;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(aa.cand_ticket + cl, 1u);
-    s_last_block = (prev == (unsigned)aa.nbatch - 1u);
-    if (s_last_block) aa.cand_ticket[cl] = 0u;
-  }
-  __syncthreads();
-  if (s_last_block) {
-    __threadfence();
-    for (int n = threadIdx.x; n < NN; n += blockDim.x) {
-      int total = 0, nelig = 0;
-      for (int b = 0; b < aa.nbatch; ++b) {
-        total += __ldcg(aa.colsum + ((size_t)cl * aa.nbatch + b) * NN + n);
-        nelig += __ldcg(aa.colelig + ((size_t)cl * aa.nbatch + b) * NN + n);
-      }
-      if (nelig >= 2 || total > (int)s_cap[n]) {
-        const unsigned slot = atomicAdd(aa.list_count, 1u);
-        aa.list[slot] = ((uint32_t)cl << 13) | (uint32_t)n;
-      }
-    }
-  }
-}
-
 // Column pass: warps take nodes from the work list the row kernel built (any order: columns are
 // independent) and repair them.
 __global__ void __launch_bounds__(128, 4) colrepair_kernel(ColfixArgs a) {
@@ -1202,6 +888,417 @@ __global__ void __launch_bounds__(128, 4) colrepair_kernel(ColfixArgs a) {
     repair_column_list(a, cl, n, total, nelig, cp, lane);
     __syncwarp();
   }
+}
+
+// ---------------------------------------------------------------------------------------
+// A whole child per block: row pass and repair in one launch, rows of any width up to 512 nodes and any alignment
+// (the dense entry points called on their own).
+//
+// Almost every entry of a population is zero and almost every row is copied unchanged, so a warp takes a tile
+// of rows (as many as touch 160 aligned vectors of their sources and hold 1024 entries), reads each row's aligned
+// vectors from the parent it comes from, and lays the tile out in shared memory, shifted to where the child lies
+// between two 16-byte boundaries: zeros, and the entries of the vectors that hold something, which are queued
+// (ballot + popc) and looked at one lane per entry.  Rows that are perturbed or break a row cap are
+// edited there by the warp; then the tile goes out in whole vectors.  Column totals and occupant lists stay in
+// shared memory, and once the block's rows are out its groups of 16 lanes decide the nodes that need repair and
+// write the few entries that change.
+// A child is a cluster of up to eight blocks where there are few children: every block lists the occupants that its
+// rows bring, and the nodes are then decided from all their lists, over distributed shared memory.
+// Bound: for large children instruction issue (55 % of the slots) and the loads' latency between two tiles, for small
+// ones the chain of one block's steps.  Measured with the fitness behind it (us, before: kernels for the rows
+// and for the columns): 512 children of 1024 x 256 178 -> 171, 256 of 1000 x 250 760 -> 132, 57 of 748 x 255 255 -> 45
+// (83 with one block per child), 200 of 300 x 72 46 -> 29, 100 of 48 x 16 31 -> 18.5.  Tiles of 128 vectors where rows are
+// not aligned: 177 us for 1000 x 250 (a tile costs the same whether it has three rows or four).
+// ---------------------------------------------------------------------------------------
+constexpr int CHILD_WARPS = 8;
+constexpr int CHILD_TILE = 1024;        // entries a warp lays out at a time
+constexpr int CHILD_OCC = 16;           // occupants listed per node: a group of lanes
+constexpr int CHILD_SPLIT = 8;          // blocks of a child, at most
+__host__ __device__ constexpr int child_vectors(bool whole) { return whole ? 128 : 160; }   // a warp reads at a time
+
+struct ChildArgs {
+  RowsArgs r;
+  ColfixArgs col;                       // for nodes with more occupants than a list holds
+  const int16_t *src_lo, *src_hi;       // what may be read: [src_lo, src_hi)
+  int row_vecs;                         // aligned vectors a row may touch
+  int split;                            // blocks of a child: a power of two
+  int tile_rows, chunk_rows;            // rows laid out at a time; rows whose draws are made at a time
+};
+
+template <bool WHOLE>
+struct ChildWarp {                      // shared memory of a warp
+  uint4 tile[WHOLE ? 64 : CHILD_TILE / 8 + 1];       // the tile; WHOLE: the row being edited
+  uint4 qvec[child_vectors(WHOLE)];
+  uint32_t qmeta[child_vectors(WHOLE)];          // row of the tile (bits 0..4) | place of its first entry in the row, + 8 unless WHOLE (8..17) | alive (31)
+  uint32_t row[32];                     // of the tile: GPUs | occupied nodes << 22
+  int bad[32];                          // an entry is out of range
+};
+
+inline size_t child_smem_bytes(int NN, bool whole) {
+  return CHILD_WARPS * (whole ? sizeof(ChildWarp<true>) : sizeof(ChildWarp<false>)) + (size_t)NN * (CHILD_OCC * 4 + 4 + 4 + 2);
+}
+
+// WHOLE: rows are whole vectors on 16-byte boundaries.  Their vectors go straight out again, and only a row
+// that is edited (perturbed, over a cap, an entry out of range) is laid out, from its queued vectors, and written once more.
+template <bool WHOLE>
+__global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(const __grid_constant__ ChildArgs aa) {
+  extern __shared__ __align__(16) unsigned char child_smem[];
+  const RowsArgs &a = aa.r;
+  const int NN = a.num_nodes, J = a.J, P = a.P;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  ChildWarp<WHOLE> &w = ((ChildWarp<WHOLE> *)child_smem)[warp];
+  uint32_t *s_occ = (uint32_t *)(child_smem + CHILD_WARPS * sizeof(ChildWarp<WHOLE>));   // job | GPUs << 16 | distributed << 31
+  int32_t *s_tot = (int32_t *)(s_occ + (size_t)NN * CHILD_OCC);                      // GPUs placed on the node
+  uint32_t *s_cnt = (uint32_t *)(s_tot + NN);                                        // distributed jobs on it | occupants << 16
+  int16_t *s_cap = (int16_t *)(s_cnt + NN);
+  __shared__ int s_parent[2];
+  // a cluster of `split` blocks to a child; gw: this warp among all of them
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int split = aa.split, part = (int)blockIdx.x & (split - 1), cl = (int)blockIdx.x / split;
+  const int gw = part * CHILD_WARPS + warp, nwarps = split * CHILD_WARPS;
+  const uint32_t c = a.first_cand + (uint32_t)cl, round = round_of(a.key);
+  const bool bred = a.mode == ROWS_GENERATION && (int)c >= a.num_elite;
+  for (int i = tid; i < NN; i += blockDim.x) {
+    s_tot[i] = 0;
+    s_cnt[i] = 0u;
+    s_cap[i] = (int16_t)max((int)a.cap[i], 0);
+  }
+
+  // ---- the draws of this warp's next rows, a lane each -----------------------------------------------
+  bool act_l = false, mut_l = false, sec_l = false;
+  int kc_l = 0;
+  u32x4 mw = {0, 0, 0, 0};
+  auto draw_rows = [&](int j0) {
+    act_l = mut_l = sec_l = false;
+    const int j = j0 + lane;
+    if (lane >= aa.chunk_rows || j >= J) return;
+    act_l = !a.active || a.active[j];
+    kc_l = max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max));
+    if (bred) {
+      uint32_t x;
+      draw_two(a.key.k0, round, (uint32_t)j, c, a.gen, SLOT_XOVER, SLOT_MUTATE, x, mw);
+      sec_l = (x >> 31) != 0u;
+      mut_l = mw.x < a.thr;
+    } else if (a.mode == ROWS_INIT && c > 0u) {
+      mw = draw_one(a.key.k0, round, (uint32_t)j, c, GEN_INIT, SLOT_INIT);
+      mut_l = mw.x < a.thr;
+    }
+  };
+  draw_rows(gw * aa.chunk_rows);
+
+  // ---- parents (generation mode): the candidate of its rank for an elite child, else the better-ranked of two
+  // random pairs ---------------------------------------------------------------------------------------
+  if (bred) {
+    if (warp == 0) {
+      const u32x4 sel = draw_one(a.key.k0, round, 0u, c, a.gen, SLOT_SELECT);
+      const int i = (int)bounded(lane == 0 ? sel.x : lane == 1 ? sel.y : lane == 2 ? sel.z : sel.w, (uint32_t)P);
+      const uint32_t k = order_key(__ldg(a.fitness_bits + i));
+      const int io = __shfl_down_sync(0xffffffffu, i, 1);
+      const uint32_t ko = __shfl_down_sync(0xffffffffu, k, 1);
+      if (lane == 0 || lane == 2) s_parent[lane >> 1] = tournament_winner(k, i, ko, io);
+    }
+  } else if (a.mode == ROWS_GENERATION) {
+    if ((size_t)P * 6 <= CHILD_WARPS * sizeof(ChildWarp<WHOLE>)) {       // keys, and a list of candidates behind them
+      uint32_t *keys = (uint32_t *)child_smem;
+      for (int i = tid; i < P; i += blockDim.x) keys[i] = order_key(__ldg(a.fitness_bits + i));
+      __syncthreads();
+      if (warp == 0) {
+        const int i = candidate_of_rank(keys, P, (int)c, (uint16_t *)(keys + P), lane);
+        if (lane == 0) s_parent[0] = s_parent[1] = i;
+      }
+    } else {
+      for (int i = tid; i < P; i += blockDim.x) {
+        const uint32_t ki = order_key(a.fitness_bits[i]);
+        int rk = 0;
+        for (int o = 0; o < P; ++o) {
+          const uint32_t ko = order_key(__ldg(a.fitness_bits + o));
+          rk += (ko > ki || (ko == ki && o < i)) ? 1 : 0;
+        }
+        if (rk == (int)c) s_parent[0] = s_parent[1] = i;
+      }
+    }
+  }
+  __syncthreads();
+
+  const size_t mat = (size_t)J * NN;
+  int16_t *child = a.dst + (size_t)cl * mat;
+  const int16_t *src_a = a.src, *src_b;           // NULL: the rows start empty
+  if (a.mode == ROWS_GENERATION) {
+    src_b = a.src + (size_t)s_parent[1] * mat;
+    src_a += (size_t)s_parent[0] * mat;
+  } else {
+    if (a.mode == ROWS_REPAIR) src_a = child;
+    src_b = src_a;
+  }
+  auto add_occupant = [&](int j, int n, int v, bool dist) {
+    atomicAdd(&s_tot[n], v);
+    const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
+    if (k < CHILD_OCC) s_occ[n * CHILD_OCC + k] = (uint32_t)j | ((uint32_t)v << 16) | (dist ? 0x80000000u : 0u);
+  };
+  constexpr int B = child_vectors(WHOLE) / 32;
+  int16_t *tile = (int16_t *)w.tile;
+  // the lane's vectors of a tile: row | place in the row << 8 (that of its first entry, before the row's skew)
+  uint32_t at_q[B];
+  {
+    const uint32_t inv = (65536u + (uint32_t)aa.row_vecs - 1u) / (uint32_t)aa.row_vecs;   // t / row_vecs = t * inv >> 16 (t < 160)
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const uint32_t t = (uint32_t)(q * 32 + lane), r = (t * inv) >> 16;
+      at_q[q] = min(r, 31u) | ((8u * (t - r * (uint32_t)aa.row_vecs)) << 8) | (r < (uint32_t)aa.tile_rows ? 0u : 0x80000000u);
+    }
+  }
+
+#pragma unroll 1
+  for (int j0 = gw * aa.chunk_rows; j0 < J; j0 += nwarps * aa.chunk_rows) {
+    const int nrows = min(aa.chunk_rows, J - j0);
+    const unsigned act_mask = __ballot_sync(0xffffffffu, act_l), sec_mask = __ballot_sync(0xffffffffu, sec_l);
+    const unsigned mut_mask = __ballot_sync(0xffffffffu, mut_l && act_l);
+#pragma unroll 1
+    for (int r0 = 0; r0 < nrows; r0 += aa.tile_rows) {
+      const int rows = min(aa.tile_rows, nrows - r0), ent = rows * NN, jt = j0 + r0;
+      int16_t *out = child + (size_t)jt * NN;
+      const int skew = WHOLE ? 0 : (int)(((uintptr_t)out & 15) >> 1);      // entry e of the tile lies at skew + e
+      const int out_vecs = (skew + ent + 7) >> 3;
+      // ---- in: four or five vectors a lane, queued if they hold anything ---------------------------------
+      const int16_t *const from_a = src_a + (size_t)jt * NN, *const from_b = src_b + (size_t)jt * NN;
+      const unsigned load_rows = src_a ? act_mask >> r0 : 0u, sec_rows = sec_mask >> r0;
+      uint4 x[B];
+      uint32_t meta[B];
+      if (WHOLE) {
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+          const uint32_t r = at_q[q] & 31u;
+          x[q] = make_uint4(0u, 0u, 0u, 0u);
+          meta[q] = at_q[q] | 0x80000000u;
+          if (q * 32 + lane < out_vecs && ((load_rows >> r) & 1u))
+            x[q] = *((const uint4 *)(((sec_rows >> r) & 1u) ? from_b : from_a) + (q * 32 + lane));
+        }
+      } else {
+        // (vectors reach up to seven entries beyond their rows: not beyond the sources)
+        const bool inside = from_a - 7 >= aa.src_lo && from_b - 7 >= aa.src_lo && from_a + ent + 7 <= aa.src_hi &&
+                            from_b + ent + 7 <= aa.src_hi;
+        const int skew_a = (int)((uintptr_t)from_a >> 1), skew_b = (int)((uintptr_t)from_b >> 1);
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+          const int r = (int)(at_q[q] & 31u), first = r * NN;
+          const bool sec = (sec_rows >> r) & 1u;
+          const int e = (int)((at_q[q] >> 8) & 0x3FFu) - (((sec ? skew_b : skew_a) + first) & 7);
+          x[q] = make_uint4(0u, 0u, 0u, 0u);
+          meta[q] = (uint32_t)r | ((uint32_t)(e + 8) << 8) | 0x80000000u;
+          if ((int)at_q[q] >= 0 && r < rows && e < NN && ((load_rows >> r) & 1u)) {
+            const int16_t *const p = (sec ? from_b : from_a) + first + e;
+            if (inside || (p >= aa.src_lo && p + 8 <= aa.src_hi)) {
+              x[q] = *(const uint4 *)p;
+            } else {
+              uint32_t y[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+              for (int h = max(0, -e); h < 8 && e + h < NN; ++h)
+                y[h >> 1] |= (uint32_t)(uint16_t)p[h] << (16 * (h & 1));
+              x[q] = make_uint4(y[0], y[1], y[2], y[3]);
+            }
+          }
+        }
+      }
+      if (!WHOLE)
+        for (int v = lane; v < out_vecs; v += 32) w.tile[v] = make_uint4(0u, 0u, 0u, 0u);
+      w.row[lane] = 0u;
+      if (WHOLE) w.bad[lane] = 0;
+      int qn = 0;
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const bool nz = (x[q].x | x[q].y | x[q].z | x[q].w) != 0u;
+        const unsigned bal = __ballot_sync(0xffffffffu, nz);
+        if (nz) {
+          const int pos = qn + __popc(bal & ((1u << lane) - 1u));
+          w.qvec[pos] = x[q];
+          w.qmeta[pos] = meta[q];
+        }
+        qn += __popc(bal);
+        if (WHOLE && q * 32 + lane < out_vecs) ((uint4 *)out)[q * 32 + lane] = x[q];
+      }
+      __syncwarp();
+      // ---- first look: entries (those of the vector's own row, forced into [0, node size]) to their places, the
+      // rows' K and N ------------------------------------------------------------------------------------
+      for (int e = lane; e < qn * 8; e += 32) {
+        const int val = (int)((const int16_t *)w.qvec)[e];
+        const uint32_t m = w.qmeta[e >> 3];
+        const int r = (int)(m & 31u), n = (int)((m >> 8) & 0x3FFu) - (WHOLE ? 0 : 8) + (e & 7);
+        if (WHOLE ? val != 0 : val > 0 && n >= 0 && n < NN) {
+          const int cv = min(max(val, 0), (int)s_cap[n]);
+          if (!WHOLE) tile[skew + r * NN + n] = (int16_t)cv;
+          else if (cv != val) w.bad[r] = 1;
+          if (cv > 0) atomicAdd(&w.row[r], (uint32_t)cv | (1u << 22));
+        }
+      }
+      __syncwarp();
+      // ---- rows that are perturbed or break a row cap: edited where they lie ----------------------------
+      bool need_l = false;
+      const int kc_r = __shfl_sync(0xffffffffu, kc_l, (r0 + lane) & 31);      // the cap of the tile's lane-th row
+      if (lane < rows)
+        need_l = ((act_mask >> (r0 + lane)) & 1u) &&
+                 (((mut_mask >> (r0 + lane)) & 1u) || (int)(w.row[lane] & 0x3FFFFFu) > kc_r || (int)(w.row[lane] >> 22) > a.n_max ||
+                  (WHOLE && w.bad[lane]));
+      unsigned need = __ballot_sync(0xffffffffu, need_l);
+#pragma unroll 1
+      while (need) {
+        const int rl = __ffs(need) - 1, rr = r0 + rl;
+        need &= need - 1;
+        int16_t *row = WHOLE ? tile : tile + skew + rl * NN;
+        if (WHOLE) {                    // laid out from its vectors
+          for (int v = lane; v < aa.row_vecs; v += 32) w.tile[v] = make_uint4(0u, 0u, 0u, 0u);
+          __syncwarp();
+          for (int e = lane; e < qn * 8; e += 32) {
+            const int n = (int)((w.qmeta[e >> 3] >> 8) & 0x3FFu) + (e & 7);
+            if ((w.qmeta[e >> 3] & 31u) == (uint32_t)rl)
+              row[n] = (int16_t)min(max((int)((const int16_t *)w.qvec)[e], 0), (int)s_cap[n]);
+          }
+          __syncwarp();
+        }
+        int rK = (int)(w.row[rl] & 0x3FFFFFu), rN = (int)(w.row[rl] >> 22);
+        if ((mut_mask >> rr) & 1u) {
+          const uint32_t m1 = __shfl_sync(0xffffffffu, mw.y, rr), m2 = __shfl_sync(0xffffffffu, mw.z, rr),
+                         m3 = __shfl_sync(0xffffffffu, mw.w, rr);
+          const uint32_t op = bounded(m1, 3u);
+          if (op == 0u) {
+            const int n = (int)bounded(m3, (uint32_t)NN);
+            if (lane == 0) row[n] = (int16_t)min((int)row[n] + 1, (int)s_cap[n]);
+          } else if (rN > 0) {
+            const int ns = nth_occupied(row, NN, bounded(m2, (uint32_t)rN), lane);
+            if (op == 1u) {
+              if (lane == 0) row[ns] = (int16_t)(row[ns] - 1);
+            } else {
+              const int nd = (int)bounded(m3, (uint32_t)NN);
+              if (nd != ns && lane == 0) {
+                row[nd] = (int16_t)min((int)row[nd] + (int)row[ns], (int)s_cap[nd]);
+                row[ns] = 0;
+              }
+            }
+          }
+          __syncwarp();
+          rK = 0; rN = 0;
+          for (int n = lane; n < NN; n += 32) { rK += row[n]; rN += row[n] > 0; }
+          rK = __reduce_add_sync(0xffffffffu, rK);
+          rN = __reduce_add_sync(0xffffffffu, rN);
+        }
+        const int rkc = __shfl_sync(0xffffffffu, kc_l, rr);
+        if (rK > rkc || rN > a.n_max) {
+          if (lane == 0) {
+            int excess = rK - rkc;
+            for (int n = NN - 1; n >= 0 && excess > 0; --n) {
+              const int take = min((int)row[n], excess);
+              row[n] = (int16_t)(row[n] - take);
+              excess -= take;
+            }
+            int occ = 0;
+            for (int n = 0; n < NN; ++n)
+              if (row[n] > 0 && ++occ > a.n_max) row[n] = 0;
+            rN = min(occ, a.n_max);
+          }
+          rN = __shfl_sync(0xffffffffu, rN, 0);
+          __syncwarp();
+        }
+        // its queued vectors are dropped, its occupants added from where it lies
+        if (lane == 0) w.row[rl] = (uint32_t)rN << 22;
+        for (int e = lane; e < qn; e += 32)
+          if ((w.qmeta[e] & 31u) == (uint32_t)rl) w.qmeta[e] &= 0x7FFFFFFFu;
+        for (int n = lane; n < NN; n += 32)
+          if (row[n] > 0) add_occupant(jt + rl, n, (int)row[n], rN >= 2);
+        if (WHOLE)
+          for (int v = lane; v < aa.row_vecs; v += 32) ((uint4 *)(out + (size_t)rl * NN))[v] = w.tile[v];
+        __syncwarp();
+      }
+      // ---- second look: column totals and occupant lists; out -------------------------------------------
+      for (int e = lane; e < qn * 8; e += 32) {
+        const int val = (int)((const int16_t *)w.qvec)[e];
+        const uint32_t m = w.qmeta[e >> 3];
+        const int r = (int)(m & 31u), n = (int)((m >> 8) & 0x3FFu) - (WHOLE ? 0 : 8) + (e & 7);
+        if ((m >> 31) && val > 0 && (WHOLE || (n >= 0 && n < NN))) {
+          const int cv = min(val, (int)s_cap[n]);
+          if (cv > 0) add_occupant(jt + r, n, cv, (w.row[r] >> 23) != 0u);
+        }
+      }
+      if (!WHOLE) {
+        for (int v = lane + (skew ? 1 : 0); 8 * v + 8 <= skew + ent; v += 32) ((uint4 *)(out - skew))[v] = w.tile[v];
+        // the two vectors shared with the rows next to the tile, an entry each
+        const int i = lane < 8 ? lane : ((skew + ent) & ~7) + (lane & 7);
+        if (lane < 16 && i >= skew && i < skew + ent && (lane < 8 ? skew != 0 : (skew == 0 || i >= 8))) out[i - skew] = tile[i];
+      }
+      if (lane < rows) a.dflag[(size_t)cl * J + jt + lane] = (w.row[lane] >> 23) != 0u ? 1 : 0;
+      __syncwarp();
+    }
+    draw_rows(j0 + nwarps * aa.chunk_rows);
+  }
+  if (split > 1) cluster.sync();
+  else __syncthreads();
+
+  // ---- repair: the nodes are dealt out to all warps; a lane looks at a node, groups of 16 lanes decide those
+  // that hold two distributed jobs or more GPUs than they have, from the occupants that the child's blocks have
+  // listed; a node with more occupants than a group has lanes is walked by a warp ----------------------
+  auto of_part = [&](auto *p, int q) { return split > 1 ? cluster.map_shared_rank(p, q) : p; };
+#pragma unroll 1
+  for (int n0 = gw; n0 < NN; n0 += 32 * nwarps) {
+    const int n_l = n0 + lane * nwarps;
+    int tot_l = 0, cap_l = 0;
+    uint32_t cnt_l = 0u;                // (a sum over all blocks: at most J of each, below 65536)
+    if (n_l < NN) {
+      cap_l = (int)s_cap[n_l];
+#pragma unroll 1
+      for (int q = 0; q < split; ++q) {
+        tot_l += of_part(s_tot, q)[n_l];
+        cnt_l += of_part(s_cnt, q)[n_l];
+      }
+    }
+    const bool bad = (cnt_l & 0xFFFFu) >= 2u || tot_l > cap_l;
+    unsigned todo = __ballot_sync(0xffffffffu, bad);
+    if (todo == 0u) continue;
+    uint32_t rep_l = 0u;                // the two rotation offsets
+    if (bad) {
+      uint32_t x;
+      u32x4 y;
+      draw_two(a.key.k0, round, (uint32_t)n_l, c, a.gen, SLOT_REPAIR_INTF, SLOT_REPAIR_CAP, x, y);
+      rep_l = bounded(x, (uint32_t)J) | (bounded(y.x, (uint32_t)J) << 16);
+    }
+    __syncwarp();
+#pragma unroll 1
+    while (todo) {
+      const int b0 = __ffs(todo) - 1;
+      todo &= todo - 1;
+      int b1 = -1;
+      if (todo) { b1 = __ffs(todo) - 1; todo &= todo - 1; }
+      const int b = (lane & 16) ? b1 : b0, sub = lane & 15, from = max(b, 0);
+      const uint32_t rep = __shfl_sync(0xffffffffu, rep_l, from), cnt = __shfl_sync(0xffffffffu, cnt_l, from);
+      const int tot = __shfl_sync(0xffffffffu, tot_l, from), cap_n = __shfl_sync(0xffffffffu, cap_l, from);
+      const int n = n0 + from * nwarps, count = b >= 0 ? (int)(cnt >> 16) : 0;
+      const bool listed = count <= CHILD_OCC, have = listed && sub < count;
+      uint32_t e = 0u;
+      if (have) {                       // the sub-th of the blocks' lists, one behind the other
+        int q = 0, k = sub;
+#pragma unroll 1
+        for (; q < split - 1; ++q) {
+          const int here = (int)(of_part(s_cnt, q)[n] >> 16);
+          if (k < here) break;
+          k -= here;
+        }
+        e = of_part(s_occ, q)[n * CHILD_OCC + k];
+      }
+      const int j = (int)(e & 0xFFFFu), v_old = (int)((e >> 16) & 0x7FFu);
+      int ri = j - (int)(rep & 0xFFFFu), rc = have ? j - (int)(rep >> 16) : 0x3fffffff;
+      if (ri < 0) ri += J;
+      if (rc < 0) rc += J;
+      const int most = max(__shfl_sync(0xffffffffu, count, 0), __shfl_sync(0xffffffffu, count, 16));
+      const int v = decide(v_old, (e >> 31) != 0u, have, min(most, CHILD_OCC), (cnt & 0xFFFFu) >= 2u, tot, cap_n, ri, rc);
+      if (have && v != v_old) child[(size_t)j * NN + n] = (int16_t)v;
+#pragma unroll 1
+      for (unsigned walk = __ballot_sync(0xffffffffu, !listed && sub == 0); walk; walk &= walk - 1) {
+        const int l = __ffs(walk) - 1;
+        const uint32_t cw = __shfl_sync(0xffffffffu, cnt, l);
+        repair_column_any(aa.col, nullptr, cl, __shfl_sync(0xffffffffu, n, l), __shfl_sync(0xffffffffu, tot, l),
+                          (int)(cw & 0xFFFFu), __shfl_sync(0xffffffffu, cap_n, l), lane);
+        __syncwarp();
+      }
+    }
+  }
+  if (split > 1) cluster.sync();        // (the other blocks may still read this one's lists)
 }
 
 int launch_rows(sched_ctx *ctx, RowsArgs &a) {
@@ -1225,12 +1322,12 @@ int launch_rows(sched_ctx *ctx, RowsArgs &a) {
   return SCHED_OK;
 }
 
-int launch_cols(sched_ctx *ctx, int16_t *pop, int count, uint32_t first_cand, uint32_t gen) {
+int launch_cols(sched_ctx *ctx, const RngKey &key, int16_t *pop, int count, uint32_t first_cand, uint32_t gen) {
   if (count == 0 || ctx->cfg.num_jobs == 0) return SCHED_OK;
   ColsArgs a;
   a.pop = pop; a.dflag = ctx->d_dflag; a.cap = ctx->d_cap;
   a.J = ctx->cfg.num_jobs; a.num_nodes = ctx->cfg.num_nodes;
-  a.gen = gen; a.key = make_key(ctx->cfg.seed, ctx->d_round);
+  a.gen = gen; a.key = key;
   for (int first = 0; first < count; first += 65535) {
     const int n = min(65535, count - first);
     a.count = n;
@@ -1244,9 +1341,52 @@ int launch_cols(sched_ctx *ctx, int16_t *pop, int count, uint32_t first_cand, ui
   return SCHED_OK;
 }
 
-// Row pass + column pass of `count` candidates.  Rows of a multiple of 8 and at most 512
-// nodes (16-byte vectors, <= 2 per lane) with node sizes <= 2047 take the batched kernels
-// with fused column sums; everything else the general warp-per-row / thread-per-column pair.
+// Row pass and repair in one launch (child_kernel).
+int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first_cand, uint32_t gen) {
+  const int NN = a.num_nodes;
+  ChildArgs ca = {};
+  ca.r = a;
+  ca.col.pop = a.dst; ca.col.dflag = a.dflag; ca.col.cap = a.cap;
+  ca.col.J = a.J; ca.col.num_nodes = NN;
+  ca.col.gen = gen; ca.col.first_cand = first_cand; ca.col.key = a.key;
+  const size_t mat = (size_t)a.J * NN;
+  ca.src_lo = a.src;
+  ca.src_hi = a.src + mat * (a.mode == ROWS_GENERATION ? a.P : a.mode == ROWS_REPAIR ? count : a.src ? 1 : 0);
+  const bool whole = NN % 8 == 0 && (((uintptr_t)a.dst | (uintptr_t)a.src) & 15) == 0;
+  // a child is split over blocks while that leaves none of them without a place on the GPU and every warp a few rows
+  ca.split = 1;
+  while (ca.split < CHILD_SPLIT && (long long)count * ca.split * 2 <= 3LL * ctx->num_sms && ca.split * 2 * CHILD_WARPS * 4 <= a.J) ca.split *= 2;
+  ca.row_vecs = whole ? NN / 8 : (NN + 14) / 8;
+  const int warps = CHILD_WARPS * ca.split, turns = (a.J + 32 * warps - 1) / (32 * warps);
+  ca.chunk_rows = (a.J + warps * turns - 1) / (warps * turns);
+  ca.tile_rows = std::min(ca.chunk_rows, whole ? child_vectors(true) / ca.row_vecs
+                                               : std::min(child_vectors(false) / ca.row_vecs, CHILD_TILE / NN));
+  void (*const kernel)(ChildArgs) = whole ? child_kernel<true> : child_kernel<false>;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)count * (unsigned)ca.split);
+  lc.blockDim = dim3(CHILD_WARPS * 32);
+  lc.dynamicSmemBytes = child_smem_bytes(NN, whole);
+  lc.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ca.split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1u;
+  lc.attrs = attr;
+  lc.numAttrs = ca.split > 1 ? 1 : 0;
+  if (lc.dynamicSmemBytes > 48 * 1024)
+    SCHED_CUDA_CHECK(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes));
+  {
+    TimedLaunch tl_(ctx, KK_ROWS);
+    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, kernel, ca));
+  }
+  SCHED_LAUNCH_CHECK(ctx);
+  return SCHED_OK;
+}
+
+// Row pass + column pass of `count` candidates.  Rounds on dense matrices want per-row summaries: rows of whole
+// 16-byte vectors take the batched kernels with fused column sums.  Without summaries every width takes a block (or
+// a few) per child, up to 512 nodes (a tile holds two rows), sizes <= 2047 (an occupant's word) and 65535 jobs (a
+// node's counters); beyond those the general warp-per-row / thread-per-column pair.
 int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint32_t first_cand, uint32_t gen) {
   if (count == 0 || a.J == 0) return SCHED_OK;
   const int NN = a.num_nodes;
@@ -1254,6 +1394,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   const bool fused = (NN % 8 == 0) && NN <= 512 && aligned && ctx->cap_max <= 2047 && count <= 65535 &&
                      a.J <= (1 << 20);
   ctx->summ_valid = fused && a.summ != nullptr;
+  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535) return launch_children(ctx, a, count, first_cand, gen);
   if (!fused) {
     if (a.mode == ROWS_GENERATION) {
       {
@@ -1264,7 +1405,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
     }
     int rc = launch_rows(ctx, a);
     if (rc != SCHED_OK) return rc;
-    return launch_cols(ctx, pop, count, first_cand, gen);
+    return launch_cols(ctx, a.key, pop, count, first_cand, gen);
   }
   const int nbatch = (a.J + 255) / 256;
   int rc = ensure_colscratch(ctx, (size_t)count * nbatch * NN);
@@ -1275,34 +1416,6 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   aa.list_count = ctx->d_colcount; aa.list = ctx->d_collist; aa.cand_ticket = ctx->d_rowticket;
   aa.occ_count = ctx->d_occcount; aa.occ_list = ctx->d_occlist;
   dim3 grid((unsigned)nbatch, (unsigned)count);
-  const int row_vecs_all = NN / 8;
-  if (a.summ == nullptr && (row_vecs_all & (row_vecs_all - 1)) == 0) {
-    // no per-row summaries wanted (the entry points called on their own): the streaming kernel
-    const size_t smem = stream_smem_bytes(NN);
-    if (smem > 24 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(rows_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) {
-        set_error(ctx, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e));
-        return SCHED_ERR_CUDA;
-      }
-    }
-    SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(ctx->d_colcount, 0, sizeof(unsigned int), ctx->stream));
-    {
-      TimedLaunch tl_(ctx, KK_ROWS);
-      rows_stream_kernel<<<grid, 256, smem, ctx->stream>>>(aa);
-    }
-    SCHED_LAUNCH_CHECK(ctx);
-    ColfixArgs f;
-    f.pop = pop; f.dflag = ctx->d_dflag; f.cap = ctx->d_cap;
-    f.colsum = ctx->d_colsum; f.colelig = ctx->d_colelig; f.summ = nullptr;
-    f.J = a.J; f.num_nodes = NN; f.nbatch = nbatch;
-    f.gen = gen; f.first_cand = first_cand; f.key = make_key(ctx->cfg.seed, ctx->d_round);
-    f.list = ctx->d_collist; f.list_count = ctx->d_colcount;
-    f.cur = nullptr; f.occ_count = ctx->d_occcount; f.occ_list = ctx->d_occlist;
-    { TimedLaunch tl_(ctx, KK_COLS); colrepair_kernel<<<ctx->num_sms * 4, 128, 0, ctx->stream>>>(f); }
-    SCHED_LAUNCH_CHECK(ctx);
-    return SCHED_OK;
-  }
   SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(ctx->d_colcount, 0, sizeof(unsigned int), ctx->stream));
   {
     TimedLaunch tl_(ctx, KK_ROWS);
@@ -1333,7 +1446,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   f.pop = pop; f.dflag = ctx->d_dflag; f.cap = ctx->d_cap;
   f.colsum = ctx->d_colsum; f.colelig = ctx->d_colelig; f.summ = a.summ;
   f.J = a.J; f.num_nodes = NN; f.nbatch = nbatch;
-  f.gen = gen; f.first_cand = first_cand; f.key = make_key(ctx->cfg.seed, ctx->d_round);
+  f.gen = gen; f.first_cand = first_cand; f.key = a.key;
   f.list = ctx->d_collist; f.list_count = ctx->d_colcount;
   f.cur = a.cur; f.occ_count = ctx->d_occcount; f.occ_list = ctx->d_occlist;
   { TimedLaunch tl_(ctx, KK_COLS); colrepair_kernel<<<ctx->num_sms * 4, 128, 0, ctx->stream>>>(f); }
@@ -1341,7 +1454,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   return SCHED_OK;
 }
 
-RowsArgs base_rows_args(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int count) {
+RowsArgs base_rows_args(sched_ctx *ctx, const RngKey &key, const int32_t *d_k_cap, const uint8_t *d_active, int count) {
   RowsArgs a;
   const sched_config &c = ctx->cfg;
   a.cap = ctx->d_cap; a.k_cap = d_k_cap; a.active = d_active;
@@ -1349,7 +1462,7 @@ RowsArgs base_rows_args(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
   a.P = c.population; a.J = c.num_jobs; a.num_nodes = c.num_nodes;
   a.k_max = c.k_max; a.n_max = c.n_max; a.num_elite = c.num_elite; a.count = count;
   a.thr = 0; a.gen = 0; a.first_cand = 0;
-  a.key = make_key(c.seed, ctx->d_round);
+  a.key = key;
   a.src = nullptr; a.dst = nullptr; a.mode = ROWS_REPAIR; a.fitness_bits = nullptr;
   a.cur = nullptr; a.summ = nullptr; a.summ_in = nullptr;
   return a;
@@ -1357,41 +1470,41 @@ RowsArgs base_rows_args(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d
 
 }  // namespace
 
-int launch_repair(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
+int launch_repair(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active, int16_t *d_pop,
                   int32_t count, uint32_t first_candidate, uint32_t generation) {
   int rc = ensure_dflag(ctx, count);
   if (rc != SCHED_OK) return rc;
-  RowsArgs a = base_rows_args(ctx, d_k_cap, d_active, count);
+  RowsArgs a = base_rows_args(ctx, key, d_k_cap, d_active, count);
   a.mode = ROWS_REPAIR; a.src = d_pop; a.dst = d_pop;
-  a.first_cand = first_candidate; a.gen = generation; a.key = make_key(ctx->cfg.seed, ctx->d_round);
+  a.first_cand = first_candidate; a.gen = generation;
   return launch_rows_cols(ctx, a, d_pop, count, first_candidate, generation);
 }
 
-int launch_init_population(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active,
+int launch_init_population(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active,
                            const int16_t *d_cur, int16_t *d_pop_out) {
   const int P = ctx->cfg.population;
   int rc = ensure_dflag(ctx, P);
   if (rc != SCHED_OK) return rc;
-  RowsArgs a = base_rows_args(ctx, d_k_cap, d_active, P);
+  RowsArgs a = base_rows_args(ctx, key, d_k_cap, d_active, P);
   a.mode = ROWS_INIT; a.src = d_cur; a.dst = d_pop_out;
-  a.thr = ctx->cfg.thr_init; a.gen = GEN_INIT; a.key = make_key(ctx->cfg.seed, ctx->d_round);
+  a.thr = ctx->cfg.thr_init; a.gen = GEN_INIT;
   a.cur = ctx->round_cur; a.summ = ctx->round_summ;
   return launch_rows_cols(ctx, a, d_pop_out, P, 0u, GEN_INIT);
 }
 
 // children first_child .. first_child + num_children - 1 (num_children < 0: all of them)
-int launch_generation(sched_ctx *ctx, const int32_t *d_k_cap, const uint8_t *d_active,
+int launch_generation(sched_ctx *ctx, RngKey key, const int32_t *d_k_cap, const uint8_t *d_active,
                       const int16_t *d_pop_in, const float *d_fitness_in, int16_t *d_pop_out,
                       uint32_t generation, int first_child, int num_children) {
   const int P = num_children < 0 ? ctx->cfg.population : num_children;
   if (P == 0) return SCHED_OK;
   int rc = ensure_dflag(ctx, P);
   if (rc != SCHED_OK) return rc;
-  RowsArgs a = base_rows_args(ctx, d_k_cap, d_active, P);
+  RowsArgs a = base_rows_args(ctx, key, d_k_cap, d_active, P);
   a.first_cand = (uint32_t)first_child;
   a.mode = ROWS_GENERATION; a.src = d_pop_in; a.dst = d_pop_out;
   a.fitness_bits = (const uint32_t *)d_fitness_in;
-  a.thr = ctx->cfg.thr_mutate; a.gen = generation; a.key = make_key(ctx->cfg.seed, ctx->d_round);
+  a.thr = ctx->cfg.thr_mutate; a.gen = generation;
   a.cur = ctx->round_cur; a.summ = ctx->round_summ; a.summ_in = ctx->round_summ_in;
   return launch_rows_cols(ctx, a, d_pop_out, P, (uint32_t)first_child, generation);
 }

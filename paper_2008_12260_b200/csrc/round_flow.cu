@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "fitness_common.cuh"
+#include "search_common.cuh"
 
 namespace {
 
@@ -93,53 +94,6 @@ __device__ __forceinline__ Record load_record(const uint32_t *p) {
 __device__ __forceinline__ void store_record(uint32_t *p, const Record &r) {
   asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(r.w[0]), "r"(r.w[1]), "r"(r.w[2]),
                "r"(r.w[3]), "r"(r.w[4]), "r"(r.w[5]), "r"(r.w[6]), "r"(r.w[7]) : "memory");
-}
-
-// ---- the random stream -------------------------------------------------------------------------
-__device__ __noinline__ u32x4 draw_one(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot) {
-  const u32x4 c = {idx, cand, gen, slot};
-  return philox4x32_10(c, k0, k1);
-}
-
-// Two calls that differ only in their slot (the last counter word), side by side: of the first call word
-// x, of the second all.  What does not see the slot is worked out once - the first round, the first product
-// of the second, the second product of the third - and of the first call's last two rounds only what its
-// word x needs.
-__device__ __noinline__ void draw_two(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot_a,
-                                      uint32_t slot_b, uint32_t &a_x, u32x4 &b) {
-  constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u, W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
-#define HI(m, v) __umulhi((m), (v))
-#define LO(m, v) ((m) * (v))
-  u32x4 ca, cb, na, nb;
-  {
-    const uint32_t x = HI(M1, gen) ^ cand ^ k0, y = LO(M1, gen), w = LO(M0, idx), h0 = HI(M0, idx);
-    const uint32_t za = h0 ^ slot_a ^ k1, zb = h0 ^ slot_b ^ k1;
-    k0 += W0; k1 += W1;
-    ca.x = HI(M1, za) ^ y ^ k0; ca.y = LO(M1, za);
-    cb.x = HI(M1, zb) ^ y ^ k0; cb.y = LO(M1, zb);
-    ca.z = HI(M0, x) ^ w ^ k1; ca.w = LO(M0, x);
-    k0 += W0; k1 += W1;
-    const uint32_t h1 = HI(M1, ca.z), l1 = LO(M1, ca.z);
-    na.x = h1 ^ ca.y ^ k0; na.y = l1; na.z = HI(M0, ca.x) ^ ca.w ^ k1; na.w = LO(M0, ca.x);
-    nb.x = h1 ^ cb.y ^ k0; nb.y = l1; nb.z = HI(M0, cb.x) ^ ca.w ^ k1; nb.w = LO(M0, cb.x);
-    ca = na; cb = nb;
-    k0 += W0; k1 += W1;
-  }
-#pragma unroll
-  for (int r = 3; r < 8; ++r) {
-    na.x = HI(M1, ca.z) ^ ca.y ^ k0; na.y = LO(M1, ca.z); na.z = HI(M0, ca.x) ^ ca.w ^ k1; na.w = LO(M0, ca.x);
-    nb.x = HI(M1, cb.z) ^ cb.y ^ k0; nb.y = LO(M1, cb.z); nb.z = HI(M0, cb.x) ^ cb.w ^ k1; nb.w = LO(M0, cb.x);
-    ca = na; cb = nb;
-    k0 += W0; k1 += W1;
-  }
-  // ninth round: of the first call y and z
-  na.y = LO(M1, ca.z); na.z = HI(M0, ca.x) ^ ca.w ^ k1;
-  nb.x = HI(M1, cb.z) ^ cb.y ^ k0; nb.y = LO(M1, cb.z); nb.z = HI(M0, cb.x) ^ cb.w ^ k1; nb.w = LO(M0, cb.x);
-  k0 += W0; k1 += W1;
-  a_x = HI(M1, na.z) ^ na.y ^ k0;
-  b.x = HI(M1, nb.z) ^ nb.y ^ k0; b.y = LO(M1, nb.z); b.z = HI(M0, nb.x) ^ nb.w ^ k1; b.w = LO(M0, nb.x);
-#undef HI
-#undef LO
 }
 
 // ---- waiting and publishing --------------------------------------------------------------------
@@ -484,34 +438,6 @@ constexpr int INFO_DIST = 1;        // the row spanned two nodes or more after t
 constexpr int INFO_CHANGED = 2;     // a node's decision changes it
 constexpr int INFO_WIDE = 4;
 
-// What the repair decides for the occupant in this lane of a group of 16 (entry: an occupant as listed): the GPUs it keeps on the node.  rot_i, rot_c: the row's place in the node's two
-// rotated job orders.  Called by whole warps, two nodes at a time (shuffles under the full mask; a group
-// without a node has no occupants).
-__device__ __forceinline__ int decide(uint32_t entry, bool have, int most, bool intf, int tot, int cap_n, int rot_i, int rot_c) {
-  int v = have ? (int)((entry >> 13) & 0x7FFu) : 0;
-  const bool dist = have && intf && (entry >> 31);
-  int removed = 0;
-  if (__any_sync(0xffffffffu, intf)) {
-    int first = dist ? rot_i : 0x7fffffff;
-#pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) first = min(first, __shfl_xor_sync(0xffffffffu, first, off));
-    if (dist && rot_i != first) { removed = v; v = 0; }
-#pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, off);
-  }
-  const int excess = tot - removed - cap_n;
-  int ahead = 0;                         // GPUs of the occupants that come first in rotated order
-  if (__any_sync(0xffffffffu, excess > 0)) {
-#pragma unroll 1
-    for (int k = 0; k < most; ++k) {
-      const int rk = __shfl_sync(0xffffffffu, rot_c, k, 16), vk = __shfl_sync(0xffffffffu, v, k, 16);
-      if (rk < rot_c) ahead += vk;
-    }
-  }
-  if (have && excess > 0) v -= min(v, max(excess - ahead, 0));
-  return v;
-}
-
 // Block-wide minimum and exclusive prefix sum (s_red: a word per warp); both end with a barrier.
 __device__ __noinline__ int block_min(int v, int *s_red, int nwarps) {
   v = __reduce_min_sync(0xffffffffu, v);
@@ -553,46 +479,6 @@ __device__ __noinline__ int row_at(const uint32_t *rec, const int16_t *wide, int
 #pragma unroll
   for (int k = 0; k < ENTRIES; ++k) v = entry_node(r.w[k]) == node ? entry_gpus(r.w[k]) : v;
   return v;
-}
-
-// The candidate of rank c (fitness key descending, index ascending) of P keys in shared memory, by one
-// warp.  The (c + 1)-th largest of the lanes' own maxima is no larger than the key wanted, so only the
-// keys from there on (about twice c) are ranked; list: room for P.
-__device__ __noinline__ int candidate_of_rank(const uint32_t *key, int P, int c, uint16_t *list, int lane) {
-  uint32_t top = 0u;
-#pragma unroll 4
-  for (int i = lane; i < P; i += 32) top = max(top, key[i]);
-  int before = 0;                       // lanes whose maximum comes first
-#pragma unroll 1
-  for (int l = 0; l < 32; ++l) {
-    const uint32_t o = __shfl_sync(0xffffffffu, top, l);
-    before += o > top || (o == top && l < lane) ? 1 : 0;
-  }
-  uint32_t bound = 0u;                  // (more ranks than lanes: every key)
-  if (c < 32) bound = __shfl_sync(0xffffffffu, top, __ffs(__ballot_sync(0xffffffffu, before == c)) - 1);
-  int n = 0;
-#pragma unroll 1
-  for (int i0 = 0; i0 < P; i0 += 32) {
-    const bool in = i0 + lane < P && key[i0 + lane] >= bound;
-    const unsigned m = __ballot_sync(0xffffffffu, in);
-    if (in) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(i0 + lane);
-    n += __popc(m);
-  }
-  __syncwarp();
-  int found = 0x7fffffff;
-#pragma unroll 1
-  for (int x = lane; x < n; x += 32) {
-    const int i = list[x];
-    const uint32_t k = key[i];
-    int rank = 0;
-#pragma unroll 2
-    for (int y = 0; y < n; ++y) {
-      const uint32_t o = key[list[y]];
-      rank += o > k || (o == k && y < x) ? 1 : 0;
-    }
-    if (rank == c) found = i;
-  }
-  return __reduce_min_sync(0xffffffffu, found);
 }
 
 // everything a block knows about the candidate it is working on
@@ -1018,7 +904,7 @@ __global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const
           if (ri < 0) ri += J;
           if (rc < 0) rc += J;
           const int most = max(__shfl_sync(0xffffffffu, count, 0), __shfl_sync(0xffffffffu, count, 16));
-          const int v = decide(e, have, min(most, a.occ), (s_cnt[n] & 0xFFFFu) >= 2u, s_tot[n], (int)s_cap[n], ri, rc);
+          const int v = decide(have ? (int)((e >> 13) & 0x7FFu) : 0, (e >> 31) != 0u, have, min(most, a.occ), (s_cnt[n] & 0xFFFFu) >= 2u, s_tot[n], (int)s_cap[n], ri, rc);
           const bool changed = have && v != (int)((e >> 13) & 0x7FFu);
           if (changed) {
             set_entry(jc, (int)((e >> 25) & 7u), n, v);

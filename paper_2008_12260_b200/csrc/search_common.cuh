@@ -1,0 +1,119 @@
+// Pieces of the population search (Sec. 4.3) that the one-launch round and the dense operators share: draws of the
+// counter-based stream, the candidate of a rank, the repair's decision for a node.
+#pragma once
+
+#include "common.cuh"
+
+static __device__ __noinline__ u32x4 draw_one(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot) {
+  const u32x4 c = {idx, cand, gen, slot};
+  return philox4x32_10(c, k0, k1);
+}
+
+// Two calls that differ only in their slot (the last counter word), side by side: of the first call word
+// x, of the second all.  What does not see the slot is worked out once - the first round, the first product
+// of the second, the second product of the third - and of the first call's last two rounds only what its
+// word x needs.
+static __device__ __noinline__ void draw_two(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot_a,
+                                      uint32_t slot_b, uint32_t &a_x, u32x4 &b) {
+  constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u, W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
+#define HI(m, v) __umulhi((m), (v))
+#define LO(m, v) ((m) * (v))
+  u32x4 ca, cb, na, nb;
+  {
+    const uint32_t x = HI(M1, gen) ^ cand ^ k0, y = LO(M1, gen), w = LO(M0, idx), h0 = HI(M0, idx);
+    const uint32_t za = h0 ^ slot_a ^ k1, zb = h0 ^ slot_b ^ k1;
+    k0 += W0; k1 += W1;
+    ca.x = HI(M1, za) ^ y ^ k0; ca.y = LO(M1, za);
+    cb.x = HI(M1, zb) ^ y ^ k0; cb.y = LO(M1, zb);
+    ca.z = HI(M0, x) ^ w ^ k1; ca.w = LO(M0, x);
+    k0 += W0; k1 += W1;
+    const uint32_t h1 = HI(M1, ca.z), l1 = LO(M1, ca.z);
+    na.x = h1 ^ ca.y ^ k0; na.y = l1; na.z = HI(M0, ca.x) ^ ca.w ^ k1; na.w = LO(M0, ca.x);
+    nb.x = h1 ^ cb.y ^ k0; nb.y = l1; nb.z = HI(M0, cb.x) ^ ca.w ^ k1; nb.w = LO(M0, cb.x);
+    ca = na; cb = nb;
+    k0 += W0; k1 += W1;
+  }
+#pragma unroll
+  for (int r = 3; r < 8; ++r) {
+    na.x = HI(M1, ca.z) ^ ca.y ^ k0; na.y = LO(M1, ca.z); na.z = HI(M0, ca.x) ^ ca.w ^ k1; na.w = LO(M0, ca.x);
+    nb.x = HI(M1, cb.z) ^ cb.y ^ k0; nb.y = LO(M1, cb.z); nb.z = HI(M0, cb.x) ^ cb.w ^ k1; nb.w = LO(M0, cb.x);
+    ca = na; cb = nb;
+    k0 += W0; k1 += W1;
+  }
+  // ninth round: of the first call y and z
+  na.y = LO(M1, ca.z); na.z = HI(M0, ca.x) ^ ca.w ^ k1;
+  nb.x = HI(M1, cb.z) ^ cb.y ^ k0; nb.y = LO(M1, cb.z); nb.z = HI(M0, cb.x) ^ cb.w ^ k1; nb.w = LO(M0, cb.x);
+  k0 += W0; k1 += W1;
+  a_x = HI(M1, na.z) ^ na.y ^ k0;
+  b.x = HI(M1, nb.z) ^ nb.y ^ k0; b.y = LO(M1, nb.z); b.z = HI(M0, nb.x) ^ nb.w ^ k1; b.w = LO(M0, nb.x);
+#undef HI
+#undef LO
+}
+
+// What the repair decides for the occupant in this lane of a group of 16 (`have`: there is one; v: its GPUs on the
+// node, 0 without; distributed: its row spans two nodes or more): the GPUs it keeps there.  rot_i, rot_c: the
+// row's place in the node's two rotated job orders.  Called by whole warps, two nodes at a time (shuffles under the full mask; a group
+// without a node has no occupants).
+__device__ __forceinline__ int decide(int v, bool distributed, bool have, int most, bool intf, int tot, int cap_n, int rot_i, int rot_c) {
+  const bool dist = have && intf && distributed;
+  int removed = 0;
+  if (__any_sync(0xffffffffu, intf)) {
+    int first = dist ? rot_i : 0x7fffffff;
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) first = min(first, __shfl_xor_sync(0xffffffffu, first, off));
+    if (dist && rot_i != first) { removed = v; v = 0; }
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, off);
+  }
+  const int excess = tot - removed - cap_n;
+  int ahead = 0;                         // GPUs of the occupants that come first in rotated order
+  if (__any_sync(0xffffffffu, excess > 0)) {
+#pragma unroll 1
+    for (int k = 0; k < most; ++k) {
+      const int rk = __shfl_sync(0xffffffffu, rot_c, k, 16), vk = __shfl_sync(0xffffffffu, v, k, 16);
+      if (rk < rot_c) ahead += vk;
+    }
+  }
+  if (have && excess > 0) v -= min(v, max(excess - ahead, 0));
+  return v;
+}
+
+// The candidate of rank c (fitness key descending, index ascending) of P keys in shared memory, by one
+// warp.  The (c + 1)-th largest of the lanes' own maxima is no larger than the key wanted, so only the
+// keys from there on (about twice c) are ranked; list: room for P.
+static __device__ __noinline__ int candidate_of_rank(const uint32_t *key, int P, int c, uint16_t *list, int lane) {
+  uint32_t top = 0u;
+#pragma unroll 4
+  for (int i = lane; i < P; i += 32) top = max(top, key[i]);
+  int before = 0;                       // lanes whose maximum comes first
+#pragma unroll 1
+  for (int l = 0; l < 32; ++l) {
+    const uint32_t o = __shfl_sync(0xffffffffu, top, l);
+    before += o > top || (o == top && l < lane) ? 1 : 0;
+  }
+  uint32_t bound = 0u;                  // (more ranks than lanes: every key)
+  if (c < 32) bound = __shfl_sync(0xffffffffu, top, __ffs(__ballot_sync(0xffffffffu, before == c)) - 1);
+  int n = 0;
+#pragma unroll 1
+  for (int i0 = 0; i0 < P; i0 += 32) {
+    const bool in = i0 + lane < P && key[i0 + lane] >= bound;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (in) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(i0 + lane);
+    n += __popc(m);
+  }
+  __syncwarp();
+  int found = 0x7fffffff;
+#pragma unroll 1
+  for (int x = lane; x < n; x += 32) {
+    const int i = list[x];
+    const uint32_t k = key[i];
+    int rank = 0;
+#pragma unroll 2
+    for (int y = 0; y < n; ++y) {
+      const uint32_t o = key[list[y]];
+      rank += o > k || (o == k && y < x) ? 1 : 0;
+    }
+    if (rank == c) found = i;
+  }
+  return __reduce_min_sync(0xffffffffu, found);
+}

@@ -1,0 +1,76 @@
+"""Dense operators with a block (or a cluster of blocks) per child: rows of every width relative to a 16-byte vector,
+buffers that begin between two vectors, crowded nodes (more occupants than a list holds), entries out of range,
+full rows (every vector of a tile queued), children split over several blocks.  Bit-exact against the oracle,
+whose code knows none of these cases."""
+import numpy as np
+import pytest
+
+from paper_2008_12260_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+class _Jobs:
+    def __init__(self, k_cap, active):
+        self.k_cap, self.active = k_cap, active
+
+
+def _unaligned(torch, a, shift):
+    """A device copy of `a` that begins `shift` entries behind a 16-byte boundary, with guards around it."""
+    flat = torch.full((a.size + 32,), 77, dtype=torch.int16, device="cuda:0")
+    view = flat[8 + shift:8 + shift + a.size].view(a.shape)
+    view.copy_(torch.from_numpy(a))
+    return flat, view
+
+
+def _guards_ok(flat, shift, size):
+    return bool((flat[:8 + shift] == 77).all()) and bool((flat[8 + shift + size:] == 77).all())
+
+
+# nodes, jobs, population, density of the raw matrices, shifts of parents and children
+CASES = [
+    (1, 3, 5, 0.9, 1, 0), (7, 33, 9, 0.3, 0, 3), (8, 33, 9, 0.3, 0, 0), (8, 33, 9, 0.3, 4, 0), (9, 1, 4, 0.5, 7, 2),
+    (31, 40, 7, 0.2, 0, 0), (33, 257, 200, 0.05, 5, 6), (75, 300, 3, 0.1, 0, 0), (255, 70, 5, 0.02, 1, 7),
+    (256, 130, 4, 0.02, 0, 0), (256, 64, 4, 1.0, 0, 5), (257, 65, 3, 0.02, 0, 0), (448, 40, 3, 0.05, 3, 3), (504, 33, 3, 0.05, 0, 0),
+    (511, 37, 3, 0.05, 0, 1), (512, 37, 3, 1.0, 0, 0), (512, 37, 3, 0.3, 0, 0), (512, 37, 3, 0.3, 2, 0), (16, 1000, 2, 0.2, 0, 0),
+]
+
+
+@pytest.mark.parametrize("nodes,J,P,density,shift_in,shift_out", CASES)
+def test_children_of_any_width(oracle, nodes, J, P, density, shift_in, shift_out):
+    import torch
+    from paper_2008_12260_b200 import api
+
+    rng = np.random.default_rng(nodes * 1000 + J)
+    cl = synth.Cluster(rng.integers(0, 9, nodes).astype(np.int16)) if nodes > 1 else synth.uniform_cluster(1, 4)
+    if int(np.maximum(cl.node_capacity, 0).sum()) == 0:
+        cl = synth.uniform_cluster(nodes, 4)
+    raw = synth.random_raw_population(P, J, cl, seed=nodes + J, density=density, v_hi=9)
+    raw[-1, 0, -1], raw[0, 0, 0] = 30000, -5                # out of range, at both ends of the buffer
+    k_cap = rng.integers(0, cl.k_max + 3, J).astype(np.int32)
+    active = (rng.uniform(size=J) < 0.85).astype(np.uint8)
+    fit = rng.uniform(0.1, 1.0, P).astype(np.float32)
+    thr, elite, seed = synth.prob_to_threshold(0.3), min(2, P - 1), 77
+    s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=thr,
+                      thr_init=thr, num_elite=elite, seed=seed, stream=torch.cuda.current_stream().cuda_stream)
+    dj = api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch)
+    _, parents = _unaligned(torch, raw, shift_in)
+    out_flat, out = _unaligned(torch, np.full(raw.shape, 5, np.int16), shift_out)
+
+    s.ga_generation(dj, parents, torch.from_numpy(fit).cuda(), out, round=2, generation=3)
+    ref = oracle.ga_generation(raw, fit, cl.node_capacity, k_cap, cl.k_max, cl.n_max, elite, thr, seed, 2, 3, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+
+    s.init_population(dj, parents[0], out, round=4)
+    ref = oracle.init_population(P, raw[0], J, cl.node_capacity, k_cap, cl.k_max, cl.n_max, thr, seed, 4, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+
+    out.copy_(torch.from_numpy(raw))
+    s.repair_population(dj, out, round=5, generation=6, first_candidate=9)
+    got = out.cpu().numpy()
+    for c in range(P):
+        ref = oracle.repair(raw[c], cl.node_capacity, k_cap, cl.k_max, cl.n_max, seed, 5, 9 + c, 6, active=active)
+        assert np.array_equal(got[c], ref), c
+    assert _guards_ok(out_flat, shift_out, raw.size)
+    s.sync_status()
+    s.close()
