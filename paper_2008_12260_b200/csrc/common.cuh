@@ -116,8 +116,9 @@ struct sched_ctx {
   // Rounds whose blocks stay on the GPU (round_flow.cu): one allocation, with the tables in it
   void *fl_arena;
   int fl_blocks;           // blocks of the launch, 0: rounds run on the other kernels
+  int fl_warps, fl_draw_warps;   // of a block: that work on rows, that draw a step ahead
+  bool fl_terms;           // the rows' terms are looked up in shared memory
   int fl_generations;      // generations of the last round
-  bool fl_ahead;           // blocks have threads that draw a step ahead
   unsigned int fl_wait_limit;   // sched_set_wait_limit
 
   // staging for the *_host entry points (allocated on first use)
@@ -210,19 +211,16 @@ struct u32x4 {
   uint32_t x, y, z, w;
 };
 
+__host__ __device__ __forceinline__ u32x4 philox_round(u32x4 c, uint32_t k0, uint32_t k1) {
+  // one 32 x 32 -> 64 bit multiply per product (a single wide multiply-add on the device)
+  const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+  return {(uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0};
+}
+
 __host__ __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    // one 32 x 32 -> 64 bit multiply per product (a single wide multiply-add on the device)
-    const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
-    const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
-    const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
-    u32x4 n;
-    n.x = hi1 ^ c.y ^ k0;
-    n.y = lo1;
-    n.z = hi0 ^ c.w ^ k1;
-    n.w = lo0;
-    c = n;
+    c = philox_round(c, k0, k1);
     k0 += 0x9E3779B9u;
     k1 += 0xBB67AE85u;
   }

@@ -13,8 +13,9 @@
 // A row is a 32-byte record: up to six occupied nodes (node << 16 | GPUs, ascending) and the row's term
 // of the fitness sum (a row always serves the same job, so the term is fixed for the round).  A child copies
 // the records of its parents' rows; only a row with more occupied nodes ("wide") also has contents.
-// Rows of inactive jobs are left out.  One block works on one candidate at a time: a thread per row, a
-// warp of its own for the perturbed rows, whose path is long and whose number is small.
+// Rows of inactive jobs are left out.  One block works on one candidate at a time: eight lanes take a row, a word
+// of its record each, so that what is done to a row's nodes is done to all of them at once, four rows a warp;
+// perturbed rows and rows that the repair changes are dealt out like that, too.  Warps of their own draw a step ahead.
 // Operators, draws and the order of the fitness sums are those of the dense kernels: identical populations
 // and fitness bits.
 #include <algorithm>
@@ -31,20 +32,36 @@ constexpr uint32_t NO_NODE = 0xFFFFFFFFu;       // an entry that is not used
 constexpr uint32_t WIDE = 0xFFFFFFFEu;          // first entry of a row with more: its contents are elsewhere
 constexpr int REC_TERM = 6;
 constexpr int DEPTH = 4;                        // generations kept
-constexpr int MAX_ROW_THREADS = 256;            // as the dense fitness kernel: the order of its sums
-constexpr int STASH = 128;                      // perturbed rows whose draws are kept, further ones draw again
+constexpr int SUM_THREADS = 256;                // as the dense fitness kernel: the order of its sums
+constexpr int LANES = 8;                        // lanes of a row
+constexpr int STASH = 128;                      // perturbed rows of many whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
+constexpr int FLOW_MAX_WARPS = 20;
+constexpr int FLOW_OCC = 16;                    // occupants listed per node: a group of lanes
 constexpr int FLOW_MAX_JOBS = 8192, FLOW_MAX_NODES = 512;
 
+// Kinds of the generation kernel.  Not MANY: the child's records and what its rows' terms are made of are kept in shared
+// memory, too.  FEW_ALONE, SOME_ALONE: no two blocks share an SM (a population of at most as many), up to 256 and up to
+// 1024 jobs.  Registers: 142 for FEW_ALONE's 12 warps (testbed round 490 us; 522 with 96, 555 with 64, that is with
+// spills, which lie in the L1 that every acquire empties), 96 for SOME_ALONE's 20 (12 warps for 881 jobs: 826 us, 20: 730),
+// 64 for FEW, 56 for MANY.
+constexpr int FEW_ALONE = 0, SOME_ALONE = 1, FEW = 2, MANY = 3;
+__host__ __device__ constexpr bool few(int kind) { return kind != MANY; }
+__host__ __device__ constexpr int kind_threads(int kind) { return kind == FEW_ALONE ? 384 : kind == SOME_ALONE ? 640 : kind == FEW ? 512 : 288; }
+__host__ __device__ constexpr int kind_blocks(int kind) { return kind == MANY ? 4 : kind == FEW ? 2 : 1; }
+
 __host__ __device__ inline int wide_stride(int NN) { return (NN + 7) & ~7; }
+__host__ __device__ inline int stash_rows(int J) { return J <= SMEM_RECORDS ? J : STASH; }
 
 struct FlowRows {
   uint32_t *rec;             // [DEPTH][P][J][REC_WORDS]; rows of active jobs only, one behind the other
   int16_t *wide;             // [DEPTH][P][J][wide_stride] contents of wide rows
   uint32_t *cur_rec;         // [2][J][REC_WORDS] the current allocation after the row caps, and before them
   int16_t *cur_wide;         // [2][J][wide_stride]
-  uint32_t *same;            // [J][REC_WORDS] entries of a row that equals the current allocation's (first one
-                             // NO_NODE - 2: there is none with six nodes or fewer)
+  uint32_t *same;            // [J][REC_WORDS] a row that counts as unchanged, with its term (first entry NEVER: there is none
+                             // with six nodes or fewer)
+  float *terms;              // [J][classes][k_max + 1] term of a row that counts as changed (or of any, without the penalty), by
+                             // its GPUs and where they are: one node, several, several racks
   float *pen;                // [J] penalty factor of a row that differs from the current allocation's
   uint16_t *act;             // [J] active jobs, ascending; act[J] .. : see num_act
   int *num_act;
@@ -52,6 +69,12 @@ struct FlowRows {
   uint32_t *base;            // tag of the round's initial population
 };
 constexpr uint32_t NEVER = 0xFFFFFFFDu;
+
+// Places in the generation kernel's shared memory, behind what the warps tell each other (terms: -1 where they are not kept there).
+struct FlowSmem {
+  int act, term, info, node, occ, viol, cap, rack, mut, mod, wide, slow, stash, flag, dense, rep, keys, sums, scratch, rec, same,
+      terms, total;
+};
 
 struct FlowArgs {
   FlowRows r;
@@ -65,8 +88,11 @@ struct FlowArgs {
   const float *table_rack;
   TermParams tp;             // tp.pen: r.pen when the penalty is on
   float delta;
-  int P, J, NN, k_max, n_max, num_elite, generations, occ;
-  int row_threads;           // then the warp of the perturbed rows, then the threads that draw (or none: the row threads do)
+  const int32_t *nmin;       // [k_max + 1] fewest nodes, two or more, that K replicas fit on
+  int P, J, NN, k_max, n_max, num_elite, generations;
+  int warps;                 // warps that work on the rows; the others draw
+  int classes;               // 2, or 3 with racks
+  FlowSmem at;
   uint32_t thr_init, thr_mutate;
   RngKey key;
   int rows_per_chunk, chunks;   // the dense fitness kernel's chunking, reproduced for identical sums
@@ -97,22 +123,18 @@ __device__ __forceinline__ void store_record(uint32_t *p, const Record &r) {
 }
 
 // ---- waiting and publishing --------------------------------------------------------------------
-// The key published under `tag`; false when it has not come within the limit (the caller returns: the
+// The word (tag << 32 | key) published under `tag`; 0 when it has not come within the limit (the caller returns: the
 // other blocks' waits run out the same way).  A thread that has waited calls waited() before the barrier
 // behind which the block reads the rows, or before it publishes in its turn.
-__device__ __noinline__ bool wait_tag(const unsigned long long *p, uint32_t tag, uint32_t &key, unsigned int limit, int *status) {
+__device__ __forceinline__ unsigned long long wait_tag(const unsigned long long *p, uint32_t tag, unsigned int limit, int *status) {
 #pragma unroll 1
   for (unsigned int n = 0; n < limit; ++n) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    if ((uint32_t)(v >> 32) == tag) {
-      key = (uint32_t)v;
-      return true;
-    }
+    if ((uint32_t)(v >> 32) == tag) return v;
   }
   atomicCAS(status, 0, SCHED_ERR_TIMEOUT);
-  key = 0u;
-  return false;
+  return 0ull;
 }
 // Acquire: with the publisher's fence (release) and the block's barrier, what was written before the tag
 // was published is seen by every thread of this block, and what was read before it lies behind it.  One
@@ -125,147 +147,9 @@ __device__ __forceinline__ void publish(unsigned long long *p, uint32_t tag, uin
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// ---- a row as its sorted list of occupied nodes, in registers -------------------------------------
-constexpr int LIST = ENTRIES + 1;       // one more than a record holds: a perturbation may add before the caps take
-
-__device__ __forceinline__ void list_totals(const uint32_t (&e)[LIST], int &K, int &N) {
-  K = 0;
-  N = 0;
-#pragma unroll
-  for (int k = 0; k < LIST; ++k) {
-    const bool on = e[k] != NO_NODE;
-    K += on ? entry_gpus(e[k]) : 0;
-    N += on ? 1 : 0;
-  }
-}
-
-// GPUs on a node, 0 when it is not occupied
-__device__ __forceinline__ int list_at(const uint32_t (&e)[LIST], int node) {
-  int v = 0;
-#pragma unroll
-  for (int k = 0; k < LIST; ++k) v = entry_node(e[k]) == node ? entry_gpus(e[k]) : v;
-  return v;
-}
-
-// A[j][node] = v
-__device__ __forceinline__ void list_set(uint32_t (&e)[LIST], int node, int v) {
-  bool found = false;
-#pragma unroll
-  for (int k = 0; k < LIST; ++k)
-    if (entry_node(e[k]) == node) {
-      found = true;
-      e[k] = v > 0 ? ((uint32_t)node << 16) | (uint32_t)v : NO_NODE;
-    }
-  uint32_t x = !found && v > 0 ? ((uint32_t)node << 16) | (uint32_t)v : NO_NODE;
-#pragma unroll
-  for (int k = 0; k < LIST; ++k) {      // a new entry to its place, a hole to the end
-    const uint32_t lo = min(e[k], x);
-    x = max(e[k], x);
-    e[k] = lo;
-  }
-#pragma unroll
-  for (int k = 0; k + 1 < LIST; ++k) {
-    const uint32_t lo = min(e[k], e[k + 1]);
-    e[k + 1] = max(e[k], e[k + 1]);
-    e[k] = lo;
-  }
-}
-
-// grow / shrink / relocate (Sec. 4.3), chosen by the row's draw
-__device__ __forceinline__ void list_perturb(uint32_t (&e)[LIST], int N, uint32_t wy, uint32_t wz, uint32_t ww, int NN,
-                                             const int16_t *s_cap) {
-  const uint32_t op = bounded(wy, 3u);
-  const int nd = (int)bounded(ww, (uint32_t)NN);
-  int ns = -1, vs = 0;
-  if (op != 0u && N > 0) {
-    const int t = (int)bounded(wz, (uint32_t)N);
-#pragma unroll
-    for (int k = 0; k < LIST; ++k)
-      if (k == t) { ns = entry_node(e[k]); vs = entry_gpus(e[k]); }
-  }
-  int node0 = -1, v0 = 0, node1 = -1;
-  if (op == 0u) {
-    node0 = nd;
-    v0 = min(list_at(e, nd) + 1, (int)s_cap[nd]);
-  } else if (ns >= 0) {
-    if (op == 1u) {
-      node0 = ns;
-      v0 = vs - 1;
-    } else if (nd != ns) {
-      node0 = nd;
-      v0 = min(list_at(e, nd) + vs, (int)s_cap[nd]);
-      node1 = ns;
-    }
-  }
-#pragma unroll 1
-  for (int q = 0; q < 2; ++q) {
-    const int node = q ? node1 : node0;
-    if (node >= 0) list_set(e, node, q ? 0 : v0);
-  }
-}
-
-// row caps: replicas above kc leave from the highest node index down, then occupied nodes beyond n_max
-// are cleared from the highest index down
-__device__ __forceinline__ void list_caps(uint32_t (&e)[LIST], int K, int kc, int n_max) {
-  int excess = K - kc;
-#pragma unroll
-  for (int k = LIST - 1; k >= 0; --k) {
-    if (e[k] != NO_NODE && excess > 0) {
-      const int v = entry_gpus(e[k]), take = min(v, excess);
-      excess -= take;
-      e[k] = take == v ? NO_NODE : e[k] - (uint32_t)take;
-    }
-    if (k >= n_max) e[k] = NO_NODE;
-  }
-}
-
-// ---- fitness terms ------------------------------------------------------------------------------
+// ---- fitness terms of rows laid out in shared memory ----------------------------------------------
 // table of a row by the racks its nodes lie in
 __device__ __forceinline__ const float *table_of(const FlowArgs &a, int lo, int hi) { return lo < hi ? a.table_rack : a.tp.table; }
-
-__device__ __forceinline__ const float *list_table(const FlowArgs &a, const uint32_t (&e)[LIST]) {
-  if (!a.rack) return a.tp.table;
-  int lo = 0x7fffffff, hi = -1;
-#pragma unroll
-  for (int k = 0; k < ENTRIES; ++k)
-    if (e[k] != NO_NODE && sched_index_ok(a.status, entry_node(e[k]) < a.NN, SCHED_CHK_NODE)) {
-      const int r = (int)__ldg(a.rack + entry_node(e[k]));
-      lo = min(lo, r);
-      hi = max(hi, r);
-    }
-  return table_of(a, lo, hi);
-}
-
-// What a finished list's term needs from memory, asked for together (the table's entry, the job's penalty
-// factor, the current allocation's entries), and the record it gives.
-struct TermLoads {
-  float speedup, pen;
-  uint4 lo;
-  uint2 hi;
-};
-__device__ __forceinline__ TermLoads list_loads(const FlowArgs &a, const uint32_t (&e)[LIST], int j, int K, int N) {
-  TermLoads t;
-  t.pen = 1.f;
-  t.lo = make_uint4(0u, 0u, 0u, 0u);
-  t.hi = make_uint2(0u, 0u);
-  if (a.tp.pen) {
-    t.lo = __ldg((const uint4 *)(a.r.same + (size_t)j * REC_WORDS));
-    t.hi = __ldg((const uint2 *)(a.r.same + (size_t)j * REC_WORDS + 4));
-    t.pen = __ldg(a.r.pen + j);
-  }
-  if (!sched_index_ok(a.status, j < a.J && K >= 0 && N >= 0 && N <= ENTRIES, SCHED_CHK_ENTRY)) K = N = 0;
-  t.speedup = __ldg(list_table(a, e) + fitness_table_index(a.tp, j, K, N));
-  return t;
-}
-__device__ __forceinline__ Record list_record(const FlowArgs &a, const uint32_t (&e)[LIST], const TermLoads &t) {
-  const bool changed = t.lo.x != e[0] || t.lo.y != e[1] || t.lo.z != e[2] || t.lo.w != e[3] || t.hi.x != e[4] || t.hi.y != e[5];
-  Record r;
-#pragma unroll
-  for (int k = 0; k < ENTRIES; ++k) r.w[k] = e[k];
-  r.w[REC_TERM] = __float_as_uint(fitness_term_with(a.tp, t.speedup, t.pen, changed));
-  r.w[7] = 0u;
-  return r;
-}
 
 // ---- rows laid out in shared memory, a warp each (wide rows, and lists that overflow) --------------
 __device__ __forceinline__ void dense_from_list(int16_t *row, int NS, const Record &r, int lane, int *status) {
@@ -382,7 +266,22 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) raw += __shfl_xor_sync(0xffffffffu, raw, off);
     in_range = __all_sync(0xffffffffu, in_range);
-    if (a.tp.pen && lane == 0) a.r.pen[j] = raw > 0 ? realloc_factor(a.age[j], a.restarts[j], a.delta) : 1.f;
+    const float pen = a.tp.pen && raw > 0 ? realloc_factor(a.age[j], a.restarts[j], a.delta) : 1.f;
+    if (a.tp.pen && lane == 0) a.r.pen[j] = pen;
+    // (what a row of the search can be: on one node, or on as many as its GPUs need at least; the table has one
+    // value for all of those)
+    const int KD = a.k_max + 1, ND = a.n_max + 1;
+#pragma unroll 1
+    for (int K = lane; K < KD; K += 32) {
+      const int many = K >= 2 ? a.nmin[K] : ND;
+#pragma unroll 1
+      for (int cls = 0; cls < a.classes; ++cls) {
+        const int N = cls ? many : K >= 1 ? 1 : ND;
+        const float *table = cls == 2 ? a.table_rack : a.tp.table;
+        const float x = N < ND ? table[((size_t)j * KD + K) * ND + N] : 0.f;
+        a.r.terms[((size_t)j * a.classes + cls) * KD + K] = fitness_term_with(a.tp, x, pen, true);
+      }
+    }
     __syncwarp();
     int K, N;
     dense_totals(row, NN, lane, K, N);
@@ -394,7 +293,7 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
       Record r = dense_record(a, row, j, K, N, a.r.cur_wide + at * NS, lane);
       if (lane == 0) store_record(a.r.cur_rec + at * REC_WORDS, r);
       if (caps && lane == 0) {
-        if (!in_range || N > ENTRIES) r.w[0] = NEVER;
+        if (!a.tp.pen || !in_range || N > ENTRIES) r.w[0] = NEVER;
         store_record(a.r.same + (size_t)j * REC_WORDS, r);
       }
       __syncwarp();
@@ -402,51 +301,86 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
   }
 }
 
-// ---- shared memory of the generation kernel -----------------------------------------------------
-struct FlowSmem {
-  size_t act, term, info, node, occ, viol, cap, mut, mod, wide, slow, stash, flag, dense, rep, keys, sums, rec, total;
-};
-
-__host__ __device__ inline FlowSmem flow_smem(int P, int J, int NN, int occ, int warps, int chunks) {
-  FlowSmem L;
-  size_t off = 0;
-#define TAKE(field, bytes) do { L.field = off; off += ((size_t)(bytes) + 15) & ~(size_t)15; } while (0)
-  TAKE(act, (size_t)J * 2);
-  TAKE(term, (size_t)J * 4);
-  TAKE(info, (size_t)J);
-  TAKE(node, (size_t)NN * 8);
-  TAKE(occ, (size_t)NN * occ * 4);
-  TAKE(viol, (size_t)NN);
-  TAKE(cap, (size_t)NN * 2);
-  TAKE(mut, 2 * (size_t)J * 2);
-  TAKE(mod, (size_t)J * 2);
-  TAKE(wide, (size_t)J * 2);
-  TAKE(slow, (size_t)J * 2);
-  TAKE(stash, 2 * (size_t)STASH * 16);
-  TAKE(flag, 2 * (size_t)J);
-  TAKE(dense, (size_t)warps * wide_stride(NN) * 2);
-  TAKE(rep, 2 * (size_t)NN * 4);
-  TAKE(keys, (size_t)P * 6);      // and a list of candidates behind them
-  TAKE(sums, (size_t)chunks * 8 * 8);
-  TAKE(rec, J <= SMEM_RECORDS ? (size_t)J * REC_WORDS * 4 : 0);
-#undef TAKE
-  L.total = off;
-  return L;
-}
-
 constexpr int INFO_DIST = 1;        // the row spanned two nodes or more after the row pass (interference snapshot)
 constexpr int INFO_CHANGED = 2;     // a node's decision changes it
 constexpr int INFO_WIDE = 4;
 
-// Block-wide minimum and exclusive prefix sum (s_red: a word per warp); both end with a barrier.
+// The candidate a block is working on.
+struct Work {
+  int src[2];                         // parents' first rows, counted in records from the population's first (initial population:
+                                      // the current allocation's rows after and before the caps, by job)
+  int dst;                            // the child's first row
+  uint32_t c, gen;
+  bool init;
+};
+
+// What the warps of a block tell each other.  Two sets where a candidate's draws are made while the one before
+// it is worked on.
+struct FlowCtl {
+  int4 hand[2];                       // parents' first rows, 0: a wait ran out
+  int nmut[2];
+  int nwide, nslow, nmod, walk, po;
+  uint32_t sel[2][4];
+  unsigned long long word;            // what is published
+  int red[FLOW_MAX_WARPS];
+};
+
+// The block's shared memory.
+struct FlowView {
+  FlowCtl &ctl;
+  uint16_t *act;                      // active jobs
+  float *term;                        // by job, 0 where there is none
+  uint8_t *info;                      // by row
+  uint32_t *node;                     // by node: GPUs placed on it; distributed jobs on it | occupants << 16
+  uint32_t *occ;                      // row | GPUs << 13 | place in the record (7: wide) << 25 | distributed << 31
+  uint8_t *viol;                      // the node's column is to be walked
+  int16_t *cap, *rack;
+  uint16_t *mut, *mod, *wide, *slow;  // mut: two sets
+  uint4 *stash;                       // two sets
+  uint8_t *flag;                      // two sets, by row: 1 from the second parent, 2 perturbed
+  int16_t *dense;                     // a row per warp
+  uint32_t *rep;                      // two sets, by node: the two rotation offsets
+  uint32_t *keys;
+  double *sums;
+  uint32_t *scratch;                  // a record's place per eight lanes
+  uint32_t *rec, *same;               // by row: the child's records, the unchanged rows (few jobs)
+  float *terms;                       // by row (where they fit)
+};
+
+// (memory: its address in the shared window, so that functions that are called know what it points to)
+__device__ __forceinline__ FlowView flow_view(const FlowArgs &a, uint32_t memory) {
+  const FlowSmem &L = a.at;
+  unsigned char *const s = (unsigned char *)__cvta_shared_to_generic(memory);
+  return FlowView{*(FlowCtl *)s, (uint16_t *)(s + L.act), (float *)(s + L.term), s + L.info, (uint32_t *)(s + L.node),
+                  (uint32_t *)(s + L.occ), s + L.viol, (int16_t *)(s + L.cap), (int16_t *)(s + L.rack),
+                  (uint16_t *)(s + L.mut), (uint16_t *)(s + L.mod), (uint16_t *)(s + L.wide), (uint16_t *)(s + L.slow),
+                  (uint4 *)(s + L.stash), s + L.flag, (int16_t *)(s + L.dense), (uint32_t *)(s + L.rep), (uint32_t *)(s + L.keys),
+                  (double *)(s + L.sums), (uint32_t *)(s + L.scratch), (uint32_t *)(s + L.rec), (uint32_t *)(s + L.same),
+                  (float *)(s + L.terms)};
+}
+
+__device__ __forceinline__ uint32_t *rec_row(const FlowArgs &a, int row) { return a.r.rec + (ptrdiff_t)row * REC_WORDS; }
+__device__ __forceinline__ int16_t *wide_row(const FlowArgs &a, int row) { return a.r.wide + (ptrdiff_t)row * wide_stride(a.NN); }
+// contents of row jc (job j) of a parent
+__device__ __forceinline__ const int16_t *wide_source(const FlowArgs &a, const Work &w, int from, int jc, int j) {
+  return w.init ? a.r.cur_wide + ((size_t)from * a.J + j) * wide_stride(a.NN) : wide_row(a, (from ? w.src[1] : w.src[0]) + jc);
+}
+
+// Barriers: 0 is the whole block's.
+constexpr int BAR_ROWS = 1;           // the warps that work on rows
+constexpr int BAR_SUMS = 2;           // all of them but the last
+constexpr int BAR_KEY = 3;            // the first and the last of them
+__device__ __forceinline__ void bar(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
+// Minimum and exclusive prefix sum over the warps that work on rows; both end with a barrier.
 __device__ __noinline__ int block_min(int v, int *s_red, int nwarps) {
   v = __reduce_min_sync(0xffffffffu, v);
   if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-  __syncthreads();
+  bar(BAR_ROWS, nwarps * 32);
   int r = s_red[0];
 #pragma unroll 1
   for (int w = 1; w < nwarps; ++w) r = min(r, s_red[w]);
-  __syncthreads();
+  bar(BAR_ROWS, nwarps * 32);
   return r;
 }
 __device__ __noinline__ int block_exscan(int v, int *s_red, int nwarps, int &total) {
@@ -458,7 +392,7 @@ __device__ __noinline__ int block_exscan(int v, int *s_red, int nwarps, int &tot
     if (lane >= off) incl += u;
   }
   if (lane == 31) s_red[warp] = incl;
-  __syncthreads();
+  bar(BAR_ROWS, nwarps * 32);
   int before = 0;
   total = 0;
 #pragma unroll 1
@@ -467,643 +401,760 @@ __device__ __noinline__ int block_exscan(int v, int *s_red, int nwarps, int &tot
     if (w < warp) before += t;
     total += t;
   }
-  __syncthreads();
+  bar(BAR_ROWS, nwarps * 32);
   return before + incl - v;
 }
 
 // GPUs of a finished row of this block's candidate on a node
-__device__ __noinline__ int row_at(const uint32_t *rec, const int16_t *wide, int NS, int jc, int node) {
-  const Record r = load_record(rec + (size_t)jc * REC_WORDS);
-  if (r.w[0] == WIDE) return (int)__ldcg(wide + (size_t)jc * NS + node);
+template <int KIND>
+__device__ __noinline__ int row_at(const FlowArgs &a, int row, int node) {
+  const Record r = load_record(rec_row(a, row));
+  if (r.w[0] == WIDE) return (int)__ldcg(wide_row(a, row) + node);
   int v = 0;
 #pragma unroll
   for (int k = 0; k < ENTRIES; ++k) v = entry_node(r.w[k]) == node ? entry_gpus(r.w[k]) : v;
   return v;
 }
 
-// everything a block knows about the candidate it is working on
-struct Work {
-  const uint32_t *src_a, *src_b;      // parents' records (initial population: the current allocation after and before the caps)
-  const int16_t *wide_a, *wide_b;     // and contents
-  uint32_t *rec;                      // the child's
-  int16_t *wide;
-  uint32_t c, gen, round;
-  bool init;
-};
+// ---- rows, eight lanes each: lane k has word k of the record --------------------------------------
+// Called by whole warps; `live`: this lane's row is one.
+
+// of a warp's ballot, the bits of this lane's row
+__device__ __forceinline__ unsigned row_bits(bool p, int lane) { return (__ballot_sync(0xffffffffu, p) >> (lane & 24)) & 0xFFu; }
+
+__device__ __forceinline__ int row_sum(int v) {
+#pragma unroll
+  for (int off = LANES / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// a row's occupant into the nodes' totals and lists
+__device__ __forceinline__ void add_occupant(const FlowArgs &a, const FlowView &v, int jc, int k_rec, uint32_t e, bool dist) {
+  const int n = entry_node(e);
+  if (!sched_index_ok(a.status, n < a.NN && jc < a.J && entry_gpus(e) <= 2047, SCHED_CHK_NODE)) return;
+  atomicAdd(&v.node[2 * n], (uint32_t)entry_gpus(e));
+  const uint32_t k = atomicAdd(&v.node[2 * n + 1], (dist ? 1u : 0u) | (1u << 16)) >> 16;
+  if (k < (uint32_t)FLOW_OCC)
+    v.occ[n * FLOW_OCC + k] = (uint32_t)jc | ((uint32_t)entry_gpus(e) << 13) | ((uint32_t)k_rec << 25) | (dist ? 0x80000000u : 0u);
+}
+
+// A word of a finished row goes to its place: the child's records, the term by job.
+template <int KIND>
+__device__ __forceinline__ void put_word(const FlowArgs &a, const FlowView &v, int dst, int jc, int k, uint32_t word) {
+  rec_row(a, dst + jc)[k] = word;
+  if (few(KIND)) v.rec[jc * REC_WORDS + k] = word;
+  if (k == REC_TERM) v.term[v.act[jc]] = __uint_as_float(word);
+}
+
+// Eight words of a warp's own, for a row whose entries are to be put in order: emptied, filled (by all lanes of the row that
+// have one), read.
+__device__ __forceinline__ uint32_t *empty_place(const FlowView &v, int warp, int lane) {
+  uint32_t *place = v.scratch + warp * 32 + (lane & 24);
+  place[lane & 7] = NO_NODE;
+  __syncwarp();
+  return place;
+}
+
+// A row's finished list becomes its record, the term from the classes' terms or the unchanged row's; in the row pass
+// (`fresh`) its occupants are added up.  e: this lane's entry, in any order; K, N: their GPUs and number; place: the entries in
+// order.
+template <int KIND>
+__device__ __forceinline__ void settle_row(const FlowArgs &a, const FlowView &v, int dst, int jc, uint32_t e, const uint32_t *place, int K, int N,
+                                           bool live, bool fresh, int lane) {
+  const int k = lane & 7;
+  int cls = N >= 2 ? 1 : 0;
+  if (a.rack) {
+    const bool on = e != NO_NODE && sched_index_ok(a.status, entry_node(e) < a.NN, SCHED_CHK_NODE);
+    const int r = on ? (int)v.rack[entry_node(e)] : -1;
+    const unsigned have = row_bits(on, lane);
+    const int first = __shfl_sync(0xffffffffu, r, have ? __ffs(have) - 1 : 0, LANES);
+    if (row_bits(on && r != first, lane)) cls = 2;
+  }
+  if (!live || !sched_index_ok(a.status, K >= 0 && K <= a.k_max && jc < a.J, SCHED_CHK_ENTRY)) K = 0;
+  const int row = a.classes * (a.k_max + 1), at = cls * (a.k_max + 1) + K, j = v.act[jc];
+  const uint32_t same = few(KIND) ? v.same[jc * REC_WORDS + k] : __ldg(a.r.same + (size_t)j * REC_WORDS + k);
+  const float changed = few(KIND) && a.at.terms >= 0 ? v.terms[jc * row + at] : __ldg(a.r.terms + (size_t)j * row + at);
+  __syncwarp();
+  const uint32_t word = place[k];
+  const uint32_t unchanged = __shfl_sync(0xffffffffu, same, REC_TERM, LANES);
+  const bool equal = (row_bits(word == same, lane) & 0x3Fu) == 0x3Fu;
+  if (live) {
+    put_word<KIND>(a, v, dst, jc, k, k < ENTRIES ? word : k == REC_TERM ? (equal ? unchanged : __float_as_uint(changed)) : 0u);
+    if (fresh && k < ENTRIES && word != NO_NODE) add_occupant(a, v, jc, k, word, N >= 2);
+    if (fresh && k == 0) v.info[jc] = N >= 2 ? INFO_DIST : 0;
+  }
+  __syncwarp();
+}
+
+// Row caps: replicas above kc leave from the highest node index down, then occupied nodes beyond n_max from the
+// highest index down.  The list in place; its GPUs and entries then.
+__device__ __noinline__ int2 cap_list(uint32_t *place, int K, int N, int kc, int n_max, bool over, int lane) {
+  __syncwarp();
+  const int k = lane & 7;
+  uint32_t e = place[k];
+  const int gpus = e != NO_NODE ? entry_gpus(e) : 0;
+  int upto = gpus;
+#pragma unroll
+  for (int off = 1; off < LANES; off <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, upto, off, LANES);
+    if (k >= off) upto += u;
+  }
+  if (over && e != NO_NODE) {
+    const int take = min(gpus, max(upto - kc, 0));
+    e = take == gpus || k >= n_max ? NO_NODE : e - (uint32_t)take;
+    place[k] = e;
+  }
+  return make_int2(row_sum(e != NO_NODE ? entry_gpus(e) : 0), __popc(row_bits(e != NO_NODE, lane)));
+}
+
+// The row pass for up to four perturbed rows: perturbation (grow, shrink, relocate, chosen by the row's draw), row caps,
+// the new record.  x0: the first of them in the list.
+template <int KIND>
+__device__ __forceinline__ void perturb_rows(const FlowArgs &a, const FlowView &v, const Work &w, uint32_t round, int set, int x0, int nmut,
+                                             int warp, int lane) {
+  uint32_t *const place = empty_place(v, warp, lane);
+  const int k = lane & 7, i = x0 + (lane >> 3), NN = a.NN;
+  const unsigned below = (1u << k) - 1u;
+  bool live = i < nmut;
+  const int m = live ? v.mut[set * a.J + i] : 0, jc = m & 0x7FFF;
+  live = live && sched_index_ok(a.status, i < a.J && jc < a.J, SCHED_CHK_LIST);
+  uint32_t e = NO_NODE;
+  if (live && k < ENTRIES) e = __ldcg(rec_row(a, (w.init || (m >> 15) ? w.src[1] : w.src[0]) + (w.init ? (int)v.act[jc] : jc)) + k);
+  uint4 st = make_uint4(0u, 0u, 0u, 0u);
+  if (i < stash_rows(a.J)) {
+    st = v.stash[set * stash_rows(a.J) + i];
+  } else if (live) {
+    const int j = v.act[jc];
+    const u32x4 d = draw_one(a.key.k0, round, (uint32_t)j, w.c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE);
+    st = make_uint4(d.y, d.z, d.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)));
+  }
+  __syncwarp();
+  const uint32_t op = bounded(st.x, 3u);
+  const int nd = (int)bounded(st.z, (uint32_t)NN), cap_nd = (int)v.cap[nd];
+  const bool wide = (row_bits(k == 0 && e == WIDE, lane) & 1u) != 0u;
+  int N = __popc(row_bits(e != NO_NODE, lane));
+  const uint32_t es = __shfl_sync(0xffffffffu, e, N > 0 ? (int)bounded(st.y, (uint32_t)N) : 0, LANES);
+  const int ns = entry_node(es), vs = entry_gpus(es);
+  const unsigned at_nd = row_bits(e != NO_NODE && entry_node(e) == nd, lane);
+  const uint32_t end = __shfl_sync(0xffffffffu, e, at_nd ? __ffs(at_nd) - 1 : 0, LANES);
+  const int v_nd = at_nd ? entry_gpus(end) : 0;
+  const bool change = op == 0u || (N > 0 && (op == 1u || nd != ns));
+  const int X = op == 1u ? ns : nd, V = op == 0u ? min(v_nd + 1, cap_nd) : op == 1u ? vs - 1 : min(v_nd + vs, cap_nd);
+  const uint32_t x = ((uint32_t)X << 16) | (uint32_t)V;
+  const bool insert = change && op != 1u && !at_nd && V > 0;
+  if (change && e != NO_NODE) {
+    if (entry_node(e) == X) e = V > 0 ? x : NO_NODE;
+    else if (op == 2u && entry_node(e) == ns) e = NO_NODE;
+  }
+  const unsigned there = row_bits(e != NO_NODE, lane);
+  const int extra = insert ? 1 : 0, extra_at = __popc(row_bits(e != NO_NODE && e < x, lane));
+  if (e != NO_NODE) place[__popc(there & below) + (e > x ? extra : 0)] = e;
+  if (insert && k == 7) {                     // (a record has no seventh entry: the lane of the new one)
+    place[extra_at] = x;
+    e = x;
+  }
+  int K = row_sum(e != NO_NODE ? entry_gpus(e) : 0);
+  N = __popc(there) + extra;
+  const bool over = live && !wide && (K > (int)st.w || N > a.n_max);
+  if (__any_sync(0xffffffffu, over)) {
+    const int2 now = cap_list(place, K, N, (int)st.w, a.n_max, over, lane);
+    K = now.x;
+    N = now.y;
+    __syncwarp();
+    e = place[k];
+  }
+  const bool slow = live && (wide || N > ENTRIES);
+  live = live && !slow;
+  if (slow && k == 0) {
+    const int at = atomicAdd(&v.ctl.nslow, 1);
+    if (sched_index_ok(a.status, at < a.J, SCHED_CHK_LIST)) v.slow[at] = (uint16_t)m;
+  }
+  settle_row<KIND>(a, v, w.dst, jc, live ? e : NO_NODE, place, K, N, live, true, lane);
+}
+
+// A row without the entries that decisions took out (0 GPUs), and its new term.
+template <int KIND>
+__device__ __forceinline__ void finish_row(const FlowArgs &a, const FlowView &v, int dst, int jc, bool live, int warp, int lane) {
+  uint32_t *const place = empty_place(v, warp, lane);
+  const int k = lane & 7;
+  uint32_t e = NO_NODE;
+  if (live && k < ENTRIES) e = few(KIND) ? v.rec[jc * REC_WORDS + k] : __ldcg(rec_row(a, dst + jc) + k);
+  if (entry_gpus(e) == 0) e = NO_NODE;
+  const unsigned there = row_bits(e != NO_NODE, lane);
+  if (e != NO_NODE) place[__popc(there & ((1u << k) - 1u))] = e;
+  settle_row<KIND>(a, v, dst, jc, e, place, row_sum(e != NO_NODE ? entry_gpus(e) : 0), __popc(there), live, false, lane);
+}
+
+// A wide row that decisions changed, by a warp.
+template <int KIND>
+__device__ __noinline__ void finish_wide(const FlowArgs &a, uint32_t memory, int dst, int jc, int warp, int lane) {
+  const FlowView v = flow_view(a, memory);
+  int16_t *dense = v.dense + (size_t)warp * wide_stride(a.NN), *row = wide_row(a, dst + jc);
+#pragma unroll 1
+  for (int n = lane; n < a.NN; n += 32) dense[n] = __ldcg(row + n);
+  __syncwarp();
+  int K, N;
+  dense_totals(dense, a.NN, lane, K, N);
+  const Record out = dense_record(a, dense, v.act[jc], K, N, row, lane);
+#pragma unroll
+  for (int k = 0; k < REC_WORDS; ++k)
+    if (lane == k) put_word<KIND>(a, v, dst, jc, k, out.w[k]);
+  if (lane == 0 && N <= ENTRIES) v.info[jc] &= ~INFO_WIDE;
+  __syncwarp();
+}
+
+// The row pass for wide rows, and for perturbed ones that are or may become wide: a warp each.
+template <int KIND>
+__device__ __noinline__ void wide_rows(const FlowArgs &a, uint32_t memory, Work w, uint32_t round, int warp, int lane) {
+  const FlowView v = flow_view(a, memory);
+  const int NN = a.NN, NS = wide_stride(NN), nwide = v.ctl.nwide;
+  int16_t *dense = v.dense + (size_t)warp * NS;
+#pragma unroll 1
+  for (int i = warp; i < nwide + v.ctl.nslow; i += a.warps) {
+    const bool slow = i >= nwide;
+    const int x = slow ? v.slow[i - nwide] : v.wide[i], jc = x & 0x7FFF;
+    if (!sched_index_ok(a.status, jc < a.J, SCHED_CHK_LIST)) continue;
+    const int j = v.act[jc];
+    const int from = (x >> 15) || (w.init && slow);
+    const Record rec = load_record(rec_row(a, (from ? w.src[1] : w.src[0]) + (w.init ? j : jc)));
+    int16_t *const mine = wide_row(a, w.dst + jc);
+    if (rec.w[0] == WIDE) {
+      const int16_t *contents = wide_source(a, w, from, jc, j);
+#pragma unroll 1
+      for (int n = lane; n < NS; n += 32) {
+        const int16_t e = __ldcg(contents + n);
+        dense[n] = e;
+        if (!slow) mine[n] = e;
+      }
+      __syncwarp();
+    } else {
+      dense_from_list(dense, NS, rec, lane, a.status);
+    }
+    if (slow) {
+      int K, N;
+      dense_totals(dense, NN, lane, K, N);
+      const u32x4 m = draw_one(a.key.k0, round, (uint32_t)j, w.c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE);
+      const uint32_t op = bounded(m.y, 3u);
+      const int nd = (int)bounded(m.w, (uint32_t)NN);
+      if (op == 0u) {
+        if (lane == 0) dense[nd] = (int16_t)min((int)dense[nd] + 1, (int)v.cap[nd]);
+      } else if (N > 0) {
+        int ns = nth_occupied(dense, NN, bounded(m.z, (uint32_t)N), lane);
+        if (!sched_index_ok(a.status, ns >= 0 && ns < NN && nd < NN, SCHED_CHK_NODE)) ns = nd;
+        if (lane == 0 && op == 1u) dense[ns] = (int16_t)(dense[ns] - 1);
+        if (lane == 0 && op == 2u && nd != ns) {
+          dense[nd] = (int16_t)min((int)dense[nd] + (int)dense[ns], (int)v.cap[nd]);
+          dense[ns] = 0;
+        }
+      }
+      __syncwarp();
+      dense_totals(dense, NN, lane, K, N);
+      dense_caps(dense, NN, K, N, max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)), a.n_max, lane);
+      const Record out = dense_record(a, dense, j, K, N, mine, lane);
+#pragma unroll
+      for (int k = 0; k < REC_WORDS; ++k)
+        if (lane == k) put_word<KIND>(a, v, w.dst, jc, k, out.w[k]);
+      if (lane == 0) v.info[jc] = (N >= 2 ? INFO_DIST : 0) | (N > ENTRIES ? INFO_WIDE : 0);
+      __syncwarp();
+    }
+    const bool dist = (v.info[jc] & INFO_DIST) != 0, wide = (v.info[jc] & INFO_WIDE) != 0;
+    int before = 0;
+#pragma unroll 1
+    for (int n0 = 0; n0 < NN; n0 += 32) {
+      const int n = n0 + lane, e = n < NN ? (int)dense[n] : 0;
+      const unsigned m = __ballot_sync(0xffffffffu, e > 0);
+      const int k = before + __popc(m & ((1u << lane) - 1u));
+      if (e > 0) add_occupant(a, v, jc, wide ? 7 : k, ((uint32_t)n << 16) | (uint32_t)e, dist);
+      before += __popc(m);
+    }
+    __syncwarp();
+  }
+}
+
+// A decision goes straight into the row: entry k of its record (0 GPUs: taken out when the row is
+// finished), or its contents.  Decisions of different nodes touch different words.
+template <int KIND>
+__device__ __forceinline__ void set_entry(const FlowArgs &a, const FlowView &v, int dst, int jc, int k, int n, int gpus) {
+  if (!sched_index_ok(a.status, jc < a.J && n < a.NN && (k == 7 || k < ENTRIES), SCHED_CHK_ENTRY)) return;
+  const uint32_t e = ((uint32_t)n << 16) | (uint32_t)gpus;
+  if (k == 7) wide_row(a, dst + jc)[n] = (int16_t)gpus;
+  else if (few(KIND)) v.rec[jc * REC_WORDS + k] = e;
+  else rec_row(a, dst + jc)[k] = e;
+}
+
+// Nodes with more occupants than a list holds: the warps walk the column, node by node.  Thread t looks after the
+// consecutive rows [t * rpt, (t + 1) * rpt).  Interference: the first distributed occupant in rotated job
+// order stays.  Capacity: a prefix sum in job order gives every row the GPUs that come before it in rotated
+// order.
+template <int KIND>
+__device__ __noinline__ void walk_columns(const FlowArgs &a, uint32_t memory, int dst, int set, int JA, int warp, int lane) {
+  const FlowView v = flow_view(a, memory);
+  const int tid = threadIdx.x, threads = a.warps * 32, J = a.J;
+  bar(BAR_ROWS, threads);
+  const int rpt = (JA + threads - 1) / threads;
+  const int lo = min(JA, tid * rpt), hi = min(JA, lo + rpt);
+#pragma unroll 1
+  for (int n = 0; n < a.NN; ++n) {
+    if (!v.viol[n]) continue;
+    const uint32_t rep = v.rep[set * a.NN + n];
+    const bool intf = (v.node[2 * n + 1] & 0xFFFFu) >= 2u;
+    auto dist = [&](int jc) { return (v.info[jc] & INFO_DIST) != 0; };
+    int keep = -1;
+    if (intf) {
+      int best = 0x7fffffff;
+#pragma unroll 1
+      for (int jc = lo; jc < hi; ++jc)
+        if (dist(jc) && row_at<KIND>(a, dst + jc, n) > 0) {
+          int t = (int)v.act[jc] - (int)(rep & 0xFFFFu);
+          if (t < 0) t += J;
+          best = min(best, t);
+        }
+      keep = (int)(rep & 0xFFFFu) + block_min(best, v.ctl.red, a.warps);     // the job that stays
+      if (keep >= J) keep -= J;
+    }
+    auto stays = [&](int jc) {
+      const int g = row_at<KIND>(a, dst + jc, n);
+      return intf && dist(jc) && g > 0 && (int)v.act[jc] != keep ? 0 : g;
+    };
+    int mine = 0, total;
+#pragma unroll 1
+    for (int jc = lo; jc < hi; ++jc) mine += stays(jc);
+    int running = block_exscan(mine, v.ctl.red, a.warps, total);
+    const int excess = total - (int)v.cap[n], o = (int)(rep >> 16);
+    int p_o = 0;                          // GPUs of the rows before the offset in job order
+    if (excess > 0) {
+      if (tid == 0) v.ctl.po = total;     // (no active job at or behind the offset)
+      bar(BAR_ROWS, threads);
+      int p = running;
+#pragma unroll 1
+      for (int jc = lo; jc < hi; ++jc) {
+        if ((int)v.act[jc] >= o && (jc == 0 || (int)v.act[jc - 1] < o)) v.ctl.po = p;
+        p += stays(jc);
+      }
+      bar(BAR_ROWS, threads);
+      p_o = v.ctl.po;
+    }
+#pragma unroll 1
+    for (int jc = lo; jc < hi; ++jc) {
+      const int g = row_at<KIND>(a, dst + jc, n), g_eff = stays(jc);
+      int take = 0;
+      if (excess > 0) {
+        const int ahead = (int)v.act[jc] >= o ? running - p_o : total - p_o + running;
+        take = min(g_eff, max(excess - ahead, 0));
+      }
+      running += g_eff;
+      v.mod[jc] = g_eff - take == g ? 0 : 1;
+      if (g_eff - take != g) {            // into the row
+        int k = 7;
+        if (!(v.info[jc] & INFO_WIDE)) {
+          const Record rec = load_record(rec_row(a, dst + jc));
+#pragma unroll
+          for (int z = 0; z < ENTRIES; ++z) k = entry_node(rec.w[z]) == n ? z : k;
+        }
+        set_entry<KIND>(a, v, dst, jc, k, n, g_eff - take);
+      }
+    }
+    bar(BAR_ROWS, threads);
+#pragma unroll 1
+    for (int i = warp * 4; i < JA; i += a.warps * 4) {
+      const int jc = min(i + (lane >> 3), JA - 1);
+      const bool live = i + (lane >> 3) < JA && v.mod[jc] && !(v.info[jc] & INFO_WIDE);
+      if (__any_sync(0xffffffffu, live)) finish_row<KIND>(a, v, dst, jc, live, warp, lane);
+    }
+    bar(BAR_ROWS, threads);
+#pragma unroll 1
+    for (int jc = warp; jc < JA; jc += a.warps)
+      if (v.mod[jc] && (v.info[jc] & INFO_WIDE)) finish_wide<KIND>(a, memory, dst, jc, warp, lane);
+    bar(BAR_ROWS, threads);
+  }
+}
 
 // An elite child: the records (and contents) of the candidate of its rank, as they are.
-__device__ __noinline__ void copy_candidate(const FlowArgs &a, const uint32_t *from, const int16_t *wide_from, uint32_t *to,
-                                            int16_t *wide_to, int rows) {
-  const int NS = wide_stride(a.NN);
+template <int KIND>
+__device__ __noinline__ void copy_candidate(const FlowArgs &a, int from, int to, int rows) {
 #pragma unroll 4
-  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-    const Record r = load_record(from + (size_t)i * REC_WORDS);
-    store_record(to + (size_t)i * REC_WORDS, r);
+  for (int i = threadIdx.x; i < rows; i += a.warps * 32) {
+    const Record r = load_record(rec_row(a, from + i));
+    store_record(rec_row(a, to + i), r);
     if (r.w[0] == WIDE) {
 #pragma unroll 1
-      for (int v = 0; v < NS / 8; ++v)
-        ((uint4 *)(wide_to + (size_t)i * NS))[v] = __ldcg((const uint4 *)(wide_from + (size_t)i * NS) + v);
+      for (int v = 0; v < wide_stride(a.NN) / 8; ++v)
+        ((uint4 *)wide_row(a, to + i))[v] = __ldcg((const uint4 *)wide_row(a, from + i) + v);
     }
   }
 }
 
-__global__ void __launch_bounds__(2 * MAX_ROW_THREADS + 32, 2) flow_kernel(const __grid_constant__ FlowArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int J = a.J, NN = a.NN, NS = wide_stride(NN), P = a.P;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5, T = a.row_threads;
-  const int draw_t = (int)blockDim.x > T + 32 ? tid - (T + 32) : tid < T ? tid : -1;    // place among the drawing threads
-  const FlowSmem L = flow_smem(P, J, NN, a.occ, nwarps, a.chunks);
-  uint16_t *s_act = (uint16_t *)(smem + L.act);
-  float *s_term = (float *)(smem + L.term);                   // by job, 0 where there is none
-  uint8_t *s_info = smem + L.info;                            // by row
-  int *s_tot = (int *)(smem + L.node);                        // GPUs placed on the node
-  uint32_t *s_cnt = (uint32_t *)(s_tot + NN);                 // distributed jobs on it | occupants << 16
-  uint32_t *s_occ = (uint32_t *)(smem + L.occ);               // row | GPUs << 13 | place in the record (7: wide) << 25 | distributed << 31
-  uint8_t *s_viol = smem + L.viol;                            // the node's column is to be walked
-  int16_t *s_cap = (int16_t *)(smem + L.cap);
-  uint16_t *s_mut2 = (uint16_t *)(smem + L.mut), *s_mod = (uint16_t *)(smem + L.mod);
-  uint16_t *s_wide = (uint16_t *)(smem + L.wide), *s_slow = (uint16_t *)(smem + L.slow);
-  uint4 *s_stash2 = (uint4 *)(smem + L.stash);
-  uint8_t *s_flag2 = smem + L.flag;                          // by row: 1 from the second parent, 2 perturbed
-  uint32_t *s_rec = J <= SMEM_RECORDS ? (uint32_t *)(smem + L.rec) : nullptr;
-  int16_t *s_dense = (int16_t *)(smem + L.dense) + (size_t)warp * NS;
-  uint32_t *s_rep2 = (uint32_t *)(smem + L.rep);
-  uint32_t *s_keys = (uint32_t *)(smem + L.keys);
-  double *s_sums = (double *)(smem + L.sums);
-  __shared__ int s_nmut2[2], s_nwide, s_nslow, s_nmod, s_walk, s_ok, s_po;
-  __shared__ uint32_t s_par[2], s_sel[2][4];
-  __shared__ int s_red[2 * MAX_ROW_THREADS / 32 + 1];
+// Two calls that differ in their slot, a round at a time: a twelfth of the code of draw_two for half again its instructions.
+// A small round's blocks have issue slots to spare and no room for code: what all its warps go through in a
+// generation should stay in the SM's instruction cache.
+__device__ __forceinline__ void draw_two_rolled(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot_a,
+                                                uint32_t slot_b, uint32_t &a_x, u32x4 &b) {
+  u32x4 x = {idx, cand, gen, slot_a}, y = {idx, cand, gen, slot_b};
+#pragma unroll 1
+  for (int r = 0; r < 10; ++r) {
+    x = philox_round(x, k0, k1);
+    y = philox_round(y, k0, k1);
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+  }
+  a_x = x.x;
+  b = y;
+}
+
+// The warps that draw: a candidate's random numbers of a step (each row's parent and whether it is perturbed, the
+// perturbed rows' list, the nodes' offsets).  Nothing in it waits for another block, so it is done while the
+// item before is worked on; the block's barrier hands it over.
+template <int KIND>
+__device__ __noinline__ void draw_items(const FlowArgs &a, uint32_t memory, uint32_t round, int JA) {
+  const FlowView v = flow_view(a, memory);
+  const int J = a.J, NN = a.NN, P = a.P, lane = threadIdx.x & 31;
+  const int D = (int)blockDim.x - a.warps * 32, d = (int)threadIdx.x - a.warps * 32;
+  int set = 0;
+  uint32_t c = blockIdx.x;
+#pragma unroll 1
+  for (int s = 0; s <= a.generations; set ^= 1) {
+    const bool init = s == 0;
+    const uint32_t gen = (uint32_t)(s - 1);                 // (GEN_INIT is -1)
+    const uint32_t c_next = c + gridDim.x < (uint32_t)P ? c + gridDim.x : blockIdx.x;
+    const int s_next = c_next > c ? s : s + 1;
+    // the candidates of the next item's tournaments: looked at before the barrier that hands that item over
+    if (d < 32 && s_next > 0) {
+      u32x4 sel;
+      uint32_t unused;
+      if (few(KIND)) draw_two_rolled(a.key.k0, round, 0u, c_next, (uint32_t)(s_next - 1), SLOT_SELECT, SLOT_SELECT, unused, sel);
+      else sel = draw_one(a.key.k0, round, 0u, c_next, (uint32_t)(s_next - 1), SLOT_SELECT);
+      if (lane < 4) v.ctl.sel[set ^ 1][lane] = bounded(lane == 0 ? sel.x : lane == 1 ? sel.y : lane == 2 ? sel.z : sel.w, (uint32_t)P);
+    }
+    if (init || (int)c >= a.num_elite) {
+#pragma unroll 1
+      for (int i = d; i < JA + NN; i += D) {
+        const bool row = i < JA;
+        const int jc = row ? i : 0;
+        const uint32_t idx = row ? v.act[jc] : (uint32_t)(i - JA);
+        u32x4 m;
+        uint32_t x = 0u;
+        const uint32_t slot_a = row ? SLOT_XOVER : SLOT_REPAIR_INTF, slot_b = !row ? SLOT_REPAIR_CAP : init ? SLOT_INIT : SLOT_MUTATE;
+        if (few(KIND)) draw_two_rolled(a.key.k0, round, idx, c, gen, slot_a, slot_b, x, m);
+        else draw_two(a.key.k0, round, idx, c, gen, slot_a, slot_b, x, m);
+        if (!row) {
+          v.rep[set * NN + (int)idx] = bounded(x, (uint32_t)J) | (bounded(m.x, (uint32_t)J) << 16);
+          continue;
+        }
+        const bool sec = !init && (x >> 31) != 0u, mut = init ? c > 0u && m.x < a.thr_init : m.x < a.thr_mutate;
+        v.flag[set * J + jc] = (sec ? 1 : 0) | (mut ? 2 : 0);
+        if (mut) {
+          const int at = atomicAdd(&v.ctl.nmut[set], 1);
+          if (!sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) continue;
+          v.mut[set * J + at] = (uint16_t)(jc | (sec ? 0x8000 : 0));
+          if (at < stash_rows(J))
+            v.stash[set * stash_rows(J) + at] = make_uint4(m.y, m.z, m.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[idx] : a.k_max, a.k_max)));
+        }
+      }
+    }
+    __syncthreads();
+    if (!v.ctl.hand[set].z) return;
+    c = c_next;
+    s = s_next;
+  }
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_kernel(const __grid_constant__ FlowArgs a) {
+  extern __shared__ __align__(16) unsigned char flow_memory[];
+  const uint32_t memory = (uint32_t)__cvta_generic_to_shared(flow_memory);
+  const FlowView v = flow_view(a, memory);
+  const int J = a.J, NN = a.NN, P = a.P;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = a.warps;
 
   const uint32_t round = __ldg(a.key.round_ptr), base = __ldg(a.r.base);
   const int JA = *a.r.num_act;
 #pragma unroll 1
-  for (int i = tid; i < JA; i += blockDim.x) s_act[i] = a.r.act[i];
+  for (int i = tid; i < JA; i += blockDim.x) v.act[i] = a.r.act[i];
 #pragma unroll 1
-  for (int i = tid; i < J; i += blockDim.x) s_term[i] = 0.f;
+  for (int i = tid; i < J; i += blockDim.x) v.term[i] = 0.f;
 #pragma unroll 1
-  for (int i = tid; i < a.chunks * 8; i += blockDim.x) s_sums[i] = 0.0;
-#pragma unroll 1
-  for (int i = tid; i < NN; i += blockDim.x) { s_cap[i] = (int16_t)max((int)a.cap[i], 0); s_tot[i] = 0; s_cnt[i] = 0u; s_viol[i] = 0; }
-  if (tid == 0) { s_nmut2[0] = s_nmut2[1] = 0; s_nwide = 0; s_nslow = 0; s_nmod = 0; s_walk = 0; s_ok = 1; }
+  for (int i = tid; i < NN; i += blockDim.x) {
+    v.cap[i] = (int16_t)max((int)a.cap[i], 0);
+    if (a.rack) v.rack[i] = a.rack[i];
+    v.node[2 * i] = v.node[2 * i + 1] = 0u;
+    v.viol[i] = 0;
+  }
+  if (tid == 0) {
+    FlowCtl &c = v.ctl;
+    c.nmut[0] = c.nmut[1] = c.nwide = c.nslow = c.nmod = c.walk = 0;
+    c.hand[0] = c.hand[1] = make_int4(0, 0, 1, 0);
+  }
   __syncthreads();
-  const bool rep_ahead = J <= SMEM_RECORDS;       // the nodes' repair numbers are drawn ahead, too
-  const size_t cand_rec = (size_t)J * REC_WORDS, cand_wide = (size_t)J * NS;
-  auto rec_of = [&](int step, uint32_t c) { return a.r.rec + ((size_t)(step & (DEPTH - 1)) * P + c) * cand_rec; };
-  auto wide_of = [&](int step, uint32_t c) { return a.r.wide + ((size_t)(step & (DEPTH - 1)) * P + c) * cand_wide; };
-  auto pub_of = [&](int step, uint32_t c) { return a.r.pub + (size_t)(step & (DEPTH - 1)) * P + c; };
+  if (few(KIND)) {
+#pragma unroll 1
+    for (int i = tid; i < JA * REC_WORDS; i += blockDim.x)
+      v.same[i] = __ldg(a.r.same + (size_t)v.act[i / REC_WORDS] * REC_WORDS + (i & (REC_WORDS - 1)));
+    if (a.at.terms >= 0) {
+      const int row = a.classes * (a.k_max + 1);
+#pragma unroll 1
+      for (int i = warp; i < JA; i += (int)(blockDim.x >> 5))
+#pragma unroll 4
+        for (int x = lane; x < row; x += 32) v.terms[i * row + x] = __ldg(a.r.terms + (size_t)v.act[i] * row + x);
+    }
+  }
+  if (warp >= W) {
+    draw_items<KIND>(a, memory, round, JA);
+    return;
+  }
 
-  // A candidate's random numbers of a step: each row's parent and whether it is perturbed, the perturbed
-  // rows' list.  Nothing in it waits for another block, so it is done a step ahead - by threads of their
-  // own where the GPU has room for them, else by the row threads while the perturbed rows are worked on.
-  // Two sets.
-  auto draw_step = [&](int s, uint32_t c, int set) {
-    const bool init = s == 0;
-    const uint32_t gen = (uint32_t)(s - 1);                 // (GEN_INIT is -1)
-    if (!init && (int)c < a.num_elite) return;
-    uint16_t *s_mut = s_mut2 + set * J;
-    uint8_t *s_flag = s_flag2 + set * J;
+  const int threads = W * 32, g = lane >> 3, nv = (min(J, SUM_THREADS) + 31) >> 5;
+  const bool last_warp = warp == W - 1;
+  const int PJ = P * J, cur_rows = (int)((a.r.cur_rec - a.r.rec) / REC_WORDS);
+  auto pub_of = [&](int step, uint32_t cand) { return a.r.pub + (size_t)(step & (DEPTH - 1)) * P + cand; };
+  // Items: this block's candidates of step 0 (the initial population), of step 1 (generation 0), ...
+  int s = 0, set = 0;
+  Work w;
+  w.c = blockIdx.x;
 #pragma unroll 1
-    for (int jc = draw_t; jc < JA; jc += T) {
-      const uint32_t j = s_act[jc];
-      u32x4 m;
-      uint32_t x = 0u;
-      draw_two(a.key.k0, round, j, c, gen, SLOT_XOVER, init ? SLOT_INIT : SLOT_MUTATE, x, m);
-      const bool sec = !init && (x >> 31) != 0u, mut = init ? c > 0u && m.x < a.thr_init : m.x < a.thr_mutate;
-      s_flag[jc] = (sec ? 1 : 0) | (mut ? 2 : 0);
-      if (mut) {
-        const int i = atomicAdd(&s_nmut2[set], 1);
-        if (!sched_index_ok(a.status, i < J, SCHED_CHK_LIST)) continue;
-        s_mut[i] = (uint16_t)(jc | (sec ? 0x8000 : 0));
-        if (i < STASH) s_stash2[set * STASH + i] = make_uint4(m.y, m.z, m.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)));
-      }
-    }
-    if (rep_ahead) {
-#pragma unroll 1
-      for (int n = T - 1 - draw_t; n < NN; n += T) {
-        uint32_t x;
-        u32x4 y;
-        draw_two(a.key.k0, round, (uint32_t)n, c, gen, SLOT_REPAIR_INTF, SLOT_REPAIR_CAP, x, y);
-        s_rep2[set * NN + n] = bounded(x, (uint32_t)J) | (bounded(y.x, (uint32_t)J) << 16);
-      }
-    }
-    if (draw_t < 32 && !init) {
-      const u32x4 sel = draw_one(a.key.k0, round, 0u, c, gen, SLOT_SELECT);
-      if (lane < 4) s_sel[set][lane] = bounded(lane == 0 ? sel.x : lane == 1 ? sel.y : lane == 2 ? sel.z : sel.w, (uint32_t)P);
-    }
-  };
-  // Items: this block's candidates of step 0 (the initial population), of step 1 (generation 0), ...; the
-  // item before the first only draws.
-  int s_at = 0, item = -1;
-  uint32_t c_at = blockIdx.x;
-#pragma unroll 1
-  while (s_at <= a.generations) {
-      int s = s_at;
-      uint32_t c = c_at;
-      asm volatile("" : "+r"(s));               // (one copy of the code for all steps)
-      if (item >= 0) {
-        c_at += gridDim.x;
-        if (c_at >= (uint32_t)P) { c_at = blockIdx.x; ++s_at; }
-      }
-      Work w;
-      w.c = c; w.init = s == 0; w.gen = w.init ? GEN_INIT : (uint32_t)(s - 1); w.round = round;
-      w.rec = rec_of(s, c); w.wide = wide_of(s, c);
-      const bool elite = item >= 0 && !w.init && (int)c < a.num_elite;
+  while (s <= a.generations) {
+    const uint32_t c = w.c;
+    const bool init = s == 0, elite = !init && (int)c < a.num_elite;
+    w.init = init;
+    w.gen = (uint32_t)(s - 1);
+    w.dst = (s & (DEPTH - 1)) * PJ + (int)c * J;
 
-      const int set = item & 1;
-      uint16_t *const s_mut = s_mut2 + set * J;
-      const uint8_t *const s_flag = s_flag2 + set * J;
-      uint4 *const s_stash = s_stash2 + set * STASH;
-      uint32_t *const s_rep = s_rep2 + set * NN;
-      // ---- parents ----------------------------------------------------------------------------------
-      // The candidate of its rank for an elite child (which needs every key), else the better-ranked of
-      // two random pairs (which needs four).  Candidate 0 waits for every key in any case: that it has
-      // published step t tells everybody that nobody reads step t - 2 any more.
-      if (item >= 0 && !w.init) {
-        if (elite || c == 0u) {
-          bool ok = true;
+    // ---- parents ----------------------------------------------------------------------------------
+    // The candidate of its rank for an elite child (which needs every key), else the better-ranked of
+    // two random pairs (which needs four).  Candidate 0 waits for every key in any case: that it has
+    // published step t tells everybody that nobody reads step t - 2 any more.
+    if (!init && (elite || c == 0u)) {
+      bool ok = true;
 #pragma unroll 1
-          for (int i = tid; i < P && ok; i += blockDim.x) {
-            uint32_t k;
-            ok = wait_tag(pub_of(s - 1, i), base + (uint32_t)(s - 1), k, a.wait_limit, a.status);
-            s_keys[i] = k;
-          }
-          waited();
-          if (!ok) s_ok = 0;
-          __syncthreads();
-          if (elite && warp == 0 && s_ok) {
-            const int i = candidate_of_rank(s_keys, P, (int)c, (uint16_t *)(s_keys + P), lane);
-            if (lane == 0) s_par[0] = s_par[1] = (uint32_t)i;
-          }
-        }
-        if (warp == T / 32) {
-          uint32_t k = 0u;
-          bool ok = true;
-          const uint32_t mine = s_sel[set][lane & 3];
-          if (lane < 4 && !elite) ok = wait_tag(pub_of(s - 1, mine), base + (uint32_t)(s - 1), k, a.wait_limit, a.status);
-          if (lane == 4 && s >= DEPTH) ok = wait_tag(pub_of(s - 2, 0u), base + (uint32_t)(s - 2), k, a.wait_limit, a.status);
-          waited();
-          if (!__all_sync(0xffffffffu, ok) && lane == 0) s_ok = 0;
-          const uint32_t other = __shfl_down_sync(0xffffffffu, mine, 1), ko = __shfl_down_sync(0xffffffffu, k, 1);
-          if (!elite && (lane == 0 || lane == 2)) s_par[lane >> 1] = (uint32_t)tournament_winner(k, (int)mine, ko, (int)other);
-        }
+      for (int i = tid; i < P && ok; i += threads) {
+        const unsigned long long word = wait_tag(pub_of(s - 1, i), base + (uint32_t)(s - 1), a.wait_limit, a.status);
+        ok = word != 0ull;
+        v.keys[i] = (uint32_t)word;
       }
-      __syncthreads();
-      if (!s_ok) return;                        // (a wait ran out: the status says so)
-      if (!sched_index_ok(a.status, w.init || (s_par[0] < (uint32_t)P && s_par[1] < (uint32_t)P), SCHED_CHK_SLOT)) return;
-      const uint32_t elite_key = elite ? s_keys[s_par[0]] : 0u;
+      waited();
+      if (!ok) v.ctl.hand[set].z = 0;
+      bar(BAR_ROWS, threads);
+    }
+    if (last_warp) {
       // (initial population: an unperturbed row is the current allocation's after the row caps, a perturbed one
       // starts from it before them; rows of the current allocation lie by job)
-      w.src_a = w.init ? a.r.cur_rec : rec_of(s - 1, s_par[0]);
-      w.wide_a = w.init ? a.r.cur_wide : wide_of(s - 1, s_par[0]);
-      w.src_b = w.init ? a.r.cur_rec + cand_rec : rec_of(s - 1, s_par[1]);
-      w.wide_b = w.init ? a.r.cur_wide + cand_wide : wide_of(s - 1, s_par[1]);
-
-      // a row's occupants into the nodes' totals and lists
-      auto add_occupant = [&](int jc, int k_rec, uint32_t e, uint32_t dist) {
-        const int n = entry_node(e);
-        if (!sched_index_ok(a.status, n < NN && jc < JA && entry_gpus(e) <= 2047, SCHED_CHK_NODE)) return;
-        atomicAdd(&s_tot[n], entry_gpus(e));
-        const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
-        if (k < (uint32_t)a.occ) s_occ[n * a.occ + k] = (uint32_t)jc | ((uint32_t)entry_gpus(e) << 13) | ((uint32_t)k_rec << 25) | dist;
-      };
-      // small problems find a row of their own child again in shared memory
-      auto keep_record = [&](int jc, const Record &r) {
-        if (!s_rec) return;
-        ((uint4 *)(s_rec + jc * REC_WORDS))[0] = make_uint4(r.w[0], r.w[1], r.w[2], r.w[3]);
-        ((uint4 *)(s_rec + jc * REC_WORDS))[1] = make_uint4(r.w[4], r.w[5], r.w[6], r.w[7]);
-      };
-      auto own_record = [&](int jc) {
-        if (!s_rec) return load_record(w.rec + (size_t)jc * REC_WORDS);
-        const uint4 x = ((const uint4 *)(s_rec + jc * REC_WORDS))[0], y = ((const uint4 *)(s_rec + jc * REC_WORDS))[1];
-        return Record{{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w}};
-      };
-      const int nmut = item >= 0 ? s_nmut2[set] : 0;
-      if (elite) {
-        copy_candidate(a, w.src_a, w.wide_a, w.rec, w.wide, JA);
-      } else if (tid < T && item >= 0) {
-        // ---- unperturbed rows, a thread each; four at a time, so that their loads travel together ------
-        constexpr int RB = 4;
-#pragma unroll 1
-        for (int jc0 = tid; jc0 < JA; jc0 += RB * T) {
-          Record rec[RB];
-          uint32_t flag[RB];
-#pragma unroll
-          for (int q = 0; q < RB; ++q) {
-            const int jc = min(jc0 + q * T, JA - 1);
-            flag[q] = jc0 + q * T < JA ? s_flag[jc] : 2u;
-            const uint32_t *src = (flag[q] & 1u) ? w.src_b : w.src_a;
-            rec[q] = load_record(src + (size_t)(w.init ? (int)s_act[jc] : jc) * REC_WORDS);
-          }
-#pragma unroll
-          for (int q = 0; q < RB; ++q) {
-            const int jc = jc0 + q * T;
-            if (flag[q] & 2u) continue;
-            store_record(w.rec + (size_t)jc * REC_WORDS, rec[q]);
-            keep_record(jc, rec[q]);
-            s_term[s_act[jc]] = __uint_as_float(rec[q].w[REC_TERM]);
-            if (rec[q].w[0] == WIDE) {
-              s_info[jc] = INFO_DIST | INFO_WIDE;
-              const int at = atomicAdd(&s_nwide, 1);
-              if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_wide[at] = (uint16_t)(jc | ((flag[q] & 1u) ? 0x8000 : 0));
-              continue;
-            }
-            const uint32_t dist = rec[q].w[1] != NO_NODE ? 0x80000000u : 0u;
-            s_info[jc] = dist ? INFO_DIST : 0;
-            if (rec[q].w[0] != NO_NODE) add_occupant(jc, 0, rec[q].w[0], dist);
-#pragma unroll 1
-            for (int k = 1; k < ENTRIES; ++k) {           // (few rows have more: one copy of the code)
-              uint32_t e = rec[q].w[1];
-#pragma unroll
-              for (int z = 2; z < ENTRIES; ++z) e = z == k ? rec[q].w[z] : e;
-              if (e == NO_NODE) break;
-              add_occupant(jc, k, e, dist);
-            }
-          }
-        }
+      const int before = init ? cur_rows : ((s - 1) & (DEPTH - 1)) * PJ;
+      int parent = init ? lane >> 1 : 0;
+      if (!init) {
+        unsigned long long word = 1ull;
+        const uint32_t mine = v.ctl.sel[set][lane & 3], other = __shfl_down_sync(0xffffffffu, mine, 1);
+        const unsigned long long *const watched = lane == 4 ? pub_of(s - 2, 0u) : pub_of(s - 1, mine);
+        const uint32_t tag = base + (uint32_t)(lane == 4 ? s - 2 : s - 1);
+        if (lane == 4 ? s >= DEPTH : lane < 4 && !elite) word = wait_tag(watched, tag, a.wait_limit, a.status);
+        waited();
+        const uint32_t key = (uint32_t)word, ko = __shfl_down_sync(0xffffffffu, key, 1);
+        parent = tournament_winner(key, (int)mine, ko, (int)other);
+        if (word == 0ull) v.ctl.hand[set].z = 0;
+        if (elite) parent = v.ctl.hand[set].z ? candidate_of_rank(v.keys, P, (int)c, (uint16_t *)(v.keys + P), lane) : 0;
+        if (!sched_index_ok(a.status, parent >= 0 && parent < P, SCHED_CHK_SLOT)) parent = 0;
       }
-      if (draw_t >= 0) {
-        if (s_at <= a.generations) draw_step(s_at, c_at, set ^ 1);
-      } else if (tid >= T && !elite) {
-        // ---- perturbed rows: the last warp, a lane each --------------------------------------------------
-#pragma unroll 1
-        for (int i = lane; i < nmut; i += 32) {
-          const int jc = s_mut[i] & 0x7FFF;
-          if (!sched_index_ok(a.status, i < J && jc < JA, SCHED_CHK_LIST)) continue;
-          const int j = s_act[jc];
-          const uint32_t *src = (w.init || (s_mut[i] >> 15)) ? w.src_b : w.src_a;
-          const Record rec = load_record(src + (size_t)(w.init ? j : jc) * REC_WORDS);
-          uint4 st;
-          if (i < STASH) {
-            st = s_stash[i];
-          } else {
-            const u32x4 m = draw_one(a.key.k0, round, (uint32_t)j, c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE);
-            st = make_uint4(m.y, m.z, m.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)));
-          }
-          bool slow = rec.w[0] == WIDE;
-          if (!slow) {
-            uint32_t e[LIST];
-#pragma unroll
-            for (int k = 0; k < ENTRIES; ++k) e[k] = rec.w[k];
-            e[ENTRIES] = NO_NODE;
-            int K, N;
-            list_totals(e, K, N);
-            list_perturb(e, N, st.x, st.y, st.z, NN, s_cap);
-            list_totals(e, K, N);
-            if (K > (int)st.w || N > a.n_max) {
-              list_caps(e, K, (int)st.w, a.n_max);
-              list_totals(e, K, N);
-            }
-            slow = e[ENTRIES] != NO_NODE;
-            if (!slow) {
-              const uint32_t dist = N >= 2 ? 0x80000000u : 0u;
-              const TermLoads loads = list_loads(a, e, j, K, N);     // (on their way while the nodes are added up)
-              s_info[jc] = dist ? INFO_DIST : 0;
-#pragma unroll 1
-              for (int k = 0; k < N; ++k) {
-                uint32_t x = e[0];
-#pragma unroll
-                for (int z = 1; z < ENTRIES; ++z) x = z == k ? e[z] : x;
-                add_occupant(jc, k, x, dist);
-              }
-              const Record out = list_record(a, e, loads);
-              store_record(w.rec + (size_t)jc * REC_WORDS, out);
-              keep_record(jc, out);
-              s_term[j] = __uint_as_float(out.w[REC_TERM]);
-            }
-          }
-          if (slow) {
-            const int at = atomicAdd(&s_nslow, 1);
-            if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_slow[at] = s_mut[i];
-          }
-        }
-      }
-      __syncthreads();
-      if (elite || item < 0) {
-        if (elite && tid == 0) {
-          publish(pub_of(s, c), base + (uint32_t)s, elite_key);
-          if (s == a.generations) a.fitness[c] = __uint_as_float(elite_key ^ ((elite_key >> 31) ? 0x80000000u : 0xFFFFFFFFu));
-        }
-        ++item;
-        continue;
-      }
-
-      // ---- wide rows, a warp each -------------------------------------------------------------------
-      if (s_nwide | s_nslow) {
-#pragma unroll 1
-        for (int i = warp; i < s_nwide + s_nslow; i += nwarps) {
-          const bool slow = i >= s_nwide;
-          const int x = slow ? s_slow[i - s_nwide] : s_wide[i], jc = x & 0x7FFF;
-          if (!sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST)) continue;
-          const int j = s_act[jc];
-          const bool sec = (x >> 15) || (w.init && slow);
-          const int at = w.init ? j : jc;
-          const Record rec = load_record((sec ? w.src_b : w.src_a) + (size_t)at * REC_WORDS);
-          if (rec.w[0] == WIDE) {
-            const int16_t *from = (sec ? w.wide_b : w.wide_a) + (size_t)at * NS;
-#pragma unroll 1
-            for (int n = lane; n < NS; n += 32) {
-              const int16_t v = __ldcg(from + n);
-              s_dense[n] = v;
-              if (!slow) w.wide[(size_t)jc * NS + n] = v;
-            }
-            __syncwarp();
-          } else {
-            dense_from_list(s_dense, NS, rec, lane, a.status);
-          }
-          if (slow) {
-            int K, N;
-            dense_totals(s_dense, NN, lane, K, N);
-            const u32x4 m = draw_one(a.key.k0, round, (uint32_t)j, c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE);
-            const uint32_t op = bounded(m.y, 3u);
-            const int nd = (int)bounded(m.w, (uint32_t)NN);
-            if (op == 0u) {
-              if (lane == 0) s_dense[nd] = (int16_t)min((int)s_dense[nd] + 1, (int)s_cap[nd]);
-            } else if (N > 0) {
-              int ns = nth_occupied(s_dense, NN, bounded(m.z, (uint32_t)N), lane);
-              if (!sched_index_ok(a.status, ns >= 0 && ns < NN && nd < NN, SCHED_CHK_NODE)) ns = nd;
-              if (lane == 0 && op == 1u) s_dense[ns] = (int16_t)(s_dense[ns] - 1);
-              if (lane == 0 && op == 2u && nd != ns) {
-                s_dense[nd] = (int16_t)min((int)s_dense[nd] + (int)s_dense[ns], (int)s_cap[nd]);
-                s_dense[ns] = 0;
-              }
-            }
-            __syncwarp();
-            dense_totals(s_dense, NN, lane, K, N);
-            dense_caps(s_dense, NN, K, N, max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)), a.n_max, lane);
-            const Record out = dense_record(a, s_dense, j, K, N, w.wide + (size_t)jc * NS, lane);
-            if (lane == 0) {
-              store_record(w.rec + (size_t)jc * REC_WORDS, out);
-              keep_record(jc, out);
-              s_term[j] = __uint_as_float(out.w[REC_TERM]);
-              s_info[jc] = (N >= 2 ? INFO_DIST : 0) | (N > ENTRIES ? INFO_WIDE : 0);
-            }
-            __syncwarp();
-          }
-          const uint32_t dist = (s_info[jc] & INFO_DIST) ? 0x80000000u : 0u;
-          const bool wide = (s_info[jc] & INFO_WIDE) != 0;
-          int before = 0;
-#pragma unroll 1
-          for (int n0 = 0; n0 < NN; n0 += 32) {
-            const int n = n0 + lane, v = n < NN ? (int)s_dense[n] : 0;
-            const unsigned m = __ballot_sync(0xffffffffu, v > 0);
-            const int k = before + __popc(m & ((1u << lane) - 1u));
-            if (v > 0) add_occupant(jc, wide ? 7 : k, ((uint32_t)n << 16) | (uint32_t)v, dist);
-            before += __popc(m);
-          }
-          __syncwarp();
-        }
-        __syncthreads();
-      }
-
-      // A decision goes straight into the row: entry k of its record (0 GPUs: taken out when the row is
-      // finished), or its contents.  Decisions of different nodes touch different words.
-      auto set_entry = [&](int jc, int k, int n, int v) {
-        if (!sched_index_ok(a.status, jc < JA && n < NN && (k == 7 || k < ENTRIES), SCHED_CHK_ENTRY)) return;
-        if (k == 7) w.wide[(size_t)jc * NS + n] = (int16_t)v;
-        else if (s_rec) s_rec[jc * REC_WORDS + k] = ((uint32_t)n << 16) | (uint32_t)v;
-        else w.rec[(size_t)jc * REC_WORDS + k] = ((uint32_t)n << 16) | (uint32_t)v;
-      };
-
-      // ---- node decisions: a lane looks at a node, groups of 16 lanes decide the nodes that hold two
-      // distributed jobs or more GPUs than they have; nodes are dealt out round robin, so that violations
-      // spread over the warps ---------------------------------------------------------------------------
-#pragma unroll 1
-      for (int n0 = warp; n0 < NN; n0 += 32 * nwarps) {
-        const int n_l = n0 + lane * nwarps;
-        bool bad = false;
-        if (n_l < NN) bad = (s_cnt[n_l] & 0xFFFFu) >= 2u || s_tot[n_l] > (int)s_cap[n_l];
-        unsigned todo = __ballot_sync(0xffffffffu, bad);
-        if (todo == 0u) continue;
-        uint32_t rep_l = 0u;                    // the two rotation offsets, below 8192 each
-        if (bad) {
-          if (rep_ahead) {
-            rep_l = s_rep[n_l];
-          } else {
-            uint32_t x;
-            u32x4 y;
-            draw_two(a.key.k0, round, (uint32_t)n_l, c, w.gen, SLOT_REPAIR_INTF, SLOT_REPAIR_CAP, x, y);
-            rep_l = bounded(x, (uint32_t)J) | (bounded(y.x, (uint32_t)J) << 16);
-            s_rep[n_l] = rep_l;                 // (a walked column wants it again)
-          }
-        }
-        __syncwarp();
-#pragma unroll 1
-        while (todo) {
-          const int b0 = __ffs(todo) - 1;
-          todo &= todo - 1;
-          int b1 = -1;
-          if (todo) { b1 = __ffs(todo) - 1; todo &= todo - 1; }
-          const int b = (lane & 16) ? b1 : b0, sub = lane & 15;
-          const uint32_t rep = __shfl_sync(0xffffffffu, rep_l, max(b, 0));
-          const int n = n0 + max(b, 0) * nwarps, count = b >= 0 ? (int)(s_cnt[n] >> 16) : 0;
-          const bool listed = count <= a.occ, have = listed && sub < count;   // else: walked below
-          const uint32_t e = have ? s_occ[n * a.occ + sub] : 0u;
-          const int jc = (int)(e & 0x1FFFu);
-          const int j = have && sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) ? (int)s_act[jc] : 0;
-          int ri = j - (int)(rep & 0xFFFFu), rc = have ? j - (int)(rep >> 16) : 0x3fffffff;
-          if (ri < 0) ri += J;
-          if (rc < 0) rc += J;
-          const int most = max(__shfl_sync(0xffffffffu, count, 0), __shfl_sync(0xffffffffu, count, 16));
-          const int v = decide(have ? (int)((e >> 13) & 0x7FFu) : 0, (e >> 31) != 0u, have, min(most, a.occ), (s_cnt[n] & 0xFFFFu) >= 2u, s_tot[n], (int)s_cap[n], ri, rc);
-          const bool changed = have && v != (int)((e >> 13) & 0x7FFu);
-          if (changed) {
-            set_entry(jc, (int)((e >> 25) & 7u), n, v);
-            // (bytes, so the word around it is updated as a whole)
-            const uint32_t bit = (uint32_t)INFO_CHANGED << (8 * (jc & 3));
-            if (sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) && (atomicOr((uint32_t *)s_info + (jc >> 2), bit) & bit) == 0u) {
-              const int at = atomicAdd(&s_nmod, 1);
-              if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) s_mod[at] = (uint16_t)jc;
-            }
-          }
-          if (b >= 0 && sub == 0 && !listed) { s_viol[n] = 1; s_walk = 1; }
-          __syncwarp();
-        }
-      }
-      __syncthreads();
-
-      // ---- rows the decisions change ------------------------------------------------------------------
-      // a row without the entries that were taken out, and its new term; by one thread (records), one warp (wide)
-      auto finish_row = [&](int jc) {
-        const int j = s_act[jc];
-        const Record rec = own_record(jc);
-        uint32_t e[LIST];
-        int holes = 0;
-#pragma unroll
-        for (int k = 0; k < ENTRIES; ++k) {
-          const bool out = entry_gpus(rec.w[k]) == 0;       // (an unused entry is not: its low half is all ones)
-          e[k] = out ? NO_NODE : rec.w[k];
-          holes += out ? 1 : 0;
-        }
-        e[ENTRIES] = NO_NODE;
-#pragma unroll 1
-        for (int h = 0; h < holes; ++h) {
-#pragma unroll
-          for (int k = 0; k + 1 < ENTRIES; ++k) {           // the last hole to the end
-            const uint32_t lo = min(e[k], e[k + 1]);
-            e[k + 1] = max(e[k], e[k + 1]);
-            e[k] = lo;
-          }
-        }
-        int K, N;
-        list_totals(e, K, N);
-        const Record out = list_record(a, e, list_loads(a, e, j, K, N));
-        store_record(w.rec + (size_t)jc * REC_WORDS, out);
-        keep_record(jc, out);
-        s_term[j] = __uint_as_float(out.w[REC_TERM]);
-      };
-      auto finish_wide = [&](int jc) {
-        int16_t *row = w.wide + (size_t)jc * NS;
-#pragma unroll 1
-        for (int n = lane; n < NN; n += 32) s_dense[n] = __ldcg(row + n);
-        __syncwarp();
-        int K, N;
-        dense_totals(s_dense, NN, lane, K, N);
-        const Record out = dense_record(a, s_dense, s_act[jc], K, N, row, lane);
-        if (lane == 0) {
-          store_record(w.rec + (size_t)jc * REC_WORDS, out);
-          keep_record(jc, out);
-          s_term[s_act[jc]] = __uint_as_float(out.w[REC_TERM]);
-          if (N <= ENTRIES) s_info[jc] &= ~INFO_WIDE;
-        }
-        __syncwarp();
-      };
-      const int nmod = s_nmod;
-#pragma unroll 1
-      for (int i = tid; i < nmod; i += blockDim.x) {
-        const int jc = s_mod[i];
-        if (!(s_info[jc] & INFO_WIDE)) finish_row(jc);
-      }
-      if (s_nwide | s_nslow) {                  // wide rows among them
-        __syncthreads();                        // (one may turn into a record here: not to be taken for one above)
-#pragma unroll 1
-        for (int i = warp; i < nmod; i += nwarps) {
-          const int jc = s_mod[i];
-          if (s_info[jc] & INFO_WIDE) finish_wide(jc);
-        }
-      }
-
-      // ---- nodes with more occupants than a list holds: the block walks the column, node by node ------
-      // Thread t looks after the consecutive rows [t * rpt, (t + 1) * rpt).  Interference: the first
-      // distributed occupant in rotated job order stays.  Capacity: a block-wide prefix sum in job order gives
-      // every row the GPUs that come before it in rotated order.
-      if (s_walk) {
-        __syncthreads();
-        const int rpt = (JA + (int)blockDim.x - 1) / (int)blockDim.x;
-        const int lo = min(JA, tid * rpt), hi = min(JA, lo + rpt);
-#pragma unroll 1
-        for (int n = 0; n < NN; ++n) {
-          if (!s_viol[n]) continue;
-          const uint32_t rep = s_rep[n];
-          const bool intf = (s_cnt[n] & 0xFFFFu) >= 2u;
-          auto dist = [&](int jc) { return (s_info[jc] & INFO_DIST) != 0; };
-          int keep = -1;
-          if (intf) {
-            int best = 0x7fffffff;
-#pragma unroll 1
-            for (int jc = lo; jc < hi; ++jc)
-              if (dist(jc) && row_at(w.rec, w.wide, NS, jc, n) > 0) {
-                int t = (int)s_act[jc] - (int)(rep & 0xFFFFu);
-                if (t < 0) t += J;
-                best = min(best, t);
-              }
-            keep = (int)(rep & 0xFFFFu) + block_min(best, s_red, nwarps);     // the job that stays
-            if (keep >= J) keep -= J;
-          }
-          auto stays = [&](int jc) {
-            const int v = row_at(w.rec, w.wide, NS, jc, n);
-            return intf && dist(jc) && v > 0 && (int)s_act[jc] != keep ? 0 : v;
-          };
-          int mine = 0, total;
-#pragma unroll 1
-          for (int jc = lo; jc < hi; ++jc) mine += stays(jc);
-          int running = block_exscan(mine, s_red, nwarps, total);
-          const int excess = total - (int)s_cap[n], o = (int)(rep >> 16);
-          int p_o = 0;                          // GPUs of the rows before the offset in job order
-          if (excess > 0) {
-            if (tid == 0) s_po = total;         // (no active job at or behind the offset)
-            __syncthreads();
-            int p = running;
-#pragma unroll 1
-            for (int jc = lo; jc < hi; ++jc) {
-              if ((int)s_act[jc] >= o && (jc == 0 || (int)s_act[jc - 1] < o)) s_po = p;
-              p += stays(jc);
-            }
-            __syncthreads();
-            p_o = s_po;
-          }
-#pragma unroll 1
-          for (int jc = lo; jc < hi; ++jc) {
-            const int v = row_at(w.rec, w.wide, NS, jc, n), v_eff = stays(jc);
-            int take = 0;
-            if (excess > 0) {
-              const int ahead = (int)s_act[jc] >= o ? running - p_o : total - p_o + running;
-              take = min(v_eff, max(excess - ahead, 0));
-            }
-            running += v_eff;
-            s_mod[jc] = v_eff - take == v ? 0 : 1;
-            if (v_eff - take != v) {            // into the row
-              int k = 7;
-              if (!(s_info[jc] & INFO_WIDE)) {
-                const Record rec = own_record(jc);
-#pragma unroll
-                for (int z = 0; z < ENTRIES; ++z) k = entry_node(rec.w[z]) == n ? z : k;
-              }
-              set_entry(jc, k, n, v_eff - take);
-            }
-          }
-          __syncthreads();
-#pragma unroll 1
-          for (int jc = tid; jc < JA; jc += blockDim.x)
-            if (s_mod[jc] && !(s_info[jc] & INFO_WIDE)) finish_row(jc);
-          __syncthreads();
-#pragma unroll 1
-          for (int jc = warp; jc < JA; jc += nwarps)
-            if (s_mod[jc] && (s_info[jc] & INFO_WIDE)) finish_wide(jc);
-          __syncthreads();
-        }
-      }
-      __syncthreads();
-
-      // ---- fitness (Eq. 14) from the rows' terms, in the order of the dense kernel: per chunk of rows, thread
-      // t adds rows t, t + 256, ... in double, a shuffle tree per warp, the warps in index order; then the
-      // chunks in index order.  Published once all of the candidate's rows are written. ------------------
-      if (tid < T) {
-#pragma unroll 1
-        for (int ch = 0; ch < a.chunks; ++ch) {
-          const int j0 = ch * a.rows_per_chunk, j1 = min(J, j0 + a.rows_per_chunk);
-          double acc = 0.0;
-#pragma unroll 1
-          for (int j = j0 + tid; j < j1; j += MAX_ROW_THREADS) acc += (double)s_term[j];
-#pragma unroll
-          for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-          if (lane == 0) s_sums[ch * 8 + warp] = acc;
-        }
-      } else if (warp == T / 32) {
-        // everybody's rows are written: made visible to the other blocks while the sums are formed
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-      }
-#pragma unroll 1
-      for (int i = tid; i < NN; i += blockDim.x) { s_tot[i] = 0; s_cnt[i] = 0u; s_viol[i] = 0; }
-      if (tid == 0) { s_nmut2[set] = 0; s_nwide = 0; s_nslow = 0; s_nmod = 0; s_walk = 0; }
-      __syncthreads();
-      if (tid == T) {
-        double sum = 0.0;
-#pragma unroll 1
-        for (int ch = 0; ch < a.chunks; ++ch) {
-          double v[8], t = 0.0;
-#pragma unroll
-          for (int x = 0; x < 8; ++x) v[x] = s_sums[ch * 8 + x];
-#pragma unroll
-          for (int x = 0; x < 8; ++x) t += v[x];            // (warps that do not exist left zeros)
-          sum += t;
-        }
-        const float f = fitness_finalise(a.tp.mode, a.tp.p, sum, (double)JA);
-        const unsigned long long word = ((unsigned long long)(base + (uint32_t)s) << 32) | order_key(__float_as_uint(f));
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(pub_of(s, c)), "l"(word) : "memory");   // (behind this thread's fence)
-        if (s == a.generations) a.fitness[c] = f;
-      }
-      ++item;
+      if (lane == 0) v.ctl.hand[set].x = before + parent * J;
+      if (lane == 2) v.ctl.hand[set].y = before + parent * J;
+      if (elite && lane == 0) v.ctl.hand[set].w = parent;
     }
+    __syncthreads();
+    const int4 hand = v.ctl.hand[set];
+    if (!hand.z) return;                      // (a wait ran out: the status says so)
+    w.src[0] = hand.x;
+    w.src[1] = hand.y;
+
+    auto next_item = [&]() {
+      set ^= 1;
+      w.c += gridDim.x;
+      if (w.c >= (uint32_t)P) { w.c = blockIdx.x; ++s; }
+    };
+    if (elite) {
+      const uint32_t key = v.keys[hand.w];
+      copy_candidate<KIND>(a, w.src[0], w.dst, JA);
+      bar(BAR_ROWS, threads);
+      if (tid == 0) {
+        publish(pub_of(s, c), base + (uint32_t)s, key);
+        if (s == a.generations) a.fitness[c] = __uint_as_float(key ^ ((key >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+      }
+      next_item();
+      continue;
+    }
+
+    // ---- the rows: perturbed ones (from the last warp on) and the others --------------------------------
+    const uint8_t *const flag = v.flag + set * J;
+    auto note_wide = [&](int jc, uint32_t f) {
+      const int at = atomicAdd(&v.ctl.nwide, 1);
+      if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) v.wide[at] = (uint16_t)(jc | ((f & 1u) ? 0x8000 : 0));
+      v.info[jc] = INFO_DIST | INFO_WIDE;
+    };
+    const int nmut = v.ctl.nmut[set];
+#pragma unroll 1
+    for (int x = (W - 1 - warp) * 4; x < nmut; x += W * 4) perturb_rows<KIND>(a, v, w, round, set, x, nmut, warp, lane);
+    constexpr int RB = KIND == SOME_ALONE || KIND == MANY ? 2 : 1;       // rows of a thread whose loads travel together
+#pragma unroll 1
+    for (int jc0 = tid; jc0 < JA; jc0 += RB * threads) {
+      Record rec[RB];
+      uint32_t f[RB];
+#pragma unroll
+      for (int q = 0; q < RB; ++q) {
+        const int jc = min(jc0 + q * threads, JA - 1);
+        f[q] = jc0 + q * threads < JA ? (uint32_t)flag[jc] : 2u;
+        rec[q] = load_record(rec_row(a, ((f[q] & 1u) ? w.src[1] : w.src[0]) + (init ? (int)v.act[jc] : jc)));
+      }
+#pragma unroll
+      for (int q = 0; q < RB; ++q) {
+        const int jc = jc0 + q * threads;
+        if (f[q] & 2u) continue;
+        store_record(rec_row(a, w.dst + jc), rec[q]);
+        if (few(KIND)) {
+          ((uint4 *)v.rec)[2 * jc] = make_uint4(rec[q].w[0], rec[q].w[1], rec[q].w[2], rec[q].w[3]);
+          ((uint4 *)v.rec)[2 * jc + 1] = make_uint4(rec[q].w[4], rec[q].w[5], rec[q].w[6], rec[q].w[7]);
+        }
+        v.term[v.act[jc]] = __uint_as_float(rec[q].w[REC_TERM]);
+        if (rec[q].w[0] == WIDE) {
+          note_wide(jc, f[q]);
+          continue;
+        }
+        const bool dist = rec[q].w[1] != NO_NODE;
+        v.info[jc] = dist ? INFO_DIST : 0;
+        if (rec[q].w[0] != NO_NODE) add_occupant(a, v, jc, 0, rec[q].w[0], dist);
+#pragma unroll 1
+        for (int x = 1; x < ENTRIES; ++x) {           // (few rows have more: one copy of the code)
+          uint32_t e = rec[q].w[1];
+#pragma unroll
+          for (int z = 2; z < ENTRIES; ++z) e = z == x ? rec[q].w[z] : e;
+          if (e == NO_NODE) break;
+          add_occupant(a, v, jc, x, e, dist);
+        }
+      }
+    }
+    bar(BAR_ROWS, threads);
+    const bool any_wide = (v.ctl.nwide | v.ctl.nslow) != 0;
+    if (any_wide) {
+      wide_rows<KIND>(a, memory, w, round, warp, lane);
+      bar(BAR_ROWS, threads);
+    }
+
+    // ---- node decisions: a lane looks at a node, groups of 16 lanes decide the nodes that hold two
+    // distributed jobs or more GPUs than they have; nodes are dealt out round robin, so that violations
+    // spread over the warps ---------------------------------------------------------------------------
+#pragma unroll 1
+    for (int n0 = warp; n0 < NN; n0 += 32 * W) {
+      const int n_l = n0 + lane * W;
+      bool bad = false;
+      if (n_l < NN) {
+        const uint2 here = ((const uint2 *)v.node)[n_l];
+        bad = (here.y & 0xFFFFu) >= 2u || (int)here.x > (int)v.cap[n_l];
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, bad);
+#pragma unroll 1
+      while (todo) {
+        const int b0 = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int b1 = __ffs(todo) - 1;       // (-1: there is none)
+        todo &= todo - 1;
+        const int b = (lane & 16) ? b1 : b0, sub = lane & 15;
+        const int n = n0 + max(b, 0) * W;
+        const uint2 here = ((const uint2 *)v.node)[n];
+        const uint32_t rep = v.rep[set * NN + n], e = v.occ[n * FLOW_OCC + sub];
+        const int count = b >= 0 ? (int)(here.y >> 16) : 0, cap_n = (int)v.cap[n];
+        const bool listed = count <= FLOW_OCC, have = listed && sub < count;   // else: walked below
+        const int jc = have ? (int)(e & 0x1FFFu) : 0, had = have ? (int)((e >> 13) & 0x7FFu) : 0;
+        const int j = sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) ? (int)v.act[jc] : 0;
+        int ri = j - (int)(rep & 0xFFFFu), rc = j - (int)(rep >> 16);
+        if (ri < 0) ri += J;
+        if (rc < 0) rc += J;
+        const int most = max(__shfl_sync(0xffffffffu, count, 0), __shfl_sync(0xffffffffu, count, 16));
+        const int keeps = decide(had, (e >> 31) != 0u, have, min(most, FLOW_OCC), (here.y & 0xFFFFu) >= 2u, (int)here.x, cap_n, ri, rc);
+        if (have && keeps != had) {
+          set_entry<KIND>(a, v, w.dst, jc, (int)((e >> 25) & 7u), n, keeps);
+          // (bytes, so the word around it is updated as a whole)
+          const uint32_t bit = (uint32_t)INFO_CHANGED << (8 * (jc & 3));
+          if ((atomicOr((uint32_t *)v.info + (jc >> 2), bit) & bit) == 0u) {
+            const int at = atomicAdd(&v.ctl.nmod, 1);
+            if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) v.mod[at] = (uint16_t)jc;
+          }
+        }
+        if (b >= 0 && sub == 0 && !listed) { v.viol[n] = 1; v.ctl.walk = 1; }
+        __syncwarp();
+      }
+    }
+    bar(BAR_ROWS, threads);
+
+    // ---- rows the decisions change, then columns that have to be walked --------------------------------
+    const int nmod = v.ctl.nmod, walk = v.ctl.walk;
+#pragma unroll 1
+    for (int i0 = warp * 4; i0 < nmod; i0 += W * 4) {
+      const int jc = v.mod[min(i0 + g, nmod - 1)];
+      finish_row<KIND>(a, v, w.dst, jc, i0 + g < nmod && !(v.info[jc] & INFO_WIDE), warp, lane);
+    }
+    if (any_wide) {                           // wide rows among them
+      bar(BAR_ROWS, threads);                 // (one may turn into a record here: not to be taken for one above)
+#pragma unroll 1
+      for (int i = warp; i < nmod; i += W) {
+        const int jc = v.mod[i];
+        if (v.info[jc] & INFO_WIDE) finish_wide<KIND>(a, memory, w.dst, jc, warp, lane);
+      }
+    }
+    if (walk) walk_columns<KIND>(a, memory, w.dst, set, JA, warp, lane);
+    bar(BAR_ROWS, threads);
+
+    // ---- fitness (Eq. 14) from the rows' terms, in the order of the dense kernel: per chunk of rows, thread
+    // t adds rows t, t + 256, ... in double, a shuffle tree per warp, the warps in index order; then the
+    // chunks in index order.  Meanwhile the last warp makes everybody's rows visible to the other blocks; then it
+    // publishes. -----------------------------------------------------------------------------------------
+    if (last_warp) {
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      bar(BAR_KEY, 64);
+      if (lane == 0) {
+        const unsigned long long word = v.ctl.word;
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(pub_of(s, c)), "l"(word) : "memory");   // (behind this thread's fence)
+      }
+    } else {
+      constexpr bool ONE = KIND == FEW_ALONE;     // (up to 256 rows: one chunk, a row a thread)
+      const int chunks = ONE ? 1 : a.chunks;
+#pragma unroll 1
+      for (int x = warp; x < chunks * nv; x += W - 1) {
+        const int ch = ONE || chunks == 1 ? 0 : x / nv, vw = x - ch * nv;
+        double acc = 0.0;
+        if (ONE) {
+          if (vw * 32 + lane < J) acc = (double)v.term[vw * 32 + lane];
+        } else {
+          const int j0 = ch * a.rows_per_chunk, j1 = min(J, j0 + a.rows_per_chunk);
+#pragma unroll 1
+          for (int j = j0 + vw * 32 + lane; j < j1; j += SUM_THREADS) acc += (double)v.term[j];
+        }
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == 0) v.sums[ch * 8 + vw] = acc;
+      }
+      if (chunks * nv > 1) bar(BAR_SUMS, threads - 32);
+      if (warp == 0) {
+        if (lane == 0) {
+          double sum = 0.0;
+#pragma unroll 1
+          for (int ch = 0; ch < chunks; ++ch) {
+            double t = 0.0;
+#pragma unroll 1
+            for (int x = 0; x < nv; ++x) t += v.sums[ch * 8 + x];
+            sum += t;
+          }
+          const float f = fitness_finalise(a.tp.mode, a.tp.p, sum, (double)JA);
+          v.ctl.word = ((unsigned long long)(base + (uint32_t)s) << 32) | order_key(__float_as_uint(f));
+          if (s == a.generations) a.fitness[c] = f;
+        }
+        __syncwarp();
+        bar(BAR_KEY, 64);
+      }
+      // for the next candidate
+#pragma unroll 1
+      for (int i = threads - 33 - tid; i < NN; i += threads - 32) {
+        ((uint2 *)v.node)[i] = make_uint2(0u, 0u);
+        v.viol[i] = 0;
+      }
+      if (tid == threads - 33) { v.ctl.nmut[set] = 0; v.ctl.nwide = 0; v.ctl.nslow = 0; v.ctl.nmod = 0; v.ctl.walk = 0; }
+    }
+    next_item();
+  }
 }
 
 // The best candidate (largest key, lowest index on ties) and its rows as a dense matrix; the next
@@ -1192,10 +1243,6 @@ __global__ void __launch_bounds__(256) flow_gather_kernel(FlowRows f, int P, int
   }
 }
 
-int flow_row_threads(int J) { return std::min(MAX_ROW_THREADS, (J + 31) & ~31); }
-// row threads, the warp of the perturbed rows, and (ahead) as many threads again that draw the next step
-int flow_threads(int J, bool ahead) { return flow_row_threads(J) * (ahead ? 2 : 1) + 32; }
-
 }  // namespace
 
 namespace {
@@ -1206,6 +1253,8 @@ struct FlowArena {
   float *goodput, *speedup, *speedup_rack, *fitness;
   size_t total;
 };
+
+int flow_classes(const sched_ctx *ctx) { return ctx->d_rack ? 3 : 2; }
 
 FlowArena flow_arena(const sched_ctx *ctx, char *base) {
   const sched_config &c = ctx->cfg;
@@ -1219,6 +1268,7 @@ FlowArena flow_arena(const sched_ctx *ctx, char *base) {
   TAKE(fitness, float, P * 4);
   TAKE(r.cur_rec, uint32_t, 2 * J * REC_WORDS * 4);
   TAKE(r.same, uint32_t, J * REC_WORDS * 4);
+  TAKE(r.terms, float, J * flow_classes(ctx) * ctx->KD * 4);
   TAKE(r.pen, float, J * 4);
   TAKE(r.act, uint16_t, J * 2);
   TAKE(r.num_act, int, 4);
@@ -1232,13 +1282,92 @@ FlowArena flow_arena(const sched_ctx *ctx, char *base) {
   return f;
 }
 
-constexpr int FLOW_OCC = 16;      // occupants listed per node: a group of lanes
+int flow_kind(const sched_ctx *ctx) {
+  const int J = ctx->cfg.num_jobs, NN = ctx->cfg.num_nodes, P = ctx->cfg.population;
+  const bool alone = P <= ctx->num_sms, two = P <= 2 * ctx->num_sms;
+  if (J <= SMEM_RECORDS) return alone ? FEW_ALONE : FEW;
+  if (alone && J <= 4 * SMEM_RECORDS) return SOME_ALONE;
+  return two && 83 * J + 115 * NN + 6 * P <= 96 * 1024 ? FEW : MANY;      // (what two blocks find room for on an SM)
+}
 
-size_t flow_smem_bytes(const sched_ctx *ctx, bool ahead) {
-  int rows, chunks;
-  fitness_chunking(ctx, ctx->cfg.population, rows, chunks);
-  return flow_smem(ctx->cfg.population, ctx->cfg.num_jobs, ctx->cfg.num_nodes, FLOW_OCC,
-                   flow_threads(ctx->cfg.num_jobs, ahead) / 32, chunks).total;
+FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms) {
+  const sched_config &c = ctx->cfg;
+  const int J = c.num_jobs, NN = c.num_nodes, P = c.population;
+  int rows, chunks, off = 0;
+  fitness_chunking(ctx, P, rows, chunks);
+  FlowSmem L;
+  auto take = [&](size_t bytes) {
+    const int at = off;
+    off += (int)((bytes + 15) & ~(size_t)15);
+    return at;
+  };
+  take(sizeof(FlowCtl));
+  L.act = take((size_t)J * 2);
+  L.term = take((size_t)J * 4);
+  L.info = take((size_t)J);
+  L.node = take((size_t)NN * 8);
+  L.occ = take((size_t)NN * FLOW_OCC * 4);
+  L.viol = take((size_t)NN);
+  L.cap = take((size_t)NN * 2);
+  L.rack = take(ctx->d_rack ? (size_t)NN * 2 : 0);
+  L.mut = take(2 * (size_t)J * 2);
+  L.mod = take((size_t)J * 2);
+  L.wide = take((size_t)J * 2);
+  L.slow = take((size_t)J * 2);
+  L.stash = take(2 * (size_t)stash_rows(J) * 16);
+  L.flag = take(2 * (size_t)J);
+  L.dense = take((size_t)warps * wide_stride(NN) * 2);
+  L.rep = take(2 * (size_t)NN * 4);
+  L.keys = take((size_t)P * 6);      // and a list of candidates behind them
+  L.sums = take((size_t)chunks * 8 * 8);
+  L.scratch = take((size_t)warps * 32 * 4);
+  L.rec = flow_kind(ctx) != MANY ? take((size_t)J * REC_WORDS * 4) : 0;
+  L.same = flow_kind(ctx) != MANY ? take((size_t)J * REC_WORDS * 4) : 0;
+  L.terms = terms ? take((size_t)J * flow_classes(ctx) * ctx->KD * 4) : -1;
+  L.total = off;
+  return L;
+}
+
+// The launch's shape.
+struct FlowShape {
+  int warps, draw_warps, blocks;
+  FlowSmem at;
+};
+
+using FlowKernel = void (*)(FlowArgs);
+FlowKernel flow_kernel_for(const sched_ctx *ctx) {
+  const int kind = flow_kind(ctx);
+  return kind == MANY ? flow_kernel<MANY> : kind == FEW ? flow_kernel<FEW> : kind == SOME_ALONE ? flow_kernel<SOME_ALONE> : flow_kernel<FEW_ALONE>;
+}
+
+// A block for every candidate if they fit the GPU.  Warps that work on rows and warps that draw, measured: testbed (48 jobs)
+// 3 + 2 540 us, 4 + 2 513, 6 + 2 508, 8 + 2 and 8 + 4 505, 12 + 4 509; 96 jobs in racks 662, 621, 557, 547, 542, 542; two
+// blocks an SM (210 jobs) 8 + 2 760, 10 + 3 698, 12 + 3 693; 1024 jobs, four blocks an SM 6 + 2 3896, 7 + 2 3700,
+// 7 + 3 3774, 8 + 2 3740.  The terms' table is kept in shared memory where that does not cost a block its place.
+FlowShape flow_shape(const sched_ctx *ctx) {
+  const sched_config &c = ctx->cfg;
+  const bool few = flow_kind(ctx) != MANY;
+  FlowShape best = {};
+  const int per_sm = std::min(4, std::max(1, (c.population + ctx->num_sms - 1) / ctx->num_sms));
+  int warps, draw;
+  switch (flow_kind(ctx)) {
+    case MANY: warps = 7; draw = 2; break;
+    case FEW: warps = per_sm == 2 ? 12 : per_sm == 3 ? 8 : 6; draw = per_sm == 2 ? 3 : 2; break;
+    case SOME_ALONE: warps = 16; draw = 4; break;
+    default: warps = 8; draw = 4; break;
+  }
+  for (int terms = few ? 1 : 0; terms >= 0; --terms) {
+    FlowShape f = {warps, draw, 0, flow_smem(ctx, warps, terms != 0)};
+    int fit = 0;
+    if (f.at.total > 220 * 1024 ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, flow_kernel_for(ctx), (warps + draw) * 32, f.at.total) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    f.blocks = std::min(c.population, fit * ctx->num_sms);
+    if (f.blocks > best.blocks) best = f;
+  }
+  return best;
 }
 
 }  // namespace
@@ -1253,24 +1382,16 @@ int round_flow_ensure(sched_ctx *ctx) {
   if (2 * rows > ctx->rs_budget) return SCHED_OK;
   int coop = 0, blocks = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop ||
-      cudaFuncSetAttribute(flow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess) {
+      cudaFuncSetAttribute(flow_kernel_for(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess) {
     cudaGetLastError();
     return SCHED_OK;
   }
-  // threads that draw ahead where every candidate still has a block of its own (and its nodes' draws pay)
-  for (int ahead = c.num_jobs <= SMEM_RECORDS ? 1 : 0; ahead >= 0; --ahead) {
-    const size_t smem = flow_smem_bytes(ctx, ahead != 0);
-    int per_sm = 0;
-    if (smem > 220 * 1024 ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, flow_kernel, flow_threads(c.num_jobs, ahead != 0), smem) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
-    }
-    blocks = std::min(c.population, per_sm * ctx->num_sms);
-    ctx->fl_ahead = ahead != 0;
-    if (blocks == c.population) break;
-  }
+  const FlowShape shape = flow_shape(ctx);
+  blocks = shape.blocks;
   if (blocks < 1) return SCHED_OK;
+  ctx->fl_warps = shape.warps;
+  ctx->fl_draw_warps = shape.draw_warps;
+  ctx->fl_terms = shape.at.terms >= 0;
   const FlowArena size = flow_arena(ctx, nullptr);
   if (cudaMalloc((void **)&ctx->fl_arena, size.total) != cudaSuccess) {
     cudaGetLastError();
@@ -1302,7 +1423,8 @@ static FlowArgs flow_args(const sched_ctx *ctx, const sched_jobs *jobs, const in
   a.tp.active = nullptr; a.tp.k_max = c.k_max; a.tp.n_max = c.n_max; a.tp.mode = fitness_mode(c.p); a.tp.p = c.p;
   a.tp.floor_ = c.speedup_floor;
   a.P = c.population; a.J = c.num_jobs; a.NN = c.num_nodes; a.k_max = c.k_max; a.n_max = c.n_max;
-  a.num_elite = c.num_elite; a.occ = FLOW_OCC; a.row_threads = flow_row_threads(c.num_jobs);
+  a.num_elite = c.num_elite; 
+  a.nmin = ctx->d_nmin; a.classes = flow_classes(ctx);
   a.thr_init = c.thr_init; a.thr_mutate = c.thr_mutate;
   a.key = make_key(c.seed, ctx->d_round);
   fitness_chunking(ctx, c.population, a.rows_per_chunk, a.chunks);
@@ -1318,6 +1440,8 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   const sched_config &c = ctx->cfg;
   FlowArgs a = flow_args(ctx, jobs, d_cur);
   a.generations = generations;
+  a.warps = ctx->fl_warps;
+  a.at = flow_smem(ctx, ctx->fl_warps, ctx->fl_terms);
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
     TimedLaunch tl_(ctx, KK_FLOW_BUILD);
@@ -1326,8 +1450,8 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   SCHED_LAUNCH_CHECK(ctx);
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)ctx->fl_blocks);
-  lc.blockDim = dim3((unsigned)flow_threads(c.num_jobs, ctx->fl_ahead));
-  lc.dynamicSmemBytes = flow_smem_bytes(ctx, ctx->fl_ahead);
+  lc.blockDim = dim3((unsigned)(ctx->fl_warps + ctx->fl_draw_warps) * 32);
+  lc.dynamicSmemBytes = (size_t)a.at.total;
   lc.stream = ctx->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -1336,7 +1460,7 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   lc.numAttrs = 1;
   {
     TimedLaunch tl_(ctx, KK_FLOW);
-    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, flow_kernel, a));
+    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, flow_kernel_for(ctx), a));
   }
   SCHED_LAUNCH_CHECK(ctx);
   {

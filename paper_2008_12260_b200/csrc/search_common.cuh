@@ -52,26 +52,32 @@ static __device__ __noinline__ void draw_two(uint32_t k0, uint32_t k1, uint32_t 
 
 // What the repair decides for the occupant in this lane of a group of 16 (`have`: there is one; v: its GPUs on the
 // node, 0 without; distributed: its row spans two nodes or more): the GPUs it keeps there.  rot_i, rot_c: the
-// row's place in the node's two rotated job orders.  Called by whole warps, two nodes at a time (shuffles under the full mask; a group
+// row's place in the node's two rotated job orders (below 65536; GPUs below 2048).  Called by whole warps, two nodes at a time (shuffles under the full mask; a group
 // without a node has no occupants).
 __device__ __forceinline__ int decide(int v, bool distributed, bool have, int most, bool intf, int tot, int cap_n, int rot_i, int rot_c) {
   const bool dist = have && intf && distributed;
   int removed = 0;
-  if (__any_sync(0xffffffffu, intf)) {
-    int first = dist ? rot_i : 0x7fffffff;
+  if (__any_sync(0xffffffffu, intf)) {   // of the distributed ones only the first in rotated order stays
+    int first = dist ? (rot_i << 11) | v : 0x7fffffff, all = dist ? v : 0;
 #pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) first = min(first, __shfl_xor_sync(0xffffffffu, first, off));
-    if (dist && rot_i != first) { removed = v; v = 0; }
-#pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) removed += __shfl_xor_sync(0xffffffffu, removed, off);
+    for (int off = 8; off >= 1; off >>= 1) {
+      first = min(first, __shfl_xor_sync(0xffffffffu, first, off));
+      all += __shfl_xor_sync(0xffffffffu, all, off);
+    }
+    if (intf) removed = all - (first & 0x7FF);
+    if (dist && (first >> 11) != rot_i) v = 0;
   }
   const int excess = tot - removed - cap_n;
   int ahead = 0;                         // GPUs of the occupants that come first in rotated order
   if (__any_sync(0xffffffffu, excess > 0)) {
+    const int mine = have ? (rot_c << 11) | v : 0x7fffffff;
 #pragma unroll 1
-    for (int k = 0; k < most; ++k) {
-      const int rk = __shfl_sync(0xffffffffu, rot_c, k, 16), vk = __shfl_sync(0xffffffffu, v, k, 16);
-      if (rk < rot_c) ahead += vk;
+    for (int k = 0; k < most; k += 4) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int other = __shfl_sync(0xffffffffu, mine, k + q, 16);
+        if ((other >> 11) < rot_c && other != 0x7fffffff) ahead += other & 0x7FF;
+      }
     }
   }
   if (have && excess > 0) v -= min(v, max(excess - ahead, 0));
