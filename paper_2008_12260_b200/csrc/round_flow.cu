@@ -206,11 +206,12 @@ __device__ __noinline__ Record dense_record(const FlowArgs &a, const int16_t *ro
       hi = max(hi, r);
     }
     const unsigned m = __ballot_sync(0xffffffffu, v > 0);
-    if (lane >= base && lane < base + __popc(m)) {
-      const int at = (int)__fns(m, 0, lane - base + 1);
-      mine = ((uint32_t)(n0 + at) << 16) | (uint32_t)row[n0 + at];
+#pragma unroll 1
+    for (unsigned left = m; left && base < ENTRIES; left &= left - 1u, ++base) {
+      const int at = __ffs(left) - 1;
+      const uint32_t e = ((uint32_t)(n0 + at) << 16) | (uint32_t)__shfl_sync(0xffffffffu, v, at);
+      if (lane == base) mine = e;
     }
-    base += __popc(m);
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
@@ -240,9 +241,9 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
   const int J = a.J, NN = a.NN, NS = wide_stride(NN);
   if (blockIdx.x == 0 && warp == 0) {
     int n = 0;
-#pragma unroll 1
+#pragma unroll 8
     for (int j0 = 0; j0 < J; j0 += 32) {
-      const bool on = j0 + lane < J && (!a.active || a.active[j0 + lane]);
+      const bool on = j0 + lane < J && (!a.active || __ldg(a.active + j0 + lane));
       const unsigned m = __ballot_sync(0xffffffffu, on);
       if (on) a.r.act[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(j0 + lane);
       n += __popc(m);
@@ -268,37 +269,42 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
     in_range = __all_sync(0xffffffffu, in_range);
     const float pen = a.tp.pen && raw > 0 ? realloc_factor(a.age[j], a.restarts[j], a.delta) : 1.f;
     if (a.tp.pen && lane == 0) a.r.pen[j] = pen;
-    // (what a row of the search can be: on one node, or on as many as its GPUs need at least; the table has one
-    // value for all of those)
-    const int KD = a.k_max + 1, ND = a.n_max + 1;
-#pragma unroll 1
-    for (int K = lane; K < KD; K += 32) {
-      const int many = K >= 2 ? a.nmin[K] : ND;
-#pragma unroll 1
-      for (int cls = 0; cls < a.classes; ++cls) {
-        const int N = cls ? many : K >= 1 ? 1 : ND;
-        const float *table = cls == 2 ? a.table_rack : a.tp.table;
-        const float x = N < ND ? table[((size_t)j * KD + K) * ND + N] : 0.f;
-        a.r.terms[((size_t)j * a.classes + cls) * KD + K] = fitness_term_with(a.tp, x, pen, true);
-      }
-    }
     __syncwarp();
     int K, N;
     dense_totals(row, NN, lane, K, N);
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // the tables
+    // (what a row of the search can be: on one node, or on as many as its GPUs need at least; the table has one
+    // value for all of those)
+    const int KD = a.k_max + 1, ND = a.n_max + 1;
+#pragma unroll 2
+    for (int k = lane; k < KD; k += 32) {
+      const int many = k >= 2 ? __ldg(a.nmin + k) : ND, one = k >= 1 ? 1 : ND;
+      const size_t from = ((size_t)j * KD + k) * ND;
+      float *to = a.r.terms + (size_t)j * a.classes * KD + k;
+      const float x0 = one < ND ? __ldcg(a.tp.table + from + one) : 0.f, x1 = many < ND ? __ldcg(a.tp.table + from + many) : 0.f;
+      const float x2 = a.classes > 2 && many < ND ? __ldcg(a.table_rack + from + many) : 0.f;
+      to[0] = fitness_term_with(a.tp, x0, pen, true);
+      to[KD] = fitness_term_with(a.tp, x1, pen, true);
+      if (a.classes > 2) to[2 * KD] = fitness_term_with(a.tp, x2, pen, true);
+    }
     const int kc = max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max));
+    Record r;
 #pragma unroll 1
     for (int caps = 1; caps >= 0; --caps) {     // before the caps (the second set), then after them (the first)
+      const bool over = K > kc || N > a.n_max;
       if (!caps) dense_caps(row, NN, K, N, kc, a.n_max, lane);
       const size_t at = (size_t)caps * J + j;
-      Record r = dense_record(a, row, j, K, N, a.r.cur_wide + at * NS, lane);
+      if (caps || over || N > ENTRIES) r = dense_record(a, row, j, K, N, a.r.cur_wide + at * NS, lane);
       if (lane == 0) store_record(a.r.cur_rec + at * REC_WORDS, r);
       if (caps && lane == 0) {
-        if (!a.tp.pen || !in_range || N > ENTRIES) r.w[0] = NEVER;
-        store_record(a.r.same + (size_t)j * REC_WORDS, r);
+        Record same = r;
+        if (!a.tp.pen || !in_range || N > ENTRIES) same.w[0] = NEVER;
+        store_record(a.r.same + (size_t)j * REC_WORDS, same);
       }
       __syncwarp();
     }
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");        // (a block without an active job ends after the tables, too)
 }
 
 constexpr int INFO_DIST = 1;        // the row spanned two nodes or more after the row pass (interference snapshot)
@@ -1163,6 +1169,7 @@ __global__ void __launch_bounds__(256) flow_finish_kernel(FlowArgs a) {
   __shared__ unsigned long long s_best[8];
   __shared__ uint16_t s_place[FLOW_MAX_JOBS];      // place of a job's row, 0xFFFF: the job is not active
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, P = a.P, J = a.J, NN = a.NN, NS = wide_stride(NN);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   unsigned long long best = 0ull;
 #pragma unroll 1
   for (int i = tid; i < P; i += 256) {
@@ -1434,6 +1441,20 @@ static FlowArgs flow_args(const sched_ctx *ctx, const sched_jobs *jobs, const in
   return a;
 }
 
+// A launch that may begin while the kernel before it on the stream ends.
+static cudaError_t launch_beside(sched_ctx *ctx, FlowKernel kernel, int blocks, int threads, const FlowArgs &a) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)blocks);
+  lc.blockDim = dim3((unsigned)threads);
+  lc.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, a);
+}
+
 // The search of a round, after its tables.
 int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_cur, int32_t generations, int16_t *d_best,
                       float *d_best_fitness) {
@@ -1445,7 +1466,8 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
     TimedLaunch tl_(ctx, KK_FLOW_BUILD);
-    flow_build_kernel<<<(c.num_jobs + 3) / 4, 128, 0, ctx->stream>>>(a);
+    // (beside the tables' last kernel: what needs no table is done while that still writes)
+    SCHED_CUDA_CHECK(ctx, launch_beside(ctx, flow_build_kernel, (c.num_jobs + 3) / 4, 128, a));
   }
   SCHED_LAUNCH_CHECK(ctx);
   cudaLaunchConfig_t lc = {};
@@ -1465,7 +1487,7 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   SCHED_LAUNCH_CHECK(ctx);
   {
     TimedLaunch tl_(ctx, KK_FLOW_FINISH);
-    flow_finish_kernel<<<std::min((c.num_jobs + 7) / 8, ctx->num_sms), 256, 0, ctx->stream>>>(a);
+    SCHED_CUDA_CHECK(ctx, launch_beside(ctx, flow_finish_kernel, std::min((c.num_jobs + 7) / 8, ctx->num_sms), 256, a));
   }
   SCHED_LAUNCH_CHECK(ctx);
   ctx->fl_generations = generations;

@@ -490,6 +490,7 @@ template <bool SAMPLES>
 __global__ void __maxnreg__(56) table_kernel(TableArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   cg::cluster_group cl = cg::this_cluster();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // (who starts beside this waits for its end)
   const int KD = a.k_max + 1, tid = threadIdx.x, nthreads = blockDim.x;
   const int nb = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int j = a.j_first + (int)blockIdx.x / nb;
@@ -789,6 +790,7 @@ __global__ void __launch_bounds__(256, 4) sweep_kernel(TableArgs a) {
 __global__ void __launch_bounds__(256) slab_kernel(TableArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int KD = a.k_max + 1, j = a.j_first + (int)blockIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // (who starts beside this waits for its end)
   const int fair = fair_place(a, j);
   const TableSmem t = {a.g + (size_t)j * KD * 3, a.a + (size_t)j * KD * 3};
   asm volatile("griddepcontrol.wait;" ::: "memory");
