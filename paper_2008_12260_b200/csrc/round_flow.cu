@@ -32,6 +32,10 @@ constexpr uint32_t NO_NODE = 0xFFFFFFFFu;       // an entry that is not used
 constexpr uint32_t WIDE = 0xFFFFFFFEu;          // first entry of a row with more: its contents are elsewhere
 constexpr int REC_TERM = 6;
 constexpr int DEPTH = 4;                        // generations kept
+// Words from one candidate's published key to the next's.  Side by side, a hundred keys are seven lines that
+// every block polls, and polls and publications queue there: testbed round 494 us, 422 with 32 bytes between them, 415 with
+// 64, 420 with 128; 210 jobs x 150 candidates 708, 555, 549, 565; racks 528, 449, 438, 438.
+constexpr int PUB_STRIDE = 8;
 constexpr int SUM_THREADS = 256;                // as the dense fitness kernel: the order of its sums
 constexpr int LANES = 8;                        // lanes of a row
 constexpr int STASH = 128;                      // perturbed rows of many whose draws are kept, further ones draw again
@@ -65,7 +69,7 @@ struct FlowRows {
   float *pen;                // [J] penalty factor of a row that differs from the current allocation's
   uint16_t *act;             // [J] active jobs, ascending; act[J] .. : see num_act
   int *num_act;
-  unsigned long long *pub;   // [DEPTH][P] tag << 32 | fitness key
+  unsigned long long *pub;   // [DEPTH][P][PUB_STRIDE] tag << 32 | fitness key
   uint32_t *base;            // tag of the round's initial population
 };
 constexpr uint32_t NEVER = 0xFFFFFFFDu;
@@ -911,7 +915,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
   const int threads = W * 32, g = lane >> 3, nv = (min(J, SUM_THREADS) + 31) >> 5;
   const bool last_warp = warp == W - 1;
   const int PJ = P * J, cur_rows = (int)((a.r.cur_rec - a.r.rec) / REC_WORDS);
-  auto pub_of = [&](int step, uint32_t cand) { return a.r.pub + (size_t)(step & (DEPTH - 1)) * P + cand; };
+  auto pub_of = [&](int step, uint32_t cand) { return a.r.pub + ((size_t)(step & (DEPTH - 1)) * P + cand) * PUB_STRIDE; };
   // Items: this block's candidates of step 0 (the initial population), of step 1 (generation 0), ...
   int s = 0, set = 0;
   Work w;
@@ -1280,7 +1284,7 @@ FlowArena flow_arena(const sched_ctx *ctx, char *base) {
   TAKE(r.act, uint16_t, J * 2);
   TAKE(r.num_act, int, 4);
   TAKE(r.base, uint32_t, 4);
-  TAKE(r.pub, unsigned long long, DEPTH * P * 8);
+  TAKE(r.pub, unsigned long long, DEPTH * P * PUB_STRIDE * 8);
   TAKE(r.cur_wide, int16_t, 2 * J * NS * 2);
   TAKE(r.rec, uint32_t, DEPTH * P * J * REC_WORDS * 4);
   TAKE(r.wide, int16_t, DEPTH * P * J * NS * 2);
@@ -1412,7 +1416,7 @@ int round_flow_ensure(sched_ctx *ctx) {
   ctx->d_fit_buf = ctx->d_fit = f.fitness;
   ctx->scratch_epoch++;
   // no tag matches before it is published, and a record that was never written has no nodes
-  SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(f.r.pub, 0, DEPTH * (size_t)c.population * 8, ctx->stream));
+  SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(f.r.pub, 0, DEPTH * (size_t)c.population * PUB_STRIDE * 8, ctx->stream));
   SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(f.r.base, 1, 4, ctx->stream));
   ctx->fl_blocks = blocks;
   return SCHED_OK;
