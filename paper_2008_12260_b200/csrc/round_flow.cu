@@ -883,6 +883,8 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
 #pragma unroll 1
   for (int i = tid; i < J; i += blockDim.x) v.term[i] = 0.f;
 #pragma unroll 1
+  for (int i = tid; i < a.chunks * 8; i += blockDim.x) v.sums[i] = 0.0;
+#pragma unroll 1
   for (int i = tid; i < NN; i += blockDim.x) {
     v.cap[i] = (int16_t)max((int)a.cap[i], 0);
     if (a.rack) v.rack[i] = a.rack[i];
@@ -1143,9 +1145,11 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
           double sum = 0.0;
 #pragma unroll 1
           for (int ch = 0; ch < chunks; ++ch) {
-            double t = 0.0;
-#pragma unroll 1
-            for (int x = 0; x < nv; ++x) t += v.sums[ch * 8 + x];
+            double part[8], t = 0.0;            // (warps that do not exist left zeros)
+#pragma unroll
+            for (int x = 0; x < 8; ++x) part[x] = v.sums[ch * 8 + x];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) t += part[x];
             sum += t;
           }
           const float f = fitness_finalise(a.tp.mode, a.tp.p, sum, (double)JA);
