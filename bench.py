@@ -53,13 +53,13 @@ CONFIG = {
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the committed ncu
 # summaries under profiles/ (not measured in this run); None = the kernel has changed since its
 # counters were taken.
-# "rows": one dense large-workload generation of the streaming row kernel (227.7 MB read + 233.7 MB
+# "rows": one dense large-workload generation, rows and repair in one kernel (158.3 MB read + 236.4 MB
 # written: some parent rows are shared by several children and come from L2).
 # "fitness_stress": 16 dense stress candidates moved 544.8 + 3.5 MB; every candidate is streamed
 # once, so the figure is scaled by candidates / 16 to the chunk that is timed.
-# "round_search": per generation, a 201st of one large round's 12.0 MB read and 2328 MB written (records stay in
+# "round_search": per generation, a 201st of one large round's 2.4 MB read and 2162 MB written (records stay in
 # L2 or are written back from it).
-NCU_TRAFFIC_BYTES = {"rows": 461.4e6, "fitness_stress_per_candidate": 548.3e6 / 16, "round_search": 2340.3e6 / 201}
+NCU_TRAFFIC_BYTES = {"rows": 394.7e6, "fitness_stress_per_candidate": 548.3e6 / 16, "round_search": 2164.3e6 / 201}
 
 
 def measured_peaks():
