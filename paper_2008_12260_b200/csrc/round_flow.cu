@@ -234,7 +234,8 @@ __device__ __noinline__ Record dense_record(const FlowArgs &a, const int16_t *ro
 #pragma unroll 1
     for (int n = lane; n < wide_stride(NN); n += 32) wide[n] = n < NN ? row[n] : (int16_t)0;
   }
-  const float sp = __ldg(table_of(a, lo, hi) + fitness_table_index(a.tp, j, K, N));
+  // (not through the read-only path: flow_build_kernel calls this, and the tables' kernel writes them while it runs)
+  const float sp = __ldcg(table_of(a, lo, hi) + fitness_table_index(a.tp, j, K, N));
   r.w[REC_TERM] = __float_as_uint(fitness_term_with(a.tp, sp, a.tp.pen ? a.r.pen[j] : 1.f, changed));
   r.w[7] = 0u;
   return r;
