@@ -1,5 +1,5 @@
 // Pieces of the population search (Sec. 4.3) that the one-launch round and the dense operators share: draws of the
-// counter-based stream, the candidate of a rank, the repair's decision for a node.
+// counter-based stream and the repair's decision for a node.
 #pragma once
 
 #include "common.cuh"
@@ -82,44 +82,4 @@ __device__ __forceinline__ int decide(int v, bool distributed, bool have, int mo
   }
   if (have && excess > 0) v -= min(v, max(excess - ahead, 0));
   return v;
-}
-
-// The candidate of rank c (fitness key descending, index ascending) of P keys in shared memory, by one
-// warp.  The (c + 1)-th largest of the lanes' own maxima is no larger than the key wanted, so only the
-// keys from there on (about twice c) are ranked; list: room for P.
-static __device__ __noinline__ int candidate_of_rank(const uint32_t *key, int P, int c, uint16_t *list, int lane) {
-  uint32_t top = 0u;
-#pragma unroll 4
-  for (int i = lane; i < P; i += 32) top = max(top, key[i]);
-  int before = 0;                       // lanes whose maximum comes first
-#pragma unroll 1
-  for (int l = 0; l < 32; ++l) {
-    const uint32_t o = __shfl_sync(0xffffffffu, top, l);
-    before += o > top || (o == top && l < lane) ? 1 : 0;
-  }
-  uint32_t bound = 0u;                  // (more ranks than lanes: every key)
-  if (c < 32) bound = __shfl_sync(0xffffffffu, top, __ffs(__ballot_sync(0xffffffffu, before == c)) - 1);
-  int n = 0;
-#pragma unroll 1
-  for (int i0 = 0; i0 < P; i0 += 32) {
-    const bool in = i0 + lane < P && key[i0 + lane] >= bound;
-    const unsigned m = __ballot_sync(0xffffffffu, in);
-    if (in) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(i0 + lane);
-    n += __popc(m);
-  }
-  __syncwarp();
-  int found = 0x7fffffff;
-#pragma unroll 1
-  for (int x = lane; x < n; x += 32) {
-    const int i = list[x];
-    const uint32_t k = key[i];
-    int rank = 0;
-#pragma unroll 2
-    for (int y = 0; y < n; ++y) {
-      const uint32_t o = key[list[y]];
-      rank += o > k || (o == k && y < x) ? 1 : 0;
-    }
-    if (rank == c) found = i;
-  }
-  return __reduce_min_sync(0xffffffffu, found);
 }

@@ -74,3 +74,28 @@ def test_children_of_any_width(oracle, nodes, J, P, density, shift_in, shift_out
     assert _guards_ok(out_flat, shift_out, raw.size)
     s.sync_status()
     s.close()
+
+
+# population, elite children: as many as lanes, more, everybody; keys in one turn of a block and in many
+@pytest.mark.parametrize("P,elite", [(1, 1), (33, 33), (256, 40), (257, 256), (5121, 70), (7361, 33)])
+@pytest.mark.parametrize("values", [0, 5, 1])           # different fitness values (0: all of them differ)
+@pytest.mark.parametrize("nodes", [3, 8])
+def test_elite_children_of_any_rank(oracle, P, elite, values, nodes):
+    import torch
+    from paper_2008_12260_b200 import api
+
+    rng = np.random.default_rng(P + elite + values)
+    cl = synth.uniform_cluster(nodes, 4)
+    J, thr, seed = 2, synth.prob_to_threshold(0.3), 5
+    raw = synth.random_raw_population(P, J, cl, seed=P, density=0.4, v_hi=4)
+    fit = (rng.integers(0, values, P) - 2).astype(np.float32) if values else rng.permutation(P).astype(np.float32)
+    k_cap, active = np.full(J, cl.k_max, np.int32), np.ones(J, np.uint8)
+    s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=thr,
+                      num_elite=elite, seed=seed, stream=torch.cuda.current_stream().cuda_stream)
+    out = torch.empty(raw.shape, dtype=torch.int16, device="cuda:0")
+    s.ga_generation(api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch), torch.from_numpy(raw).cuda(),
+                    torch.from_numpy(fit).cuda(), out, round=1, generation=2)
+    ref = oracle.ga_generation(raw, fit, cl.node_capacity, k_cap, cl.k_max, cl.n_max, elite, thr, seed, 1, 2, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+    s.sync_status()
+    s.close()
