@@ -20,3 +20,41 @@ KINDS = [
 @pytest.mark.parametrize("start", ["none", "feasible", "raw"])
 def test_rounds_at_the_kinds_edges(shape, start):
     shapes.test_round_equals_stepwise("flow", shape, start)
+
+
+# candidates, elite children, share of rows perturbed at first and per generation: ranks of few keys above the bound, of
+# more (ties in a converged population), of as many as there are, and ranks beyond a warp's lanes
+@pytest.mark.parametrize("P,elite,init,mutate", [(64, 4, 0.0, 0.0), (65, 31, 0.0, 0.0), (300, 16, 0.01, 0.0), (300, 31, 0.01, 0.01),
+                                                 (300, 32, 0.3, 0.05), (148, 148, 0.3, 0.0), (500, 200, 0.05, 0.01)])
+def test_elite_candidates_of_a_round(P, elite, init, mutate):
+    import numpy as np
+    import torch
+    from helpers import with_fair_share
+    from paper_2008_12260_b200 import api, synth
+
+    cfg = synth.Config("ranks", 12, 4, 30, 3, 16, 8, P, 6, num_elite=elite, mutate_prob=mutate, init_prob=init, with_history=True)
+    cl = cfg.cluster()
+    jobs = with_fair_share(cfg.jobs(), cl)
+    s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
+    dj = api.DeviceJobs(jobs, "cuda", torch)
+    cur = torch.from_numpy(synth.random_feasible_allocation(cl, cfg.num_jobs, 5)).cuda()
+    best, bf = torch.empty((cfg.num_jobs, 12), dtype=torch.int16, device="cuda"), torch.zeros(1, device="cuda")
+    pop, fit = torch.empty((P, cfg.num_jobs, 12), dtype=torch.int16, device="cuda"), torch.empty(P, device="cuda")
+    sp, rf = torch.empty(s.table_shape, device="cuda"), torch.empty(cfg.num_jobs, device="cuda")
+    s.schedule_round(dj, cur, best, bf, round=2, generations=6)
+    s.get_population(pop, fit)
+    s.build_speedup_table(dj, None, sp, None)
+    s.compute_realloc_factor(dj, rf)
+    a, b, f = torch.empty_like(pop), torch.empty_like(pop), torch.empty_like(fit)
+    s.init_population(dj, cur, a, round=2)
+    for g in range(7):
+        s.eval_fitness(a, sp, f, p=cfg.p, cur=cur, realloc_factor=rf, active=dj.tensors["active"])
+        if g < 6:                 # the rank of a child's parent is checked against a plain sort as well
+            order = np.argsort(-f.cpu().numpy(), kind="stable")
+            s.ga_generation(dj, a, f, b, round=2, generation=g)
+            for c in range(0, elite, 7):
+                assert torch.equal(b[c], a[int(order[c])])
+            a, b = b, a
+    s.sync_status()
+    assert torch.equal(a, pop) and torch.equal(f.view(torch.int32), fit.view(torch.int32))
+    s.close()
