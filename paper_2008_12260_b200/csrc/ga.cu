@@ -912,7 +912,8 @@ __global__ void __launch_bounds__(128, 4) colrepair_kernel(ColfixArgs a) {
 // ---------------------------------------------------------------------------------------
 constexpr int CHILD_WARPS = 8;
 constexpr int CHILD_TILE = 1024;        // entries a warp lays out at a time
-constexpr int CHILD_OCC = 16;           // occupants listed per node: a group of lanes
+constexpr int CHILD_OCC = 16;           // occupants a group of lanes decides; listed per node of a block: at least as many
+constexpr int CHILD_CROWD = 768;        // occupants a warp decides
 constexpr int CHILD_SPLIT = 8;          // blocks of a child, at most
 __host__ __device__ constexpr int child_vectors(bool whole) { return whole ? 128 : 160; }   // a warp reads at a time
 
@@ -922,6 +923,7 @@ struct ChildArgs {
   const int16_t *src_lo, *src_hi;       // what may be read: [src_lo, src_hi)
   int row_vecs;                         // aligned vectors a row may touch
   int split;                            // blocks of a child: a power of two
+  int occ;                              // occupants a block lists per node
   int tile_rows, chunk_rows;            // rows laid out at a time; rows whose draws are made at a time
 };
 
@@ -934,8 +936,57 @@ struct ChildWarp {                      // shared memory of a warp
   int bad[32];                          // an entry is out of range
 };
 
-inline size_t child_smem_bytes(int NN, bool whole) {
-  return CHILD_WARPS * (whole ? sizeof(ChildWarp<true>) : sizeof(ChildWarp<false>)) + (size_t)NN * (CHILD_OCC * 4 + 4 + 4 + 2);
+static_assert(sizeof(ChildWarp<true>) >= CHILD_CROWD * 4 && sizeof(ChildWarp<false>) >= CHILD_CROWD * 4, "a crowded node's occupants");
+
+inline size_t child_smem_bytes(int NN, int occ, bool whole) {
+  return CHILD_WARPS * (whole ? sizeof(ChildWarp<true>) : sizeof(ChildWarp<false>)) + (size_t)NN * ((size_t)occ * 4 + 4 + 4 + 2);
+}
+
+// Behind the nodes' lists: GPUs placed on each; distributed jobs on it | occupants << 16.
+__device__ __forceinline__ const uint32_t *child_counts(const uint32_t *s_occ, int NN, int occ) { return s_occ + (size_t)NN * occ + NN; }
+
+// An entry of a list: job | GPUs << 16 | distributed << 31.
+__device__ __forceinline__ int occupant_gpus(uint32_t e) { return (int)((e >> 16) & 0x7FFu); }
+__device__ __forceinline__ int rotated(uint32_t e, uint32_t offset, int J) {
+  const int r = (int)(e & 0xFFFFu) - (int)offset;
+  return r < 0 ? r + J : r;
+}
+
+// The repair of a node with more occupants than a group of lanes has, by a warp: from the blocks' lists, gathered in `list`, or,
+// where one of those is too short, from the column (128 children of 1024 x 8, a tenth of the rows perturbed: 24.0 us
+// from lists, 32.7 from the columns where there are more than 16; three of ten, as at first, 42.9 and 51.0).
+__device__ __noinline__ void repair_crowded(const ChildArgs &aa, uint32_t *list, const uint32_t *s_occ, int cl, int n, int tot, uint32_t cnt,
+                                            int cap_n, uint32_t rep, int lane) {
+  const int J = aa.r.J, NN = aa.r.num_nodes, count = (int)(cnt >> 16);
+  const bool intf = (cnt & 0xFFFFu) >= 2u;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  bool all = count <= CHILD_CROWD;
+  if (all) {
+    int at = 0;
+#pragma unroll 1
+    for (int q = 0; q < aa.split; ++q) {
+      const uint32_t *const occ = aa.split > 1 ? cluster.map_shared_rank(s_occ, q) : s_occ;
+      const int here = (int)(child_counts(occ, NN, aa.occ)[n] >> 16);
+      all = all && here <= aa.occ;
+      for (int k = lane; k < min(here, aa.occ); k += 32) list[at + k] = occ[n * aa.occ + k];
+      at += here;
+    }
+    __syncwarp();
+  }
+  if (!all) {
+    repair_column_any(aa.col, nullptr, cl, n, tot, (int)(cnt & 0xFFFFu), cap_n, lane);
+    return;
+  }
+  const auto rot_i = [&](uint32_t e) { return rotated(e, rep & 0xFFFFu, J); };
+  const auto rot_c = [&](uint32_t e) { return rotated(e, rep >> 16, J); };
+  const CrowdPlaces at = crowd_places([=](int k) { return list[k]; }, count, J, tot, intf, cap_n, lane, occupant_gpus, rot_i, rot_c);
+  int16_t *const column = aa.r.dst + (size_t)cl * J * NN + n;
+#pragma unroll 1
+  for (int k = lane; k < count; k += 32) {
+    const uint32_t e = list[k];
+    const int v = at.keeps(e, occupant_gpus(e), rot_i(e), rot_c(e));
+    if (v != occupant_gpus(e)) column[(size_t)(e & 0xFFFFu) * NN] = (int16_t)v;
+  }
 }
 
 // The candidate of rank c (fitness key descending, index ascending) of any number, by a block: the key from its
@@ -1020,7 +1071,7 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   ChildWarp<WHOLE> &w = ((ChildWarp<WHOLE> *)child_smem)[warp];
   uint32_t *s_occ = (uint32_t *)(child_smem + CHILD_WARPS * sizeof(ChildWarp<WHOLE>));   // job | GPUs << 16 | distributed << 31
-  int32_t *s_tot = (int32_t *)(s_occ + (size_t)NN * CHILD_OCC);                      // GPUs placed on the node
+  int32_t *s_tot = (int32_t *)(s_occ + (size_t)NN * aa.occ);                         // GPUs placed on the node
   uint32_t *s_cnt = (uint32_t *)(s_tot + NN);                                        // distributed jobs on it | occupants << 16
   int16_t *s_cap = (int16_t *)(s_cnt + NN);
   __shared__ int s_parent[2];
@@ -1088,7 +1139,7 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
   auto add_occupant = [&](int j, int n, int v, bool dist) {
     atomicAdd(&s_tot[n], v);
     const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
-    if (k < CHILD_OCC) s_occ[n * CHILD_OCC + k] = (uint32_t)j | ((uint32_t)v << 16) | (dist ? 0x80000000u : 0u);
+    if (k < (uint32_t)aa.occ) s_occ[n * aa.occ + k] = (uint32_t)j | ((uint32_t)v << 16) | (dist ? 0x80000000u : 0u);
   };
   constexpr int B = child_vectors(WHOLE) / 32;
   int16_t *tile = (int16_t *)w.tile;
@@ -1288,7 +1339,7 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
 
   // ---- repair: the nodes are dealt out to all warps; a lane looks at a node, groups of 16 lanes decide those
   // that hold two distributed jobs or more GPUs than they have, from the occupants that the child's blocks have
-  // listed; a node with more occupants than a group has lanes is walked by a warp ----------------------
+  // listed; those with more than a group has lanes by a warp each --------------------------------------
   auto of_part = [&](auto *p, int q) { return split > 1 ? cluster.map_shared_rank(p, q) : p; };
 #pragma unroll 1
   for (int n0 = gw; n0 < NN; n0 += 32 * nwarps) {
@@ -1334,7 +1385,7 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
           if (k < here) break;
           k -= here;
         }
-        e = of_part(s_occ, q)[n * CHILD_OCC + k];
+        e = of_part(s_occ, q)[n * aa.occ + k];
       }
       const int j = (int)(e & 0xFFFFu), v_old = (int)((e >> 16) & 0x7FFu);
       int ri = j - (int)(rep & 0xFFFFu), rc = have ? j - (int)(rep >> 16) : 0x3fffffff;
@@ -1346,9 +1397,8 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
 #pragma unroll 1
       for (unsigned walk = __ballot_sync(0xffffffffu, !listed && sub == 0); walk; walk &= walk - 1) {
         const int l = __ffs(walk) - 1;
-        const uint32_t cw = __shfl_sync(0xffffffffu, cnt, l);
-        repair_column_any(aa.col, nullptr, cl, __shfl_sync(0xffffffffu, n, l), __shfl_sync(0xffffffffu, tot, l),
-                          (int)(cw & 0xFFFFu), __shfl_sync(0xffffffffu, cap_n, l), lane);
+        repair_crowded(aa, (uint32_t *)&w, s_occ, cl, __shfl_sync(0xffffffffu, n, l), __shfl_sync(0xffffffffu, tot, l),
+                       __shfl_sync(0xffffffffu, cnt, l), __shfl_sync(0xffffffffu, cap_n, l), __shfl_sync(0xffffffffu, rep, l), lane);
         __syncwarp();
       }
     }
@@ -1411,6 +1461,7 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   // a child is split over blocks while that leaves none of them without a place on the GPU and every warp a few rows
   ca.split = 1;
   while (ca.split < CHILD_SPLIT && (long long)count * ca.split * 2 <= 3LL * ctx->num_sms && ca.split * 2 * CHILD_WARPS * 4 <= a.J) ca.split *= 2;
+  ca.occ = std::min(CHILD_CROWD, listed_occupants(ctx, a.mode == ROWS_REPAIR ? ctx->cfg.thr_mutate : a.thr, 256 * CHILD_OCC / NN));
   ca.row_vecs = whole ? NN / 8 : (NN + 14) / 8;
   const int warps = CHILD_WARPS * ca.split, turns = (a.J + 32 * warps - 1) / (32 * warps);
   ca.chunk_rows = (a.J + warps * turns - 1) / (warps * turns);
@@ -1420,7 +1471,7 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)count * (unsigned)ca.split);
   lc.blockDim = dim3(CHILD_WARPS * 32);
-  lc.dynamicSmemBytes = child_smem_bytes(NN, whole);
+  lc.dynamicSmemBytes = child_smem_bytes(NN, ca.occ, whole);
   lc.stream = ctx->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1428,7 +1479,7 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1u;
   lc.attrs = attr;
   lc.numAttrs = ca.split > 1 ? 1 : 0;
-  if (lc.dynamicSmemBytes > 48 * 1024)
+  if (lc.dynamicSmemBytes > 47 * 1024)        // (48 KB need no asking for, the static ones among them)
     SCHED_CUDA_CHECK(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes));
   {
     TimedLaunch tl_(ctx, KK_ROWS);

@@ -2,6 +2,9 @@
 // counter-based stream and the repair's decision for a node.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
 
 static __device__ __noinline__ u32x4 draw_one(uint32_t k0, uint32_t k1, uint32_t idx, uint32_t cand, uint32_t gen, uint32_t slot) {
@@ -82,4 +85,69 @@ __device__ __forceinline__ int decide(int v, bool distributed, bool have, int mo
   }
   if (have && excess > 0) v -= min(v, max(excess - ahead, 0));
   return v;
+}
+
+// What the repair decides for a node with more occupants than decide() takes, by a warp, from their list (bit 31 of an
+// entry: distributed): of the distributed ones the first in rotated order stays; of the GPUs then left, the last that
+// the node has room for stay, in the other rotated order.
+struct CrowdPlaces {
+  int first;                             // place of the distributed occupant that stays, -1: all do
+  int upto, stay;                        // all before the place `upto` leave; of the occupant there `stay` GPUs stay
+  __device__ __forceinline__ int keeps(uint32_t e, int gpus, int place_i, int place_c) const {
+    if (first >= 0 && (e >> 31) && place_i != first) return 0;
+    return place_c < upto ? 0 : place_c == upto ? min(gpus, stay) : gpus;
+  }
+};
+
+// `upto` is found bit by bit, a pass over the list each, so the work grows with the list and not with its square.
+// list(k): its k-th entry; gpus(e), rot_i(e), rot_c(e): an entry's GPUs (below 2048) and its places (below 65536, J of them).
+template <class List, class Gpus, class RotI, class RotC>
+__device__ __forceinline__ CrowdPlaces crowd_places(List list, int count, int J, int tot, bool intf, int cap_n, int lane, Gpus gpus,
+                                                    RotI rot_i, RotC rot_c) {
+  CrowdPlaces at = {-1, -1, 0};
+  const bool one = count <= 32;          // an entry a lane, looked at once
+  const uint32_t e0 = lane < count ? list(lane) : 0u;
+  const int g0 = lane < count ? gpus(e0) : 0;
+  if (intf) {
+    int first = 0x7fffffff, all = 0;
+#pragma unroll 1
+    for (int k = lane; k < count; k += 32) {
+      const uint32_t e = one ? e0 : list(k);
+      if (!(e >> 31)) continue;
+      first = min(first, (rot_i(e) << 11) | gpus(e));
+      all += gpus(e);
+    }
+    first = __reduce_min_sync(0xffffffffu, first);
+    tot -= __reduce_add_sync(0xffffffffu, all) - (first & 0x7FF);
+    at.first = first >> 11;
+  }
+  if (tot <= cap_n) return at;
+  const int v0 = at.keeps(e0, g0, rot_i(e0), 0), place0 = rot_c(e0);
+  auto from = [&](int place) {           // GPUs from there on
+    int sum = place0 >= place ? v0 : 0;
+    if (!one)
+#pragma unroll 1
+      for (int k = lane + 32; k < count; k += 32) {
+        const uint32_t e = list(k);
+        if (rot_c(e) >= place) sum += at.keeps(e, gpus(e), rot_i(e), 0);
+      }
+    return __reduce_add_sync(0xffffffffu, sum);
+  };
+  int upto = 0;
+#pragma unroll 1
+  for (int bit = 1 << (31 - __clz(J)); bit; bit >>= 1)
+    if (from(upto | bit) > cap_n) upto |= bit;
+  const int stay = cap_n - from(upto + 1);
+  at.upto = upto;
+  at.stay = stay;
+  return at;
+}
+
+// How many occupants a node's list should hold, in steps of 16 (what decide() takes) up to `most`: jobs of two GPUs on a
+// full node, what a step brings on average (two of three perturbed rows take a node), and four standard deviations.
+inline int listed_occupants(const sched_ctx *ctx, uint32_t thr, int most) {
+  const double full = std::min(ctx->cap_max, 2 * ctx->cfg.num_jobs) / 2.0;
+  const double mean = ctx->cfg.num_jobs * (thr / 4294967296.0) * (2.0 / 3.0) / ctx->cfg.num_nodes;
+  const double want = std::min(full + mean + 4.0 * std::sqrt(full / 2.0 + mean), 1e6);
+  return std::max(16, std::min(((int)want + 15) & ~15, most & ~15));
 }

@@ -99,3 +99,40 @@ def test_elite_children_of_any_rank(oracle, P, elite, values, nodes):
     assert np.array_equal(out.cpu().numpy(), ref)
     s.sync_status()
     s.close()
+
+
+# nodes, GPUs a node, jobs, children, density: about as many occupants a node as a group of lanes takes (16), as the blocks' lists
+# hold (16 to 768, by the node's size and the rows perturbed), and more; one block and several; nodes larger than what lies on
+# them, and one without any GPUs
+CROWDS = [(1, 3, 17, 3, 1.0), (1, 3, 26, 3, 1.0), (1, 500, 600, 3, 1.0), (1, 500, 680, 3, 1.0), (1, 2047, 700, 1, 1.0), (1, 2047, 1280, 2, 1.0),
+          (3, 8, 2000, 1, 0.3), (3, 8, 2000, 1, 0.45), (8, 0, 200, 4, 0.09), (8, 40, 1024, 2, 0.06), (8, 40, 1024, 2, 0.6),
+          (9, 8, 3000, 300, 0.029), (64, 8, 700, 3, 0.028), (64, 8, 4000, 2, 0.007), (250, 4, 300, 3, 0.06), (256, 4, 300, 3, 0.06),
+          (512, 4, 120, 2, 0.14)]
+
+
+@pytest.mark.parametrize("nodes,gpus,J,P,density", CROWDS)
+def test_crowded_nodes(oracle, nodes, gpus, J, P, density):
+    import torch
+    from paper_2008_12260_b200 import api
+
+    rng = np.random.default_rng(nodes + J)
+    cap = np.full(nodes, max(gpus, 1), np.int16)
+    cap[nodes // 2] = gpus                                  # (0: a node without any)
+    raw = synth.random_raw_population(P, J, synth.Cluster(cap), seed=nodes + J, density=density, v_hi=4)
+    raw[:, :, 0] = rng.integers(0, 3, (P, J))
+    k_max, n_max = 64, min(nodes, 64)
+    k_cap, active = rng.integers(1, 40, J).astype(np.int32), (rng.uniform(size=J) < 0.9).astype(np.uint8)
+    fit, thr, seed = rng.uniform(0.1, 1.0, P).astype(np.float32), synth.prob_to_threshold(0.2), 9
+    s = api.Scheduler(node_capacity=cap, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=thr, thr_init=thr, num_elite=0,
+                      seed=seed, k_max=k_max, n_max=n_max, stream=torch.cuda.current_stream().cuda_stream)
+    dj = api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch)
+    parents, out = torch.from_numpy(raw).cuda(), torch.empty(raw.shape, dtype=torch.int16, device="cuda:0")
+    s.ga_generation(dj, parents, torch.from_numpy(fit).cuda(), out, round=2, generation=3)
+    ref = oracle.ga_generation(raw, fit, cap, k_cap, k_max, n_max, 0, thr, seed, 2, 3, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+    s.repair_population(dj, parents, round=5, generation=6, first_candidate=9)
+    got = parents.cpu().numpy()
+    for c in range(0, P, max(1, P // 4)):
+        assert np.array_equal(got[c], oracle.repair(raw[c], cap, k_cap, k_max, n_max, seed, 5, 9 + c, 6, active=active)), c
+    s.sync_status()
+    s.close()
