@@ -47,8 +47,8 @@ constexpr int LANES = 8;                        // lanes of a row
 constexpr int STASH = 128;                      // perturbed rows of many whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
 constexpr int FLOW_MAX_WARPS = 20;
-constexpr int FLOW_OCC = 16;                    // occupants listed per node: a group of lanes
-constexpr int FLOW_MAX_JOBS = 8192, FLOW_MAX_NODES = 512;
+constexpr int FLOW_OCC = 16;                    // occupants of a node that a group of lanes decides
+constexpr int FLOW_MAX_JOBS = 8192, FLOW_MAX_NODES = 512, FLOW_MAX_SMEM = 220 * 1024;
 constexpr int RANK_PAIRS = 64;                 // keys that are ranked by comparing them with one another
 
 // Kinds of the generation kernel.  Not MANY: the child's records and what its rows' terms are made of are kept in shared
@@ -56,10 +56,14 @@ constexpr int RANK_PAIRS = 64;                 // keys that are ranked by compar
 // 1024 jobs.  Registers: 142 for FEW_ALONE's 12 warps (testbed round 490 us; 522 with 96, 555 with 64, that is with
 // spills, which lie in the L1 that every acquire empties), 96 for SOME_ALONE's 20 (12 warps for 881 jobs: 826 us, 20: 730),
 // 64 for FEW, 56 for MANY.
-constexpr int FEW_ALONE = 0, SOME_ALONE = 1, FEW = 2, MANY = 3;
-__host__ __device__ constexpr bool few(int kind) { return kind != MANY; }
-__host__ __device__ constexpr int kind_threads(int kind) { return kind == FEW_ALONE ? 384 : kind == SOME_ALONE ? 640 : kind == FEW ? 512 : 288; }
-__host__ __device__ constexpr int kind_blocks(int kind) { return kind == MANY ? 4 : kind == FEW ? 2 : 1; }
+// CROWDED, with any of them: lists longer than a group of lanes, where so many occupants of a node are to be expected.
+constexpr int FEW_ALONE = 0, SOME_ALONE = 1, FEW = 2, MANY = 3, CROWDED = 4;
+__host__ __device__ constexpr int shape_of(int kind) { return kind & 3; }
+__host__ __device__ constexpr bool few(int kind) { return shape_of(kind) != MANY; }
+__host__ __device__ constexpr int kind_threads(int kind) {
+  return shape_of(kind) == FEW_ALONE ? 384 : shape_of(kind) == SOME_ALONE ? 640 : shape_of(kind) == FEW ? 512 : 288;
+}
+__host__ __device__ constexpr int kind_blocks(int kind) { return shape_of(kind) == MANY ? 4 : shape_of(kind) == FEW ? 2 : 1; }
 
 __host__ __device__ inline int wide_stride(int NN) { return (NN + 7) & ~7; }
 __host__ __device__ inline int stash_rows(int J) { return J <= SMEM_RECORDS ? J : STASH; }
@@ -83,7 +87,7 @@ constexpr uint32_t NEVER = 0xFFFFFFFDu;
 
 // Places in the generation kernel's shared memory, behind what the warps tell each other (terms: -1 where they are not kept there).
 struct FlowSmem {
-  int act, term, info, node, occ, viol, cap, rack, mut, mod, wide, slow, stash, flag, dense, rep, keys, sums, scratch, rec, same,
+  int act, term, info, node, occ, more, viol, cap, rack, mut, mod, wide, slow, stash, flag, dense, rep, keys, sums, scratch, rec, same,
       terms, total;
 };
 
@@ -102,6 +106,7 @@ struct FlowArgs {
   const int32_t *nmin;       // [k_max + 1] fewest nodes, two or more, that K replicas fit on
   int P, J, NN, k_max, n_max, num_elite, generations;
   int warps;                 // warps that work on the rows; the others draw
+  int more;                  // occupants listed per node beyond FLOW_OCC
   int classes;               // 2, or 3 with racks
   FlowSmem at;
   uint32_t thr_init, thr_mutate;
@@ -322,6 +327,7 @@ __global__ void __launch_bounds__(128) flow_build_kernel(FlowArgs a) {
 constexpr int INFO_DIST = 1;        // the row spanned two nodes or more after the row pass (interference snapshot)
 constexpr int INFO_CHANGED = 2;     // a node's decision changes it
 constexpr int INFO_WIDE = 4;
+constexpr int INFO_AGAIN = 8;       // a crowded node's decision changes it
 
 // The candidate a block is working on.
 struct Work {
@@ -351,6 +357,7 @@ struct FlowView {
   uint8_t *info;                      // by row
   uint32_t *node;                     // by node: GPUs placed on it; distributed jobs on it | occupants << 16
   uint32_t *occ;                      // row | GPUs << 13 | place in the record (7: wide) << 25 | distributed << 31
+  uint32_t *more;                     // those that do not fit
   uint8_t *viol;                      // the node's column is to be walked
   int16_t *cap, *rack;
   uint16_t *mut, *mod, *wide, *slow;  // mut: two sets
@@ -370,7 +377,7 @@ __device__ __forceinline__ FlowView flow_view(const FlowArgs &a, uint32_t memory
   const FlowSmem &L = a.at;
   unsigned char *const s = (unsigned char *)__cvta_shared_to_generic(memory);
   return FlowView{*(FlowCtl *)s, (uint16_t *)(s + L.act), (float *)(s + L.term), s + L.info, (uint32_t *)(s + L.node),
-                  (uint32_t *)(s + L.occ), s + L.viol, (int16_t *)(s + L.cap), (int16_t *)(s + L.rack),
+                  (uint32_t *)(s + L.occ), (uint32_t *)(s + L.more), s + L.viol, (int16_t *)(s + L.cap), (int16_t *)(s + L.rack),
                   (uint16_t *)(s + L.mut), (uint16_t *)(s + L.mod), (uint16_t *)(s + L.wide), (uint16_t *)(s + L.slow),
                   (uint4 *)(s + L.stash), s + L.flag, (int16_t *)(s + L.dense), (uint32_t *)(s + L.rep), (uint32_t *)(s + L.keys),
                   (double *)(s + L.sums), (uint32_t *)(s + L.scratch), (uint32_t *)(s + L.rec), (uint32_t *)(s + L.same),
@@ -519,13 +526,16 @@ __device__ __forceinline__ int row_sum(int v) {
 }
 
 // a row's occupant into the nodes' totals and lists
+template <int KIND>
 __device__ __forceinline__ void add_occupant(const FlowArgs &a, const FlowView &v, int jc, int k_rec, uint32_t e, bool dist) {
   const int n = entry_node(e);
   if (!sched_index_ok(a.status, n < a.NN && jc < a.J && entry_gpus(e) <= 2047, SCHED_CHK_NODE)) return;
   atomicAdd(&v.node[2 * n], (uint32_t)entry_gpus(e));
   const uint32_t k = atomicAdd(&v.node[2 * n + 1], (dist ? 1u : 0u) | (1u << 16)) >> 16;
-  if (k < (uint32_t)FLOW_OCC)
-    v.occ[n * FLOW_OCC + k] = (uint32_t)jc | ((uint32_t)entry_gpus(e) << 13) | ((uint32_t)k_rec << 25) | (dist ? 0x80000000u : 0u);
+  auto entry = [&] { return (uint32_t)jc | ((uint32_t)entry_gpus(e) << 13) | ((uint32_t)k_rec << 25) | (dist ? 0x80000000u : 0u); };
+  if (k < (uint32_t)FLOW_OCC) v.occ[n * FLOW_OCC + k] = entry();
+  else if constexpr ((KIND & CROWDED) != 0)
+    if (k < (uint32_t)(FLOW_OCC + a.more)) v.more[n * a.more + (int)k - FLOW_OCC] = entry();
 }
 
 // A word of a finished row goes to its place: the child's records, the term by job.
@@ -570,7 +580,7 @@ __device__ __forceinline__ void settle_row(const FlowArgs &a, const FlowView &v,
   const bool equal = (row_bits(word == same, lane) & 0x3Fu) == 0x3Fu;
   if (live) {
     put_word<KIND>(a, v, dst, jc, k, k < ENTRIES ? word : k == REC_TERM ? (equal ? unchanged : __float_as_uint(changed)) : 0u);
-    if (fresh && k < ENTRIES && word != NO_NODE) add_occupant(a, v, jc, k, word, N >= 2);
+    if (fresh && k < ENTRIES && word != NO_NODE) add_occupant<KIND>(a, v, jc, k, word, N >= 2);
     if (fresh && k == 0) v.info[jc] = N >= 2 ? INFO_DIST : 0;
   }
   __syncwarp();
@@ -754,7 +764,7 @@ __device__ __noinline__ void wide_rows(const FlowArgs &a, uint32_t memory, Work 
       const int n = n0 + lane, e = n < NN ? (int)dense[n] : 0;
       const unsigned m = __ballot_sync(0xffffffffu, e > 0);
       const int k = before + __popc(m & ((1u << lane) - 1u));
-      if (e > 0) add_occupant(a, v, jc, wide ? 7 : k, ((uint32_t)n << 16) | (uint32_t)e, dist);
+      if (e > 0) add_occupant<KIND>(a, v, jc, wide ? 7 : k, ((uint32_t)n << 16) | (uint32_t)e, dist);
       before += __popc(m);
     }
     __syncwarp();
@@ -770,6 +780,27 @@ __device__ __forceinline__ void set_entry(const FlowArgs &a, const FlowView &v, 
   if (k == 7) wide_row(a, dst + jc)[n] = (int16_t)gpus;
   else if (few(KIND)) v.rec[jc * REC_WORDS + k] = e;
   else rec_row(a, dst + jc)[k] = e;
+}
+
+// A row into the list of those that decisions have changed, once.
+__device__ __forceinline__ void add_changed(const FlowView &v, int jc, int flag, int J, int *status) {
+  // (bytes, so the word around it is updated as a whole)
+  const uint32_t bit = (uint32_t)flag << (8 * (jc & 3));
+  if ((atomicOr((uint32_t *)v.info + (jc >> 2), bit) & bit) == 0u) {
+    const int at = atomicAdd(&v.ctl.nmod, 1);
+    if (sched_index_ok(status, at < J, SCHED_CHK_LIST)) v.mod[at] = (uint16_t)jc;
+  }
+}
+
+// Place of a node in a finished row: of its record, 7: the row is wide.
+template <int KIND>
+__device__ __forceinline__ int place_of(const FlowArgs &a, const FlowView &v, int dst, int jc, int n) {
+  if (v.info[jc] & INFO_WIDE) return 7;
+  const Record rec = load_record(rec_row(a, dst + jc));
+  int k = 7;
+#pragma unroll
+  for (int z = 0; z < ENTRIES; ++z) k = entry_node(rec.w[z]) == n ? z : k;
+  return k;
 }
 
 // Nodes with more occupants than a list holds: the warps walk the column, node by node.  Thread t looks after the
@@ -835,13 +866,7 @@ __device__ __noinline__ void walk_columns(const FlowArgs &a, uint32_t memory, in
       running += g_eff;
       v.mod[jc] = g_eff - take == g ? 0 : 1;
       if (g_eff - take != g) {            // into the row
-        int k = 7;
-        if (!(v.info[jc] & INFO_WIDE)) {
-          const Record rec = load_record(rec_row(a, dst + jc));
-#pragma unroll
-          for (int z = 0; z < ENTRIES; ++z) k = entry_node(rec.w[z]) == n ? z : k;
-        }
-        set_entry<KIND>(a, v, dst, jc, k, n, g_eff - take);
+        set_entry<KIND>(a, v, dst, jc, place_of<KIND>(a, v, dst, jc, n), n, g_eff - take);
       }
     }
     bar(BAR_ROWS, threads);
@@ -857,6 +882,62 @@ __device__ __noinline__ void walk_columns(const FlowArgs &a, uint32_t memory, in
       if (v.mod[jc] && (v.info[jc] & INFO_WIDE)) finish_wide<KIND>(a, memory, dst, jc, warp, lane);
     bar(BAR_ROWS, threads);
   }
+}
+
+// Nodes with more occupants than a group of lanes has: by a warp each, from their lists, and the rows that this
+// changes; then the nodes whose lists are too short.  Behind the other nodes' rows, so that a generation without such
+// nodes does not have it on its way.
+template <int KIND>
+__device__ __noinline__ void crowded_nodes(const FlowArgs &a, uint32_t memory, int dst, int set, int JA, int warp, int lane) {
+  const FlowView v = flow_view(a, memory);
+  const int threads = a.warps * 32;
+  bar(BAR_ROWS, threads);                     // (the rows of the other nodes are finished)
+  if (threadIdx.x == 0) v.ctl.nmod = 0;
+  bar(BAR_ROWS, threads);
+#pragma unroll 1
+  for (int n = warp; n < a.NN; n += a.warps) {
+    if (!v.viol[n]) continue;
+    const uint2 here = ((const uint2 *)v.node)[n];
+    const int count = (int)(here.y >> 16);
+    if (count > FLOW_OCC + a.more) {
+      if (lane == 0) v.ctl.walk = 2;
+      continue;
+    }
+    const uint32_t rep = v.rep[set * a.NN + n];
+    auto list = [&](int i) { return i < FLOW_OCC ? v.occ[n * FLOW_OCC + i] : v.more[n * a.more + i - FLOW_OCC]; };
+    auto gpus = [&](uint32_t e) { return (int)((e >> 13) & 0x7FFu); };
+    auto place = [&](uint32_t e, uint32_t offset) {
+      const int jc = (int)(e & 0x1FFFu), r = (sched_index_ok(a.status, jc < a.J, SCHED_CHK_LIST) ? (int)v.act[jc] : 0) - (int)offset;
+      return r < 0 ? r + a.J : r;
+    };
+    auto rot_i = [&](uint32_t e) { return place(e, rep & 0xFFFFu); };
+    auto rot_c = [&](uint32_t e) { return place(e, rep >> 16); };
+    const CrowdPlaces at = crowd_places(list, count, a.J, (int)here.x, (here.y & 0xFFFFu) >= 2u, (int)v.cap[n], lane, gpus, rot_i, rot_c);
+#pragma unroll 1
+    for (int i = lane; i < count; i += 32) {
+      const uint32_t e = list(i);
+      const int jc = (int)(e & 0x1FFFu), keeps = at.keeps(e, gpus(e), rot_i(e), rot_c(e));
+      if (keeps == gpus(e)) continue;
+      set_entry<KIND>(a, v, dst, jc, place_of<KIND>(a, v, dst, jc, n), n, keeps);
+      add_changed(v, jc, INFO_AGAIN, a.J, a.status);
+    }
+    __syncwarp();
+    if (lane == 0) v.viol[n] = 0;
+  }
+  bar(BAR_ROWS, threads);
+  const int nmod = v.ctl.nmod;
+#pragma unroll 1
+  for (int i0 = warp * 4; i0 < nmod; i0 += a.warps * 4) {
+    const int jc = v.mod[min(i0 + (lane >> 3), nmod - 1)];
+    finish_row<KIND>(a, v, dst, jc, i0 + (lane >> 3) < nmod && !(v.info[jc] & INFO_WIDE), warp, lane);
+  }
+  bar(BAR_ROWS, threads);                     // (a wide one may turn into a record: not to be taken for one above)
+#pragma unroll 1
+  for (int i = warp; i < nmod; i += a.warps) {
+    const int jc = v.mod[i];
+    if (v.info[jc] & INFO_WIDE) finish_wide<KIND>(a, memory, dst, jc, warp, lane);
+  }
+  if (v.ctl.walk == 2) walk_columns<KIND>(a, memory, dst, set, JA, warp, lane);
 }
 
 // An elite child: the records (and contents) of the candidate of its rank, as they are.
@@ -1081,7 +1162,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
     const int nmut = v.ctl.nmut[set];
 #pragma unroll 1
     for (int x = (W - 1 - warp) * 4; x < nmut; x += W * 4) perturb_rows<KIND>(a, v, w, round, set, x, nmut, warp, lane);
-    constexpr int RB = KIND == SOME_ALONE || KIND == MANY ? 2 : 1;       // rows of a thread whose loads travel together
+    constexpr int RB = shape_of(KIND) == SOME_ALONE || shape_of(KIND) == MANY ? 2 : 1;       // rows of a thread whose loads travel together
 #pragma unroll 1
     for (int jc0 = tid; jc0 < JA; jc0 += RB * threads) {
       Record rec[RB];
@@ -1108,14 +1189,14 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
         }
         const bool dist = rec[q].w[1] != NO_NODE;
         v.info[jc] = dist ? INFO_DIST : 0;
-        if (rec[q].w[0] != NO_NODE) add_occupant(a, v, jc, 0, rec[q].w[0], dist);
+        if (rec[q].w[0] != NO_NODE) add_occupant<KIND>(a, v, jc, 0, rec[q].w[0], dist);
 #pragma unroll 1
         for (int x = 1; x < ENTRIES; ++x) {           // (few rows have more: one copy of the code)
           uint32_t e = rec[q].w[1];
 #pragma unroll
           for (int z = 2; z < ENTRIES; ++z) e = z == x ? rec[q].w[z] : e;
           if (e == NO_NODE) break;
-          add_occupant(a, v, jc, x, e, dist);
+          add_occupant<KIND>(a, v, jc, x, e, dist);
         }
       }
     }
@@ -1149,7 +1230,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
         const uint2 here = ((const uint2 *)v.node)[n];
         const uint32_t rep = v.rep[set * NN + n], e = v.occ[n * FLOW_OCC + sub];
         const int count = b >= 0 ? (int)(here.y >> 16) : 0, cap_n = (int)v.cap[n];
-        const bool listed = count <= FLOW_OCC, have = listed && sub < count;   // else: walked below
+        const bool listed = count <= FLOW_OCC, have = listed && sub < count;   // else: below
         const int jc = have ? (int)(e & 0x1FFFu) : 0, had = have ? (int)((e >> 13) & 0x7FFu) : 0;
         const int j = sched_index_ok(a.status, jc < JA, SCHED_CHK_LIST) ? (int)v.act[jc] : 0;
         int ri = j - (int)(rep & 0xFFFFu), rc = j - (int)(rep >> 16);
@@ -1159,12 +1240,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
         const int keeps = decide(had, (e >> 31) != 0u, have, min(most, FLOW_OCC), (here.y & 0xFFFFu) >= 2u, (int)here.x, cap_n, ri, rc);
         if (have && keeps != had) {
           set_entry<KIND>(a, v, w.dst, jc, (int)((e >> 25) & 7u), n, keeps);
-          // (bytes, so the word around it is updated as a whole)
-          const uint32_t bit = (uint32_t)INFO_CHANGED << (8 * (jc & 3));
-          if ((atomicOr((uint32_t *)v.info + (jc >> 2), bit) & bit) == 0u) {
-            const int at = atomicAdd(&v.ctl.nmod, 1);
-            if (sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) v.mod[at] = (uint16_t)jc;
-          }
+          add_changed(v, jc, INFO_CHANGED, J, a.status);
         }
         if (b >= 0 && sub == 0 && !listed) { v.viol[n] = 1; v.ctl.walk = 1; }
         __syncwarp();
@@ -1187,7 +1263,8 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
         if (v.info[jc] & INFO_WIDE) finish_wide<KIND>(a, memory, w.dst, jc, warp, lane);
       }
     }
-    if (walk) walk_columns<KIND>(a, memory, w.dst, set, JA, warp, lane);
+    if (walk && (KIND & CROWDED)) crowded_nodes<KIND>(a, memory, w.dst, set, JA, warp, lane);
+    else if (walk) walk_columns<KIND>(a, memory, w.dst, set, JA, warp, lane);
     bar(BAR_ROWS, threads);
 
     // ---- fitness (Eq. 14) from the rows' terms, in the order of the dense kernel: per chunk of rows, thread
@@ -1202,7 +1279,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
         asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(pub_of(s, c)), "l"(word) : "memory");   // (behind this thread's fence)
       }
     } else {
-      constexpr bool ONE = KIND == FEW_ALONE;     // (up to 256 rows: one chunk, a row a thread)
+      constexpr bool ONE = shape_of(KIND) == FEW_ALONE;     // (up to 256 rows: one chunk, a row a thread)
       const int chunks = ONE ? 1 : a.chunks;
 #pragma unroll 1
       for (int x = warp; x < chunks * nv; x += W - 1) {
@@ -1385,7 +1462,7 @@ int flow_kind(const sched_ctx *ctx) {
   return two && 83 * J + 115 * NN + 6 * P <= 96 * 1024 ? FEW : MANY;      // (what two blocks find room for on an SM)
 }
 
-FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms) {
+FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms, int more) {
   const sched_config &c = ctx->cfg;
   const int J = c.num_jobs, NN = c.num_nodes, P = c.population;
   int rows, chunks, off = 0;
@@ -1402,6 +1479,7 @@ FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms) {
   L.info = take((size_t)J);
   L.node = take((size_t)NN * 8);
   L.occ = take((size_t)NN * FLOW_OCC * 4);
+  L.more = take((size_t)NN * more * 4);
   L.viol = take((size_t)NN);
   L.cap = take((size_t)NN * 2);
   L.rack = take(ctx->d_rack ? (size_t)NN * 2 : 0);
@@ -1425,14 +1503,32 @@ FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms) {
 
 // The launch's shape.
 struct FlowShape {
-  int warps, draw_warps, blocks;
+  int warps, draw_warps, blocks, more;
   FlowSmem at;
 };
 
 using FlowKernel = void (*)(FlowArgs);
-FlowKernel flow_kernel_for(const sched_ctx *ctx) {
-  const int kind = flow_kind(ctx);
-  return kind == MANY ? flow_kernel<MANY> : kind == FEW ? flow_kernel<FEW> : kind == SOME_ALONE ? flow_kernel<SOME_ALONE> : flow_kernel<FEW_ALONE>;
+FlowKernel flow_kernel_for(const sched_ctx *ctx, bool crowded) {
+  switch (flow_kind(ctx) | (crowded ? CROWDED : 0)) {
+    case FEW_ALONE: return flow_kernel<FEW_ALONE>;
+    case SOME_ALONE: return flow_kernel<SOME_ALONE>;
+    case FEW: return flow_kernel<FEW>;
+    case MANY: return flow_kernel<MANY>;
+    case FEW_ALONE | CROWDED: return flow_kernel<FEW_ALONE | CROWDED>;
+    case SOME_ALONE | CROWDED: return flow_kernel<SOME_ALONE | CROWDED>;
+    case FEW | CROWDED: return flow_kernel<FEW | CROWDED>;
+    default: return flow_kernel<MANY | CROWDED>;
+  }
+}
+
+// What a node's list should hold beyond FLOW_OCC occupants, by the rows that a step (the initial population, too)
+// perturbs, in at most 16 KB.  A node with more than its list holds is walked, row by row, by the whole block.  60
+// generations with lists of 16 and with these (us): a fifth of the rows perturbed, 8 nodes x 1024 jobs x 300 candidates
+// 6435 -> 1679, 16 x 1024 x 512 2729 -> 1840, 4 x 300 x 512 1083 -> 773; a fiftieth, but three of ten at first, 4 x 1024 x 512
+// 1032 -> 870, 8 x 512 x 148 388 -> 385.  Where crowds are rare they cost up to 2 % (8 x 300 x 297 450 -> 459).
+int flow_more(const sched_ctx *ctx) {
+  const sched_config &c = ctx->cfg;
+  return listed_occupants(ctx, std::max(c.thr_mutate, c.thr_init), 256 * FLOW_OCC / c.num_nodes) - FLOW_OCC;
 }
 
 // A block for every candidate if they fit the GPU.  Warps that work on rows and warps that draw, measured: testbed (48 jobs)
@@ -1451,11 +1547,16 @@ FlowShape flow_shape(const sched_ctx *ctx) {
     case SOME_ALONE: warps = 16; draw = 4; break;
     default: warps = 8; draw = 4; break;
   }
-  for (int terms = few ? 1 : 0; terms >= 0; --terms) {
-    FlowShape f = {warps, draw, 0, flow_smem(ctx, warps, terms != 0)};
+  for (int x = few ? 3 : 1; x >= 0 && best.blocks < c.population; --x) {      // terms and long lists, terms, long lists, neither
+    const bool terms = (x & 2) != 0;
+    const int more = (x & 1) ? flow_more(ctx) : 0;
+    if ((x & 1) && more == 0) continue;
+    FlowShape f = {warps, draw, 0, more, flow_smem(ctx, warps, terms, more)};
+    const FlowKernel kernel = flow_kernel_for(ctx, more > 0);
     int fit = 0;
-    if (f.at.total > 220 * 1024 ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, flow_kernel_for(ctx), (warps + draw) * 32, f.at.total) != cudaSuccess) {
+    if (f.at.total > FLOW_MAX_SMEM ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_MAX_SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, (warps + draw) * 32, f.at.total) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -1477,8 +1578,7 @@ int round_flow_ensure(sched_ctx *ctx) {
   if (2 * rows > ctx->rs_budget) return SCHED_OK;
   if ((long long)(DEPTH + 1) * c.population * c.num_jobs >= 1ll << 31) return SCHED_OK;      // (rows are counted in 32 bits)
   int coop = 0, blocks = 0;
-  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop ||
-      cudaFuncSetAttribute(flow_kernel_for(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess) {
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop) {
     cudaGetLastError();
     return SCHED_OK;
   }
@@ -1488,6 +1588,7 @@ int round_flow_ensure(sched_ctx *ctx) {
   ctx->fl_warps = shape.warps;
   ctx->fl_draw_warps = shape.draw_warps;
   ctx->fl_terms = shape.at.terms >= 0;
+  ctx->fl_more = shape.more;
   const FlowArena size = flow_arena(ctx, nullptr);
   if (cudaMalloc((void **)&ctx->fl_arena, size.total) != cudaSuccess) {
     cudaGetLastError();
@@ -1551,7 +1652,8 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   FlowArgs a = flow_args(ctx, jobs, d_cur);
   a.generations = generations;
   a.warps = ctx->fl_warps;
-  a.at = flow_smem(ctx, ctx->fl_warps, ctx->fl_terms);
+  a.more = ctx->fl_more;
+  a.at = flow_smem(ctx, ctx->fl_warps, ctx->fl_terms, ctx->fl_more);
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
     TimedLaunch tl_(ctx, KK_FLOW_BUILD);
@@ -1571,7 +1673,7 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   lc.numAttrs = 1;
   {
     TimedLaunch tl_(ctx, KK_FLOW);
-    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, flow_kernel_for(ctx), a));
+    SCHED_CUDA_CHECK(ctx, cudaLaunchKernelEx(&lc, flow_kernel_for(ctx, ctx->fl_more > 0), a));
   }
   SCHED_LAUNCH_CHECK(ctx);
   {

@@ -22,6 +22,20 @@ def test_rounds_at_the_kinds_edges(shape, start):
     shapes.test_round_equals_stepwise("flow", shape, start)
 
 
+# nodes with more occupants than a group of lanes takes, in every kind of block: within the lists, beyond them (many GPUs a
+# node and rows everywhere), with racks, inactive jobs and rows of more nodes than a record holds
+CROWDS = [
+    (3, 8, 200, 40, 5, 0, 1.0, 0.5), (4, 4, 900, 30, 4, 2, 0.8, 0.3), (4, 4, 300, 200, 3, 0, 1.0, 0.3), (4, 8, 1100, 160, 3, 0, 1.0, 0.2),
+    (2, 300, 1300, 20, 3, 0, 1.0, 0.3), (2, 300, 250, 200, 3, 1, 1.0, 0.3), (20, 2, 250, 100, 12, 5, 1.0, 0.9), (20, 2, 250, 460, 6, 0, 1.0, 0.9),
+]
+
+
+@pytest.mark.parametrize("shape", CROWDS, ids=lambda s: "-".join(str(x) for x in s))
+@pytest.mark.parametrize("start", ["none", "feasible", "raw"])
+def test_rounds_with_crowded_nodes(shape, start):
+    shapes.test_round_equals_stepwise("flow", shape, start)
+
+
 # candidates, elite children, share of rows perturbed at first and per generation: ranks of few keys above the bound, of
 # more (ties in a converged population), of as many as there are, and ranks beyond a warp's lanes
 @pytest.mark.parametrize("P,elite,init,mutate", [(64, 4, 0.0, 0.0), (65, 31, 0.0, 0.0), (300, 16, 0.01, 0.0), (300, 31, 0.01, 0.01),
