@@ -65,11 +65,13 @@ def store_budget(cfg):
     return budget
 
 
-def check_route(s, route):
+def check_route(s, route, summaries=False):
     """What a round ran on, from the kernel timing that was on meanwhile ("flow": the one-launch search,
-    "store": the row pool)."""
+    "store": the row pool, "dense": dense matrices, with the batched rows and the work-list repair behind them where
+    the fitness is computed from row summaries)."""
     ran = {name for name, (ms, n) in s.read_kernel_timing().items() if n}
-    assert ("round_search" in ran, "generation_store" in ran, "rows" in ran) == (route == "flow", route == "store", False)
+    assert (("round_search" in ran, "generation_store" in ran, "rows" in ran, "cols" in ran)
+            == (route == "flow", route == "store", route == "dense", route == "dense" and summaries))
 
 
 def feasible(A, cap, k_cap, n_max):

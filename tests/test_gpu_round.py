@@ -81,9 +81,8 @@ def test_round_equals_stepwise_calls_and_oracle_fitness(gpu, oracle, cfg):
 
 
 def test_large_config_round_equals_stepwise(gpu, oracle):
-    """The large configuration (batched row kernel, work-list column repair, fitness from row
-    summaries) for three generations: the round must equal the entry points called one by one,
-    whose fitness reads the dense matrices; the final fitness is checked against the oracle on a
+    """The large configuration for three generations: the round (the one-launch search) must equal the entry
+    points called one by one, which work on dense matrices; the final fitness is checked against the oracle on a
     sample of candidates."""
     torch, api = gpu
     cfg = synth.LARGE

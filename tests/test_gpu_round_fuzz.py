@@ -1,5 +1,5 @@
 """Randomly drawn problem shapes through a whole round: the round's specialised kernels (the one-launch
-search, the row store) against the same round made of the dense entry points
+search, the row store, the batched dense kernels) against the same round made of the dense entry points
 called one by one - populations and fitness bit for bit - and the last generation against the
 oracle.  Shapes, probabilities, the current allocation (none / feasible / breaking every rule),
 inactive jobs and small replica caps all vary with the seed.  POLLUX_FUZZ_CASES raises the number
@@ -43,7 +43,7 @@ def gpu():
     return torch, api
 
 
-@pytest.mark.parametrize("route", ["flow", "store"])
+@pytest.mark.parametrize("route", ["flow", "store", "dense"])
 @pytest.mark.parametrize("seed", range(N_CASES))
 def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed, route):
     torch, api = gpu
@@ -69,8 +69,8 @@ def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed, route):
     penalise = cur is not None
     rnd = int(g.integers(0, 5))
     s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
-    if route == "store":
-        s.set_store_budget(store_budget(cfg))
+    if route != "flow":
+        s.set_store_budget(store_budget(cfg) if route == "store" else 0)
     s.set_kernel_timing(True)
     dj = api.DeviceJobs(jobs, "cuda:0", torch)
     d_cur = None if cur is None else torch.from_numpy(cur).cuda()
@@ -78,7 +78,7 @@ def test_random_round_equals_dense_stepwise_round(gpu, oracle, seed, route):
     bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
     s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=cfg.generations)
     s.sync_status()
-    check_route(s, route)
+    check_route(s, route, summaries=True)
     s.set_kernel_timing(False)
     pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
     fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")

@@ -1,6 +1,7 @@
 """Inside a round the generations run on specialised kernels: one launch that keeps four generations of
 row records, or, where a budget leaves no room for those, shared rows (indices into a row pool, copy
-on write; a launch per generation).  Every case runs on both.  Either way the round must equal,
+on write; a launch per generation), or, with no budget at all, dense matrices with a summary per row.  Every case runs on
+all three.  Either way the round must equal,
 bit for bit, the same round made of the dense entry points called one by one, which the other
 tests pin to the oracle; the last generation is also checked against the oracle directly
 (teacher-forced)."""
@@ -90,7 +91,7 @@ def _stepwise(torch, s, dj, cfg, d_cur, rnd, gens, penalise):
     return a.cpu().numpy(), f.cpu().numpy(), sp.cpu().numpy(), prev
 
 
-@pytest.mark.parametrize("route", ["flow", "store"])
+@pytest.mark.parametrize("route", ["flow", "store", "dense"])
 @pytest.mark.parametrize("cfg", CASES, ids=lambda c: c.name)
 def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg, route):
     torch, api = gpu
@@ -109,8 +110,8 @@ def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg, route):
     penalise = cur is not None
     rnd = 3
     s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
-    if route == "store":
-        s.set_store_budget(store_budget(cfg))
+    if route != "flow":
+        s.set_store_budget(store_budget(cfg) if route == "store" else 0)
     s.set_kernel_timing(True)
     dj = api.DeviceJobs(jobs, "cuda:0", torch)
     d_cur = None if cur is None else torch.from_numpy(cur).cuda()
@@ -118,7 +119,7 @@ def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg, route):
     bf = torch.zeros(1, dtype=torch.float32, device="cuda:0")
     s.schedule_round(dj, d_cur, best, bf, round=rnd, generations=cfg.generations)
     s.sync_status()
-    check_route(s, route)
+    check_route(s, route, summaries=True)
     s.set_kernel_timing(False)
     pop = torch.empty((cfg.population, cfg.num_jobs, cfg.num_nodes), dtype=torch.int16, device="cuda:0")
     fit = torch.empty(cfg.population, dtype=torch.float32, device="cuda:0")
@@ -134,7 +135,7 @@ def test_store_round_equals_dense_stepwise_round(gpu, oracle, cfg, route):
         assert feasible(pop[c], cl.node_capacity, jobs.k_cap, cl.n_max)
     if route == "store" and cfg.name in ("store-compaction", "store-all-perturbed"):
         assert s.store_moves() >= 3
-    elif route == "flow":
+    elif route != "store":
         assert s.store_moves() == 0
     if cfg.name == "store-crowded-nodes":
         assert (pop > 0).sum(axis=1).max() > 16      # more jobs on a node than a block lists

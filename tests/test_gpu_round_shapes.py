@@ -1,6 +1,6 @@
 """Rounds at the shapes where their kernels change: node counts that are no multiple of a row's
 pieces, racks, few and many jobs, inactive jobs, populations larger than the GPU holds blocks, elites; in one
-launch and, where a budget can ask for it, on the row store.  A round must equal, bit for bit, the same round
+launch, where a budget can ask for it on the row store, and without any budget on dense matrices.  A round must equal, bit for bit, the same round
 made of the dense entry points called one by one (which other tests pin to the oracle)."""
 import numpy as np
 import pytest
@@ -23,7 +23,8 @@ SHAPES = [
 ]
 
 
-@pytest.mark.parametrize("route,shape", [("flow", s) for s in SHAPES] + [("store", s) for s in SHAPES if s[2] > 48],
+@pytest.mark.parametrize("route,shape", [("flow", s) for s in SHAPES] + [("store", s) for s in SHAPES if s[2] > 48] +
+                         [("dense", s) for s in SHAPES],
                          ids=lambda s: s if isinstance(s, str) else "-".join(str(x) for x in s))
 @pytest.mark.parametrize("start", ["none", "feasible", "raw"])
 def test_round_equals_stepwise(route, shape, start):
@@ -48,8 +49,8 @@ def test_round_equals_stepwise(route, shape, start):
         cur = synth.random_raw_population(1, J, cl, 6, density=0.3, v_hi=2 * gpn)[0]
     dev = "cuda"
     s = api.scheduler_for(cfg, stream=torch.cuda.current_stream().cuda_stream)
-    if route == "store":
-        s.set_store_budget(store_budget(cfg))
+    if route != "flow":
+        s.set_store_budget(store_budget(cfg) if route == "store" else 0)
     s.set_kernel_timing(True)
     dj = api.DeviceJobs(jobs, dev, torch)
     ar, br = (torch.from_numpy(x).cuda() for x in synth.draw_rack_pair(jobs, 9))
@@ -62,7 +63,7 @@ def test_round_equals_stepwise(route, shape, start):
     fit = torch.empty(P, dtype=torch.float32, device=dev)
     s.schedule_round(dj, d_cur, best, bf, round=2, generations=gens)
     s.sync_status()
-    check_route(s, route)
+    check_route(s, route, summaries=NN % 8 == 0 and not per_rack)
     s.set_kernel_timing(False)
     s.get_population(pop, fit)
 
