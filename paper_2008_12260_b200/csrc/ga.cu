@@ -5,9 +5,10 @@
 //
 // Implementations of the same operators on dense matrices, chosen by shape:
 //  * child_kernel: one launch, a block or a cluster of blocks per child, rows of any width up to 512 nodes (the
-//    entry points called on their own);
-//  * rows2_kernel + colrepair_kernel: rows of whole 16-byte vectors and at most 512 nodes, with per-row summaries -
-//    batched rows with fused column sums and occupant lists, a work list of violating nodes;
+//    entry points called on their own, and dense rounds without summaries);
+//  * rows2_kernel + colrepair_kernel: rows of whole 16-byte vectors and at most 512 nodes, with per-row summaries or
+//    more jobs than child_kernel's counters hold - batched rows with fused column sums and occupant lists, a work list of
+//    violating nodes;
 //  * rows_kernel + cols_kernel (+ rank_kernel): the general pair - a warp per (candidate, job)
 //    row through shared memory, then a thread per (candidate, node) column.
 // Rounds do not use dense matrices for their generations (round_flow.cu, rowstore.cu) unless neither the
@@ -1492,7 +1493,8 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
 // Row pass + column pass of `count` candidates.  Rounds on dense matrices want per-row summaries: rows of whole
 // 16-byte vectors take the batched kernels with fused column sums.  Without summaries every width takes a block (or
 // a few) per child, up to 512 nodes (a tile holds two rows), sizes <= 2047 (an occupant's word) and 65535 jobs (a
-// node's counters); beyond those the general warp-per-row / thread-per-column pair.
+// node's counters); with more jobs, rows of whole vectors take the batched kernels, too (up to 2^20 jobs: an occupant's
+// word there).  What is left takes the general warp-per-row / thread-per-column pair.
 int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint32_t first_cand, uint32_t gen) {
   if (count == 0 || a.J == 0) return SCHED_OK;
   const int NN = a.num_nodes;

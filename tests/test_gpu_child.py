@@ -136,3 +136,39 @@ def test_crowded_nodes(oracle, nodes, gpus, J, P, density):
         assert np.array_equal(got[c], oracle.repair(raw[c], cap, k_cap, k_max, n_max, seed, 5, 9 + c, 6, active=active)), c
     s.sync_status()
     s.close()
+
+
+# beyond 65535 jobs a node's counters no longer do: rows of whole vectors on the batched kernels, others a row and a column at a time
+@pytest.mark.parametrize("nodes,shift", [(8, 0), (8, 1), (9, 0), (24, 0)])
+def test_more_jobs_than_a_nodes_counters_hold(oracle, nodes, shift):
+    import torch
+    from paper_2008_12260_b200 import api
+
+    J, P, thr, seed = 65541, 3, synth.prob_to_threshold(0.2), 4
+    rng = np.random.default_rng(nodes)
+    cl = synth.uniform_cluster(nodes, 8)
+    raw = synth.random_raw_population(P, J, cl, seed=nodes, density=0.0005, v_hi=9)
+    raw[1, :40, 2] = 3                                      # more occupants of a batch of rows than are listed
+    k_cap, active = rng.integers(0, cl.k_max + 3, J).astype(np.int32), (rng.uniform(size=J) < 0.9).astype(np.uint8)
+    fit = rng.uniform(0.1, 1.0, P).astype(np.float32)
+    s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=thr, thr_init=thr,
+                      num_elite=1, seed=seed, stream=torch.cuda.current_stream().cuda_stream)
+    dj = api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch)
+    _, parents = _unaligned(torch, raw, shift)
+    out_flat, out = _unaligned(torch, np.full(raw.shape, 5, np.int16), shift)
+    s.set_kernel_timing(True)
+    s.ga_generation(dj, parents, torch.from_numpy(fit).cuda(), out, round=2, generation=3)
+    ran = {name for name, (ms, n) in s.read_kernel_timing().items() if n}
+    assert "cols" in ran and ("rank" in ran) == (nodes % 8 != 0 or shift != 0)
+    ref = oracle.ga_generation(raw, fit, cl.node_capacity, k_cap, cl.k_max, cl.n_max, 1, thr, seed, 2, 3, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+    s.init_population(dj, parents[1], out, round=4)
+    ref = oracle.init_population(P, raw[1], J, cl.node_capacity, k_cap, cl.k_max, cl.n_max, thr, seed, 4, active=active)
+    assert np.array_equal(out.cpu().numpy(), ref)
+    s.repair_population(dj, parents, round=5, generation=6, first_candidate=9)
+    got = parents.cpu().numpy()
+    for c in range(P):
+        assert np.array_equal(got[c], oracle.repair(raw[c], cl.node_capacity, k_cap, cl.k_max, cl.n_max, seed, 5, 9 + c, 6, active=active)), c
+    assert _guards_ok(out_flat, shift, raw.size)
+    s.sync_status()
+    s.close()
