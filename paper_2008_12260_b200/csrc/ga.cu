@@ -926,6 +926,7 @@ struct ChildArgs {
   int split;                            // blocks of a child: a power of two
   int occ;                              // occupants a block lists per node
   int tile_rows, chunk_rows;            // rows laid out at a time; rows whose draws are made at a time
+  int *status;
 };
 
 template <bool WHOLE>
@@ -969,7 +970,8 @@ __device__ __noinline__ void repair_crowded(const ChildArgs &aa, uint32_t *list,
       const uint32_t *const occ = aa.split > 1 ? cluster.map_shared_rank(s_occ, q) : s_occ;
       const int here = (int)(child_counts(occ, NN, aa.occ)[n] >> 16);
       all = all && here <= aa.occ;
-      for (int k = lane; k < min(here, aa.occ); k += 32) list[at + k] = occ[n * aa.occ + k];
+      for (int k = lane; k < min(here, aa.occ); k += 32)
+        if (sched_index_ok(aa.status, at + k < CHILD_CROWD, SCHED_CHK_LIST)) list[at + k] = occ[n * aa.occ + k];
       at += here;
     }
     __syncwarp();
@@ -986,7 +988,8 @@ __device__ __noinline__ void repair_crowded(const ChildArgs &aa, uint32_t *list,
   for (int k = lane; k < count; k += 32) {
     const uint32_t e = list[k];
     const int v = at.keeps(e, occupant_gpus(e), rot_i(e), rot_c(e));
-    if (v != occupant_gpus(e)) column[(size_t)(e & 0xFFFFu) * NN] = (int16_t)v;
+    if (v != occupant_gpus(e) && sched_index_ok(aa.status, (int)(e & 0xFFFFu) < J, SCHED_CHK_NODE))
+      column[(size_t)(e & 0xFFFFu) * NN] = (int16_t)v;
   }
 }
 
@@ -1131,13 +1134,15 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
   int16_t *child = a.dst + (size_t)cl * mat;
   const int16_t *src_a = a.src, *src_b;           // NULL: the rows start empty
   if (a.mode == ROWS_GENERATION) {
-    src_b = a.src + (size_t)s_parent[1] * mat;
-    src_a += (size_t)s_parent[0] * mat;
+    const bool found = sched_index_ok(aa.status, (unsigned)s_parent[0] < (unsigned)P && (unsigned)s_parent[1] < (unsigned)P, SCHED_CHK_SLOT);
+    src_b = a.src + (found ? (size_t)s_parent[1] * mat : 0);
+    src_a += found ? (size_t)s_parent[0] * mat : 0;
   } else {
     if (a.mode == ROWS_REPAIR) src_a = child;
     src_b = src_a;
   }
   auto add_occupant = [&](int j, int n, int v, bool dist) {
+    if (!sched_index_ok(aa.status, n < NN && j < J && v <= 2047, SCHED_CHK_NODE)) return;
     atomicAdd(&s_tot[n], v);
     const uint32_t k = atomicAdd(&s_cnt[n], (dist ? 1u : 0u) | (1u << 16)) >> 16;
     if (k < (uint32_t)aa.occ) s_occ[n * aa.occ + k] = (uint32_t)j | ((uint32_t)v << 16) | (dist ? 0x80000000u : 0u);
@@ -1270,7 +1275,8 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
             const int n = (int)bounded(m3, (uint32_t)NN);
             if (lane == 0) row[n] = (int16_t)min((int)row[n] + 1, (int)s_cap[n]);
           } else if (rN > 0) {
-            const int ns = nth_occupied(row, NN, bounded(m2, (uint32_t)rN), lane);
+            int ns = nth_occupied(row, NN, bounded(m2, (uint32_t)rN), lane);
+            if (!sched_index_ok(aa.status, ns >= 0 && ns < NN, SCHED_CHK_NODE)) ns = 0;
             if (op == 1u) {
               if (lane == 0) row[ns] = (int16_t)(row[ns] - 1);
             } else {
@@ -1394,7 +1400,7 @@ __global__ void __launch_bounds__(CHILD_WARPS * 32, WHOLE ? 4 : 3) child_kernel(
       if (rc < 0) rc += J;
       const int most = max(__shfl_sync(0xffffffffu, count, 0), __shfl_sync(0xffffffffu, count, 16));
       const int v = decide(v_old, (e >> 31) != 0u, have, min(most, CHILD_OCC), (cnt & 0xFFFFu) >= 2u, tot, cap_n, ri, rc);
-      if (have && v != v_old) child[(size_t)j * NN + n] = (int16_t)v;
+      if (have && v != v_old && sched_index_ok(aa.status, j < J && n < NN, SCHED_CHK_NODE)) child[(size_t)j * NN + n] = (int16_t)v;
 #pragma unroll 1
       for (unsigned walk = __ballot_sync(0xffffffffu, !listed && sub == 0); walk; walk &= walk - 1) {
         const int l = __ffs(walk) - 1;
@@ -1452,6 +1458,7 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   const int NN = a.num_nodes;
   ChildArgs ca = {};
   ca.r = a;
+  ca.status = ctx->d_status;
   ca.col.pop = a.dst; ca.col.dflag = a.dflag; ca.col.cap = a.cap;
   ca.col.J = a.J; ca.col.num_nodes = NN;
   ca.col.gen = gen; ca.col.first_cand = first_cand; ca.col.key = a.key;

@@ -1,7 +1,7 @@
 """The range-checking build of the library (-DSCHED_CHECKED): kernels test the indices they
 compute from data - row slots, node numbers, list positions - and report a violation through
 the status word instead of touching memory.  The rounds of given and of randomly
-drawn shapes (most of them in one launch and on the row store) and the operator tests run once against it; their sync_status() calls raise if any check fired."""
+drawn shapes (in one launch, on the row store and on dense matrices) and the operator tests run once against it; their sync_status() calls raise if any check fired."""
 import os
 import subprocess
 import sys
@@ -19,7 +19,7 @@ def test_round_and_operator_tests_pass_on_the_checked_build():
     env = dict(os.environ, POLLUXSCHED_LIB=lib)
     cmd = [sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", "-p", "no:cacheprovider",
            os.path.join(ROOT, "tests", "test_gpu_round_kernels.py"), os.path.join(ROOT, "tests", "test_gpu_ga.py"),
-           os.path.join(ROOT, "tests", "test_gpu_round_fuzz.py"), os.path.join(ROOT, "tests", "test_gpu_round_shapes.py")]
+           os.path.join(ROOT, "tests", "test_gpu_child.py"), os.path.join(ROOT, "tests", "test_gpu_round_fuzz.py"), os.path.join(ROOT, "tests", "test_gpu_round_shapes.py")]
     out = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)
     assert out.returncode == 0, out.stdout[-3000:] + out.stderr[-2000:]
     assert " passed" in out.stdout
