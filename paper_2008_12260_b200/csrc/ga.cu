@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "fitness_common.cuh"
@@ -1453,6 +1454,30 @@ int launch_cols(sched_ctx *ctx, const RngKey &key, int16_t *pop, int count, uint
   return SCHED_OK;
 }
 
+bool whole_rows(const RowsArgs &a) { return a.num_nodes % 8 == 0 && (((uintptr_t)a.dst | (uintptr_t)a.src) & 15) == 0; }
+
+int child_occupants(const sched_ctx *ctx, const RowsArgs &a) {
+  return std::min(CHILD_CROWD, listed_occupants(ctx, a.mode == ROWS_REPAIR ? ctx->cfg.thr_mutate : a.thr, 256 * CHILD_OCC / a.num_nodes));
+}
+
+// Places for blocks on the GPU: three an SM (registers), four where rows are whole and their lists leave the memory for it.  Four
+// pay where a block has much to copy (128 children of 1024 x 256 with three 54 us, with four 44); small ones they only
+// cut up further (repair of 64 children of 1024 x 8 8.7 us, 10.7).
+long long child_places(const sched_ctx *ctx, const RowsArgs &a) {
+  const bool whole = whole_rows(a);
+  const size_t smem = child_smem_bytes(a.num_nodes, child_occupants(ctx, a), whole) + 1024;
+  const long long most = whole && (long long)a.J * a.num_nodes >= 1 << 17 ? 4 : 3;
+  return std::min<long long>(most, 228 * 1024 / smem) * ctx->num_sms;
+}
+
+// Blocks of a child: more than one while that leaves none of them without a place and every warp a few rows.
+int child_split(const sched_ctx *ctx, const RowsArgs &a, int count) {
+  const long long places = child_places(ctx, a);
+  int split = 1;
+  while (split < CHILD_SPLIT && (long long)count * split * 2 <= places && split * 2 * CHILD_WARPS * 4 <= a.J) split *= 2;
+  return split;
+}
+
 // Row pass and repair in one launch (child_kernel).
 int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first_cand, uint32_t gen) {
   const int NN = a.num_nodes;
@@ -1465,11 +1490,9 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   const size_t mat = (size_t)a.J * NN;
   ca.src_lo = a.src;
   ca.src_hi = a.src + mat * (a.mode == ROWS_GENERATION ? a.P : a.mode == ROWS_REPAIR ? count : a.src ? 1 : 0);
-  const bool whole = NN % 8 == 0 && (((uintptr_t)a.dst | (uintptr_t)a.src) & 15) == 0;
-  // a child is split over blocks while that leaves none of them without a place on the GPU and every warp a few rows
-  ca.split = 1;
-  while (ca.split < CHILD_SPLIT && (long long)count * ca.split * 2 <= 3LL * ctx->num_sms && ca.split * 2 * CHILD_WARPS * 4 <= a.J) ca.split *= 2;
-  ca.occ = std::min(CHILD_CROWD, listed_occupants(ctx, a.mode == ROWS_REPAIR ? ctx->cfg.thr_mutate : a.thr, 256 * CHILD_OCC / NN));
+  const bool whole = whole_rows(a);
+  ca.split = child_split(ctx, a, count);
+  ca.occ = child_occupants(ctx, a);
   ca.row_vecs = whole ? NN / 8 : (NN + 14) / 8;
   const int warps = CHILD_WARPS * ca.split, turns = (a.J + 32 * warps - 1) / (32 * warps);
   ca.chunk_rows = (a.J + warps * turns - 1) / (warps * turns);
@@ -1497,10 +1520,30 @@ int launch_children(sched_ctx *ctx, const RowsArgs &a, int count, uint32_t first
   return SCHED_OK;
 }
 
+// Whether rows of whole vectors are quicker on the batched kernels (a block per 256 rows of a child) than in
+// child_kernel, whose blocks are at most eight per child.  us, child_kernel against the batched kernels:
+//  * so few children that SMs stay empty, with many entries for each block (what a row costs beside its nodes is
+//    worth some 64 of them in a repair, 192 where rows are perturbed): generation of 1 child of 2048 x 256 25 / 32, 4096 39 / 32,
+//    32768 177 / 57; 16 children of 2048 x 512 41 / 48, 4096 x 512 75 / 56, 4096 x 128 33 / 33, 8192 x 128 44 / 39; repair of
+//    1 of 4096 x 256 26 / 23, 4 of 8192 x 64 17 / 17, 16384 x 64 27 / 20, 16 of 2048 x 512 31 / 37, 4096 x 512 50 / 42;
+//  * rows of more than 256 nodes, when a power of two of blocks a child leaves a third of the places empty: generation of 128
+//    children of 1024 x 512 89 / 76, 4096 x 512 259 / 245; 200 of 1024 x 512, which fill them, 102 / 117.
+// Not where nodes are crowded: the batched kernels list eight occupants a node and 256 rows, and 32 in all (generation of 16
+// children of 32768 x 8 74 / 279, x 64 103 / 93).
+bool batched_rows_pay(const sched_ctx *ctx, const RowsArgs &a, int count) {
+  const int split = child_split(ctx, a, count), rows = (a.J + split - 1) / split, NN = a.num_nodes;
+  const bool still = a.mode == ROWS_REPAIR || (a.mode == ROWS_INIT && count == 1);       // no row is perturbed
+  const uint32_t thr = a.mode == ROWS_REPAIR ? ctx->cfg.thr_mutate : still ? 0u : a.thr;
+  const double crowd = a.J * (thr / 4294967296.0) * (2.0 / 3.0) / NN;      // (two of three perturbed rows take a node)
+  if (crowd + 2.0 * std::sqrt(crowd) > 30.0) return false;
+  if (2LL * count * split < 3LL * ctx->num_sms) return (long long)rows * (NN + (still ? 64 : 192)) >= (still ? 155000 : 190000);
+  return NN > 256 && (long long)count * split * 10 < child_places(ctx, a) * 7 && (long long)count * a.J * NN >= 60000000;
+}
+
 // Row pass + column pass of `count` candidates.  Rounds on dense matrices want per-row summaries: rows of whole
 // 16-byte vectors take the batched kernels with fused column sums.  Without summaries every width takes a block (or
-// a few) per child, up to 512 nodes (a tile holds two rows), sizes <= 2047 (an occupant's word) and 65535 jobs (a
-// node's counters); with more jobs, rows of whole vectors take the batched kernels, too (up to 2^20 jobs: an occupant's
+// a few) per child where no other kernels pay, up to 512 nodes (a tile holds two rows), sizes <= 2047 (an occupant's word) and
+// 65535 jobs (a node's counters); with more jobs, rows of whole vectors take the batched kernels, too (up to 2^20 jobs: an occupant's
 // word there).  What is left takes the general warp-per-row / thread-per-column pair.
 int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint32_t first_cand, uint32_t gen) {
   if (count == 0 || a.J == 0) return SCHED_OK;
@@ -1509,7 +1552,8 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   const bool fused = (NN % 8 == 0) && NN <= 512 && aligned && ctx->cap_max <= 2047 && count <= 65535 &&
                      a.J <= (1 << 20);
   ctx->summ_valid = fused && a.summ != nullptr;
-  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535) return launch_children(ctx, a, count, first_cand, gen);
+  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535 && !(fused && batched_rows_pay(ctx, a, count)))
+    return launch_children(ctx, a, count, first_cand, gen);
   if (!fused) {
     if (a.mode == ROWS_GENERATION) {
       {

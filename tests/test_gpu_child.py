@@ -172,3 +172,53 @@ def test_more_jobs_than_a_nodes_counters_hold(oracle, nodes, shift):
     assert _guards_ok(out_flat, shift, raw.size)
     s.sync_status()
     s.close()
+
+
+# nodes, jobs, children, share of rows perturbed, what the three operators run on: so few children of so many rows that a block per
+# 256 rows is quicker ("cols": with the work-list repair behind it), the same with crowded nodes, and either side of that
+MANY_ROWS = [(256, 4096, 1, 0.02, "cols cols cols"), (64, 17000, 3, 0.01, "cols cols cols"), (512, 1900, 65, 0.01, "cols cols cols"),
+             (16, 8193, 4, 0.01, "cols cols rows"), (16, 17000, 2, 0.3, "rows rows rows"), (256, 1024, 2, 0.02, "rows rows rows"),
+             (512, 1000, 65, 0.01, "rows rows rows")]
+
+
+@pytest.mark.parametrize("nodes,J,P,share,routes", MANY_ROWS)
+def test_few_children_of_many_rows(oracle, nodes, J, P, share, routes):
+    _three_operators(oracle, nodes, J, P, share, routes.split())
+
+
+def _three_operators(oracle, nodes, J, P, share, routes):
+    """Initial population, generation and repair, the kernels they run on ("rows": child_kernel alone) and their results."""
+    import torch
+    from paper_2008_12260_b200 import api
+
+    thr, seed, elite = synth.prob_to_threshold(share), 11, 1 if P > 1 else 0
+    rng = np.random.default_rng(nodes + J)
+    cl = synth.uniform_cluster(nodes, 4)
+    raw = synth.random_raw_population(P, J, cl, seed=nodes + P, density=0.002 if J > 100 else 0.1, v_hi=6)
+    k_cap, active = rng.integers(0, cl.k_max + 3, J).astype(np.int32), (rng.uniform(size=J) < 0.9).astype(np.uint8)
+    fit = rng.uniform(0.1, 1.0, P).astype(np.float32)
+    s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=thr, thr_init=thr,
+                      num_elite=elite, seed=seed, stream=torch.cuda.current_stream().cuda_stream)
+    dj = api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch)
+    parents, out = torch.from_numpy(raw).cuda(), torch.empty(raw.shape, dtype=torch.int16, device="cuda:0")
+    s.set_kernel_timing(True)
+    ran = lambda: "cols" if s.read_kernel_timing()["cols"][1] else "rows"
+    some = sorted({0, 1 % P, P // 2, P - 1})                # (the oracle takes its time over large populations)
+
+    s.init_population(dj, parents[0], out, round=4)
+    used = [ran()]
+    got = out.cpu().numpy()
+    want = oracle.init_population(P, raw[0], J, cl.node_capacity, k_cap, cl.k_max, cl.n_max, thr, seed, 4, active=active)
+    assert np.array_equal(got, want)
+    s.ga_generation(dj, parents, torch.from_numpy(fit).cuda(), out, round=2, generation=3)
+    used.append(ran())
+    want = oracle.ga_generation(raw, fit, cl.node_capacity, k_cap, cl.k_max, cl.n_max, elite, thr, seed, 2, 3, active=active)
+    assert np.array_equal(out.cpu().numpy(), want)
+    s.repair_population(dj, parents, round=5, generation=6, first_candidate=9)
+    used.append(ran())
+    got = parents.cpu().numpy()
+    for c in some:
+        assert np.array_equal(got[c], oracle.repair(raw[c], cl.node_capacity, k_cap, cl.k_max, cl.n_max, seed, 5, 9 + c, 6, active=active)), c
+    assert used == routes
+    s.sync_status()
+    s.close()
