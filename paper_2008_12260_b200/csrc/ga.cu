@@ -1540,6 +1540,14 @@ bool batched_rows_pay(const sched_ctx *ctx, const RowsArgs &a, int count) {
   return NN > 256 && (long long)count * split * 10 < child_places(ctx, a) * 7 && (long long)count * a.J * NN >= 60000000;
 }
 
+// Whether children of a few rows are quicker on the general kernels, a warp a row and a thread a node, than with a block each:
+// where there are many more of them than places, and no ranks to find.  us, child_kernel against the pair: initial population of
+// 8000 children of 4 x 3 74 / 25, 16 x 3 97 / 64, 24 x 20 117 / 96, 24 x 41 123 / 107, 16 x 301 132 / 109, 2000 of 8 x 20 28 / 17;
+// 600 of 20 x 75 17 / 19, 8000 of 20 x 301 faster in child_kernel, too.
+bool tiny_children(const sched_ctx *ctx, const RowsArgs &a, int count) {
+  return a.mode != ROWS_GENERATION && !whole_rows(a) && count > 7 * ctx->num_sms && a.J <= 24 && a.J * (a.num_nodes + 300) <= 9700;
+}
+
 // Row pass + column pass of `count` candidates.  Rounds on dense matrices want per-row summaries: rows of whole
 // 16-byte vectors take the batched kernels with fused column sums.  Without summaries every width takes a block (or
 // a few) per child where no other kernels pay, up to 512 nodes (a tile holds two rows), sizes <= 2047 (an occupant's word) and
@@ -1552,7 +1560,8 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   const bool fused = (NN % 8 == 0) && NN <= 512 && aligned && ctx->cap_max <= 2047 && count <= 65535 &&
                      a.J <= (1 << 20);
   ctx->summ_valid = fused && a.summ != nullptr;
-  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535 && !(fused && batched_rows_pay(ctx, a, count)))
+  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535 && !(fused && batched_rows_pay(ctx, a, count)) &&
+      !tiny_children(ctx, a, count))
     return launch_children(ctx, a, count, first_cand, gen);
   if (!fused) {
     if (a.mode == ROWS_GENERATION) {

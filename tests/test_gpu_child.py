@@ -186,6 +186,14 @@ def test_few_children_of_many_rows(oracle, nodes, J, P, share, routes):
     _three_operators(oracle, nodes, J, P, share, routes.split())
 
 
+# many children of a few rows: a warp a row and a thread a node, unless ranks are wanted
+@pytest.mark.parametrize("nodes,J,P,routes", [(3, 1, 1100, "cols rows cols"), (20, 24, 1100, "cols rows cols"), (301, 16, 1100, "cols rows cols"),
+                                              (301, 17, 1100, "rows rows rows"), (20, 25, 1100, "rows rows rows"),
+                                              (8, 4, 1100, "rows rows rows"), (20, 4, 500, "rows rows rows")])
+def test_many_children_of_few_rows(oracle, nodes, J, P, routes):
+    _three_operators(oracle, nodes, J, P, 0.2, routes.split())
+
+
 def _three_operators(oracle, nodes, J, P, share, routes):
     """Initial population, generation and repair, the kernels they run on ("rows": child_kernel alone) and their results."""
     import torch
