@@ -44,7 +44,7 @@ constexpr int DEPTH = 4;                        // generations kept
 constexpr int PUB_STRIDE = 8;
 constexpr int SUM_THREADS = 256;                // as the dense fitness kernel: the order of its sums
 constexpr int LANES = 8;                        // lanes of a row
-constexpr int STASH = 128;                      // perturbed rows of many whose draws are kept, further ones draw again
+constexpr int STASH = 256;                      // perturbed rows of many whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
 constexpr int FLOW_MAX_WARPS = 20;
 constexpr int FLOW_OCC = 16;                    // occupants of a node that a group of lanes decides
@@ -87,7 +87,7 @@ constexpr uint32_t NEVER = 0xFFFFFFFDu;
 
 // Places in the generation kernel's shared memory, behind what the warps tell each other (terms: -1 where they are not kept there).
 struct FlowSmem {
-  int act, term, info, node, occ, more, viol, cap, rack, mut, mod, wide, slow, stash, flag, dense, rep, keys, sums, scratch, rec, same,
+  int act, term, info, node, occ, more, viol, cap, rack, mut, mod, stash, flag, dense, rep, keys, sums, scratch, rec, same,
       terms, total;
 };
 
@@ -360,8 +360,10 @@ struct FlowView {
   uint32_t *more;                     // those that do not fit
   uint8_t *viol;                      // the node's column is to be walked
   int16_t *cap, *rack;
-  uint16_t *mut, *mod, *wide, *slow;  // mut: two sets
-  uint4 *stash;                       // two sets
+  uint16_t *mut;                      // two sets
+  uint16_t *mod;                      // rows that decisions change
+  uint16_t *wide;                     // in the same place, before the decisions: wide rows from the front, slow ones from the back
+  uint2 *stash;                       // two sets: the draw that chooses a node of the row; operator | node << 2 | replica cap << 16
   uint8_t *flag;                      // two sets, by row: 1 from the second parent, 2 perturbed
   int16_t *dense;                     // a row per warp
   uint32_t *rep;                      // two sets, by node: the two rotation offsets
@@ -378,8 +380,8 @@ __device__ __forceinline__ FlowView flow_view(const FlowArgs &a, uint32_t memory
   unsigned char *const s = (unsigned char *)__cvta_shared_to_generic(memory);
   return FlowView{*(FlowCtl *)s, (uint16_t *)(s + L.act), (float *)(s + L.term), s + L.info, (uint32_t *)(s + L.node),
                   (uint32_t *)(s + L.occ), (uint32_t *)(s + L.more), s + L.viol, (int16_t *)(s + L.cap), (int16_t *)(s + L.rack),
-                  (uint16_t *)(s + L.mut), (uint16_t *)(s + L.mod), (uint16_t *)(s + L.wide), (uint16_t *)(s + L.slow),
-                  (uint4 *)(s + L.stash), s + L.flag, (int16_t *)(s + L.dense), (uint32_t *)(s + L.rep), (uint32_t *)(s + L.keys),
+                  (uint16_t *)(s + L.mut), (uint16_t *)(s + L.mod), (uint16_t *)(s + L.mod),
+                  (uint2 *)(s + L.stash), s + L.flag, (int16_t *)(s + L.dense), (uint32_t *)(s + L.rep), (uint32_t *)(s + L.keys),
                   (double *)(s + L.sums), (uint32_t *)(s + L.scratch), (uint32_t *)(s + L.rec), (uint32_t *)(s + L.same),
                   (float *)(s + L.terms)};
 }
@@ -607,33 +609,39 @@ __device__ __noinline__ int2 cap_list(uint32_t *place, int K, int N, int kc, int
   return make_int2(row_sum(e != NO_NODE ? entry_gpus(e) : 0), __popc(row_bits(e != NO_NODE, lane)));
 }
 
+// What a row's draw says that its parent's contents do not change: the operator, the node it goes to; and the row's cap.
+__device__ __forceinline__ uint2 choices_of(const FlowArgs &a, const u32x4 &m, int j) {
+  const int cap = max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max));
+  return make_uint2(m.z, bounded(m.y, 3u) | (bounded(m.w, (uint32_t)a.NN) << 2) | ((uint32_t)cap << 16));
+}
+static_assert(FLOW_MAX_NODES <= 512 && SCHED_MAX_K < 65536, "the choices' fields");
+
 // The row pass for up to four perturbed rows: perturbation (grow, shrink, relocate, chosen by the row's draw), row caps,
 // the new record.  x0: the first of them in the list.
 template <int KIND>
 __device__ __forceinline__ void perturb_rows(const FlowArgs &a, const FlowView &v, const Work &w, uint32_t round, int set, int x0, int nmut,
                                              int warp, int lane) {
   uint32_t *const place = empty_place(v, warp, lane);
-  const int k = lane & 7, i = x0 + (lane >> 3), NN = a.NN;
+  const int k = lane & 7, i = x0 + (lane >> 3);
   const unsigned below = (1u << k) - 1u;
   bool live = i < nmut;
   const int m = live ? v.mut[set * a.J + i] : 0, jc = m & 0x7FFF;
   live = live && sched_index_ok(a.status, i < a.J && jc < a.J, SCHED_CHK_LIST);
   uint32_t e = NO_NODE;
   if (live && k < ENTRIES) e = __ldcg(rec_row(a, (w.init || (m >> 15) ? w.src[1] : w.src[0]) + (w.init ? (int)v.act[jc] : jc)) + k);
-  uint4 st = make_uint4(0u, 0u, 0u, 0u);
-  if (i < stash_rows(a.J)) {
+  uint2 st = make_uint2(0u, 0u);
+  if (live && i < stash_rows(a.J)) {
     st = v.stash[set * stash_rows(a.J) + i];
   } else if (live) {
     const int j = v.act[jc];
-    const u32x4 d = draw_one(a.key.k0, round, (uint32_t)j, w.c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE);
-    st = make_uint4(d.y, d.z, d.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[j] : a.k_max, a.k_max)));
+    st = choices_of(a, draw_one(a.key.k0, round, (uint32_t)j, w.c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE), j);
   }
   __syncwarp();
-  const uint32_t op = bounded(st.x, 3u);
-  const int nd = (int)bounded(st.z, (uint32_t)NN), cap_nd = (int)v.cap[nd];
+  const uint32_t op = st.y & 3u;
+  const int nd = (int)((st.y >> 2) & 0x1FFu), cap_nd = (int)v.cap[nd], k_cap = (int)(st.y >> 16);
   const bool wide = (row_bits(k == 0 && e == WIDE, lane) & 1u) != 0u;
   int N = __popc(row_bits(e != NO_NODE, lane));
-  const uint32_t es = __shfl_sync(0xffffffffu, e, N > 0 ? (int)bounded(st.y, (uint32_t)N) : 0, LANES);
+  const uint32_t es = __shfl_sync(0xffffffffu, e, N > 0 ? (int)bounded(st.x, (uint32_t)N) : 0, LANES);
   const int ns = entry_node(es), vs = entry_gpus(es);
   const unsigned at_nd = row_bits(e != NO_NODE && entry_node(e) == nd, lane);
   const uint32_t end = __shfl_sync(0xffffffffu, e, at_nd ? __ffs(at_nd) - 1 : 0, LANES);
@@ -655,9 +663,9 @@ __device__ __forceinline__ void perturb_rows(const FlowArgs &a, const FlowView &
   }
   int K = row_sum(e != NO_NODE ? entry_gpus(e) : 0);
   N = __popc(there) + extra;
-  const bool over = live && !wide && (K > (int)st.w || N > a.n_max);
+  const bool over = live && !wide && (K > k_cap || N > a.n_max);
   if (__any_sync(0xffffffffu, over)) {
-    const int2 now = cap_list(place, K, N, (int)st.w, a.n_max, over, lane);
+    const int2 now = cap_list(place, K, N, k_cap, a.n_max, over, lane);
     K = now.x;
     N = now.y;
     __syncwarp();
@@ -667,7 +675,7 @@ __device__ __forceinline__ void perturb_rows(const FlowArgs &a, const FlowView &
   live = live && !slow;
   if (slow && k == 0) {
     const int at = atomicAdd(&v.ctl.nslow, 1);
-    if (sched_index_ok(a.status, at < a.J, SCHED_CHK_LIST)) v.slow[at] = (uint16_t)m;
+    if (sched_index_ok(a.status, at < a.J, SCHED_CHK_LIST)) v.wide[a.J - 1 - at] = (uint16_t)m;
   }
   settle_row<KIND>(a, v, w.dst, jc, live ? e : NO_NODE, place, K, N, live, true, lane);
 }
@@ -712,7 +720,7 @@ __device__ __noinline__ void wide_rows(const FlowArgs &a, uint32_t memory, Work 
 #pragma unroll 1
   for (int i = warp; i < nwide + v.ctl.nslow; i += a.warps) {
     const bool slow = i >= nwide;
-    const int x = slow ? v.slow[i - nwide] : v.wide[i], jc = x & 0x7FFF;
+    const int x = v.wide[slow ? a.J - 1 - (i - nwide) : i], jc = x & 0x7FFF;
     if (!sched_index_ok(a.status, jc < a.J, SCHED_CHK_LIST)) continue;
     const int j = v.act[jc];
     const int from = (x >> 15) || (w.init && slow);
@@ -1018,7 +1026,7 @@ __device__ __noinline__ void draw_items(const FlowArgs &a, uint32_t memory, uint
           if (!sched_index_ok(a.status, at < J, SCHED_CHK_LIST)) continue;
           v.mut[set * J + at] = (uint16_t)(jc | (sec ? 0x8000 : 0));
           if (at < stash_rows(J))
-            v.stash[set * stash_rows(J) + at] = make_uint4(m.y, m.z, m.w, (uint32_t)max(0, min(a.k_cap ? a.k_cap[idx] : a.k_max, a.k_max)));
+            v.stash[set * stash_rows(J) + at] = choices_of(a, m, (int)idx);
         }
       }
     }
@@ -1485,9 +1493,7 @@ FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms, int more) {
   L.rack = take(ctx->d_rack ? (size_t)NN * 2 : 0);
   L.mut = take(2 * (size_t)J * 2);
   L.mod = take((size_t)J * 2);
-  L.wide = take((size_t)J * 2);
-  L.slow = take((size_t)J * 2);
-  L.stash = take(2 * (size_t)stash_rows(J) * 16);
+  L.stash = take(2 * (size_t)stash_rows(J) * 8);
   L.flag = take(2 * (size_t)J);
   L.dense = take((size_t)warps * wide_stride(NN) * 2);
   L.rep = take(2 * (size_t)NN * 4);
