@@ -20,8 +20,8 @@
 // 7.2 k in all: waiting for the four keys 1.4 k (an unloaded L2 trip is 0.3 k; a fence behind a store 0.8 k), parents
 // 0.35 k, perturbed rows 1.9 k, decisions 1.4 k, changed rows 0.85 k, sum and power mean 1.15 k beside the fence
 // (0.95 k), publication 0.2 k.  13 k before perturbed and changed rows took eight lanes, draws and terms moved out of
-// the way and keys apart.  Eight lanes for the rows that are copied, too: 530 us instead of 490 for the testbed's round and
-// 7.4 ms instead of 3.65 for the large one, four times the instructions for as many rows.
+// the way and keys apart.  Eight lanes for the rows that are copied, too: 1.08 times the time of the testbed's round and twice
+// that of the large one (both measured before the keys were set apart), four times the instructions for as many rows.
 // Operators, draws and the order of the fitness sums are those of the dense kernels: identical populations
 // and fitness bits.
 #include <algorithm>
@@ -47,23 +47,29 @@ constexpr int LANES = 8;                        // lanes of a row
 constexpr int STASH = 256;                      // perturbed rows of many whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
 constexpr int FLOW_MAX_WARPS = 20;
+constexpr int MANY_TWO_JOBS = 2048;             // beyond these two blocks an SM take any population
+constexpr int SOME_WARPS = 16;                  // that work on the rows where a block has an SM for itself and more than 256 jobs
 constexpr int FLOW_OCC = 16;                    // occupants of a node that a group of lanes decides
 constexpr int FLOW_MAX_JOBS = 8192, FLOW_MAX_NODES = 512, FLOW_MAX_SMEM = 220 * 1024;
 constexpr int RANK_PAIRS = 64;                 // keys that are ranked by comparing them with one another
 
-// Kinds of the generation kernel.  Not MANY: the child's records and what its rows' terms are made of are kept in shared
-// memory, too.  FEW_ALONE, SOME_ALONE: no two blocks share an SM (a population of at most as many), up to 256 and up to
-// 1024 jobs.  Registers: 142 for FEW_ALONE's 12 warps (testbed round 490 us; 522 with 96, 555 with 64, that is with
-// spills, which lie in the L1 that every acquire empties), 96 for SOME_ALONE's 20 (12 warps for 881 jobs: 826 us, 20: 730),
-// 64 for FEW, 56 for MANY.
+// Kinds of the generation kernel.  Not MANY, MANY_TWO: the child's records and what its rows' terms are made of are kept in
+// shared memory, too.  FEW_ALONE, SOME_ALONE: no two blocks share an SM (a population of at most as many), up to 256 jobs and
+// up to what the memory holds (some 2700).  FEW: two blocks, or more with up to 256 jobs.  MANY_TWO: two blocks, or one with more
+// jobs than SOME_ALONE holds, and any number of candidates beyond 2048 jobs, where four blocks an SM have more records between
+// them than L2 holds and take more turns than their number saves (592 candidates x 2500 jobs 2441 us with MANY, 2312; 900 x 3000
+// 7247, 5472; 592 x 1500 2483, 2663).  Registers: 138 for FEW_ALONE's 12 warps (with 96 a testbed round takes 1.07 times as long, with 64
+// 1.13 times: spills lie in the L1 that every acquire empties; measured before the keys were set apart), 96 for SOME_ALONE's 20, 64
+// for FEW and MANY_TWO, 56 for MANY.  A lone candidate's block with more than 1024 jobs had 8 or 9 warps, which is 30 generations
+// of 64 x 1100 jobs 1028 us, now 642; 148 x 4000 2206, now 1374; 296 x 2400 1854, now 1135.
 // CROWDED, with any of them: lists longer than a group of lanes, where so many occupants of a node are to be expected.
-constexpr int FEW_ALONE = 0, SOME_ALONE = 1, FEW = 2, MANY = 3, CROWDED = 4;
-__host__ __device__ constexpr int shape_of(int kind) { return kind & 3; }
-__host__ __device__ constexpr bool few(int kind) { return shape_of(kind) != MANY; }
+constexpr int FEW_ALONE = 0, SOME_ALONE = 1, FEW = 2, MANY = 3, MANY_TWO = 4, CROWDED = 8;
+__host__ __device__ constexpr int shape_of(int kind) { return kind & 7; }
+__host__ __device__ constexpr bool few(int kind) { return shape_of(kind) < MANY; }
 __host__ __device__ constexpr int kind_threads(int kind) {
-  return shape_of(kind) == FEW_ALONE ? 384 : shape_of(kind) == SOME_ALONE ? 640 : shape_of(kind) == FEW ? 512 : 288;
+  return shape_of(kind) == FEW_ALONE ? 384 : shape_of(kind) == SOME_ALONE ? 640 : shape_of(kind) == MANY ? 288 : 512;
 }
-__host__ __device__ constexpr int kind_blocks(int kind) { return shape_of(kind) == MANY ? 4 : shape_of(kind) == FEW ? 2 : 1; }
+__host__ __device__ constexpr int kind_blocks(int kind) { return shape_of(kind) == MANY ? 4 : shape_of(kind) <= SOME_ALONE ? 1 : 2; }
 
 __host__ __device__ inline int wide_stride(int NN) { return (NN + 7) & ~7; }
 __host__ __device__ inline int stash_rows(int J) { return J <= SMEM_RECORDS ? J : STASH; }
@@ -155,8 +161,8 @@ __device__ __forceinline__ unsigned long long wait_tag(const unsigned long long 
 // Acquire: with the publisher's fence (release) and the block's barrier, what was written before the tag
 // was published is seen by every thread of this block, and what was read before it lies behind it.  One
 // fence after the polls that succeeded, not an acquire in each poll.  The one-way fence costs nothing that
-// can be measured (testbed round 663 us with it and without, large 3.87 ms), fence.acq_rel, which also waits
-// for this thread's own writes, 4 to 10 % (732 us, 4.03 ms).
+// can be measured, fence.acq_rel, which also waits for this thread's own writes, 10 % of a testbed round and 4 % of a
+// large one (of rounds that took 663 us and 3.87 ms).
 __device__ __forceinline__ void waited() { asm volatile("fence.acquire.gpu;" ::: "memory"); }
 __device__ __forceinline__ void publish(unsigned long long *p, uint32_t tag, uint32_t key) {
   const unsigned long long v = ((unsigned long long)tag << 32) | key;
@@ -1170,7 +1176,7 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
     const int nmut = v.ctl.nmut[set];
 #pragma unroll 1
     for (int x = (W - 1 - warp) * 4; x < nmut; x += W * 4) perturb_rows<KIND>(a, v, w, round, set, x, nmut, warp, lane);
-    constexpr int RB = shape_of(KIND) == SOME_ALONE || shape_of(KIND) == MANY ? 2 : 1;       // rows of a thread whose loads travel together
+    constexpr int RB = shape_of(KIND) == SOME_ALONE || !few(KIND) ? 2 : 1;       // rows of a thread whose loads travel together
 #pragma unroll 1
     for (int jc0 = tid; jc0 < JA; jc0 += RB * threads) {
       Record rec[RB];
@@ -1462,15 +1468,7 @@ FlowArena flow_arena(const sched_ctx *ctx, char *base) {
   return f;
 }
 
-int flow_kind(const sched_ctx *ctx) {
-  const int J = ctx->cfg.num_jobs, NN = ctx->cfg.num_nodes, P = ctx->cfg.population;
-  const bool alone = P <= ctx->num_sms, two = P <= 2 * ctx->num_sms;
-  if (J <= SMEM_RECORDS) return alone ? FEW_ALONE : FEW;
-  if (alone && J <= 4 * SMEM_RECORDS) return SOME_ALONE;
-  return two && 83 * J + 115 * NN + 6 * P <= 96 * 1024 ? FEW : MANY;      // (what two blocks find room for on an SM)
-}
-
-FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms, int more) {
+FlowSmem flow_smem(const sched_ctx *ctx, int kind, int warps, bool terms, int more) {
   const sched_config &c = ctx->cfg;
   const int J = c.num_jobs, NN = c.num_nodes, P = c.population;
   int rows, chunks, off = 0;
@@ -1500,11 +1498,20 @@ FlowSmem flow_smem(const sched_ctx *ctx, int warps, bool terms, int more) {
   L.keys = take((size_t)P * 6);      // and a list of candidates behind them
   L.sums = take((size_t)chunks * 8 * 8);
   L.scratch = take((size_t)warps * 32 * 4);
-  L.rec = flow_kind(ctx) != MANY ? take((size_t)J * REC_WORDS * 4) : 0;
-  L.same = flow_kind(ctx) != MANY ? take((size_t)J * REC_WORDS * 4) : 0;
+  L.rec = few(kind) ? take((size_t)J * REC_WORDS * 4) : 0;
+  L.same = few(kind) ? take((size_t)J * REC_WORDS * 4) : 0;
   L.terms = terms ? take((size_t)J * flow_classes(ctx) * ctx->KD * 4) : -1;
   L.total = off;
   return L;
+}
+
+int flow_kind(const sched_ctx *ctx) {
+  const int J = ctx->cfg.num_jobs, NN = ctx->cfg.num_nodes, P = ctx->cfg.population;
+  const bool alone = P <= ctx->num_sms, two = P <= 2 * ctx->num_sms;
+  if (J <= SMEM_RECORDS) return alone ? FEW_ALONE : FEW;
+  if (alone && flow_smem(ctx, SOME_ALONE, SOME_WARPS, false, 0).total <= FLOW_MAX_SMEM) return SOME_ALONE;
+  if (two && 79 * J + 115 * NN + 6 * P <= 96 * 1024) return FEW;        // (what two blocks find room for on an SM)
+  return two || J > MANY_TWO_JOBS ? MANY_TWO : MANY;
 }
 
 // The launch's shape.
@@ -1520,10 +1527,12 @@ FlowKernel flow_kernel_for(const sched_ctx *ctx, bool crowded) {
     case SOME_ALONE: return flow_kernel<SOME_ALONE>;
     case FEW: return flow_kernel<FEW>;
     case MANY: return flow_kernel<MANY>;
+    case MANY_TWO: return flow_kernel<MANY_TWO>;
     case FEW_ALONE | CROWDED: return flow_kernel<FEW_ALONE | CROWDED>;
     case SOME_ALONE | CROWDED: return flow_kernel<SOME_ALONE | CROWDED>;
     case FEW | CROWDED: return flow_kernel<FEW | CROWDED>;
-    default: return flow_kernel<MANY | CROWDED>;
+    case MANY | CROWDED: return flow_kernel<MANY | CROWDED>;
+    default: return flow_kernel<MANY_TWO | CROWDED>;
   }
 }
 
@@ -1537,27 +1546,30 @@ int flow_more(const sched_ctx *ctx) {
   return listed_occupants(ctx, std::max(c.thr_mutate, c.thr_init), 256 * FLOW_OCC / c.num_nodes) - FLOW_OCC;
 }
 
-// A block for every candidate if they fit the GPU.  Warps that work on rows and warps that draw, measured: testbed (48 jobs)
-// 3 + 2 540 us, 4 + 2 513, 6 + 2 508, 8 + 2 and 8 + 4 505, 12 + 4 509; 96 jobs in racks 662, 621, 557, 547, 542, 542; two
-// blocks an SM (210 jobs) 8 + 2 760, 10 + 3 698, 12 + 3 693; 1024 jobs, four blocks an SM 6 + 2 3896, 7 + 2 3700,
-// 7 + 3 3774, 8 + 2 3740.  The terms' table is kept in shared memory where that does not cost a block its place.
+// A block for every candidate if they fit the GPU.  Warps that work on rows and warps that draw, measured.  Before the keys were
+// set apart, which took the same off all of them: testbed (48 jobs) 3 + 2 540 us, 4 + 2 513, 6 + 2 508, 8 + 2 and 8 + 4 505, 12 + 4
+// 509; 96 jobs in racks 662, 621, 557, 547, 542, 542; two blocks an SM (210 jobs) 8 + 2 760, 10 + 3 698, 12 + 3 693; 1024 jobs, four
+// blocks an SM 6 + 2 3896, 7 + 2 3700, 7 + 3 3774, 8 + 2 3740.  Since, 30 generations: MANY_TWO, 148 candidates x 4000 jobs 10 + 3
+// 1563, 12 + 2 2143, 12 + 4 1373, 14 + 2 2137; SOME_ALONE, 64 x 1100 12 + 4 694, 14 + 6 647, 16 + 2 918, 16 + 4 642, 64 x 2000 821,
+// 759, 1391, 806 (with so many rows the draws are what takes long).  The terms' table is kept in shared memory where that does not cost a block its place.
 FlowShape flow_shape(const sched_ctx *ctx) {
   const sched_config &c = ctx->cfg;
-  const bool few = flow_kind(ctx) != MANY;
+  const int kind = flow_kind(ctx);
   FlowShape best = {};
-  const int per_sm = std::min(4, std::max(1, (c.population + ctx->num_sms - 1) / ctx->num_sms));
+  const int per_sm = std::min(4, (c.population + ctx->num_sms - 1) / ctx->num_sms);
   int warps, draw;
-  switch (flow_kind(ctx)) {
+  switch (kind) {
     case MANY: warps = 7; draw = 2; break;
-    case FEW: warps = per_sm == 2 ? 12 : per_sm == 3 ? 8 : 6; draw = per_sm == 2 ? 3 : 2; break;
-    case SOME_ALONE: warps = 16; draw = 4; break;
-    default: warps = 8; draw = 4; break;
+    case MANY_TWO: warps = 12; draw = 4; break;
+    case SOME_ALONE: warps = SOME_WARPS; draw = 4; break;
+    case FEW_ALONE: warps = 8; draw = 4; break;
+    default: warps = per_sm == 2 ? 12 : per_sm == 3 ? 8 : 6; draw = per_sm == 2 ? 3 : 2; break;
   }
-  for (int x = few ? 3 : 1; x >= 0 && best.blocks < c.population; --x) {      // terms and long lists, terms, long lists, neither
+  for (int x = few(kind) ? 3 : 1; x >= 0 && best.blocks < c.population; --x) {      // terms and long lists, terms, long lists, neither
     const bool terms = (x & 2) != 0;
     const int more = (x & 1) ? flow_more(ctx) : 0;
     if ((x & 1) && more == 0) continue;
-    FlowShape f = {warps, draw, 0, more, flow_smem(ctx, warps, terms, more)};
+    FlowShape f = {warps, draw, 0, more, flow_smem(ctx, kind, warps, terms, more)};
     const FlowKernel kernel = flow_kernel_for(ctx, more > 0);
     int fit = 0;
     if (f.at.total > FLOW_MAX_SMEM ||
@@ -1607,7 +1619,8 @@ int round_flow_ensure(sched_ctx *ctx) {
   ctx->d_tab_speedup_rack = f.speedup_rack;
   ctx->d_fit_buf = ctx->d_fit = f.fitness;
   ctx->scratch_epoch++;
-  // no tag matches before it is published, and a record that was never written has no nodes
+  // no tag matches before it is published.  (Records are not cleared: a round reads those of candidates that have published
+  // theirs, at places below the number of active jobs, and all of these are written before that.)
   SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(f.r.pub, 0, DEPTH * (size_t)c.population * PUB_STRIDE * 8, ctx->stream));
   SCHED_CUDA_CHECK(ctx, cudaMemsetAsync(f.r.base, 1, 4, ctx->stream));
   ctx->fl_blocks = blocks;
@@ -1659,7 +1672,7 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   a.generations = generations;
   a.warps = ctx->fl_warps;
   a.more = ctx->fl_more;
-  a.at = flow_smem(ctx, ctx->fl_warps, ctx->fl_terms, ctx->fl_more);
+  a.at = flow_smem(ctx, flow_kind(ctx), ctx->fl_warps, ctx->fl_terms, ctx->fl_more);
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
     TimedLaunch tl_(ctx, KK_FLOW_BUILD);

@@ -1,18 +1,28 @@
-"""Rounds on either side of the lines where the one-launch search changes its blocks: how many candidates share an SM (148
-on a B200) and how many jobs keep their records in shared memory.  Bit for bit the dense entry points one by one."""
+"""Rounds about the lines where the one-launch search changes its blocks: how many candidates share an SM and how many
+jobs keep their records in shared memory.  (Which blocks a round got is not looked at.)  Bit for bit the dense entry points one by
+one."""
 import pytest
+import torch
 
 import test_gpu_round_shapes as shapes
 
 pytestmark = pytest.mark.gpu
 
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+
 # as in test_gpu_round_shapes: nodes, GPUs per node, jobs, population, generations, nodes per rack, active, perturbation
 KINDS = [
-    (20, 4, 256, 148, 4, 0, 1.0, 0.2), (20, 4, 256, 149, 4, 6, 1.0, 0.2), (20, 4, 257, 148, 4, 6, 1.0, 0.2),
-    (20, 4, 257, 149, 4, 0, 1.0, 0.2), (12, 8, 1024, 30, 3, 4, 0.8, 0.1), (12, 8, 1025, 30, 3, 0, 1.0, 0.1),
-    (12, 8, 700, 296, 3, 0, 1.0, 0.1), (12, 8, 300, 297, 3, 0, 1.0, 0.1), (20, 4, 64, 296, 4, 0, 1.0, 0.2),
-    (20, 4, 64, 297, 4, 0, 0.5, 0.2), (20, 4, 64, 445, 4, 5, 1.0, 0.2), (64, 4, 900, 200, 3, 0, 1.0, 0.9),
-    (1, 4, 1, 3, 3, 0, 1.0, 1.0),
+    # a block or several an SM, records in shared memory or not
+    (20, 4, 256, SMS, 4, 0, 1.0, 0.2), (20, 4, 256, SMS + 1, 4, 6, 1.0, 0.2), (20, 4, 257, SMS, 4, 6, 1.0, 0.2),
+    (20, 4, 257, SMS + 1, 4, 0, 1.0, 0.2), (12, 8, 1024, 30, 3, 4, 0.8, 0.1), (12, 8, 1025, 30, 3, 0, 1.0, 0.1),
+    (3, 8, 2720, 20, 3, 0, 1.0, 0.1), (3, 8, 2810, 20, 3, 2, 0.9, 0.1), (12, 8, 1204, 2 * SMS, 2, 0, 1.0, 0.1),
+    (12, 8, 1206, 2 * SMS, 2, 0, 1.0, 0.1), (12, 8, 1206, 2 * SMS + 1, 2, 0, 1.0, 0.1), (6, 4, 8192, 7, 2, 0, 1.0, 0.1),
+    (12, 8, 700, 2 * SMS, 3, 0, 1.0, 0.1), (12, 8, 300, 2 * SMS + 1, 3, 0, 1.0, 0.1), (20, 4, 64, 2 * SMS, 4, 0, 1.0, 0.2),
+    (20, 4, 64, 2 * SMS + 1, 4, 0, 0.5, 0.2), (20, 4, 64, 3 * SMS + 1, 4, 5, 1.0, 0.2), (64, 4, 900, 200, 3, 0, 1.0, 0.9),
+    # smaller blocks, and more candidates than blocks
+    (20, 4, 30, 4 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 4 * SMS + 1, 4, 6, 1.0, 0.2), (20, 4, 30, 5 * SMS + 1, 4, 0, 0.7, 0.2),
+    (20, 4, 30, 6 * SMS + 1, 4, 6, 1.0, 0.9), (20, 4, 30, 8 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 8 * SMS + 1, 4, 6, 1.0, 0.2),
+    (20, 4, 250, 8 * SMS, 3, 0, 1.0, 0.2), (1, 4, 1, 3, 3, 0, 1.0, 1.0),
 ]
 
 
@@ -42,7 +52,6 @@ def test_rounds_with_crowded_nodes(shape, start):
                                                  (300, 32, 0.3, 0.05), (148, 148, 0.3, 0.0), (500, 200, 0.05, 0.01)])
 def test_elite_candidates_of_a_round(P, elite, init, mutate):
     import numpy as np
-    import torch
     from helpers import with_fair_share
     from paper_2008_12260_b200 import api, synth
 
