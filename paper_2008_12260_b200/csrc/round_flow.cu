@@ -1551,19 +1551,27 @@ int flow_more(const sched_ctx *ctx) {
 // 509; 96 jobs in racks 662, 621, 557, 547, 542, 542; two blocks an SM (210 jobs) 8 + 2 760, 10 + 3 698, 12 + 3 693; 1024 jobs, four
 // blocks an SM 6 + 2 3896, 7 + 2 3700, 7 + 3 3774, 8 + 2 3740.  Since, 30 generations: MANY_TWO, 148 candidates x 4000 jobs 10 + 3
 // 1563, 12 + 2 2143, 12 + 4 1373, 14 + 2 2137; SOME_ALONE, 64 x 1100 12 + 4 694, 14 + 6 647, 16 + 2 918, 16 + 4 642, 64 x 2000 821,
-// 759, 1391, 806 (with so many rows the draws are what takes long).  The terms' table is kept in shared memory where that does not cost a block its place.
+// 759, 1391, 806 (with so many rows the draws are what takes long); FEW, 54 jobs x 600 candidates 6 + 2 in two turns 628, 4 + 2
+// 447, 4 + 1 452, 3 + 1 487; x 888 703, 770, 533, 588; x 1100 753, 827, 902, 675; x 1300 in three, two, two and two turns 1040, 882,
+// 956, 1073.  The terms' table is kept in shared memory where that does not cost a block its place.
 FlowShape flow_shape(const sched_ctx *ctx) {
   const sched_config &c = ctx->cfg;
   const int kind = flow_kind(ctx);
   FlowShape best = {};
-  const int per_sm = std::min(4, (c.population + ctx->num_sms - 1) / ctx->num_sms);
   int warps, draw;
   switch (kind) {
     case MANY: warps = 7; draw = 2; break;
     case MANY_TWO: warps = 12; draw = 4; break;
     case SOME_ALONE: warps = SOME_WARPS; draw = 4; break;
     case FEW_ALONE: warps = 8; draw = 4; break;
-    default: warps = per_sm == 2 ? 12 : per_sm == 3 ? 8 : 6; draw = per_sm == 2 ? 3 : 2; break;
+    default: {
+      // up to eight blocks an SM, and no more turns than that takes; then as few blocks an SM as the turns leave
+      const int most = std::max(1, std::min(8, 227 * 1024 / (flow_smem(ctx, kind, 3, false, 0).total + 1024)));
+      const int turns = (c.population + most * ctx->num_sms - 1) / (most * ctx->num_sms);
+      const int per_sm = (c.population + turns * ctx->num_sms - 1) / (turns * ctx->num_sms);
+      warps = per_sm <= 2 ? 12 : per_sm == 3 ? 8 : per_sm == 4 ? 6 : per_sm <= 6 ? 4 : 3;
+      draw = per_sm <= 2 ? 3 : per_sm <= 5 ? 2 : 1;
+    }
   }
   for (int x = few(kind) ? 3 : 1; x >= 0 && best.blocks < c.population; --x) {      // terms and long lists, terms, long lists, neither
     const bool terms = (x & 2) != 0;
