@@ -1540,6 +1540,20 @@ bool batched_rows_pay(const sched_ctx *ctx, const RowsArgs &a, int count) {
   return NN > 256 && (long long)count * split * 10 < child_places(ctx, a) * 7 && (long long)count * a.J * NN >= 60000000;
 }
 
+size_t batched_scratch(const RowsArgs &a, int count) { return (size_t)count * ((a.J + 255) / 256) * a.num_nodes; }
+
+// What the batched kernels need beside the matrices. child_kernel does without: a call that could take either is not refused
+// for the lack of it, nor while its stream is captured.
+bool have_batched_scratch(sched_ctx *ctx, const RowsArgs &a, int count) {
+  if (batched_scratch(a, count) <= ctx->col_cap) return true;
+  cudaStreamCaptureStatus capture;
+  if (cudaStreamIsCapturing(ctx->stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+      ensure_colscratch(ctx, batched_scratch(a, count)) == SCHED_OK)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
 // Whether children of a few rows are quicker on the general kernels, a warp a row and a thread a node, than with a block each:
 // where there are many more of them than places, and no ranks to find.  us, child_kernel against the pair: initial population of
 // 8000 children of 4 x 3 74 / 25, 16 x 3 97 / 64, 24 x 20 117 / 96, 24 x 41 123 / 107, 16 x 301 132 / 109, 2000 of 8 x 20 28 / 17;
@@ -1560,8 +1574,8 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
   const bool fused = (NN % 8 == 0) && NN <= 512 && aligned && ctx->cap_max <= 2047 && count <= 65535 &&
                      a.J <= (1 << 20);
   ctx->summ_valid = fused && a.summ != nullptr;
-  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535 && !(fused && batched_rows_pay(ctx, a, count)) &&
-      !tiny_children(ctx, a, count))
+  if (!ctx->summ_valid && NN <= 512 && ctx->cap_max <= 2047 && a.J <= 65535 && !tiny_children(ctx, a, count) &&
+      !(fused && batched_rows_pay(ctx, a, count) && have_batched_scratch(ctx, a, count)))
     return launch_children(ctx, a, count, first_cand, gen);
   if (!fused) {
     if (a.mode == ROWS_GENERATION) {
@@ -1576,7 +1590,7 @@ int launch_rows_cols(sched_ctx *ctx, RowsArgs &a, int16_t *pop, int count, uint3
     return launch_cols(ctx, a.key, pop, count, first_cand, gen);
   }
   const int nbatch = (a.J + 255) / 256;
-  int rc = ensure_colscratch(ctx, (size_t)count * nbatch * NN);
+  int rc = ensure_colscratch(ctx, batched_scratch(a, count));
   if (rc != SCHED_OK) return rc;
   Rows2Args aa;
   aa.r = a;

@@ -186,6 +186,40 @@ def test_few_children_of_many_rows(oracle, nodes, J, P, share, routes):
     _three_operators(oracle, nodes, J, P, share, routes.split())
 
 
+def test_few_children_of_many_rows_without_scratch(oracle):
+    """A captured call whose scratch is not there yet: one launch a child instead."""
+    import torch
+    from paper_2008_12260_b200 import api
+
+    nodes, J, P, seed = 256, 4096, 2, 3
+    cl = synth.uniform_cluster(nodes, 4)
+    raw = synth.random_raw_population(P, J, cl, seed=1, density=0.002, v_hi=6)
+    k_cap, active = np.full(J, cl.k_max, np.int32), np.ones(J, np.uint8)
+    stream = torch.cuda.Stream()
+    s = api.Scheduler(node_capacity=cl.node_capacity, num_jobs=J, grid_m=1, grid_s=1, population=P, thr_mutate=1 << 26, seed=seed,
+                      stream=stream.cuda_stream)
+    dj = api.DeviceJobs(_Jobs(k_cap, active), "cuda:0", torch)
+    _, aside = _unaligned(torch, raw, 1)
+    pop = torch.from_numpy(raw).cuda()
+    torch.cuda.synchronize()
+    s.repair_population(dj, aside, round=5, generation=6)   # (rows between two vectors: no scratch)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        s.repair_population(dj, pop, round=5, generation=6)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(pop, aside)
+    got = pop.cpu().numpy()
+    for c in range(P):
+        assert np.array_equal(got[c], oracle.repair(raw[c], cl.node_capacity, k_cap, cl.k_max, cl.n_max, seed, 5, c, 6, active=active)), c
+    s.sync_status()
+    s.set_kernel_timing(True)
+    s.repair_population(dj, pop, round=5, generation=6)
+    assert s.read_kernel_timing()["cols"][1] == 1
+    s.close()
+
+
 # many children of a few rows: a warp a row and a thread a node, unless ranks are wanted
 @pytest.mark.parametrize("nodes,J,P,routes", [(3, 1, 1100, "cols rows cols"), (20, 24, 1100, "cols rows cols"), (301, 16, 1100, "cols rows cols"),
                                               (301, 17, 1100, "rows rows rows"), (20, 25, 1100, "rows rows rows"),
