@@ -117,7 +117,7 @@ struct sched_ctx {
   void *fl_arena;
   int fl_blocks;           // blocks of the launch, 0: rounds run on the other kernels
   int fl_warps, fl_draw_warps;   // of a block: that work on rows, that draw a step ahead
-  bool fl_terms;           // the rows' terms are looked up in shared memory
+  bool fl_terms;           // there is room for the rows' terms in shared memory
   int fl_more;             // occupants its lists hold per node beyond 16
   int fl_generations;      // generations of the last round
   unsigned int fl_wait_limit;   // sched_set_wait_limit

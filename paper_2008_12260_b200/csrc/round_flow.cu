@@ -47,6 +47,11 @@ constexpr int LANES = 8;                        // lanes of a row
 constexpr int STASH = 256;                      // perturbed rows of many whose draws are kept, further ones draw again
 constexpr int SMEM_RECORDS = 256;              // up to this many jobs the child's records are kept in shared memory, too
 constexpr int FLOW_MAX_WARPS = 20;
+// With more generations than this, or with so few jobs and no fewer generations than jobs, a block copies the rows' terms to
+// shared memory where they fit.  The copy takes 0.11 us a job, a generation then up to 0.27 us less: 8 candidates x 200 jobs, none, 10 and
+// 100 generations with the copy 54, 96 and 466 us, without 32, 79 and 470; 148 x 250 63, 113 and 543, 36, 89 and 542; 100 x 48
+// 34, 73 and 419, 30, 67 and 414; but 59 x 18, 30 generations, 122 and 126, 32 x 8, 10 generations, 55.1 and 55.8.
+constexpr int TERMS_FROM = 100, TERMS_JOBS = 40;
 constexpr int MANY_TWO_JOBS = 2048;             // beyond these two blocks an SM take any population
 constexpr int SOME_WARPS = 16;                  // that work on the rows where a block has an SM for itself and more than 256 jobs
 constexpr int FLOW_OCC = 16;                    // occupants of a node that a group of lanes decides
@@ -1553,7 +1558,7 @@ int flow_more(const sched_ctx *ctx) {
 // 1563, 12 + 2 2143, 12 + 4 1373, 14 + 2 2137; SOME_ALONE, 64 x 1100 12 + 4 694, 14 + 6 647, 16 + 2 918, 16 + 4 642, 64 x 2000 821,
 // 759, 1391, 806 (with so many rows the draws are what takes long); FEW, 54 jobs x 600 candidates 6 + 2 in two turns 628, 4 + 2
 // 447, 4 + 1 452, 3 + 1 487; x 888 703, 770, 533, 588; x 1100 753, 827, 902, 675; x 1300 in three, two, two and two turns 1040, 882,
-// 956, 1073.  The terms' table is kept in shared memory where that does not cost a block its place.
+// 956, 1073.  The terms' table finds room in shared memory where that does not cost a block its place.
 FlowShape flow_shape(const sched_ctx *ctx) {
   const sched_config &c = ctx->cfg;
   const int kind = flow_kind(ctx);
@@ -1680,7 +1685,8 @@ int launch_round_flow(sched_ctx *ctx, const sched_jobs *jobs, const int16_t *d_c
   a.generations = generations;
   a.warps = ctx->fl_warps;
   a.more = ctx->fl_more;
-  a.at = flow_smem(ctx, flow_kind(ctx), ctx->fl_warps, ctx->fl_terms, ctx->fl_more);
+  const bool terms = ctx->fl_terms && (generations > TERMS_FROM || (c.num_jobs <= TERMS_JOBS && generations >= c.num_jobs));
+  a.at = flow_smem(ctx, flow_kind(ctx), ctx->fl_warps, terms, ctx->fl_more);
   a.best = d_best; a.best_fitness = d_best_fitness;
   {
     TimedLaunch tl_(ctx, KK_FLOW_BUILD);

@@ -23,6 +23,10 @@ KINDS = [
     (20, 4, 30, 4 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 4 * SMS + 1, 4, 6, 1.0, 0.2), (20, 4, 30, 5 * SMS + 1, 4, 0, 0.7, 0.2),
     (20, 4, 30, 6 * SMS + 1, 4, 6, 1.0, 0.9), (20, 4, 30, 8 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 8 * SMS + 1, 4, 6, 1.0, 0.2),
     (20, 4, 250, 8 * SMS, 3, 0, 1.0, 0.2), (1, 4, 1, 3, 3, 0, 1.0, 1.0),
+    # enough generations for the terms to be copied, and one fewer
+    (6, 4, 41, 20, 100, 2, 1.0, 0.1), (6, 4, 41, 20, 101, 2, 0.9, 0.1), (6, 4, 41, SMS + 5, 101, 0, 1.0, 0.1),
+    (6, 4, 40, 20, 39, 0, 1.0, 0.1), (6, 4, 40, SMS + 5, 40, 2, 0.9, 0.1),
+    (2, 4, 300, 12, 101, 0, 1.0, 0.1), (3, 2, 280, 2 * SMS, 101, 2, 1.0, 0.1),
 ]
 
 
