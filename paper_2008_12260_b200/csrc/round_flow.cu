@@ -15,7 +15,7 @@
 // the records of its parents' rows; only a row with more occupied nodes ("wide") also has contents.
 // Rows of inactive jobs are left out.  One block works on one candidate at a time: a thread per row that is copied as it
 // is; eight lanes per row that is perturbed or that the repair changes, an entry each, so that what is done
-// to a row's nodes is done to all of them at once, four rows a warp.  Warps of their own draw a step ahead.
+// to a row's nodes is done to all of them at once, four rows a warp (a thread per row where there are very many).  Warps of their own draw a step ahead.
 // Bound: the length of a block's chain of steps.  A generation of the testbed (48 jobs x 100 candidates) in cycles,
 // 7.2 k in all: waiting for the four keys 1.4 k (an unloaded L2 trip is 0.3 k; a fence behind a store 0.8 k), parents
 // 0.35 k, perturbed rows 1.9 k, decisions 1.4 k, changed rows 0.85 k, sum and power mean 1.15 k beside the fence
@@ -52,6 +52,10 @@ constexpr int FLOW_MAX_WARPS = 20;
 // 100 generations with the copy 54, 96 and 466 us, without 32, 79 and 470; 148 x 250 63, 113 and 543, 36, 89 and 542; 100 x 48
 // 34, 73 and 419, 30, 67 and 414; but 59 x 18, 30 generations, 122 and 126, 32 x 8, 10 generations, 55.1 and 55.8.
 constexpr int TERMS_FROM = 100, TERMS_JOBS = 40;
+// More perturbed or changed rows a warp than this have a thread each instead of eight lanes, in blocks of many jobs that share their SM:
+// three rounds of four rows take a warp longer than one of 32, and the issue slots are full.  30 generations of 512 candidates x
+// 1024 jobs on 64 nodes, a tenth of the rows perturbed 1329 us with eight lanes, 1124, a fifth 1795, 1332; 832 x 2224, a fifth 6035, 4257.
+constexpr int LISTS_FROM = 12;
 constexpr int MANY_TWO_JOBS = 2048;             // beyond these two blocks an SM take any population
 constexpr int SOME_WARPS = 16;                  // that work on the rows where a block has an SM for itself and more than 256 jobs
 constexpr int FLOW_OCC = 16;                    // occupants of a node that a group of lanes decides
@@ -704,6 +708,168 @@ __device__ __forceinline__ void finish_row(const FlowArgs &a, const FlowView &v,
   settle_row<KIND>(a, v, dst, jc, e, place, row_sum(e != NO_NODE ? entry_gpus(e) : 0), __popc(there), live, false, lane);
 }
 
+// ---- rows, a thread each: a third of the instructions that eight lanes take for a row, and a longer chain ------------
+// Where a block has many such rows for its warps and shares its SM's issue slots with others.
+constexpr int LIST = ENTRIES + 1;       // one more than a record holds: a perturbation may add before the caps take
+
+__device__ __forceinline__ void list_totals(const uint32_t (&e)[LIST], int &K, int &N) {
+  K = 0;
+  N = 0;
+#pragma unroll
+  for (int k = 0; k < LIST; ++k) {
+    const bool on = e[k] != NO_NODE;
+    K += on ? entry_gpus(e[k]) : 0;
+    N += on ? 1 : 0;
+  }
+}
+
+// `gpus` of a node: the entry replaced, put in its place or taken out
+__device__ __forceinline__ void list_set(uint32_t (&e)[LIST], int node, int gpus) {
+  bool found = false;
+  const uint32_t entry = gpus > 0 ? ((uint32_t)node << 16) | (uint32_t)gpus : NO_NODE;
+#pragma unroll
+  for (int k = 0; k < LIST; ++k)
+    if (entry_node(e[k]) == node) {
+      found = true;
+      e[k] = entry;
+    }
+  uint32_t x = found ? NO_NODE : entry;
+#pragma unroll
+  for (int k = 0; k < LIST; ++k) {      // a new entry to its place, then a hole to the end
+    const uint32_t lo = min(e[k], x);
+    x = max(e[k], x);
+    e[k] = lo;
+  }
+#pragma unroll
+  for (int k = 0; k + 1 < LIST; ++k) {
+    const uint32_t lo = min(e[k], e[k + 1]);
+    e[k + 1] = max(e[k], e[k + 1]);
+    e[k] = lo;
+  }
+}
+
+// As settle_row, for a list of up to six entries in order.
+template <int KIND>
+__device__ __forceinline__ void settle_list(const FlowArgs &a, const FlowView &v, int dst, int jc, const uint32_t (&e)[LIST], int K, int N, bool fresh) {
+  const int j = v.act[jc], row = a.classes * (a.k_max + 1);
+  int cls = N >= 2 ? 1 : 0;
+  if (a.rack) {
+    int first = -1;
+#pragma unroll
+    for (int k = 0; k < ENTRIES; ++k)
+      if (e[k] != NO_NODE && sched_index_ok(a.status, entry_node(e[k]) < a.NN, SCHED_CHK_NODE)) {
+        const int r = (int)v.rack[entry_node(e[k])];
+        if (first < 0) first = r;
+        if (r != first) cls = 2;
+      }
+  }
+  if (!sched_index_ok(a.status, K >= 0 && K <= a.k_max && jc < a.J, SCHED_CHK_ENTRY)) return;
+  const uint4 lo = __ldg((const uint4 *)(a.r.same + (size_t)j * REC_WORDS)), hi = __ldg((const uint4 *)(a.r.same + (size_t)j * REC_WORDS) + 1);
+  const float changed = __ldg(a.r.terms + (size_t)j * row + cls * (a.k_max + 1) + K);
+  if (fresh) {
+    v.info[jc] = N >= 2 ? INFO_DIST : 0;
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) {
+      uint32_t x = e[0];
+#pragma unroll
+      for (int z = 1; z < ENTRIES; ++z) x = z == k ? e[z] : x;
+      add_occupant<KIND>(a, v, jc, k, x, N >= 2);
+    }
+  }
+  const bool equal = lo.x == e[0] && lo.y == e[1] && lo.z == e[2] && lo.w == e[3] && hi.x == e[4] && hi.y == e[5];
+  Record r;
+#pragma unroll
+  for (int k = 0; k < ENTRIES; ++k) r.w[k] = e[k];
+  r.w[REC_TERM] = equal ? hi.z : __float_as_uint(changed);
+  r.w[7] = 0u;
+  store_record(rec_row(a, dst + jc), r);
+  v.term[j] = __uint_as_float(r.w[REC_TERM]);
+}
+
+// As perturb_rows, for up to 32 rows.
+template <int KIND>
+__device__ __noinline__ void perturb_lists(const FlowArgs &a, uint32_t memory, Work w, uint32_t round, int set, int x0, int nmut, int lane) {
+  const FlowView v = flow_view(a, memory);
+  const int i = x0 + lane;
+  if (i >= nmut || !sched_index_ok(a.status, i < a.J, SCHED_CHK_LIST)) return;
+  const int m = v.mut[set * a.J + i], jc = m & 0x7FFF;
+  if (!sched_index_ok(a.status, jc < a.J, SCHED_CHK_LIST)) return;
+  const int j = v.act[jc];
+  const Record rec = load_record(rec_row(a, (w.init || (m >> 15) ? w.src[1] : w.src[0]) + (w.init ? j : jc)));
+  uint2 st;
+  if (i < stash_rows(a.J)) st = v.stash[set * stash_rows(a.J) + i];
+  else st = choices_of(a, draw_one(a.key.k0, round, (uint32_t)j, w.c, w.gen, w.init ? SLOT_INIT : SLOT_MUTATE), j);
+  bool slow = rec.w[0] == WIDE;
+  if (!slow) {
+    uint32_t e[LIST];
+#pragma unroll
+    for (int k = 0; k < ENTRIES; ++k) e[k] = rec.w[k];
+    e[ENTRIES] = NO_NODE;
+    int K, N;
+    list_totals(e, K, N);
+    const uint32_t op = st.y & 3u;
+    const int nd = (int)((st.y >> 2) & 0x1FFu), cap_nd = (int)v.cap[nd], k_cap = (int)(st.y >> 16);
+    int ns = -1, vs = 0, v_nd = 0;
+    const int t = N > 0 ? (int)bounded(st.x, (uint32_t)N) : 0;
+#pragma unroll
+    for (int k = 0; k < ENTRIES; ++k) {
+      if (k == t && N > 0) { ns = entry_node(e[k]); vs = entry_gpus(e[k]); }
+      v_nd = entry_node(e[k]) == nd ? entry_gpus(e[k]) : v_nd;
+    }
+    if (op == 0u || (N > 0 && (op == 1u || nd != ns))) {
+      const bool move = op == 2u;
+#pragma unroll 1
+      for (int q = 0; q < (move ? 2 : 1); ++q)
+        list_set(e, op == 1u || q ? ns : nd, q ? 0 : op == 0u ? min(v_nd + 1, cap_nd) : op == 1u ? vs - 1 : min(v_nd + vs, cap_nd));
+      list_totals(e, K, N);
+    }
+    if (K > k_cap || N > a.n_max) {     // replicas above the cap leave from the highest node down, then nodes beyond n_max
+      int excess = K - k_cap;
+#pragma unroll
+      for (int k = LIST - 1; k >= 0; --k) {
+        if (e[k] != NO_NODE && excess > 0) {
+          const int gpus = entry_gpus(e[k]), take = min(gpus, excess);
+          excess -= take;
+          e[k] = take == gpus ? NO_NODE : e[k] - (uint32_t)take;
+        }
+        if (k >= a.n_max) e[k] = NO_NODE;
+      }
+      list_totals(e, K, N);
+    }
+    slow = e[ENTRIES] != NO_NODE;
+    if (!slow) settle_list<KIND>(a, v, w.dst, jc, e, K, N, true);
+  }
+  if (slow) {
+    const int at = atomicAdd(&v.ctl.nslow, 1);
+    if (sched_index_ok(a.status, at < a.J, SCHED_CHK_LIST)) v.wide[a.J - 1 - at] = (uint16_t)m;
+  }
+}
+
+// As finish_row, for up to 32 of the changed rows.
+template <int KIND>
+__device__ __noinline__ void finish_lists(const FlowArgs &a, uint32_t memory, int dst, int i0, int nmod, int lane) {
+  const FlowView v = flow_view(a, memory);
+  if (i0 + lane >= nmod) return;
+  const int jc = v.mod[i0 + lane];
+  if (v.info[jc] & INFO_WIDE) return;
+  const Record rec = load_record(rec_row(a, dst + jc));
+  uint32_t e[LIST];
+#pragma unroll
+  for (int k = 0; k < ENTRIES; ++k) e[k] = entry_gpus(rec.w[k]) == 0 ? NO_NODE : rec.w[k];
+  e[ENTRIES] = NO_NODE;
+#pragma unroll
+  for (int n = ENTRIES - 1; n > 0; --n)
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const uint32_t lo = min(e[k], e[k + 1]);
+      e[k + 1] = max(e[k], e[k + 1]);
+      e[k] = lo;
+    }
+  int K, N;
+  list_totals(e, K, N);
+  settle_list<KIND>(a, v, dst, jc, e, K, N, false);
+}
+
 // A wide row that decisions changed, by a warp.
 template <int KIND>
 __device__ __noinline__ void finish_wide(const FlowArgs &a, uint32_t memory, int dst, int jc, int warp, int lane) {
@@ -1180,7 +1346,12 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
     };
     const int nmut = v.ctl.nmut[set];
 #pragma unroll 1
-    for (int x = (W - 1 - warp) * 4; x < nmut; x += W * 4) perturb_rows<KIND>(a, v, w, round, set, x, nmut, warp, lane);
+    for (int x = (W - 1 - warp) * 4; x < nmut && !(!few(KIND) && nmut > LISTS_FROM * W); x += W * 4)
+      perturb_rows<KIND>(a, v, w, round, set, x, nmut, warp, lane);
+    if constexpr (!few(KIND))
+      if (nmut > LISTS_FROM * W)
+#pragma unroll 1
+        for (int x = (W - 1 - warp) * 32; x < nmut; x += W * 32) perturb_lists<KIND>(a, memory, w, round, set, x, nmut, lane);
     constexpr int RB = shape_of(KIND) == SOME_ALONE || !few(KIND) ? 2 : 1;       // rows of a thread whose loads travel together
 #pragma unroll 1
     for (int jc0 = tid; jc0 < JA; jc0 += RB * threads) {
@@ -1270,10 +1441,14 @@ __global__ void __launch_bounds__(kind_threads(KIND), kind_blocks(KIND)) flow_ke
     // ---- rows the decisions change, then columns that have to be walked --------------------------------
     const int nmod = v.ctl.nmod, walk = v.ctl.walk;
 #pragma unroll 1
-    for (int i0 = warp * 4; i0 < nmod; i0 += W * 4) {
+    for (int i0 = warp * 4; i0 < nmod && !(!few(KIND) && nmod > LISTS_FROM * W); i0 += W * 4) {
       const int jc = v.mod[min(i0 + g, nmod - 1)];
       finish_row<KIND>(a, v, w.dst, jc, i0 + g < nmod && !(v.info[jc] & INFO_WIDE), warp, lane);
     }
+    if constexpr (!few(KIND))
+      if (nmod > LISTS_FROM * W)
+#pragma unroll 1
+        for (int i0 = warp * 32; i0 < nmod; i0 += W * 32) finish_lists<KIND>(a, memory, w.dst, i0, nmod, lane);
     if (any_wide) {                           // wide rows among them
       bar(BAR_ROWS, threads);                 // (one may turn into a record here: not to be taken for one above)
 #pragma unroll 1

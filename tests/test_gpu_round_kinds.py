@@ -19,6 +19,8 @@ KINDS = [
     (12, 8, 1206, 2 * SMS, 2, 0, 1.0, 0.1), (12, 8, 1206, 2 * SMS + 1, 2, 0, 1.0, 0.1), (6, 4, 8192, 7, 2, 0, 1.0, 0.1),
     (12, 8, 700, 2 * SMS, 3, 0, 1.0, 0.1), (12, 8, 300, 2 * SMS + 1, 3, 0, 1.0, 0.1), (20, 4, 64, 2 * SMS, 4, 0, 1.0, 0.2),
     (20, 4, 64, 2 * SMS + 1, 4, 0, 0.5, 0.2), (20, 4, 64, 3 * SMS + 1, 4, 5, 1.0, 0.2), (64, 4, 900, 200, 3, 0, 1.0, 0.9),
+    # a thread per changed row: more perturbed rows than draws are kept of, racks, wide rows
+    (64, 2, 900, 2 * SMS + 1, 3, 16, 0.8, 0.9), (30, 4, 600, 2 * SMS + 1, 3, 0, 1.0, 0.14),
     # smaller blocks, and more candidates than blocks
     (20, 4, 30, 4 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 4 * SMS + 1, 4, 6, 1.0, 0.2), (20, 4, 30, 5 * SMS + 1, 4, 0, 0.7, 0.2),
     (20, 4, 30, 6 * SMS + 1, 4, 6, 1.0, 0.9), (20, 4, 30, 8 * SMS, 4, 0, 1.0, 0.2), (20, 4, 30, 8 * SMS + 1, 4, 6, 1.0, 0.2),
